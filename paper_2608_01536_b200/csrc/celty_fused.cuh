@@ -30,86 +30,6 @@
 // waits are bounded: when one runs out the kernel sets kStatusTimeout in the status word and carries on to a clean
 // exit.
 
-// Shared-memory carve-up of the fused kernel, computed by ONE function for the kernel and for the host
-// (which sizes the launch with .total), so that the two can never disagree.
-struct FusedSmem {
-    size_t acc, ring, bars, flag, items, imeta, zero, keep, wrel, blk, blkw, total;
-};
-
-__host__ __device__ inline FusedSmem fused_smem_layout(int R, int K, int teams, int D, int slot_bytes, int cap)
-{
-    FusedSmem l;
-    uint32_t off = 0;
-    l.acc = off;       off += (uint32_t)teams * (R + kTileSlack) * 32 * 4;   // FP32 accumulators, one slab per team
-    l.ring = off;      off += (uint32_t)teams * D * slot_bytes;              // bulk-copy ring slots (multiples of 128 bytes)
-    l.bars = off;      off += (uint32_t)teams * D * 8 + 8;                   // one "full" mbarrier per slot, one for the offset window
-    l.flag = off;      off += (uint32_t)teams * 4;                           // per team: a wait of one of its warps ran out
-    off = (off + 15) / 16 * 16;
-    l.items = off;     off += (uint32_t)teams * cap * 8;                     // {column, x bits} per looked-up item
-    l.imeta = off;     off += (uint32_t)teams * cap * 8;                     // {offset/16, bytes} of its sub-block
-    l.zero = off;      off += 16;                                          // the all-zero group that idle lanes fetch
-    l.keep = off;      off += ((uint32_t)((K + 31) / 32) * 4 + 15) / 16 * 16;   // one keep bit per activation
-    l.wrel = off;      off += ((uint32_t)((K + 31) / 32) * 4 + 15) / 16 * 16;   // survivors before each keep word, in its block of 32
-    l.blk = off;       off += ((uint32_t)((K + 1023) / 1024) * 4 + 15) / 16 * 16; // survivors in each block of 32 keep words
-    l.blkw = off;      off += 16 * (((uint32_t)((K + 1023) / 1024) * 4 + 15) / 16 * 16);   // per warp: survivors before each block
-    l.total = off;
-    return l;
-}
-
-struct FusedParams {
-    const uint32_t *meta;      // [K*S + 1] offset/16 of sub-block (j, s) in the stream
-    const uint8_t *stream;
-    const uint16_t *x;         // K FP16
-    float tau;
-    float *y;                  // M
-    int32_t *idx;              // global compacted list (API output)
-    uint16_t *val;
-    int32_t *count;
-    uint32_t *status;
-    uint32_t *tickets;         // [0] y cleared / partial stored, [1] adds done (work after the merge) / departed
-    float *partials;           // gridDim.x vectors of Sc * R * 32 floats (accumulator layout)
-    int M, K, R, S, C;         // rows, columns, local rows per tile, slabs, chunk of the row map (tile_row)
-    int G, Sc, P, D;           // teams per slab, slabs per block, row parts, ring depth
-    int cl;                    // thread blocks per cluster (1, 2 or 4); blocks of a cluster share a row part
-    int pp;                    // 1: two warps per team that take turns at the team's accumulator (see the kernel)
-    // mix >= 2 (bulk reduce-add merge without clusters): the gridDim mod P blocks that are left when every row part
-    // has floor(gridDim / P) blocks are not given to the first parts (which would then finish early, one slice
-    // ahead of the others); each of them serves mix = P / (gridDim mod P) consecutive parts instead, with G / mix
-    // teams per slab, so that every part is shared by the same number of teams.  units_inv then holds
-    // floor(2^32 / (floor(gridDim / P) * G + G / mix)).
-    int mix;
-    int slot_bytes;            // ring slot size, multiple of 128
-    int cap;                   // columns a team looks up per batch
-    int win_cols;              // columns of the offset table a block copies into shared memory at its start
-    FusedSmem lay;             // the block's shared memory, worked out once on the host (fused_smem_layout)
-    int clear_rows, clear_extra;   // M / gridDim.x and M mod gridDim.x: block b clears clear_rows (+ 1 if b < clear_extra) rows of y
-    // teams that share the survivor list of a row part: units = (column slices of the part) * G;
-    // units_inv = floor(2^32 / units) for parts with gridDim / cl / P clusters, units_inv_long for those with
-    // one cluster more
-    uint32_t units_inv, units_inv_long;
-    int merge;                 // 0: partial vectors + ordered final sum; 1: bulk reduce-add of row segments into y
-    uint32_t spin_limit;       // polls a bounded wait makes before it gives up
-    // a1 done by the producer of the activations: when list_count is not null the surviving columns and their
-    // values come from this list (any order, every column at most once) and x and tau are not looked at
-    const int32_t *list_idx;
-    const uint16_t *list_val;
-    const int32_t *list_count;
-    // The activations are not given but made on the fly from the FP32 result of a stacked [gate; up] product
-    // (2K values, gate first): x_j = SiLU(g_j) * u_j rounded to FP16, for the down projection.  h_out (may be
-    // null) receives the K FP16 values.
-    const float *swiglu_in;
-    uint16_t *h_out;
-    // Work on y after the merge (bulk reduce-add merge only): 0 none; 1 an FP16 copy of y; 2 y holds a stacked
-    // [gate; up] product of 2I rows: h_i = SiLU(y_i) * y_{I+i} rounded to FP16, stored, and the (i, h_i) with
-    // |h_i| > ep_tau appended to a list that the next product takes as its survivors
-    int ep_kind;
-    uint16_t *ep_out;
-    float ep_tau;
-    int32_t *ep_idx;
-    uint16_t *ep_val;
-    int32_t *ep_count;
-};
-
 constexpr uint32_t kSpinLimit = 1u << 21;   // default for FusedParams::spin_limit
 
 __device__ __forceinline__ uint32_t smem_u32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -415,12 +335,17 @@ __device__ __noinline__ void fused_epilogue(const EpilogueArgs p)
 // taken branch over code that is not run costs a trip to L2 (250 cycles and more, measured with stand-alone loops:
 // a cliff at about 24 KB of code touched per launch); what falls through in sequence is prefetched and costs
 // nothing.
-template <bool kExtras, int kRegRows, int kLean = 0>
+// kBatch: one launch for several activation vectors, the blocks dealt out among them (FusedParams::ldx).
+template <bool kExtras, int kRegRows, int kLean = 0, bool kBatch = false>
 __global__ void __launch_bounds__(kRegRows > 0 ? 256 : 512, 1) k_spmspv_fused(const FusedParams p)
 {
     const int pp = kLean ? (kLean == 2 ? 1 : 0) : p.pp;
     const int merge = kLean ? 1 : p.merge;
     const int cl = kLean ? 1 : p.cl;
+    const uint16_t *const x = kBatch ? p.x + (size_t)blockIdx.y * p.ldx : p.x;
+    float *const y = kBatch ? p.y + (size_t)blockIdx.y * p.ldy : p.y;
+    uint32_t *const tickets = kBatch ? p.tickets + blockIdx.y : p.tickets;
+    const bool lists = !kBatch || blockIdx.y + 1 == gridDim.y;    // the survivor list reported is the last vector's
     extern __shared__ __align__(128) uint8_t smem[];
     const int tid = threadIdx.x, lane = tid & 31, nthreads = blockDim.x, nwarps = nthreads >> 5;
     // the warp index through a shuffle: the compiler then knows that it (and every team, slab and loop bound
@@ -524,14 +449,14 @@ __global__ void __launch_bounds__(kRegRows > 0 ? 256 : 512, 1) k_spmspv_fused(co
         const int b = (int)blockIdx.x;
         const int r0 = b * p.clear_rows + min(b, p.clear_extra), r1 = r0 + p.clear_rows + (b < p.clear_extra ? 1 : 0);
 #pragma unroll 1
-        for (int i = r0 + lane; i < r1; i += 32) p.y[i] = 0.f;
+        for (int i = r0 + lane; i < r1; i += 32) y[i] = 0.f;
         if (kExtras && p.ep_kind == 2 && blockIdx.x == 0 && lane == 0) *p.ep_count = 0;   // appended to after the merge
         __syncwarp();
         if (lane == 0) {
             __threadfence();
             // The ticket counts modulo 2 * gridDim.x, so it never has to be reset: calls alternate between
             // waiting for the lower and for the upper half.
-            y_ticket = atomicInc(&p.tickets[0], 2u * gridDim.x - 1u);
+            y_ticket = atomicInc(&tickets[0], 2u * gridDim.x - 1u);
         }
     }
     // ---- a1: threshold all of x.  A thread takes 32 activations (four 128-bit loads) and makes one keep word,
@@ -584,10 +509,10 @@ __global__ void __launch_bounds__(kRegRows > 0 ? 256 : 512, 1) k_spmspv_fused(co
                             }
                         }
                     } else if (8 * q + 8 <= p.K) {
-                        const uint4 v = __ldg(reinterpret_cast<const uint4 *>(p.x + 8 * q));
+                        const uint4 v = __ldg(reinterpret_cast<const uint4 *>(x + 8 * q));
                         h[c][0] = v.x; h[c][1] = v.y; h[c][2] = v.z; h[c][3] = v.w;
                     } else if (__builtin_expect(q < ngroups, 0)) {
-                        const uint4 v = ragged_group(p.x, p.K, q);     // the one group that K cuts short
+                        const uint4 v = ragged_group(x, p.K, q);     // the one group that K cuts short
                         h[c][0] = v.x; h[c][1] = v.y; h[c][2] = v.z; h[c][3] = v.w;
                     }
                 }
@@ -646,7 +571,7 @@ __global__ void __launch_bounds__(kRegRows > 0 ? 256 : 512, 1) k_spmspv_fused(co
         }
         __syncwarp();
         n_surv = carry;
-        if (blockIdx.x == 0 && warp == 0 && lane == 0) *p.count = carry;
+        if (lists && blockIdx.x == 0 && warp == 0 && lane == 0) *p.count = carry;
     }
 
     if (streams) {
@@ -727,10 +652,10 @@ __global__ void __launch_bounds__(kRegRows > 0 ? 256 : 512, 1) k_spmspv_fused(co
                 }
                 j = 32 * w + pos;
                 if (kExtras && p.swiglu_in) xb = (uint16_t)swiglu_half_bits(__ldg(p.swiglu_in + j), __ldg(p.swiglu_in + p.K + j));
-                else xb = __ldg(p.x + j);                            // x went through L1 in the thresholding pass
+                else xb = __ldg(x + j);                            // x went through L1 in the thresholding pass
                 }
                 items[i] = make_int2(j, (int)xb);
-                if (!from_list && part == 0 && sl == 0) {
+                if (!from_list && lists && part == 0 && sl == 0) {
                     p.idx[r] = j;
                     p.val[r] = xb;
                 }
@@ -879,7 +804,7 @@ __global__ void __launch_bounds__(kRegRows > 0 ? 256 : 512, 1) k_spmspv_fused(co
             const bool low_half = y_ticket < gridDim.x;
             bool ok = false;
             for (uint32_t it = 0; it < p.spin_limit; ++it) {
-                const uint32_t cur = ld_relaxed_u32(&p.tickets[0]);
+                const uint32_t cur = ld_relaxed_u32(&tickets[0]);
                 if (low_half ? (cur >= gridDim.x) : (cur < gridDim.x)) { ok = true; break; }
                 __nanosleep(64);
             }
@@ -943,19 +868,19 @@ __global__ void __launch_bounds__(kRegRows > 0 ? 256 : 512, 1) k_spmspv_fused(co
                 const uint32_t bytes = ((uint32_t)nrows * 4u) & ~15u;
                 const float *src = acc + (size_t)fsl * slab_words + (size_t)i0 * 32;
                 if (bytes)
-                    asm volatile("cp.reduce.async.bulk.global.shared::cta.bulk_group.add.f32 [%0], [%1], %2;" ::"l"(p.y + row0),
+                    asm volatile("cp.reduce.async.bulk.global.shared::cta.bulk_group.add.f32 [%0], [%1], %2;" ::"l"(y + row0),
                                  "r"(smem_u32(src)), "r"(bytes)
                                  : "memory");
 #pragma unroll 1
                 for (int i = (int)(bytes >> 2); i < nrows; ++i)
-                    if (src[i] != 0.f) atomicAdd(p.y + row0 + i, src[i]);
+                    if (src[i] != 0.f) atomicAdd(y + row0 + i, src[i]);
             }
             asm volatile("cp.async.bulk.commit_group;" ::: "memory");
             asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");   // shared memory may go once it has been read
         }
         if (cl > 1) cluster_sync();                               // no block leaves while a peer may still read it
         if (!kExtras || p.ep_kind == 0) return;
-        fused_epilogue(EpilogueArgs{p.y, p.tickets, p.status, p.spin_limit, p.M, p.ep_kind, p.ep_out, p.ep_tau, p.ep_idx,
+        fused_epilogue(EpilogueArgs{y, tickets, p.status, p.spin_limit, p.M, p.ep_kind, p.ep_out, p.ep_tau, p.ep_idx,
                                     p.ep_val, p.ep_count});
         return;
     }
@@ -980,10 +905,10 @@ __global__ void __launch_bounds__(kRegRows > 0 ? 256 : 512, 1) k_spmspv_fused(co
         __syncthreads();
         if (tid == 0) {
             __threadfence();                                          // the block's stores, ordered by the barrier above
-            atomicAdd(&p.tickets[0], 1u);
+            atomicAdd(&tickets[0], 1u);
             bool ok = false;
             for (uint32_t it = 0; it < p.spin_limit; ++it) {
-                if (ld_acquire_u32(&p.tickets[0]) >= gridDim.x) { ok = true; break; }
+                if (ld_acquire_u32(&tickets[0]) >= gridDim.x) { ok = true; break; }
                 __nanosleep(32);
             }
             if (__builtin_expect(!ok, 0)) atomicOr(p.status, kStatusTimeout);
@@ -1030,7 +955,7 @@ __global__ void __launch_bounds__(kRegRows > 0 ? 256 : 512, 1) k_spmspv_fused(co
                         const int fsl = w2 / tile_words, rem = w2 - fsl * tile_words;
                         const int sfull = part * p.Sc + fsl;
                         const int64_t row = tile_row(p.S, p.C, sfull, rem & 31, rem >> 5);
-                        if (sfull < p.S && row < p.M) p.y[row] = total;
+                        if (sfull < p.S && row < p.M) y[row] = total;
                     }
                 }
                 __syncthreads();
@@ -1039,20 +964,10 @@ __global__ void __launch_bounds__(kRegRows > 0 ? 256 : 512, 1) k_spmspv_fused(co
     }
     __syncthreads();
     if (tid == 0) {
-        const uint32_t t = atomicAdd(&p.tickets[1], 1u);
+        const uint32_t t = atomicAdd(&tickets[1], 1u);
         if (t == gridDim.x - 1) {                                  // last one out resets both tickets
-            atomicExch(&p.tickets[0], 0u);
-            atomicExch(&p.tickets[1], 0u);
+            atomicExch(&tickets[0], 0u);
+            atomicExch(&tickets[1], 0u);
         }
     }
-}
-
-struct FusedPlan {
-    int G, Sc, P, D, cl, pp, mix, slot_bytes, cap, threads, grid, merge;
-    size_t smem;
-};
-
-inline size_t fused_smem_bytes(int R, int K, int G, int Sc, int D, int slot_bytes, int cap)
-{
-    return fused_smem_layout(R, K, G * Sc, D, slot_bytes, cap).total;
 }

@@ -285,6 +285,7 @@ extern "C" int celty_clone(const celty_matrix *m, celty_matrix **out)
         copy->d_ws = nullptr;
         copy->last_grid = 0;
         copy->last_merge = -1;
+        for (int32_t &g : copy->last_batch_grid) g = 0;
         *out = copy.release();
         return CELTY_OK;
     } catch (const std::bad_alloc &) {

@@ -68,11 +68,119 @@ inline WorkspaceLayout workspace_layout(int64_t K, int64_t T, int64_t part_words
     return w;
 }
 
+// Shared-memory carve-up of the fused kernel, computed by ONE function for the kernel and for the host
+// (which sizes the launch with .total), so that the two can never disagree.
+struct FusedSmem {
+    size_t acc, ring, bars, flag, items, imeta, zero, keep, wrel, blk, blkw, total;
+};
+
+CELTY_HD inline FusedSmem fused_smem_layout(int R, int K, int teams, int D, int slot_bytes, int cap)
+{
+    FusedSmem l;
+    uint32_t off = 0;
+    l.acc = off;       off += (uint32_t)teams * (R + kTileSlack) * 32 * 4;   // FP32 accumulators, one slab per team
+    l.ring = off;      off += (uint32_t)teams * D * slot_bytes;              // bulk-copy ring slots (multiples of 128 bytes)
+    l.bars = off;      off += (uint32_t)teams * D * 8 + 8;                   // one "full" mbarrier per slot, one for the offset window
+    l.flag = off;      off += (uint32_t)teams * 4;                           // per team: a wait of one of its warps ran out
+    off = (off + 15) / 16 * 16;
+    l.items = off;     off += (uint32_t)teams * cap * 8;                     // {column, x bits} per looked-up item
+    l.imeta = off;     off += (uint32_t)teams * cap * 8;                     // {offset/16, bytes} of its sub-block
+    l.zero = off;      off += 16;                                          // the all-zero group that idle lanes fetch
+    l.keep = off;      off += ((uint32_t)((K + 31) / 32) * 4 + 15) / 16 * 16;   // one keep bit per activation
+    l.wrel = off;      off += ((uint32_t)((K + 31) / 32) * 4 + 15) / 16 * 16;   // survivors before each keep word, in its block of 32
+    l.blk = off;       off += ((uint32_t)((K + 1023) / 1024) * 4 + 15) / 16 * 16; // survivors in each block of 32 keep words
+    l.blkw = off;      off += 16 * (((uint32_t)((K + 1023) / 1024) * 4 + 15) / 16 * 16);   // per warp: survivors before each block
+    l.total = off;
+    return l;
+}
+
+struct FusedParams {
+    const uint32_t *meta;      // [K*S + 1] offset/16 of sub-block (j, s) in the stream
+    const uint8_t *stream;
+    const uint16_t *x;         // K FP16
+    float tau;
+    float *y;                  // M
+    int32_t *idx;              // global compacted list (API output)
+    uint16_t *val;
+    int32_t *count;
+    uint32_t *status;
+    uint32_t *tickets;         // [0] y cleared / partial stored, [1] adds done (work after the merge) / departed
+    float *partials;           // gridDim.x vectors of Sc * R * 32 floats (accumulator layout)
+    int M, K, R, S, C;         // rows, columns, local rows per tile, slabs, chunk of the row map (tile_row)
+    int G, Sc, P, D;           // teams per slab, slabs per block, row parts, ring depth
+    int cl;                    // thread blocks per cluster (1, 2 or 4); blocks of a cluster share a row part
+    int pp;                    // 1: two warps per team that take turns at the team's accumulator (see the kernel)
+    // mix >= 2 (bulk reduce-add merge without clusters): the gridDim mod P blocks that are left when every row part
+    // has floor(gridDim / P) blocks are not given to the first parts (which would then finish early, one slice
+    // ahead of the others); each of them serves mix = P / (gridDim mod P) consecutive parts instead, with G / mix
+    // teams per slab, so that every part is shared by the same number of teams.  units_inv then holds
+    // floor(2^32 / (floor(gridDim / P) * G + G / mix)).
+    int mix;
+    int slot_bytes;            // ring slot size, multiple of 128
+    int cap;                   // columns a team looks up per batch
+    int win_cols;              // columns of the offset table a block copies into shared memory at its start
+    FusedSmem lay;             // the block's shared memory, worked out once on the host (fused_smem_layout)
+    int clear_rows, clear_extra;   // M / gridDim.x and M mod gridDim.x: block b clears clear_rows (+ 1 if b < clear_extra) rows of y
+    // teams that share the survivor list of a row part: units = (column slices of the part) * G;
+    // units_inv = floor(2^32 / units) for parts with gridDim / cl / P clusters, units_inv_long for those with
+    // one cluster more
+    uint32_t units_inv, units_inv_long;
+    int merge;                 // 0: partial vectors + ordered final sum; 1: bulk reduce-add of row segments into y
+    // kBatch: gridDim.y vectors against the same matrix, gridDim.x blocks each (all of them resident at once);
+    // vector v = blockIdx.y takes x + v * ldx, y + v * ldy and ticket v
+    int64_t ldx, ldy;
+    uint32_t spin_limit;       // polls a bounded wait makes before it gives up
+    // a1 done by the producer of the activations: when list_count is not null the surviving columns and their
+    // values come from this list (any order, every column at most once) and x and tau are not looked at
+    const int32_t *list_idx;
+    const uint16_t *list_val;
+    const int32_t *list_count;
+    // The activations are not given but made on the fly from the FP32 result of a stacked [gate; up] product
+    // (2K values, gate first): x_j = SiLU(g_j) * u_j rounded to FP16, for the down projection.  h_out (may be
+    // null) receives the K FP16 values.
+    const float *swiglu_in;
+    uint16_t *h_out;
+    // Work on y after the merge (bulk reduce-add merge only): 0 none; 1 an FP16 copy of y; 2 y holds a stacked
+    // [gate; up] product of 2I rows: h_i = SiLU(y_i) * y_{I+i} rounded to FP16, stored, and the (i, h_i) with
+    // |h_i| > ep_tau appended to a list that the next product takes as its survivors
+    int ep_kind;
+    uint16_t *ep_out;
+    float ep_tau;
+    int32_t *ep_idx;
+    uint16_t *ep_val;
+    int32_t *ep_count;
+};
+
+// Shape of a fused launch (plan_fused).
+struct FusedPlan {
+    int G, Sc, P, D, cl, pp, mix, slot_bytes, cap, threads, grid, merge;
+    int lean;                  // 0: every option compiled in; 1 / 2: the builds for the default launch (without / with warp pairs)
+    size_t smem;
+};
+
+inline size_t fused_smem_bytes(int R, int K, int G, int Sc, int D, int slot_bytes, int cap)
+{
+    return fused_smem_layout(R, K, G * Sc, D, slot_bytes, cap).total;
+}
+
+// Launch choices of a handle (celty_set_launch and its neighbours); a default-constructed one is the library's.
+struct LaunchKnobs {
+    int32_t grid = 0, variant = 0, groups = 0, depth = 0, cluster = 0;
+    int32_t pairs = -1;                       // fused kernel, two warps per team that take turns at its accumulator:
+                                              // -1 = library's choice, 0 = never, 1 = always
+    int32_t reg_rows = 0;                     // register-accumulation study: local rows per lane summed in registers
+    uint32_t spin_limit = 0;                  // bounded waits inside the kernels: 0 = the library's limit
+    int32_t mix = -1;       // fused kernel, left-over blocks shared between row parts: 0 never, 1 wherever it is even, -1 where it pays
+    int32_t lean = -1;      // fused kernel: 0 = always the build with every option compiled in
+    int32_t no_overlap = 0; // fused kernel: 1 = plain launch (no programmatic dependent launch)
+    int32_t merge = -1;     // fused kernel: -1 = library's choice, 0 = ordered two-stage sum, 1 = bulk reduce-add
+};
+
 }  // namespace celty
 
 // The handle.  Host side: logical block pointers and the packed image exactly as it is copied to
 // the device.  Device side: caller-owned buffers recorded by celty_bind_device.
-struct celty_matrix {
+struct celty_matrix : celty::LaunchKnobs {
     int64_t M = 0, K = 0;
     int32_t layout = 0;
     int32_t R = 0;          // local rows per tile (LANE_TILE) or M (COLUMN)
@@ -95,14 +203,6 @@ struct celty_matrix {
     uint8_t *d_image = nullptr;
     uint8_t *d_ws = nullptr;
     celty::WorkspaceLayout ws{};
-    int32_t grid = 0, variant = 0, groups = 0, depth = 0, cluster = 0;
-    int32_t pairs = -1;                       // fused kernel, two warps per team that take turns at its accumulator:
-                                              // -1 = library's choice, 0 = never, 1 = always
-    int32_t reg_rows = 0;                     // register-accumulation study: local rows per lane summed in registers
-    uint32_t spin_limit = 0;                  // bounded waits inside the kernels: 0 = the library's limit
     int32_t last_grid = 0, last_merge = -1;   // what the tickets in the workspace were last used with
-    int32_t mix = -1;       // fused kernel, left-over blocks shared between row parts: 0 never, 1 wherever it is even, -1 where it pays
-    int32_t lean = -1;      // fused kernel: 0 = always the build with every option compiled in
-    int32_t no_overlap = 0; // fused kernel: 1 = plain launch (no programmatic dependent launch)
-    int32_t merge = -1;     // fused kernel: -1 = library's choice, 0 = ordered two-stage sum, 1 = bulk reduce-add
+    int32_t last_batch_grid[9] = {};          // the same for the tickets of launches that serve 2 .. 8 vectors
 };

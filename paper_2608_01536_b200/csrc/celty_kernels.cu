@@ -488,7 +488,7 @@ __global__ void k_decode_lane(const uint32_t *__restrict__ meta, const uint8_t *
 // asked for), so that steady-state calls make no attribute calls.  The attribute belongs to the kernel,
 // so every entry point that launches a kernel shares that kernel's cache (g_granted_*): two caches for
 // one kernel could disagree about what the runtime currently allows.
-int g_granted_fused[64], g_granted_lean[2][64], g_granted_fused_extras[64], g_granted_lean_extras[2][64], g_granted_column[64], g_granted_lane[64], g_granted_reg[4][64];
+int g_granted_fused[64], g_granted_lean[2][64], g_granted_fused_extras[64], g_granted_lean_extras[2][64], g_granted_batch[2][64], g_granted_column[64], g_granted_lane[64], g_granted_reg[4][64];
 
 template <typename Kernel>
 int ensure_smem(Kernel kernel, size_t bytes, int *granted /* [64], per device */)
@@ -513,8 +513,9 @@ int launch_compact(const void *x, int64_t K, float tau, int32_t *idx, uint16_t *
 }
 
 // Shape of the fused launch: P row parts of Sc slabs, G teams per slab (teams = G * Sc warps, one accumulator
-// slab and one ring of D slots each), clusters of cl thread blocks that add their accumulators on chip.
-int plan_fused(const celty_matrix *m, const DeviceInfo &di, FusedPlan *out)
+// slab and one ring of D slots each), clusters of cl thread blocks that add their accumulators on chip.  The launch
+// serves `vectors` activation vectors, each with an equal share of the device's blocks.
+int plan_fused(const celty_matrix *m, const LaunchKnobs &knobs, const DeviceInfo &di, int vectors, FusedPlan *out)
 {
     FusedPlan pl{};
     pl.P = m->P;
@@ -522,12 +523,12 @@ int plan_fused(const celty_matrix *m, const DeviceInfo &di, FusedPlan *out)
     if (pl.Sc > 16) return CELTY_EINVAL;      // one warp per team, 16 warps per block
     pl.slot_bytes = (int)round_up((size_t)m->max_unit16 * 16, 128);
     pl.cap = 64;
-    const int reg_rows = m->reg_rows;          // register-accumulation study: 256 threads, eight teams at most
+    const int reg_rows = knobs.reg_rows;          // register-accumulation study: 256 threads, eight teams at most
     const size_t budget = (size_t)di.max_smem_optin;
-    int blocks = std::min(di.sms, kMaxBlocks);  // every block must be resident: they wait for one another's tickets
-    if (m->grid > 0) blocks = std::min(blocks, (int)m->grid);
+    int blocks = std::min(di.sms / vectors, kMaxBlocks);  // every block must be resident: they wait for one another's tickets
+    if (knobs.grid > 0) blocks = std::min(blocks, (int)knobs.grid);
     pl.grid = std::max(blocks, pl.P);           // any number of blocks >= P: parts may differ by one column slice
-    if (pl.grid > di.sms) return CELTY_EINVAL;
+    if (pl.grid * vectors > di.sms) return CELTY_EINVAL;
     // Teams first (each needs its own accumulator), then as many ring slots as still fit (at least two, to
     // keep a copy in flight).  With warp pairs (two warps take turns at a team's accumulator, each with ring slots
     // of its own) there are eight teams at most and an even number of slots.
@@ -542,10 +543,10 @@ int plan_fused(const celty_matrix *m, const DeviceInfo &di, FusedPlan *out)
         // at 88 rows per tile, 110 columns to a block: 12.7 us with 10 teams, 12.3 with 8 pairs).
         const int most = (reg_rows > 0 || pairs || cols_per_block < 128) ? 8 : 16;
         const int g_cap = (int)std::max<int64_t>(1, std::min<int64_t>(most / pl.Sc, cols_per_block));
-        const int g_max = std::max(1, std::min(g_cap, m->groups > 0 ? m->groups : g_cap));
+        const int g_max = std::max(1, std::min(g_cap, knobs.groups > 0 ? knobs.groups : g_cap));
         // two ring slots per team unless asked otherwise: deeper rings measured no faster anywhere, and slower where
         // they only add set-up (4096 x 4096 at 64 rows per tile, eight teams: 8.5 us with two slots, 8.7 with four)
-        int d_min = m->depth > 0 ? m->depth : 2, d_max = m->depth > 0 ? m->depth : 2;
+        int d_min = knobs.depth > 0 ? knobs.depth : 2, d_max = knobs.depth > 0 ? knobs.depth : 2;
         if (pairs) {
             d_min = std::max(2, d_min + (d_min & 1));
             d_max = std::max(d_min, d_max & ~1);
@@ -566,15 +567,15 @@ int plan_fused(const celty_matrix *m, const DeviceInfo &di, FusedPlan *out)
     // 11008 x 4096 and 13824 x 5120, -1 % at 5120 x 5120, -5 % at 4096 x 4096; and they must not cost teams (5120 x 13824
     // runs 11 teams of one warp faster than 8 pairs).  The number of survivors is not known here, so the rule goes
     // by the columns: a dozen or more per team, and no more than eight teams to begin with.
-    if (reg_rows == 0 && m->pairs != 0 && pl.G > 0 && pl.Sc <= 8) {             // a pair is warps t and t + 8
+    if (reg_rows == 0 && knobs.pairs != 0 && pl.G > 0 && pl.Sc <= 8) {             // a pair is warps t and t + 8
         const int teams_per_part = std::max(1, pl.grid / pl.P) * pl.G;
-        if (m->pairs > 0 || (pl.G * pl.Sc <= 8 && m->K / teams_per_part >= 12)) {
+        if (knobs.pairs > 0 || (pl.G * pl.Sc <= 8 && m->K / teams_per_part >= 12)) {
             const FusedPlan keep = pl;
             fit(1);
             if (pl.G == 0) pl = keep;
         }
     }
-    if (pl.G == 0 && m->depth == 0 && fused_smem_bytes(m->R, (int)m->K, 1, pl.Sc, 1, pl.slot_bytes, pl.cap) <= budget) {
+    if (pl.G == 0 && knobs.depth == 0 && fused_smem_bytes(m->R, (int)m->K, 1, pl.Sc, 1, pl.slot_bytes, pl.cap) <= budget) {
         pl.G = 1;
         pl.D = 1;
         pl.pp = 0;
@@ -582,11 +583,12 @@ int plan_fused(const celty_matrix *m, const DeviceInfo &di, FusedPlan *out)
     if (pl.G == 0) return CELTY_EINVAL;
     pl.threads = reg_rows > 0 ? 256 : 512;
     pl.smem = fused_smem_bytes(m->R, (int)m->K, pl.G, pl.Sc, pl.D, pl.slot_bytes, pl.cap);
-    pl.merge = (m->merge >= 0 ? m->merge : 1);
+    pl.merge = (knobs.merge >= 0 ? knobs.merge : 1);
     // Clusters (bulk reduce-add merge only, on request): as long as the grid is made of whole clusters, every row
     // part gets at least one, and the device can hold them all at once.
-    pl.cl = pl.merge == 1 ? (m->cluster > 0 ? m->cluster : 1) : 1;
+    pl.cl = pl.merge == 1 ? (knobs.cluster > 0 ? knobs.cluster : 1) : 1;
     while (pl.cl > 1 && (pl.grid % pl.cl != 0 || pl.grid / pl.cl < pl.P)) pl.cl >>= 1;
+    pl.mix = 1;
     *out = pl;
     return CELTY_OK;
 }
@@ -642,21 +644,99 @@ int fit_clusters_only(FusedPlan *plan)
 
 // the cluster size the device can hold; then, without clusters, whether the blocks that are left over when the grid
 // is dealt to the row parts serve several parts each (FusedParams::mix): only where they can be shared evenly
-int fit_clusters(const celty_matrix *m, FusedPlan *plan)
+int fit_clusters(const LaunchKnobs &knobs, FusedPlan *plan)
 {
-    const int rc = fit_clusters_only(plan);
+    int rc = CELTY_OK;
+    if (plan->cl > 1) {                                     // the runtime is asked about the build that has clusters
+        rc = ensure_smem(k_spmspv_fused<false, 0>, plan->smem, g_granted_fused);
+        if (rc == CELTY_OK) rc = fit_clusters_only(plan);
+    }
     plan->mix = 1;
     const int left = plan->grid % plan->P;
-    if (rc == CELTY_OK && plan->cl == 1 && plan->merge == 1 && m->mix != 0 && left > 0 && plan->P % left == 0) {
+    if (rc == CELTY_OK && plan->cl == 1 && plan->merge == 1 && knobs.mix != 0 && left > 0 && plan->P % left == 0) {
         const int mix = plan->P / left;
         // Sharing evens the parts out by 1 / (mix * blocks per part) of the streaming time, and a shared block adds
         // mix times the bytes into y at the end, which takes it mix times as long (the adders in L2 are shared by
         // all blocks): measured 2.2 % faster at 1 / 36 (28672 x 8192), 3 % slower at 1 / 147 (three parts)
-        const bool pays = m->mix > 0 || (int64_t)mix * (plan->grid / plan->P) <= 48;
+        const bool pays = knobs.mix > 0 || (int64_t)mix * (plan->grid / plan->P) <= 48;
         if (pays && plan->G % mix == 0 && plan->Sc * mix <= 16) plan->mix = mix;
     }
+    // the library's default launch has builds of its own (k_spmspv_fused, kLean)
+    plan->lean = (knobs.reg_rows == 0 && plan->merge == 1 && plan->cl == 1 && knobs.lean != 0) ? 1 + plan->pp : 0;
     return rc;
 }
+
+int plan_launch(const celty_matrix *m, const LaunchKnobs &knobs, const DeviceInfo &di, int vectors, FusedPlan *out)
+{
+    const int rc = plan_fused(m, knobs, di, vectors, out);
+    return rc ? rc : fit_clusters(knobs, out);
+}
+
+// What of FusedParams follows from the matrix and the plan alone.
+FusedParams plan_params(const celty_matrix *m, const LaunchKnobs &knobs, const FusedPlan &plan, const uint8_t *image)
+{
+    FusedParams fp{};
+    fp.meta = reinterpret_cast<const uint32_t *>(image);
+    fp.stream = image + m->meta_bytes;
+    fp.M = (int)m->M; fp.K = (int)m->K; fp.R = m->R; fp.S = (int)m->S; fp.C = m->C;
+    fp.G = plan.G; fp.Sc = plan.Sc; fp.P = plan.P; fp.D = plan.D; fp.cl = plan.cl; fp.pp = plan.pp;
+    fp.mix = plan.mix;
+    fp.slot_bytes = plan.slot_bytes; fp.cap = plan.cap;
+    {
+        // offset window: as many columns as 32 KB (or the accumulator area, or the table) hold
+        const size_t acc_bytes = (size_t)plan.G * plan.Sc * (m->R + kTileSlack) * 128;
+        const size_t words = std::min<size_t>(std::min<size_t>(acc_bytes, 32768) / 4, (size_t)m->K * m->S + 4);
+        fp.win_cols = (int)std::min<int64_t>(m->K, words >= 8 ? (int64_t)((words - 8) / m->S) : 0);
+    }
+    fp.merge = plan.merge;
+    fp.lay = fused_smem_layout(m->R, (int)m->K, plan.G * plan.Sc, plan.D, plan.slot_bytes, plan.cap);
+    fp.clear_rows = (int)(m->M / plan.grid);
+    fp.clear_extra = (int)(m->M % plan.grid);
+    fp.spin_limit = knobs.spin_limit ? knobs.spin_limit : kSpinLimit;
+    auto inverse = [](uint64_t units) { return units == 1 ? 0xFFFFFFFFu : (uint32_t)(0x100000000ull / units); };
+    const int nclusters = plan.grid / plan.cl;
+    fp.units_inv = plan.mix >= 2 ? inverse((uint64_t)(plan.grid / plan.P) * plan.G + plan.G / plan.mix)
+                                 : inverse((uint64_t)plan.cl * std::max(1, nclusters / plan.P) * plan.G);
+    fp.units_inv_long = inverse((uint64_t)plan.cl * (nclusters / plan.P + 1) * plan.G);
+    return fp;
+}
+
+// Programmatic dependent launch: the kernel may be scheduled while the previous kernel of the stream drains; it
+// waits for that kernel (griddepcontrol.wait) before it reads or writes anything of the call.
+int launch_fused(void (*kernel)(FusedParams), int *granted, const LaunchKnobs &knobs, const FusedPlan &plan, int vectors,
+                 const FusedParams &fp, cudaStream_t st)
+{
+    const int rc = ensure_smem(kernel, plan.smem, granted);
+    if (rc) return rc;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)plan.grid, (unsigned)vectors);
+    cfg.blockDim = dim3((unsigned)plan.threads);
+    cfg.dynamicSmemBytes = plan.smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[2];
+    int na = 0;
+    if (!knobs.no_overlap) {
+        attr[na].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[na].val.programmaticStreamSerializationAllowed = 1;
+        ++na;
+    }
+    if (plan.cl > 1) {
+        attr[na].id = cudaLaunchAttributeClusterDimension;
+        attr[na].val.clusterDim.x = (unsigned)plan.cl;
+        attr[na].val.clusterDim.y = 1;
+        attr[na].val.clusterDim.z = 1;
+        ++na;
+    }
+    cfg.attrs = attr;
+    cfg.numAttrs = na;
+    CELTY_CUDA(cudaLaunchKernelEx(&cfg, kernel, fp));
+    return CELTY_OK;
+}
+
+// The tickets of launches that serve `vectors` vectors each (one ticket per vector) in the status words.
+constexpr int kBatchTicketWord = 16;
+inline int batch_ticket_word(int vectors) { return kBatchTicketWord + vectors * (vectors - 1) / 2; }
+static_assert(kBatchTicketWord + 9 * 8 / 2 <= (int)kAlign / 4, "the batch tickets must fit the status words");
 
 }  // namespace
 
@@ -670,11 +750,7 @@ extern "C" int celty_launch_plan(const celty_matrix *m, int32_t *out, int32_t n)
     int rc = device_info(&di);
     if (rc) return rc;
     FusedPlan plan;
-    rc = plan_fused(m, di, &plan);
-    if (rc) return rc;
-    rc = ensure_smem(k_spmspv_fused<false, 0>, plan.smem, g_granted_fused);
-    if (rc) return rc;
-    rc = fit_clusters(m, &plan);
+    rc = plan_launch(m, *m, di, 1, &plan);
     if (rc) return rc;
     const int32_t v[10] = {plan.grid, plan.threads, (int32_t)plan.smem, plan.G, plan.D, plan.cl, plan.P, plan.Sc,
                            plan.slot_bytes, plan.merge + 16 * plan.pp + 256 * plan.mix};
@@ -749,28 +825,10 @@ int run_product(celty_matrix *m, const void *x_dev, float tau, const ListInput *
     const uint8_t *stream_base = m->d_image + m->meta_bytes;
     if (m->layout == CELTY_LAYOUT_LANE_TILE && m->variant == 0) {
         FusedPlan plan;
-        rc = plan_fused(m, di, &plan);
+        rc = plan_launch(m, *m, di, 1, &plan);
         if (rc) return rc;
         if (extras && m->reg_rows) return CELTY_EINVAL;
-        rc = extras ? ensure_smem(k_spmspv_fused<true, 0>, plan.smem, g_granted_fused_extras)
-             : m->reg_rows == 32 ? ensure_smem(k_spmspv_fused<false, 32>, plan.smem, g_granted_reg[0])
-             : m->reg_rows == 64 ? ensure_smem(k_spmspv_fused<false, 64>, plan.smem, g_granted_reg[1])
-             : m->reg_rows == 96 ? ensure_smem(k_spmspv_fused<false, 96>, plan.smem, g_granted_reg[2])
-             : m->reg_rows == 128 ? ensure_smem(k_spmspv_fused<false, 128>, plan.smem, g_granted_reg[3])
-                                  : ensure_smem(k_spmspv_fused<false, 0>, plan.smem, g_granted_fused);
-        if (rc) return rc;
-        rc = fit_clusters(m, &plan);
-        if (rc) return rc;
-        // the library's default launch has builds of its own (k_spmspv_fused, kLean)
-        const int lean = (m->reg_rows == 0 && plan.merge == 1 && plan.cl == 1 && m->lean != 0) ? 1 + plan.pp : 0;
-        if (lean) {
-            rc = extras ? (lean == 2 ? ensure_smem(k_spmspv_fused<true, 0, 2>, plan.smem, g_granted_lean_extras[1])
-                                     : ensure_smem(k_spmspv_fused<true, 0, 1>, plan.smem, g_granted_lean_extras[0]))
-                        : (lean == 2 ? ensure_smem(k_spmspv_fused<false, 0, 2>, plan.smem, g_granted_lean[1])
-                                     : ensure_smem(k_spmspv_fused<false, 0, 1>, plan.smem, g_granted_lean[0]));
-            if (rc) return rc;
-        }
-        FusedParams fp{};
+        FusedParams fp = plan_params(m, *m, plan, m->d_image);
         if (list) {
             fp.list_idx = list->idx;
             fp.list_val = list->val;
@@ -788,73 +846,31 @@ int run_product(celty_matrix *m, const void *x_dev, float tau, const ListInput *
             fp.ep_val = ep->list_val;
             fp.ep_count = ep->list_count;
         }
-        fp.meta = reinterpret_cast<const uint32_t *>(m->d_image);
-        fp.stream = stream_base;
         fp.x = static_cast<const uint16_t *>(x_dev);           // not looked at when the survivors come as a list
         fp.tau = tau;
         fp.y = y;
         fp.idx = idx; fp.val = val; fp.count = count; fp.status = status; fp.tickets = status + 2;
         fp.partials = reinterpret_cast<float *>(m->d_ws + m->ws.partial_off);
-        fp.M = (int)m->M; fp.K = (int)m->K; fp.R = m->R; fp.S = (int)m->S; fp.C = m->C;
-        fp.G = plan.G; fp.Sc = plan.Sc; fp.P = plan.P; fp.D = plan.D; fp.cl = plan.cl; fp.pp = plan.pp;
-        fp.mix = plan.mix;
-        fp.slot_bytes = plan.slot_bytes; fp.cap = plan.cap;
-        {
-            // offset window: as many columns as 32 KB (or the accumulator area, or the table) hold
-            const size_t acc_bytes = (size_t)plan.G * plan.Sc * (m->R + kTileSlack) * 128;
-            const size_t words = std::min<size_t>(std::min<size_t>(acc_bytes, 32768) / 4, (size_t)m->K * m->S + 4);
-            fp.win_cols = (int)std::min<int64_t>(m->K, words >= 8 ? (int64_t)((words - 8) / m->S) : 0);
-        }
-        fp.merge = plan.merge;
-        fp.lay = fused_smem_layout(m->R, (int)m->K, plan.G * plan.Sc, plan.D, plan.slot_bytes, plan.cap);
-        fp.clear_rows = (int)(m->M / plan.grid);
-        fp.clear_extra = (int)(m->M % plan.grid);
-        fp.spin_limit = m->spin_limit ? m->spin_limit : kSpinLimit;
-        auto inverse = [](uint64_t units) { return units == 1 ? 0xFFFFFFFFu : (uint32_t)(0x100000000ull / units); };
-        const int nclusters = plan.grid / plan.cl;
-        fp.units_inv = plan.mix >= 2 ? inverse((uint64_t)(plan.grid / plan.P) * plan.G + plan.G / plan.mix)
-                                     : inverse((uint64_t)plan.cl * std::max(1, nclusters / plan.P) * plan.G);
-        fp.units_inv_long = inverse((uint64_t)plan.cl * (nclusters / plan.P + 1) * plan.G);
         // the tickets count blocks of one launch shape: start them over when the shape changes
         if (m->last_grid != plan.grid || m->last_merge != plan.merge) {
             CELTY_CUDA(cudaMemsetAsync(m->d_ws + m->ws.status_off + 8, 0, 8, st));
             m->last_grid = plan.grid;
             m->last_merge = plan.merge;
         }
-        // Programmatic dependent launch: the kernel may be scheduled while the previous kernel of the stream
-        // drains; it waits for that kernel (griddepcontrol.wait) before it reads or writes anything of the call.
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3((unsigned)plan.grid);
-        cfg.blockDim = dim3((unsigned)plan.threads);
-        cfg.dynamicSmemBytes = plan.smem;
-        cfg.stream = st;
-        cudaLaunchAttribute attr[2];
-        int na = 0;
-        if (!m->no_overlap) {
-            attr[na].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-            attr[na].val.programmaticStreamSerializationAllowed = 1;
-            ++na;
+        if (extras)
+            return plan.lean == 2 ? launch_fused(k_spmspv_fused<true, 0, 2>, g_granted_lean_extras[1], *m, plan, 1, fp, st)
+                 : plan.lean == 1 ? launch_fused(k_spmspv_fused<true, 0, 1>, g_granted_lean_extras[0], *m, plan, 1, fp, st)
+                                  : launch_fused(k_spmspv_fused<true, 0>, g_granted_fused_extras, *m, plan, 1, fp, st);
+        switch (m->reg_rows) {
+            case 32: return launch_fused(k_spmspv_fused<false, 32>, g_granted_reg[0], *m, plan, 1, fp, st);
+            case 64: return launch_fused(k_spmspv_fused<false, 64>, g_granted_reg[1], *m, plan, 1, fp, st);
+            case 96: return launch_fused(k_spmspv_fused<false, 96>, g_granted_reg[2], *m, plan, 1, fp, st);
+            case 128: return launch_fused(k_spmspv_fused<false, 128>, g_granted_reg[3], *m, plan, 1, fp, st);
+            default: break;
         }
-        if (plan.cl > 1) {
-            attr[na].id = cudaLaunchAttributeClusterDimension;
-            attr[na].val.clusterDim.x = (unsigned)plan.cl;
-            attr[na].val.clusterDim.y = 1;
-            attr[na].val.clusterDim.z = 1;
-            ++na;
-        }
-        cfg.attrs = attr;
-        cfg.numAttrs = na;
-        if (extras && lean == 2) CELTY_CUDA(cudaLaunchKernelEx(&cfg, k_spmspv_fused<true, 0, 2>, fp));
-        else if (extras && lean == 1) CELTY_CUDA(cudaLaunchKernelEx(&cfg, k_spmspv_fused<true, 0, 1>, fp));
-        else if (extras) CELTY_CUDA(cudaLaunchKernelEx(&cfg, k_spmspv_fused<true, 0>, fp));
-        else if (m->reg_rows == 32) CELTY_CUDA(cudaLaunchKernelEx(&cfg, k_spmspv_fused<false, 32>, fp));
-        else if (m->reg_rows == 64) CELTY_CUDA(cudaLaunchKernelEx(&cfg, k_spmspv_fused<false, 64>, fp));
-        else if (m->reg_rows == 96) CELTY_CUDA(cudaLaunchKernelEx(&cfg, k_spmspv_fused<false, 96>, fp));
-        else if (m->reg_rows == 128) CELTY_CUDA(cudaLaunchKernelEx(&cfg, k_spmspv_fused<false, 128>, fp));
-        else if (lean == 2) CELTY_CUDA(cudaLaunchKernelEx(&cfg, k_spmspv_fused<false, 0, 2>, fp));
-        else if (lean == 1) CELTY_CUDA(cudaLaunchKernelEx(&cfg, k_spmspv_fused<false, 0, 1>, fp));
-        else CELTY_CUDA(cudaLaunchKernelEx(&cfg, k_spmspv_fused<false, 0>, fp));
-        return CELTY_OK;
+        return plan.lean == 2 ? launch_fused(k_spmspv_fused<false, 0, 2>, g_granted_lean[1], *m, plan, 1, fp, st)
+             : plan.lean == 1 ? launch_fused(k_spmspv_fused<false, 0, 1>, g_granted_lean[0], *m, plan, 1, fp, st)
+                              : launch_fused(k_spmspv_fused<false, 0>, g_granted_fused, *m, plan, 1, fp, st);
     }
     // two launches: compaction (which also clears y), then the product.  Sizes are checked and the
     // shared-memory limit is raised before the first launch, so that an error return leaves y untouched.
@@ -987,6 +1003,77 @@ extern "C" int celty_spmspv_static(const celty_matrix *m, const void *image_dev,
     return CELTY_OK;
 }
 
+namespace {
+
+// A batch through the single-launch kernel.  One launch serves several vectors at once, each with its share of the
+// blocks: a vector's product streams no faster than before on as much of the chip as it has, but the part of a call
+// that does not stream -- thresholding, look-ups, the latency of the first copies, the merge, the change of kernels,
+// some 5 us -- is paid once for all of them (4096 x 4096, 50 % / 50 %, four vectors: 33.1 us in four launches,
+// 15.6 us in one; 8192 x 4096, eight vectors: 84.4 -> 41.0).  How many vectors share a launch is chosen by that trade: fixed time against what the division
+// of the blocks loses when they do not divide by vectors and row parts (5 vectors of a layer of 8 row parts: 29
+// blocks for 8 parts leaves five parts with one block more than the other three).
+int run_batch(celty_matrix *m, const uint16_t *x, int64_t ldx, int N, float tau, float *y, int64_t ldy,
+              celty_stream_t stream)
+{
+    cudaStream_t st = static_cast<cudaStream_t>(stream);
+    DeviceInfo di;
+    int rc = device_info(&di);
+    if (rc) return rc;
+    FusedPlan plans[9];
+    double cost[9] = {};
+    // streaming time of one vector on the whole chip: half of the columns at 5 TB/s
+    const double stream_us = 0.5 * 2.5 * (double)(m->nnz + m->n_pad) / 5e6, fixed_us = 5.0;
+    int most = 1;
+    for (int v = 1; v <= N; ++v) {
+        if (plan_launch(m, *m, di, v, &plans[v]) != CELTY_OK || (v > 1 && plans[v].lean == 0)) break;
+        const FusedPlan &pl = plans[v];
+        // teams that share a part's columns, in blocks of G teams
+        const double per_part = pl.grid / pl.P + (pl.mix >= 2 ? 1.0 / pl.mix : 0.0);
+        cost[v] = fixed_us + stream_us * di.sms / (per_part * pl.P);
+        most = v;
+    }
+    // the cheapest way to cut N into launches of nearly equal size
+    int launches = N;
+    double best = 0;
+    for (int n = (N + most - 1) / most; n <= N; ++n) {
+        const int lo = N / n, extra = N % n;
+        const double c = extra * (extra ? cost[lo + 1] : 0.0) + (n - extra) * cost[lo];
+        if (n == (N + most - 1) / most || c < best) { best = c; launches = n; }
+    }
+    for (int first = 0, l = 0; l < launches; ++l) {
+        const int v = N / launches + (l < N % launches ? 1 : 0);
+        const uint16_t *xv = x + (size_t)first * ldx;
+        float *yv = y + (size_t)first * ldy;
+        first += v;
+        if (v == 1) {
+            rc = celty_spmspv(m, xv, tau, yv, stream);
+            if (rc) return rc;
+            continue;
+        }
+        const FusedPlan &plan = plans[v];
+        uint32_t *status = reinterpret_cast<uint32_t *>(m->d_ws + m->ws.status_off);
+        FusedParams fp = plan_params(m, *m, plan, m->d_image);
+        fp.x = xv; fp.ldx = ldx;
+        fp.y = yv; fp.ldy = ldy;
+        fp.tau = tau;
+        fp.status = status;
+        fp.count = reinterpret_cast<int32_t *>(status + 1);
+        fp.idx = reinterpret_cast<int32_t *>(m->d_ws + m->ws.idx_off);
+        fp.val = reinterpret_cast<uint16_t *>(m->d_ws + m->ws.val_off);
+        fp.tickets = status + batch_ticket_word(v);
+        if (m->last_batch_grid[v] != plan.grid) {
+            CELTY_CUDA(cudaMemsetAsync(fp.tickets, 0, (size_t)v * 4, st));
+            m->last_batch_grid[v] = plan.grid;
+        }
+        rc = plan.lean == 2 ? launch_fused(k_spmspv_fused<false, 0, 2, true>, g_granted_batch[1], *m, plan, v, fp, st)
+                            : launch_fused(k_spmspv_fused<false, 0, 1, true>, g_granted_batch[0], *m, plan, v, fp, st);
+        if (rc) return rc;
+    }
+    return CELTY_OK;
+}
+
+}  // namespace
+
 extern "C" int celty_spmspv_batch(celty_matrix *m, const void *x_dev, int64_t ldx, int32_t N, float tau, void *y_dev,
                                   int64_t ldy, void *list_scratch_dev, size_t scratch_bytes, celty_stream_t stream)
 {
@@ -1004,12 +1091,7 @@ extern "C" int celty_spmspv_batch(celty_matrix *m, const void *x_dev, int64_t ld
     // on): unless the two-launch variant is asked for, the batch is N launches of the single-launch kernel, where the
     // handle has its workspace and every row of x and y starts on a 16-byte boundary.
     if (m->variant == 0 && m->d_ws && !(((uintptr_t)x_dev | (uintptr_t)(ldx * 2) | (uintptr_t)y_dev | (uintptr_t)(ldy * 4)) & 15)) {
-        for (int32_t n = 0; n < N; ++n) {
-            const int rc1 = celty_spmspv(m, static_cast<const uint16_t *>(x_dev) + (size_t)n * ldx, tau,
-                                         static_cast<float *>(y_dev) + (size_t)n * ldy, stream);
-            if (rc1) return rc1;
-        }
-        return CELTY_OK;
+        return run_batch(m, static_cast<const uint16_t *>(x_dev), ldx, N, tau, static_cast<float *>(y_dev), ldy, stream);
     }
     DeviceInfo di;
     int rc = device_info(&di);
@@ -1101,9 +1183,10 @@ extern "C" int celty_last_status(celty_matrix *m, celty_stream_t stream)
     if (word) {
         // also reset the fused kernel's tickets, which a run that gave up may have left mid-count
         CELTY_CUDA(cudaMemsetAsync(m->d_ws + m->ws.status_off, 0, 4, st));
-        CELTY_CUDA(cudaMemsetAsync(m->d_ws + m->ws.status_off + 8, 0, 8, st));
+        CELTY_CUDA(cudaMemsetAsync(m->d_ws + m->ws.status_off + 8, 0, kAlign - 8, st));
         CELTY_CUDA(cudaStreamSynchronize(st));
         m->last_grid = 0;
+        for (int32_t &g : m->last_batch_grid) g = 0;
     }
     if (word & kStatusTimeout) return CELTY_ETIMEOUT;
     if (word & kStatusBounds) return CELTY_EBOUNDS;

@@ -64,6 +64,31 @@ def test_batch_integer_data_is_bit_exact_and_strided():
     assert torch.count_nonzero(yb[2, :M]).item() == 0
 
 
+@pytest.mark.parametrize("M,K,tile_rows", [(4096, 700, 0), (20000, 90, 0), (28672, 64, 0), (40, 33, 8), (9000, 257, 40)])
+def test_batches_of_changing_size_on_one_handle(M, K, tile_rows):
+    """Vectors that share a launch, on a handle that serves batches of every size and single vectors in turn (the
+    tickets of one launch shape must not disturb another's), row parts that do not divide the blocks of a vector,
+    more blocks than columns; integer data, so every sum is exact.  The list reported is the last vector's."""
+    W = synth.integer_weights(5, M, K)
+    mask = synth.mask_bernoulli(5, M, K, 0.5)
+    X = np.stack([synth.integer_activations(40 + n, K) for n in range(8)])
+    ref = np.stack([orc.masked_gemv(W, mask, X[n], 1.0, threads=8)[0] for n in range(8)])
+    m = celty.Matrix(W, mask, tile_rows=tile_rows, device="cuda")
+    wide = torch.zeros(8, (K + 7) // 8 * 8, dtype=torch.float16, device="cuda")
+    wide[:, :K] = _dev(X)
+    for N in (2, 8, 3, 1, 5, 8, 2, 7, 4, 6, 1, 3):
+        y = torch.full((N, (M + 3) // 4 * 4), 9.0, device="cuda")[:, :M]
+        m.spmspv_batch(wide[:N, :K], 1.0, y=y)
+        torch.cuda.synchronize()
+        assert m.last_status() == 0
+        assert np.array_equal(y.cpu().numpy().astype(np.float64), ref[:N]), N
+        idx, val = m.last_compaction()
+        oi, ov, _ = orc.compact(X[N - 1], 1.0)
+        assert np.array_equal(idx.cpu().numpy(), oi) and np.array_equal(val.cpu().numpy().view(np.uint16), ov), N
+        y1 = m.spmspv(wide[N % 8, :K].contiguous(), 1.0)
+        assert np.array_equal(y1.cpu().numpy().astype(np.float64), ref[N % 8]), N
+
+
 def test_batch_argument_errors():
     m = celty.Matrix(synth.weights(1, 64, 40), None, device="cuda")
     x = torch.zeros(9, 40, dtype=torch.float16, device="cuda")
