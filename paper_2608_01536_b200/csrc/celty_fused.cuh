@@ -3,6 +3,8 @@
 //
 // One launch does the whole call (Sections 3.1-3.3):
 //   a0  the last warp of every block clears its share of y and takes a ticket (the merge at the end adds into y);
+//   (with swiglu_in: x = SiLU(gate) * up is made here, every block a share of it, and the ticket of a0 tells when all
+//       of it is there)
 //   a1  every block thresholds all of x (K <= a few 10k values, served by L2) into one keep bit per
 //       activation and ranks the survivors (popcounts + warp scans); each warp team then looks up the
 //       columns whose ranks belong to it -- the list is balanced over all teams by count -- and their
@@ -121,6 +123,37 @@ __device__ __forceinline__ uint32_t ld_acquire_u32(const uint32_t *p)
 {
     uint32_t v;
     asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
+
+// Wait until all gridDim.x blocks have taken their ticket (this block's was `mine`; the count runs modulo
+// 2 * gridDim.x, so calls alternate between waiting for its upper and for its lower half), bounded; what the others
+// wrote before theirs is visible to this block after its next barrier.
+__device__ __forceinline__ bool ticket_wait(const uint32_t *ticket, uint32_t mine, uint32_t limit)
+{
+    const bool low_half = mine < gridDim.x;
+    bool ok = false;
+    for (uint32_t it = 0; it < limit; ++it) {
+        const uint32_t cur = ld_relaxed_u32(ticket);
+        if (low_half ? (cur >= gridDim.x) : (cur < gridDim.x)) { ok = true; break; }
+        __nanosleep(it < 64 ? 20 : 64);
+    }
+    __threadfence();
+    return ok;
+}
+
+// Loads of values that other blocks of this launch may have written (not through the read-only path).
+__device__ __forceinline__ uint4 ld_plain_v4(const uint16_t *p)
+{
+    uint4 v;
+    asm volatile("ld.global.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p) : "memory");
+    return v;
+}
+
+__device__ __forceinline__ uint16_t ld_plain_u16(const uint16_t *p)
+{
+    uint16_t v;
+    asm volatile("ld.global.u16 %0, [%1];" : "=h"(v) : "l"(p) : "memory");
     return v;
 }
 
@@ -342,7 +375,7 @@ __global__ void __launch_bounds__(kRegRows > 0 ? 256 : 512, 1) k_spmspv_fused(co
     const int pp = kLean ? (kLean == 2 ? 1 : 0) : p.pp;
     const int merge = kLean ? 1 : p.merge;
     const int cl = kLean ? 1 : p.cl;
-    const uint16_t *const x = kBatch ? p.x + (size_t)blockIdx.y * p.ldx : p.x;
+    const uint16_t *const x = kBatch ? p.x + (size_t)blockIdx.y * p.ldx : kExtras && p.swiglu_in ? p.h_ws : p.x;
     float *const y = kBatch ? p.y + (size_t)blockIdx.y * p.ldy : p.y;
     uint32_t *const tickets = kBatch ? p.tickets + blockIdx.y : p.tickets;
     const bool lists = !kBatch || blockIdx.y + 1 == gridDim.y;    // the survivor list reported is the last vector's
@@ -443,6 +476,19 @@ __global__ void __launch_bounds__(kRegRows > 0 ? 256 : 512, 1) k_spmspv_fused(co
     }
     asm volatile("griddepcontrol.wait;" ::: "memory");
     uint32_t y_ticket = 0;
+    // x made from the FP32 gate / up result: every block evaluates a share (32 values per warp, dealt to the blocks in
+    // turn) into the workspace, and takes its ticket once the share is stored.  The alternative, every block
+    // evaluating all of x for itself, cost 18.6 us at 4096 x 11008 (each thread 32 SiLUs in a row, 148 times
+    // the expf work); this is one block barrier and one trip to L2 and back: 16.3 us.
+    if (kExtras && p.swiglu_in) {
+#pragma unroll 1
+        for (uint32_t i = ((uint32_t)warp * gridDim.x + blockIdx.x) * 32u + lane; i < (uint32_t)p.K; i += nthreads * gridDim.x) {
+            const uint16_t h = (uint16_t)swiglu_half_bits(__ldg(p.swiglu_in + i), __ldg(p.swiglu_in + p.K + i));
+            p.h_ws[i] = h;
+            if (p.h_out) p.h_out[i] = h;
+        }
+        __syncthreads();
+    }
     // Bulk reduce-add merge: the adds at the end need a cleared y.  The last warp clears this block's share
     // and announces it right away, so that the fence and the ticket overlap the loads of a1.
     if (merge == 1 && warp == nwarps - 1) {
@@ -457,8 +503,10 @@ __global__ void __launch_bounds__(kRegRows > 0 ? 256 : 512, 1) k_spmspv_fused(co
             // The ticket counts modulo 2 * gridDim.x, so it never has to be reset: calls alternate between
             // waiting for the lower and for the upper half.
             y_ticket = atomicInc(&tickets[0], 2u * gridDim.x - 1u);
+            if (kExtras && p.swiglu_in && !ticket_wait(tickets, y_ticket, p.spin_limit)) atomicOr(p.status, kStatusTimeout);
         }
     }
+    if (kExtras && p.swiglu_in) __syncthreads();
     // ---- a1: threshold all of x.  A thread takes 32 activations (four 128-bit loads) and makes one keep word,
     // and the warp scans the survivor counts of its block of 32 words:
     //   kbw[w]  keep bits of activations 32w .. 32w+31,
@@ -479,37 +527,8 @@ __global__ void __launch_bounds__(kRegRows > 0 ? 256 : 512, 1) k_spmspv_fused(co
                 for (int c = 0; c < 4; ++c) {                          // four independent 128-bit loads per thread
                     const int q = 4 * w + c;
                     h[c][0] = h[c][1] = h[c][2] = h[c][3] = 0u;        // zero past the end of x: never kept (tau >= 0)
-                    if (kExtras && p.swiglu_in) {                      // the activations are made here, from FP32 gate / up
-                        if (q < ngroups) {
-                            float gt[8], up[8];
-                            if (8 * q + 8 <= p.K && (p.K & 3) == 0) {  // 128-bit loads (the up half starts 16-byte aligned)
-                                const float4 a0 = __ldg(reinterpret_cast<const float4 *>(p.swiglu_in + 8 * q));
-                                const float4 a1 = __ldg(reinterpret_cast<const float4 *>(p.swiglu_in + 8 * q + 4));
-                                const float4 b0 = __ldg(reinterpret_cast<const float4 *>(p.swiglu_in + p.K + 8 * q));
-                                const float4 b1 = __ldg(reinterpret_cast<const float4 *>(p.swiglu_in + p.K + 8 * q + 4));
-                                gt[0] = a0.x; gt[1] = a0.y; gt[2] = a0.z; gt[3] = a0.w; gt[4] = a1.x; gt[5] = a1.y; gt[6] = a1.z; gt[7] = a1.w;
-                                up[0] = b0.x; up[1] = b0.y; up[2] = b0.z; up[3] = b0.w; up[4] = b1.x; up[5] = b1.y; up[6] = b1.z; up[7] = b1.w;
-                            } else {
-#pragma unroll
-                                for (int k = 0; k < 8; ++k) {
-                                    const int j = 8 * q + k;
-                                    gt[k] = j < p.K ? __ldg(p.swiglu_in + j) : 0.f;          // SiLU(0) * 0 = 0: never kept
-                                    up[k] = j < p.K ? __ldg(p.swiglu_in + p.K + j) : 0.f;
-                                }
-                            }
-#pragma unroll
-                            for (int k = 0; k < 4; ++k) {
-                                const uint32_t lo = swiglu_half_bits(gt[2 * k], up[2 * k]), hi = swiglu_half_bits(gt[2 * k + 1], up[2 * k + 1]);
-                                h[c][k] = lo | (hi << 16);
-                                // every block makes all of h; the blocks share the writing of it
-                                if (p.h_out && (q % gridDim.x) == blockIdx.x) {
-                                    if (8 * q + 2 * k < p.K) p.h_out[8 * q + 2 * k] = (uint16_t)lo;
-                                    if (8 * q + 2 * k + 1 < p.K) p.h_out[8 * q + 2 * k + 1] = (uint16_t)hi;
-                                }
-                            }
-                        }
-                    } else if (8 * q + 8 <= p.K) {
-                        const uint4 v = __ldg(reinterpret_cast<const uint4 *>(x + 8 * q));
+                    if (8 * q + 8 <= p.K) {
+                        const uint4 v = kExtras ? ld_plain_v4(x + 8 * q) : __ldg(reinterpret_cast<const uint4 *>(x + 8 * q));
                         h[c][0] = v.x; h[c][1] = v.y; h[c][2] = v.z; h[c][3] = v.w;
                     } else if (__builtin_expect(q < ngroups, 0)) {
                         const uint4 v = ragged_group(x, p.K, q);     // the one group that K cuts short
@@ -651,8 +670,7 @@ __global__ void __launch_bounds__(kRegRows > 0 ? 256 : 512, 1) k_spmspv_fused(co
                     if (k >= c) { k -= c; pos += sh; }
                 }
                 j = 32 * w + pos;
-                if (kExtras && p.swiglu_in) xb = (uint16_t)swiglu_half_bits(__ldg(p.swiglu_in + j), __ldg(p.swiglu_in + p.K + j));
-                else xb = __ldg(x + j);                            // x went through L1 in the thresholding pass
+                xb = kExtras ? ld_plain_u16(x + j) : __ldg(x + j);   // x went through L1 in the thresholding pass
                 }
                 items[i] = make_int2(j, (int)xb);
                 if (!from_list && lists && part == 0 && sl == 0) {
@@ -801,14 +819,7 @@ __global__ void __launch_bounds__(kRegRows > 0 ? 256 : 512, 1) k_spmspv_fused(co
         // (cp.reduce.async.bulk, FP32 add at L2).  y was cleared by all blocks at the start; the ticket makes
         // sure of it.
         if (warp == nwarps - 1 && lane == 0) {                      // every block's share of y is cleared by now
-            const bool low_half = y_ticket < gridDim.x;
-            bool ok = false;
-            for (uint32_t it = 0; it < p.spin_limit; ++it) {
-                const uint32_t cur = ld_relaxed_u32(&tickets[0]);
-                if (low_half ? (cur >= gridDim.x) : (cur < gridDim.x)) { ok = true; break; }
-                __nanosleep(64);
-            }
-            __threadfence();
+            const bool ok = ticket_wait(tickets, y_ticket, p.spin_limit);
             // the clearing stores of the other blocks (generic proxy) come before this block's reduce-adds
             // (asynchronous proxy) to the same addresses
             asm volatile("fence.proxy.async.global;" ::: "memory");

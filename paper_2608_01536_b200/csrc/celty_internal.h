@@ -52,7 +52,8 @@ struct WorkspaceLayout {
     size_t idx_off;      // int32[K]
     size_t val_off;      // uint16[K]
     size_t scratch_off;  // uint32[T + 2] for celty_decode_device
-    size_t partial_off;  // float[kMaxBlocks][part_words]: per-block partial sums of the fused kernel
+    size_t partial_off;  // float[kMaxBlocks][part_words]: per-block partial sums of the fused kernel (ordered merge), or
+                         // uint16[K]: the activations a down projection makes from gate and up (bulk merge)
     size_t total;
 };
 
@@ -64,7 +65,8 @@ inline WorkspaceLayout workspace_layout(int64_t K, int64_t T, int64_t part_words
     w.val_off = w.idx_off + round_up((size_t)K * 4, kAlign);
     w.scratch_off = w.val_off + round_up((size_t)K * 2, kAlign);
     w.partial_off = w.scratch_off + round_up((size_t)(T + 2) * 4, kAlign);
-    w.total = w.partial_off + round_up((size_t)kMaxBlocks * part_words * 4, kAlign);
+    const size_t partials = (size_t)kMaxBlocks * part_words * 4, h = part_words ? (size_t)K * 2 : 0;
+    w.total = w.partial_off + round_up(partials > h ? partials : h, kAlign);
     return w;
 }
 
@@ -135,11 +137,11 @@ struct FusedParams {
     const int32_t *list_idx;
     const uint16_t *list_val;
     const int32_t *list_count;
-    // The activations are not given but made on the fly from the FP32 result of a stacked [gate; up] product
-    // (2K values, gate first): x_j = SiLU(g_j) * u_j rounded to FP16, for the down projection.  h_out (may be
-    // null) receives the K FP16 values.
+    // The activations are not given but made from the FP32 result of a stacked [gate; up] product (2K values, gate
+    // first): x_j = SiLU(g_j) * u_j rounded to FP16, for the down projection, into the workspace (h_ws, K values).
+    // h_out (may be null) receives a copy.
     const float *swiglu_in;
-    uint16_t *h_out;
+    uint16_t *h_ws, *h_out;
     // Work on y after the merge (bulk reduce-add merge only): 0 none; 1 an FP16 copy of y; 2 y holds a stacked
     // [gate; up] product of 2I rows: h_i = SiLU(y_i) * y_{I+i} rounded to FP16, stored, and the (i, h_i) with
     // |h_i| > ep_tau appended to a list that the next product takes as its survivors

@@ -836,6 +836,7 @@ int run_product(celty_matrix *m, const void *x_dev, float tau, const ListInput *
         }
         if (sw) {
             fp.swiglu_in = sw->gate_up;
+            fp.h_ws = reinterpret_cast<uint16_t *>(m->d_ws + m->ws.partial_off);
             fp.h_out = sw->h_out;
         }
         if (ep && ep->kind != CELTY_EPILOGUE_NONE) {
