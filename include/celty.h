@@ -47,7 +47,8 @@ typedef enum {
  * defines, one run per value; they differ in how entries are grouped for the kernel.
  *   CELTY_LAYOUT_COLUMN     tile_rows must be 0: runs are counted along the whole column.
  *                           A warp decodes 256 consecutive entries at a time with the intra-warp
- *                           prefix sum of Algorithm 1 and scatters with shared-memory atomics.
+ *                           prefix sum of Algorithm 1; the warps that share a column (and the block's
+ *                           accumulator with it) hold different rows, so they add without atomics.
  *   CELTY_LAYOUT_LANE_TILE  tile_rows = R > 0: the rows are partitioned into tiles of R rows (the
  *                           row partition of Section 3.1 taken down to one tile per lane) and the
  *                           rule of Section 3.2 is applied to every tile separately.  Lane L of the
@@ -176,7 +177,8 @@ int celty_compact(const void *x_dev, int64_t K, float tau, int32_t *idx_dev, uin
  * the surviving columns, decodes their runs to rows, accumulates value * x_j in shared memory in
  * FP32 (one rounding per multiply-add) and merges the thread blocks' results into y (FP32 adds in L2
  * by bulk reduce-add copies; celty_set_launch can select a sum in a fixed order instead); the COLUMN
- * layout uses a compaction kernel followed by the SpMSpV kernel.  On a stream of calls the kernel's
+ * layout has one kernel of the same outline, behind a compaction kernel where K is so large that its keep bits leave
+ * no room in shared memory.  On a stream of calls the kernel's
  * set-up overlaps the end of the previous kernel (programmatic dependent launch); it waits for that
  * kernel before it reads x or touches y or the workspace.
  *   x_dev  K FP16 (device, 16-byte aligned), not modified

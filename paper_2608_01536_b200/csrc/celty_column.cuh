@@ -1,0 +1,291 @@
+// The SpMSpV kernel for the COLUMN layout: the formulation of Sections 3.1-3.3 as published, whole columns decoded
+// with the intra-warp prefix sum of Algorithm 1 (included by celty_kernels.cu inside its anonymous namespace, after
+// celty_fused.cuh).
+//
+// A thread block takes an equal share of the surviving columns; inside it, groups of W warps take one column at a
+// time, warp w of a group the chunks w, W + w, ... of 256 entries.  The entries of one column are different rows, so
+// the warps of a group add into one accumulator of M floats with plain load / fma / store: no two of them ever hold
+// the same row, and no atomics are needed (a shared-memory FP32 atomic add is a compare-and-swap loop).  What the
+// warps do exchange is where their chunk starts: each scans its own chunk (Algorithm 1), posts the rows it spans and
+// meets the others at a named barrier, which also keeps the group's columns apart (nobody scatters column i + 1
+// before everybody has scattered column i).  Two chunks per warp are loaded ahead of the one being scattered.
+//
+// What bounds it: shared memory.  The rows of the 32 lanes fall on the banks as good as at random (8 entries, or
+// some 16 rows at 50 % density, lie between two lanes), so a load or store takes 3 to 4 wavefronts where the lane
+// tiles' takes one; entries per SM / 32 x 7 wavefronts is 3.2 us at 4096 x 4096, 50 % / 50 %.  Measured there:
+// 16.0 us against 41.6 us for warps that each took whole columns and added with shared-memory atomics, behind a
+// one-block compaction kernel.
+//
+// a0 and a1 as in the fused kernel: every block clears its share of y and takes a ticket, and thresholds all of x.
+// Where K's keep words leave no room the list comes from k_compact, which also clears y; more blocks than fit the
+// device at once cannot wait for one another's tickets, and k_clear comes before them.
+
+struct ColumnParams {
+    const uint2 *meta;          // [K] {offset/16, entries}
+    const uint8_t *stream;
+    const uint16_t *x;
+    float tau;
+    int32_t *idx;               // the compacted list: written here, or read when own_list is 0
+    uint16_t *val;
+    int32_t *count;
+    float *y;
+    uint32_t *status;
+    uint32_t *ticket;           // null: the kernel before this one cleared y
+    uint32_t spin_limit;
+    int M, K;
+    int W, groups;              // warps per column, columns in flight per block (W * groups <= 32, groups <= 15 if W > 1)
+    int cap;                    // columns a block looks up at a time
+    int own_list;               // 1: threshold x here
+};
+
+constexpr int kColumnThreads = 1024;
+
+struct ColumnSmem { uint32_t acc, spans, items, imeta, warps, keep, rank, total; };
+
+__host__ __device__ inline ColumnSmem column_smem_layout(int M, int K, int groups, int cap, int own_list)
+{
+    ColumnSmem l;
+    uint32_t off = 0;
+    l.acc = off;    off += (uint32_t)groups * ((M + 3) & ~3) * 4u;    // one accumulator per group
+    l.items = off;  off += (uint32_t)cap * 8u;                       // {column, x bits}
+    l.imeta = off;  off += (uint32_t)cap * 8u;                       // {offset/16, entries}
+    l.spans = off;  off += 2u * 32u * 4u;                            // rows spanned by each warp's chunk, two columns deep
+    l.warps = off;  off += 33u * 4u;                                 // survivors before each warp's words, and of all
+    l.keep = off;   off += own_list ? (uint32_t)((K + 31) / 32) * 4u : 0u;
+    l.rank = off;   off += own_list ? (uint32_t)((K + 31) / 32) * 4u : 0u;   // survivors before each keep word
+    l.total = (off + 15u) & ~15u;
+    return l;
+}
+
+// One keep bit per activation of x[32w .. 32w+31] (zero past the end of x).
+__device__ __forceinline__ uint32_t keep_word(const uint16_t *x, int K, int w, __half2 tau2)
+{
+    const int ngroups = (K + 7) >> 3;
+    uint32_t word = 0;
+    uint4 h[4];
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+        const int q = 4 * w + c;
+        h[c] = make_uint4(0u, 0u, 0u, 0u);                          // never kept (tau >= 0)
+        if (8 * q + 8 <= K) h[c] = __ldg(reinterpret_cast<const uint4 *>(x + 8 * q));
+        else if (q < ngroups) h[c] = ragged_group(x, K, q);
+    }
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+        const uint32_t v[4] = {h[c].x, h[c].y, h[c].z, h[c].w};
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const uint32_t le = __hle2_mask(__habs2(*reinterpret_cast<const __half2 *>(&v[k])), tau2);
+            word |= ((~le & 1u) | ((~le >> 15) & 2u)) << (8 * c + 2 * k);
+        }
+    }
+    if (32 * w + 32 > K) word &= 32 * w < K ? 0xFFFFFFFFu >> (32 * w + 32 - K) : 0u;
+    return word;
+}
+
+__global__ void __launch_bounds__(kColumnThreads, 1) k_spmspv_column(const ColumnParams p)
+{
+    extern __shared__ __align__(128) uint8_t smem[];
+    const ColumnSmem lay = column_smem_layout(p.M, p.K, p.groups, p.cap, p.own_list);
+    float *acc = reinterpret_cast<float *>(smem + lay.acc);
+    int2 *items = reinterpret_cast<int2 *>(smem + lay.items);
+    uint2 *imeta = reinterpret_cast<uint2 *>(smem + lay.imeta);
+    int *warp_tot = reinterpret_cast<int *>(smem + lay.warps);
+    uint32_t *keep = reinterpret_cast<uint32_t *>(smem + lay.keep);
+    int *rank = reinterpret_cast<int *>(smem + lay.rank);
+    const int tid = threadIdx.x, lane = tid & 31;
+    const int warp = __shfl_sync(kFull, tid >> 5, 0);
+    const int Mp = (p.M + 3) & ~3;
+
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    for (int i = tid; i < p.groups * Mp / 4; i += kColumnThreads)
+        reinterpret_cast<float4 *>(acc)[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+
+    uint32_t y_ticket = 0;
+    if (p.ticket && warp == kColumnThreads / 32 - 1) {
+        for (int i = blockIdx.x * 32 + lane; i < p.M; i += gridDim.x * 32) p.y[i] = 0.f;
+        __syncwarp();
+        if (lane == 0) {
+            __threadfence();
+            y_ticket = atomicInc(p.ticket, 2u * gridDim.x - 1u);
+        }
+    }
+    // ---- a1: keep words and the survivors before each of them
+    int n = 0;
+    if (p.own_list) {
+        const __half2 tau2 = __half2half2(__float2half_rd(p.tau));   // |x| > tau decided in FP16, as in the fused kernel
+        const int nwords = (p.K + 31) >> 5;
+        for (int w0 = 0; w0 < nwords; w0 += kColumnThreads) {          // the same trip count for every thread
+            const int w = w0 + tid;
+            const uint32_t word = w < nwords ? keep_word(p.x, p.K, w, tau2) : 0u;
+            const int cnt = __popc(word);
+            int incl = cnt;
+#pragma unroll
+            for (int d = 1; d < 32; d <<= 1) {
+                const int up = __shfl_up_sync(kFull, incl, d);
+                if (lane >= d) incl += up;
+            }
+            if (lane == 31) warp_tot[warp] = incl;
+            __syncthreads();
+            const int t = warp_tot[lane];
+            const int before = __reduce_add_sync(kFull, lane < warp ? t : 0), all = __reduce_add_sync(kFull, t);
+            if (w < nwords) {
+                keep[w] = word;
+                rank[w] = n + before + incl - cnt;
+            }
+            n += all;
+            __syncthreads();
+        }
+        if (blockIdx.x == 0 && tid == 0) *p.count = n;
+    } else {
+        n = __ldcg(p.count);
+    }
+
+    const int p0 = (int)((int64_t)blockIdx.x * n / gridDim.x), p1 = (int)((int64_t)(blockIdx.x + 1) * n / gridDim.x);
+    const int g = warp / p.W, w = warp - g * p.W;
+    const bool works = g < p.groups;
+    float *const a = acc + (size_t)(works ? g : 0) * Mp;
+    volatile uint32_t *const spans = reinterpret_cast<uint32_t *>(smem + lay.spans) + (works ? g * p.W : 0);
+    uint32_t parity = 0;
+    bool out_of_range = false;
+    for (int b0 = p0; b0 < p1; b0 += p.cap) {
+        // ---- the columns of ranks b0 .. b0 + cnt - 1
+        const int cnt = min(p.cap, p1 - b0);
+        if (p.own_list) {
+            const int nwords = (p.K + 31) >> 5;
+            for (int i = tid; i < nwords; i += kColumnThreads) {
+                uint32_t word = keep[i];
+                int r = rank[i] - b0;
+                if (r >= cnt || r + __popc(word) <= 0) continue;
+                for (; word; word &= word - 1, ++r)
+                    if (r >= 0 && r < cnt) items[r].x = 32 * i + __ffs(word) - 1;
+            }
+            __syncthreads();
+            for (int i = tid; i < cnt; i += kColumnThreads) {
+                const int j = items[i].x;
+                const uint16_t xb = __ldg(p.x + j);
+                items[i].y = (int)xb;
+                imeta[i] = __ldg(p.meta + j);
+                p.idx[b0 + i] = j;
+                p.val[b0 + i] = xb;
+            }
+        } else {
+            for (int i = tid; i < cnt; i += kColumnThreads) {
+                const int j = __ldcg(p.idx + b0 + i);
+                items[i] = make_int2(j, (int)__ldcg(p.val + b0 + i));
+                imeta[i] = __ldg(p.meta + j);
+            }
+        }
+        __syncthreads();
+        // ---- a2 - a4: this group's columns of the batch
+        if (works) {
+            const int i1 = (int)((int64_t)(g + 1) * cnt / p.groups);
+            int li = (int)((int64_t)g * cnt / p.groups), lc = 0;       // what is loaded next: column, first chunk
+            int pi = li, pc = 0;                                       // what is scattered next
+            struct Chunk { uint4 v; uint32_t runs; };
+            auto next = [&](int &i, int &c) {                          // the group's next W chunks
+                c += p.W;
+                if ((uint32_t)c * (kChunkGroups * kGroup) >= imeta[i].y) { ++i; c = 0; }
+            };
+            auto load = [&](Chunk &ch) {
+                ch.v = make_uint4(0u, 0u, 0u, 0u);
+                ch.runs = 0u;
+                if (li >= i1) return;
+                const uint2 mj = imeta[li];
+                const uint32_t ng = (mj.y + kGroup - 1) / kGroup, c = (uint32_t)(lc + w), first = c * kChunkGroups;
+                if (first + lane < ng) {
+                    const uint32_t gc = min((uint32_t)kChunkGroups, ng - first);
+                    const uint8_t *chunk = p.stream + (size_t)mj.x * 16 + (size_t)c * (kChunkGroups * 20);
+                    ch.v = __ldg(reinterpret_cast<const uint4 *>(chunk + 16 * lane));
+                    ch.runs = __ldg(reinterpret_cast<const uint32_t *>(chunk + 16 * gc + 4 * lane));
+                }
+                next(li, lc);
+            };
+            Chunk c0, c1, c2;
+            load(c0);
+            load(c1);
+            uint32_t carry = 0;                                        // rows of the column before the group's chunks
+            while (pi < i1) {
+                load(c2);
+                const uint32_t nent = imeta[pi].y, e0 = ((uint32_t)(pc + w) * kChunkGroups + lane) * kGroup;
+                uint32_t even, odd, total;
+                decode_group(c0.runs, even, odd, total);
+                const uint32_t span = e0 < nent ? total + kGroup : 0u;
+                uint32_t sum = span;                                   // Algorithm 1: inclusive scan over the lanes
+#pragma unroll
+                for (int d = 1; d < 32; d <<= 1) {
+                    const uint32_t prev = __shfl_up_sync(kFull, sum, d);
+                    if (lane >= d) sum += prev;
+                }
+                uint32_t row0 = carry + sum - span;
+                const uint32_t mine = __shfl_sync(kFull, sum, 31);
+                if (p.W > 1) {
+                    if (lane == 0) spans[32 * parity + w] = mine;
+                    asm volatile("bar.sync %0, %1;" ::"r"(1 + g), "r"(32 * p.W) : "memory");
+                    const uint32_t t = lane < p.W ? spans[32 * parity + lane] : 0u;
+                    row0 += __reduce_add_sync(kFull, lane < w ? t : 0u);
+                    carry += __reduce_add_sync(kFull, t);
+                    parity ^= 1u;
+                } else {
+                    carry += mine;
+                    __syncwarp();                                      // the lanes' stores of the column before this one
+                }
+                const float xj = __half2float(__ushort_as_half((uint16_t)items[pi].y));
+                const uint32_t have = nent > e0 ? min(nent - e0, (uint32_t)kGroup) : 0u;
+                uint32_t row[kGroup];
+                float sumv[kGroup];
+#pragma unroll
+                for (int e = 0; e < kGroup; ++e) {
+                    row[e] = row0 + entry_offset(even, odd, e);
+                    const bool ok = (uint32_t)e < have;
+                    if (ok && row[e] >= (uint32_t)p.M) out_of_range = true;
+                    if (!ok || row[e] >= (uint32_t)p.M) row[e] = 0xFFFFFFFFu;
+                    sumv[e] = row[e] != 0xFFFFFFFFu ? a[row[e]] : 0.f;
+                }
+#pragma unroll
+                for (int e = 0; e < kGroup; ++e)
+                    if (row[e] != 0xFFFFFFFFu) a[row[e]] = fmaf(entry_value(c0.v, e), xj, sumv[e]);
+                const int before = pi;
+                next(pi, pc);
+                if (pi != before) carry = 0;
+                c0 = c1;
+                c1 = c2;
+            }
+        }
+        __syncthreads();
+    }
+    if (out_of_range) atomicOr(p.status, kStatusBounds);
+    if (p0 >= p1) return;                                              // (the same for the whole block)
+    if (p.ticket && warp == kColumnThreads / 32 - 1) {
+        if (lane == 0 && !ticket_wait(p.ticket, y_ticket, p.spin_limit)) atomicOr(p.status, kStatusTimeout);
+        __syncwarp();
+    }
+    // ---- a5: the groups' accumulators, then one bulk reduce-add per 512 rows of y
+    if (p.groups > 1) {
+        float4 *acc4 = reinterpret_cast<float4 *>(acc);
+        for (int i = tid; i < Mp / 4; i += kColumnThreads) {
+            float4 v = acc4[i];
+            for (int gg = 1; gg < p.groups; ++gg) {
+                const float4 t = acc4[gg * (Mp / 4) + i];
+                v.x += t.x; v.y += t.y; v.z += t.z; v.w += t.w;
+            }
+            acc4[i] = v;
+        }
+    }
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    __syncthreads();
+    for (int r0 = tid * 512; r0 < p.M; r0 += kColumnThreads * 512) {
+        // the clearing of y by other blocks or another kernel (generic proxy) comes before these adds (asynchronous proxy)
+        asm volatile("fence.proxy.async.global;" ::: "memory");
+        const int nrows = min(512, p.M - r0);
+        const uint32_t bytes = ((uint32_t)nrows * 4u) & ~15u;
+        if (bytes)
+            asm volatile("cp.reduce.async.bulk.global.shared::cta.bulk_group.add.f32 [%0], [%1], %2;" ::"l"(p.y + r0),
+                         "r"(smem_u32(acc + r0)), "r"(bytes)
+                         : "memory");
+        for (int i = (int)(bytes >> 2); i < nrows; ++i) atomicAdd(p.y + r0 + i, acc[r0 + i]);
+    }
+    asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+    asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+}

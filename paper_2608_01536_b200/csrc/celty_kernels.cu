@@ -155,14 +155,8 @@ k_compact(const uint16_t *__restrict__ x, int K, float tau, int32_t *__restrict_
     if (tid == 0) *count = base;
 }
 
-// ------------------------------------------------------------------------------------------------
-// COLUMN layout kernel: the formulation of Sections 3.1-3.3 as published.  A thread block owns a
-// slice of the surviving-column list and an M-float accumulator in shared memory.  Each warp takes
-// whole columns; per chunk of 256 entries every lane loads 8 values (one 128-bit load) and their 8
-// runs, the warp reconstructs rows with the intra-warp prefix sum of Algorithm 1 (per-lane sum,
-// five shfl_up steps, back-fill), and scatters value * x_j with shared-memory atomic adds.  The
-// accumulator is flushed to y once, with global atomic adds (split-K merge, Section 3.1).
-// ------------------------------------------------------------------------------------------------
+// One chunk of a whole column (COLUMN layout): Algorithm 1 for the parity decoder; the product's own kernel is in
+// celty_column.cuh.
 struct ColumnChunk {
     uint4 v;
     uint32_t even, odd;
@@ -194,45 +188,6 @@ __device__ __forceinline__ ColumnChunk load_column_chunk(const uint8_t *col, uin
     ch.row0 = carry + sum - span;
     carry += __shfl_sync(kFull, sum, 31);
     return ch;
-}
-
-__global__ void __launch_bounds__(256)
-k_spmspv_column(const uint2 *__restrict__ meta, const uint8_t *__restrict__ stream,
-                const int32_t *__restrict__ idx, const uint16_t *__restrict__ val,
-                const int32_t *__restrict__ count, float *__restrict__ y, int M, uint32_t *status)
-{
-    extern __shared__ float acc[];
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = blockDim.x >> 5;
-    for (int i = tid; i < M; i += blockDim.x) acc[i] = 0.f;
-    __syncthreads();
-    const int n = *count;
-    const int p0 = (int)((int64_t)blockIdx.x * n / gridDim.x);
-    const int p1 = (int)((int64_t)(blockIdx.x + 1) * n / gridDim.x);
-    for (int p = p0 + warp; p < p1; p += nwarps) {
-        const int j = idx[p];
-        const float xj = __half2float(__ushort_as_half(val[p]));
-        const uint2 mj = meta[j];
-        const uint8_t *col = stream + (size_t)mj.x * 16;
-        const uint32_t nent = mj.y, groups = (nent + kGroup - 1) / kGroup;
-        uint32_t carry = 0;
-        for (uint32_t c = 0; c * kChunkGroups < groups; ++c) {
-            const ColumnChunk ch = load_column_chunk(col, groups, c, lane, carry);
-            const uint32_t e0 = (c * kChunkGroups + lane) * kGroup;
-#pragma unroll
-            for (int e = 0; e < kGroup; ++e) {
-                if (e0 + e < nent) {
-                    const uint32_t row = ch.row0 + entry_offset(ch.even, ch.odd, e);
-                    if (row < (uint32_t)M) atomicAdd(&acc[row], entry_value(ch.v, e) * xj);
-                    else atomicOr(status, kStatusBounds);
-                }
-            }
-        }
-    }
-    __syncthreads();
-    for (int i = tid; i < M; i += blockDim.x) {
-        const float v = acc[i];
-        if (v != 0.f) atomicAdd(&y[i], v);
-    }
 }
 
 __global__ void k_decode_column(const uint2 *__restrict__ meta, const uint8_t *__restrict__ stream, int j,
@@ -503,6 +458,34 @@ int ensure_smem(Kernel kernel, size_t bytes, int *granted /* [64], per device */
 }
 
 #include "celty_fused.cuh"
+#include "celty_column.cuh"
+
+// y = 0, for the products whose blocks do not clear y themselves.  Bound by its launch: it may be scheduled while the
+// previous kernel of the stream drains and lets the next one do the same.
+__global__ void __launch_bounds__(256) k_clear(float *__restrict__ y, int M)
+{
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    const int i = (blockIdx.x * 256 + threadIdx.x) * 4;
+    if (i + 3 < M) *reinterpret_cast<float4 *>(y + i) = make_float4(0.f, 0.f, 0.f, 0.f);
+    else
+        for (int k = i; k < M; ++k) y[k] = 0.f;
+}
+
+int launch_clear(float *y, int64_t M, cudaStream_t st)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)((M + 1023) / 1024));
+    cfg.blockDim = dim3(256);
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    CELTY_CUDA(cudaLaunchKernelEx(&cfg, k_clear, y, (int)M));
+    return CELTY_OK;
+}
 
 int launch_compact(const void *x, int64_t K, float tau, int32_t *idx, uint16_t *val, int32_t *count, float *y,
                    int64_t M, cudaStream_t st)
@@ -591,6 +574,33 @@ int plan_fused(const celty_matrix *m, const LaunchKnobs &knobs, const DeviceInfo
     pl.mix = 1;
     *out = pl;
     return CELTY_OK;
+}
+
+// Warps per column and columns in flight of the COLUMN kernel.
+struct ColumnShape { int W, groups, cap, own_list; size_t smem; };
+
+ColumnShape column_shape(const celty_matrix *m, const DeviceInfo &di, int grid)
+{
+    ColumnShape s{};
+    const size_t budget = (size_t)di.max_smem_optin;
+    // as many warps as a column of average length has chunks of 256 entries (a tenth of a chunk does not get a warp
+    // of its own), in as few passes over the column as 32 warps allow
+    const double chunks = (double)m->stream_bytes / 20.0 / (double)m->K / kChunkGroups;
+    const int passes = std::max(1, (int)std::ceil((chunks - 0.1) / 32.0));
+    s.W = std::min(32, std::max(1, (int)std::ceil((chunks - 0.1) / passes)));
+    const int64_t columns = (m->K + grid - 1) / grid;                     // a block has, at most
+    s.cap = (int)std::min<int64_t>(1024, columns + 1);
+    s.groups = (int)std::min<int64_t>(columns, s.W > 1 ? std::min(15, 32 / s.W) : 32);   // 15: named barriers
+    for (s.own_list = 1; s.own_list >= 0; --s.own_list) {
+        // thresholding in the blocks needs 8 bytes per 32 activations; where they leave no room: k_compact
+        if (s.own_list && m->K > 262144) continue;
+        for (int g = s.groups; g >= 1; --g) {
+            s.smem = column_smem_layout((int)m->M, (int)m->K, g, s.cap, s.own_list).total;
+            if (s.smem <= budget) { s.groups = g; return s; }
+        }
+    }
+    s.groups = 0;
+    return s;
 }
 
 // How many clusters of `cl` blocks of the fused kernel (with `smem` bytes of dynamic shared memory each) the
@@ -876,16 +886,42 @@ int run_product(celty_matrix *m, const void *x_dev, float tau, const ListInput *
     // two launches: compaction (which also clears y), then the product.  Sizes are checked and the
     // shared-memory limit is raised before the first launch, so that an error return leaves y untouched.
     if (m->layout == CELTY_LAYOUT_COLUMN) {
-        const size_t smem = (size_t)m->M * 4;
-        if (smem > (size_t)di.max_smem_optin) return CELTY_EINVAL;
-        rc = ensure_smem(k_spmspv_column, smem, g_granted_column);
+        const int grid = m->grid > 0 ? m->grid : di.sms;
+        const ColumnShape shape = column_shape(m, di, grid);
+        if (shape.groups == 0) return CELTY_EINVAL;
+        ColumnParams cp{};
+        cp.meta = reinterpret_cast<const uint2 *>(m->d_image);
+        cp.stream = stream_base;
+        cp.x = static_cast<const uint16_t *>(x_dev);
+        cp.tau = tau;
+        cp.idx = idx; cp.val = val; cp.count = count; cp.status = status;
+        cp.y = y;
+        cp.spin_limit = m->spin_limit ? m->spin_limit : kSpinLimit;
+        if (shape.own_list && grid <= di.sms) {
+            cp.ticket = status + 2;
+            if (m->last_grid != grid || m->last_merge != 1) {   // the ticket counts blocks of one launch shape
+                CELTY_CUDA(cudaMemsetAsync(cp.ticket, 0, 4, st));
+                m->last_grid = grid;
+                m->last_merge = 1;
+            }
+        }
+        cp.M = (int)m->M; cp.K = (int)m->K;
+        cp.W = shape.W; cp.groups = shape.groups; cp.cap = shape.cap; cp.own_list = shape.own_list;
+        rc = ensure_smem(k_spmspv_column, shape.smem, g_granted_column);
         if (rc) return rc;
-        rc = launch_compact(x_dev, m->K, tau, idx, val, count, y, m->M, st);
+        if (!cp.ticket) rc = shape.own_list ? launch_clear(y, m->M, st) : launch_compact(x_dev, m->K, tau, idx, val, count, y, m->M, st);
         if (rc) return rc;
-        const int per_sm = (int)std::max<size_t>(1, std::min<size_t>(8, (size_t)(di.max_smem_optin) / (smem + 1024)));
-        const int grid = m->grid > 0 ? m->grid : di.sms * per_sm;
-        k_spmspv_column<<<grid, 256, smem, st>>>(reinterpret_cast<const uint2 *>(m->d_image), stream_base, idx, val,
-                                                  count, y, (int)m->M, status);
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3((unsigned)grid);
+        cfg.blockDim = dim3(kColumnThreads);
+        cfg.dynamicSmemBytes = shape.smem;
+        cfg.stream = st;
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[0].val.programmaticStreamSerializationAllowed = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        CELTY_CUDA(cudaLaunchKernelEx(&cfg, k_spmspv_column, cp));
     } else {
         const size_t group_bytes = (size_t)m->S * (m->R + kTileSlack) * 32 * 4;
         if (group_bytes > (size_t)di.max_smem_optin) return CELTY_EINVAL;

@@ -570,3 +570,38 @@ def test_host_buffer_entry_point():
     xh2 = torch.from_numpy(xo).pin_memory()
     m2.spmspv_host(xh2, tau, yh, xs, ys)
     _check_y(yh.numpy(), Wo, mo, xo, tau)
+
+
+@pytest.mark.parametrize("M,K,d_w,d_a,grid", [
+    (256, 150, 1.0, 1.0, 0),          # every column exactly one chunk of 256 entries, one warp per column
+    (257, 40, 1.0, 1.0, 0),           # ... and one entry more
+    (511, 2000, 0.9, 0.9, 3),         # more columns per block than it looks up at a time (three blocks)
+    (3, 5000, 0.5, 0.5, 1),           # one block, tiny columns
+    (8192, 64, 1.0, 1.0, 0),          # 32 warps per column
+    (8200, 64, 1.0, 1.0, 0),          # a second pass over the column for one group of entries
+    (49152, 37, 0.4, 1.0, 0),         # the tallest accumulator
+    (40001, 300, 0.02, 0.7, 0),       # padding entries; M not a multiple of 4
+    (2, 262145, 0.5, 0.001, 0),       # the list comes from the compaction kernel
+])
+def test_column_kernel_over_its_range(M, K, d_w, d_a, grid):
+    """Integer data, so every sum is exact: the edges of a chunk and of a pass over a column, warps per column from
+    one to 32, batches of columns, both ways to the list (which is compared as well)."""
+    W = synth.integer_weights(21, M, K)
+    mask = synth.mask_bernoulli(21, M, K, d_w) if d_w < 1 else np.ones((M, K), np.uint8)
+    x = synth.integer_activations(22, K)
+    if d_a == 1.0:
+        x[x == 0] = 2
+    elif d_a < 0.1:
+        x[np.arange(K) % int(1 / d_a) != 0] = 0
+    m = celty.Matrix(W, mask, layout=celty.LAYOUT_COLUMN, device="cuda")
+    m.set_launch(grid=grid)
+    y_ref, _ = orc.masked_gemv(W, mask, x, 0.5, threads=8)
+    oi, ov, _ = orc.compact(x, 0.5)
+    xd = torch.from_numpy(x).cuda()
+    for _ in range(2):
+        y = m.spmspv(xd, 0.5, y=torch.full((M,), 5.0, device="cuda"))
+        torch.cuda.synchronize()
+        assert m.last_status() == 0
+        assert np.array_equal(y.cpu().numpy().astype(np.float64), y_ref)
+        idx, val = m.last_compaction()
+        assert np.array_equal(idx.cpu().numpy(), oi) and np.array_equal(val.cpu().numpy().view(np.uint16), ov)
