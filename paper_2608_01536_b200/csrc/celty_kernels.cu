@@ -1024,15 +1024,34 @@ extern "C" int celty_spmspv_static(const celty_matrix *m, const void *image_dev,
     const int G = (int)std::max<size_t>(1, std::min<size_t>((size_t)di.max_smem_optin / group_bytes,
                                                              (size_t)std::max<int64_t>(1, 8 / m->S)));
     const size_t smem = group_bytes * G;
-    rc = ensure_smem(k_spmspv_lane, smem, g_granted_lane);
-    if (rc) return rc;
     int32_t *count = reinterpret_cast<int32_t *>(scratch) + 1;
     int32_t *idx = reinterpret_cast<int32_t *>(scratch + 256);
     uint16_t *val = reinterpret_cast<uint16_t *>(scratch + 256 + (size_t)kStaticMaxK * 4);
     float *y = static_cast<float *>(y_dev);
+    const uint8_t *image = static_cast<const uint8_t *>(image_dev);
+    // The single-launch kernel with its ticket in the shared array.  Every block of every call takes the ticket exactly
+    // once and all calls have one block per SM, so the count is back at a multiple of that after any call, also after
+    // calls that overlapped in spite of the rule above.  4096 x 4096, 50 % / 50 %: 28.7 us with the two kernels below,
+    // 8.4 us this way.  The handle's launch choices are for its workspace's calls and are not looked at.
+    FusedPlan plan;
+    const LaunchKnobs knobs;
+    rc = plan_launch(m, knobs, di, 1, &plan);
+    if (rc == CELTY_OK && plan.lean && plan.grid == std::min(di.sms, kMaxBlocks)) {
+        FusedParams fp = plan_params(m, knobs, plan, image);
+        fp.x = static_cast<const uint16_t *>(x_dev);
+        fp.tau = tau;
+        fp.y = y;
+        fp.idx = idx; fp.val = val; fp.count = count;
+        fp.status = reinterpret_cast<uint32_t *>(scratch);
+        fp.tickets = fp.status + 2;
+        return plan.lean == 2 ? launch_fused(k_spmspv_fused<false, 0, 2>, g_granted_lean[1], knobs, plan, 1, fp, st)
+                              : launch_fused(k_spmspv_fused<false, 0, 1>, g_granted_lean[0], knobs, plan, 1, fp, st);
+    }
+    // tiles and slabs per block for which not even one team's accumulators and ring slots fit together
+    rc = ensure_smem(k_spmspv_lane, smem, g_granted_lane);
+    if (rc) return rc;
     rc = launch_compact(x_dev, m->K, tau, idx, val, count, y, m->M, st);     // also clears y
     if (rc) return rc;
-    const uint8_t *image = static_cast<const uint8_t *>(image_dev);
     k_spmspv_lane<<<di.sms, 32 * (int)m->S * G, smem, st>>>(reinterpret_cast<const uint32_t *>(image),
                                                             image + m->meta_bytes, idx, val, count, y, (int)m->M, m->R,
                                                             (int)m->S, m->C, G);

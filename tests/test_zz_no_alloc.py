@@ -91,6 +91,26 @@ def test_static_and_two_launch_entry_points_share_one_kernel_attribute():
         assert np.all(np.abs(y.cpu().numpy().astype(np.float64) - y_ref) <= 2e-3 * a_ref + 1e-6), (W.shape, static)
 
 
+@pytest.mark.parametrize("M,K,kw", [(1, 1, {}), (33, 8, {}), (1025, 2049, {}), (49152, 16, {}), (300, 32768, {}),
+                                     (28672, 64, {}), (20000, 100, {}), (3000, 40, dict(tile_rows=240)),
+                                     (7000, 40, dict(tile_rows=200, slabs_per_block=2)),
+                                     (40000, 24, dict(tile_rows=240, slabs_per_block=6))])   # the last: two launches
+def test_static_entry_point_over_its_range(M, K, kw):
+    """Integer data, so every sum is exact: the smallest sizes, the limits, row parts that leave blocks over, and a
+    shape that the single-launch kernel has no room for; the handle's launch choices change nothing."""
+    build.build()
+    W = synth.integer_weights(3, M, K)
+    mask = synth.mask_bernoulli(3, M, K, 0.6)
+    x = synth.integer_activations(4, K)
+    m = celty.Matrix(W, mask, device="cuda", **kw)
+    y_ref, _ = orc.masked_gemv(W, mask, x, 1.0, threads=8)
+    xd = torch.from_numpy(x).cuda()
+    for variant in (0, 2, 1, 0):
+        m.set_launch(variant=variant)
+        y = m.spmspv_static(xd, 1.0, y=torch.full((M,), 7.0, device="cuda"))
+        assert np.array_equal(y.cpu().numpy().astype(np.float64), y_ref), variant
+
+
 def test_static_scratch_entry_point_rejects_what_it_cannot_hold():
     build.build()
     lib = celty.load()
