@@ -195,7 +195,7 @@ int celty_compact(const void *x_dev, int64_t K, float tau, int32_t *idx_dev, uin
 int celty_spmspv(celty_matrix *m, const void *x_dev, float tau, void *y_dev, celty_stream_t stream);
 
 /*
- * Work on y after the merge, inside the same launch (LANE_TILE handles, single-launch kernel, bulk reduce-add
+ * Work on y after the merge, by a small kernel enqueued behind the product's in the same call (LANE_TILE handles, single-launch kernel, bulk reduce-add
  * merge).  Section 6.2 times the seven products of a decode layer; between the gate/up and the down projection of
  * its MLP sits SiLU(gate) * up, and every product's output feeds FP16 consumers.
  *   CELTY_EPILOGUE_FP16    out_fp16[i] = y[i] rounded to FP16 (nearest even), i < M; y keeps the FP32 values.
@@ -221,7 +221,7 @@ typedef struct {
 } celty_epilogue;
 
 /*
- * celty_spmspv_ex -- celty_spmspv followed, in the same launch, by the work `ep` describes (NULL = none).
+ * celty_spmspv_ex -- celty_spmspv followed, in the same call, by the work `ep` describes (NULL = none).
  * Errors: those of celty_spmspv; CELTY_EINVAL also for a COLUMN handle, the two-launch or the ordered-merge
  * variant, a missing output pointer, an odd M with SWIGLU.
  */

@@ -22,8 +22,8 @@
 //       their sums through distributed shared memory, each block then sending only the segments it owns
 //       (measured: no faster, so off by default); per-block partial vectors, a bounded grid-wide ticket
 //       barrier and a sum in a fixed order (bit-reproducible, no clearing of y).
-//   then, on request: an FP16 copy of y, or SiLU(gate) * up of a stacked [gate; up] product with its
-//       thresholded list (fused_epilogue), once a second ticket shows that every block's adds are done.
+//   then, on request, in a kernel of its own: an FP16 copy of y, or SiLU(gate) * up of a stacked [gate; up] product
+//       with its thresholded list (k_epilogue).
 //
 // Rows are split over P parts of Sc slabs each, columns over the blocks of a part and, inside a block, over
 // G teams per slab; a team = one warp (or, with pp, two warps that take turns) with its own accumulator slab.
@@ -252,8 +252,6 @@ __device__ __forceinline__ void step_finish(const StepBuf &b, uint16_t xj)
     for (int e = 0; e < 8; ++e) sts_f32(b.a[e], d[e]);
 }
 
-// Work on the finished y (FusedParams::ep_kind), every block on an equal share of the rows.  A function of its own
-// (not inlined), so that what it needs in registers does not weigh on the streaming loop of the kernel.
 // SiLU(gate) * up evaluated in FP32 and rounded once to FP16 (bit pattern): the one formula behind the work after
 // a gate/up product and behind the down projection that makes its activations on the fly.
 __device__ __forceinline__ uint32_t swiglu_half_bits(float gate, float up)
@@ -275,89 +273,71 @@ __device__ __noinline__ uint4 ragged_group(const uint16_t *x, int K, int q)
     return make_uint4(h[0], h[1], h[2], h[3]);
 }
 
+// Work on the finished y (celty_epilogue), a kernel of its own behind the product:
+//   kind 1  out = y rounded to FP16;
+//   kind 2  y holds a stacked [gate; up] product of 2I rows: out_i = SiLU(y_i) * y_{I+i} rounded to FP16, and the (i,
+//           out_i) with |out_i| > tau appended to a list that the next product takes as its survivors (the product's
+//           kernel has set the count to zero).
+// As a programmatic dependent launch its few small blocks sit beside the product's while that runs, and what is left
+// of the step is one trip to L2 for y after the product's last block is gone.  As the end of the product's own launch
+// it needed a second ticket of all blocks, a poll of it and a block barrier on either side, and the larger build of
+// the streaming loop: 11008 x 4096 with the FP16 copy 16.1 us in one launch, 13.6 us this way (plain product
+// 11.8).
 struct EpilogueArgs {
     const float *y;
-    uint32_t *tickets, *status;
-    uint32_t spin_limit;
-    int M, ep_kind;
-    uint16_t *ep_out;
-    float ep_tau;
-    int32_t *ep_idx;
-    uint16_t *ep_val;
-    int32_t *ep_count;
+    int M, kind;
+    uint16_t *out;
+    float tau;
+    int32_t *idx;
+    uint16_t *val;
+    int32_t *count;
 };
 
-__device__ __noinline__ void fused_epilogue(const EpilogueArgs p)
+constexpr int kEpilogueThreads = 256;
+
+__global__ void __launch_bounds__(kEpilogueThreads) k_epilogue(const EpilogueArgs p)
 {
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nthreads = blockDim.x, nwarps = nthreads >> 5;
-    // ---- work on the finished y.  This block's adds must have been performed (not merely read out of shared
-    // memory), then every block's: a second wrap-around ticket, as for the clearing of y.
-    asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
-    __threadfence();
-    __syncthreads();
-    __shared__ int ep_warp[17];
-    if (tid == 0) {
-        __threadfence();
-        const uint32_t t = atomicInc(&p.tickets[1], 2u * gridDim.x - 1u);
-        const bool low_half = t < gridDim.x;
-        bool ok = false;
-        for (uint32_t it = 0; it < p.spin_limit; ++it) {
-            const uint32_t cur = ld_relaxed_u32(&p.tickets[1]);
-            if (low_half ? (cur >= gridDim.x) : (cur < gridDim.x)) { ok = true; break; }
-            __nanosleep(64);
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    if (p.kind == 1) {
+        const int i = (blockIdx.x * kEpilogueThreads + tid) * 4;
+        if (i + 3 < p.M && ((uintptr_t)p.out & 7) == 0) {
+            const float4 v = __ldcg(reinterpret_cast<const float4 *>(p.y + i));
+            const __half2 a = __floats2half2_rn(v.x, v.y), b = __floats2half2_rn(v.z, v.w);
+            *reinterpret_cast<uint2 *>(p.out + i) = make_uint2(*reinterpret_cast<const uint32_t *>(&a), *reinterpret_cast<const uint32_t *>(&b));
+        } else {
+            for (int k = i; k < min(i + 4, p.M); ++k) p.out[k] = __half_as_ushort(__float2half_rn(__ldcg(p.y + k)));
         }
-        __threadfence();
-        if (!ok) atomicOr(p.status, kStatusTimeout);
-    }
-    __syncthreads();
-    // every block takes an equal share of the rows; y is read past L1 (it was written by adds in L2)
-    if (p.ep_kind == 1) {
-        // (shares without a 64-bit division: n / blocks rows each, the first n mod blocks one more)
-        const int per = p.M / (int)gridDim.x, extra = p.M - per * (int)gridDim.x, b = (int)blockIdx.x;
-        const int r0 = b * per + min(b, extra), r1 = r0 + per + (b < extra ? 1 : 0);
-        for (int i = r0 + tid; i < r1; i += nthreads) p.ep_out[i] = __half_as_ushort(__float2half_rn(__ldcg(p.y + i)));
         return;
     }
-    const int half_rows = p.M / 2;
-    const int per = half_rows / (int)gridDim.x, extra = half_rows - per * (int)gridDim.x, b = (int)blockIdx.x;
-    const int r0 = b * per + min(b, extra), r1 = r0 + per + (b < extra ? 1 : 0);
-    for (int base = r0; base < r1; base += nthreads) {          // the same trip count for every thread
-        const int i = base + tid;
-        bool keep = false;
-        uint16_t hb = 0;
-        if (i < r1) {
-            const float gt = __ldcg(p.y + i), up = __ldcg(p.y + half_rows + i);
-            const __half h = __float2half_rn(gt / (1.f + expf(-gt)) * up);       // SiLU(gate) * up, one FP16 value
-            hb = __half_as_ushort(h);
-            p.ep_out[i] = hb;
-            keep = !(fabsf(__half2float(h)) <= p.ep_tau);                       // the comparator of a1
-        }
-        // positions in the list: within the warp by ballot, across the warps by a small scan, across the blocks
-        // by one atomic add per block and pass (the list comes out in no particular order)
-        const uint32_t bal = __ballot_sync(kFull, keep);
-        if (lane == 0) ep_warp[warp] = __popc(bal);
-        __syncthreads();
-        if (tid == 0) {
-            int total = 0;
-            for (int w = 0; w < nwarps; ++w) {
-                const int c = ep_warp[w];
-                ep_warp[w] = total;
-                total += c;
-            }
-            ep_warp[16] = total ? atomicAdd(p.ep_count, total) : 0;
-        }
-        __syncthreads();
-        if (keep) {
-            const int pos = ep_warp[16] + ep_warp[warp] + __popc(bal & ((1u << lane) - 1u));
-            p.ep_idx[pos] = i;
-            p.ep_val[pos] = hb;
-        }
-        __syncthreads();
+    __shared__ int warp_tot[kEpilogueThreads / 32], base;
+    const int rows = p.M / 2, i = blockIdx.x * kEpilogueThreads + tid;
+    bool keep = false;
+    uint16_t hb = 0;
+    if (i < rows) {
+        hb = (uint16_t)swiglu_half_bits(__ldcg(p.y + i), __ldcg(p.y + rows + i));
+        p.out[i] = hb;
+        keep = !(fabsf(__half2float(__ushort_as_half(hb))) <= p.tau);        // the comparator of a1
+    }
+    // positions in the list: within the warp by ballot, across the warps by a sum, across the blocks by one atomic add
+    // per block (the list comes out in no particular order)
+    const uint32_t bal = __ballot_sync(kFull, keep);
+    if (lane == 0) warp_tot[warp] = __popc(bal);
+    __syncthreads();
+    const int t = lane < kEpilogueThreads / 32 ? warp_tot[lane] : 0;
+    const int before = __reduce_add_sync(kFull, lane < warp ? t : 0), all = __reduce_add_sync(kFull, t);
+    if (tid == 0) base = all ? atomicAdd(p.count, all) : 0;
+    __syncthreads();
+    if (keep) {
+        const int pos = base + before + __popc(bal & ((1u << lane) - 1u));
+        p.idx[pos] = i;
+        p.val[pos] = hb;
     }
 }
 
-// kExtras = false compiles the list input and the work after the merge out: the plain product keeps its
-// register budget (92 registers against 128 with them), which the streaming loop's scheduling depends on.
+// kExtras = false compiles the list input and the making of x from gate and up out: the plain product keeps its
+// register budget, which the streaming loop's scheduling depends on.
 // kRegRows > 0 is the software analogue of register-file accumulation (Section 4.1, the register / shared-memory
 // split of Section 6.4): the first kRegRows local rows of every lane are summed in registers across the team's
 // columns and written to the accumulator slab once, at the end.  Those builds run 256 threads per block (eight
@@ -496,7 +476,7 @@ __global__ void __launch_bounds__(kRegRows > 0 ? 256 : 512, 1) k_spmspv_fused(co
         const int r0 = b * p.clear_rows + min(b, p.clear_extra), r1 = r0 + p.clear_rows + (b < p.clear_extra ? 1 : 0);
 #pragma unroll 1
         for (int i = r0 + lane; i < r1; i += 32) y[i] = 0.f;
-        if (kExtras && p.ep_kind == 2 && blockIdx.x == 0 && lane == 0) *p.ep_count = 0;   // appended to after the merge
+        if (!kBatch && blockIdx.x == 0 && lane == 0 && p.ep_count) *p.ep_count = 0;      // k_epilogue appends to it
         __syncwarp();
         if (lane == 0) {
             __threadfence();
@@ -890,9 +870,6 @@ __global__ void __launch_bounds__(kRegRows > 0 ? 256 : 512, 1) k_spmspv_fused(co
             asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");   // shared memory may go once it has been read
         }
         if (cl > 1) cluster_sync();                               // no block leaves while a peer may still read it
-        if (!kExtras || p.ep_kind == 0) return;
-        fused_epilogue(EpilogueArgs{y, tickets, p.status, p.spin_limit, p.M, p.ep_kind, p.ep_out, p.ep_tau, p.ep_idx,
-                                    p.ep_val, p.ep_count});
         return;
     }
     {

@@ -106,7 +106,7 @@ struct FusedParams {
     uint16_t *val;
     int32_t *count;
     uint32_t *status;
-    uint32_t *tickets;         // [0] y cleared / partial stored, [1] adds done (work after the merge) / departed
+    uint32_t *tickets;         // [0] y cleared / partial stored, [1] departed (ordered merge)
     float *partials;           // gridDim.x vectors of Sc * R * 32 floats (accumulator layout)
     int M, K, R, S, C;         // rows, columns, local rows per tile, slabs, chunk of the row map (tile_row)
     int G, Sc, P, D;           // teams per slab, slabs per block, row parts, ring depth
@@ -142,15 +142,7 @@ struct FusedParams {
     // h_out (may be null) receives a copy.
     const float *swiglu_in;
     uint16_t *h_ws, *h_out;
-    // Work on y after the merge (bulk reduce-add merge only): 0 none; 1 an FP16 copy of y; 2 y holds a stacked
-    // [gate; up] product of 2I rows: h_i = SiLU(y_i) * y_{I+i} rounded to FP16, stored, and the (i, h_i) with
-    // |h_i| > ep_tau appended to a list that the next product takes as its survivors
-    int ep_kind;
-    uint16_t *ep_out;
-    float ep_tau;
-    int32_t *ep_idx;
-    uint16_t *ep_val;
-    int32_t *ep_count;
+    int32_t *ep_count;         // not null: set to zero for the list that k_epilogue appends to after this kernel
 };
 
 // Shape of a fused launch (plan_fused).

@@ -807,6 +807,30 @@ int check_epilogue(const celty_matrix *m, const celty_epilogue *ep)
     return CELTY_OK;
 }
 
+int launch_epilogue(const celty_matrix *m, const celty_epilogue *ep, const float *y, cudaStream_t st)
+{
+    EpilogueArgs a{};
+    a.y = y;
+    a.M = (int)m->M;
+    a.kind = ep->kind;
+    a.out = static_cast<uint16_t *>(ep->out_fp16);
+    a.tau = ep->tau;
+    a.idx = ep->list_idx; a.val = ep->list_val; a.count = ep->list_count;
+    const int per_block = ep->kind == CELTY_EPILOGUE_FP16 ? 4 * kEpilogueThreads : kEpilogueThreads;
+    const int64_t n = ep->kind == CELTY_EPILOGUE_FP16 ? m->M : m->M / 2;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)((n + per_block - 1) / per_block));
+    cfg.blockDim = dim3(kEpilogueThreads);
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = m->no_overlap ? 0 : 1;
+    CELTY_CUDA(cudaLaunchKernelEx(&cfg, k_epilogue, a));
+    return CELTY_OK;
+}
+
 // The product for every entry point: x thresholded by the kernel (list == nullptr) or the survivors given as a
 // list; optional work on y after the merge.
 int run_product(celty_matrix *m, const void *x_dev, float tau, const ListInput *list, void *y_dev,
@@ -849,14 +873,8 @@ int run_product(celty_matrix *m, const void *x_dev, float tau, const ListInput *
             fp.h_ws = reinterpret_cast<uint16_t *>(m->d_ws + m->ws.partial_off);
             fp.h_out = sw->h_out;
         }
-        if (ep && ep->kind != CELTY_EPILOGUE_NONE) {
-            fp.ep_kind = ep->kind;
-            fp.ep_out = static_cast<uint16_t *>(ep->out_fp16);
-            fp.ep_tau = ep->tau;
-            fp.ep_idx = ep->list_idx;
-            fp.ep_val = ep->list_val;
-            fp.ep_count = ep->list_count;
-        }
+        const bool after = ep && ep->kind != CELTY_EPILOGUE_NONE;
+        if (after && ep->kind == CELTY_EPILOGUE_SWIGLU) fp.ep_count = ep->list_count;
         fp.x = static_cast<const uint16_t *>(x_dev);           // not looked at when the survivors come as a list
         fp.tau = tau;
         fp.y = y;
@@ -868,20 +886,21 @@ int run_product(celty_matrix *m, const void *x_dev, float tau, const ListInput *
             m->last_grid = plan.grid;
             m->last_merge = plan.merge;
         }
-        if (extras)
-            return plan.lean == 2 ? launch_fused(k_spmspv_fused<true, 0, 2>, g_granted_lean_extras[1], *m, plan, 1, fp, st)
-                 : plan.lean == 1 ? launch_fused(k_spmspv_fused<true, 0, 1>, g_granted_lean_extras[0], *m, plan, 1, fp, st)
-                                  : launch_fused(k_spmspv_fused<true, 0>, g_granted_fused_extras, *m, plan, 1, fp, st);
-        switch (m->reg_rows) {
-            case 32: return launch_fused(k_spmspv_fused<false, 32>, g_granted_reg[0], *m, plan, 1, fp, st);
-            case 64: return launch_fused(k_spmspv_fused<false, 64>, g_granted_reg[1], *m, plan, 1, fp, st);
-            case 96: return launch_fused(k_spmspv_fused<false, 96>, g_granted_reg[2], *m, plan, 1, fp, st);
-            case 128: return launch_fused(k_spmspv_fused<false, 128>, g_granted_reg[3], *m, plan, 1, fp, st);
-            default: break;
-        }
-        return plan.lean == 2 ? launch_fused(k_spmspv_fused<false, 0, 2>, g_granted_lean[1], *m, plan, 1, fp, st)
-             : plan.lean == 1 ? launch_fused(k_spmspv_fused<false, 0, 1>, g_granted_lean[0], *m, plan, 1, fp, st)
-                              : launch_fused(k_spmspv_fused<false, 0>, g_granted_fused, *m, plan, 1, fp, st);
+        // the list input and the making of x from gate and up have builds of their own
+        if (list || sw)
+            rc = plan.lean == 2 ? launch_fused(k_spmspv_fused<true, 0, 2>, g_granted_lean_extras[1], *m, plan, 1, fp, st)
+               : plan.lean == 1 ? launch_fused(k_spmspv_fused<true, 0, 1>, g_granted_lean_extras[0], *m, plan, 1, fp, st)
+                                : launch_fused(k_spmspv_fused<true, 0>, g_granted_fused_extras, *m, plan, 1, fp, st);
+        else if (m->reg_rows)
+            rc = m->reg_rows == 32 ? launch_fused(k_spmspv_fused<false, 32>, g_granted_reg[0], *m, plan, 1, fp, st)
+               : m->reg_rows == 64 ? launch_fused(k_spmspv_fused<false, 64>, g_granted_reg[1], *m, plan, 1, fp, st)
+               : m->reg_rows == 96 ? launch_fused(k_spmspv_fused<false, 96>, g_granted_reg[2], *m, plan, 1, fp, st)
+                                   : launch_fused(k_spmspv_fused<false, 128>, g_granted_reg[3], *m, plan, 1, fp, st);
+        else
+            rc = plan.lean == 2 ? launch_fused(k_spmspv_fused<false, 0, 2>, g_granted_lean[1], *m, plan, 1, fp, st)
+               : plan.lean == 1 ? launch_fused(k_spmspv_fused<false, 0, 1>, g_granted_lean[0], *m, plan, 1, fp, st)
+                                : launch_fused(k_spmspv_fused<false, 0>, g_granted_fused, *m, plan, 1, fp, st);
+        return rc || !after ? rc : launch_epilogue(m, ep, y, st);
     }
     // two launches: compaction (which also clears y), then the product.  Sizes are checked and the
     // shared-memory limit is raised before the first launch, so that an error return leaves y untouched.
