@@ -2,6 +2,8 @@
 #pragma once
 #include <cstddef>
 #include <cstdint>
+#include <cstring>
+#include <memory>
 #include <vector>
 
 #include "celty.h"
@@ -45,6 +47,22 @@ CELTY_HD inline int64_t tile_row(int64_t S, int64_t C, int64_t s, int64_t lane, 
 {
     return (((i / C) * S + s) * C + i % C) * 32 + lane;
 }
+
+// Host bytes that are not cleared when they are allocated: the encoder's threads write (and so first touch) all of them.
+class Bytes {
+public:
+    Bytes() = default;
+    Bytes(const Bytes &o) { allocate(o.n_); if (n_) std::memcpy(p_.get(), o.p_.get(), n_); }
+    Bytes &operator=(const Bytes &) = delete;
+    void allocate(size_t n) { p_.reset(new uint8_t[n]); n_ = n; }
+    uint8_t *data() { return p_.get(); }
+    const uint8_t *data() const { return p_.get(); }
+    size_t size() const { return n_; }
+
+private:
+    std::unique_ptr<uint8_t[]> p_;
+    size_t n_ = 0;
+};
 
 // Workspace layout (device): all offsets multiples of 256.
 struct WorkspaceLayout {
@@ -188,7 +206,7 @@ struct celty_matrix : celty::LaunchKnobs {
     // image = [meta | stream]
     //   COLUMN:    meta = uint2[K]  {offset/16 of the column block in the stream, entries}
     //   LANE_TILE: meta = uint32[K*S + 1]  offset/16 of sub-block (j, s); sub-blocks are contiguous
-    std::vector<uint8_t> image;
+    celty::Bytes image;
     size_t meta_bytes = 0;             // stream starts at image[meta_bytes]
     size_t stream_bytes = 0;
     uint32_t max_unit16 = 0;           // largest column block / sub-block in 16-byte units

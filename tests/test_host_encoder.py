@@ -85,6 +85,37 @@ def test_encoder_matches_oracle_on_random_draws(case):
         assert np.array_equal(vals, ovals) and np.array_equal(runs, oruns) and np.array_equal(pad, opad)
 
 
+@pytest.mark.parametrize("M,K,d_w,layout,tile_rows", [
+    (4100, 65, 0.5, celty.LAYOUT_LANE_TILE, 0),       # a second block of 64 columns with one column, several threads
+    (4100, 64, 0.03, celty.LAYOUT_COLUMN, 0),         # padding entries across the 64-row words
+    (2100, 127, 0.05, celty.LAYOUT_LANE_TILE, 65),    # tiles of one word and one row
+    (2100, 129, 1.0, celty.LAYOUT_LANE_TILE, 64),
+    (24000, 17, 0.7, celty.LAYOUT_LANE_TILE, 0),      # tall enough for the encoder to look at the density
+])
+@pytest.mark.parametrize("with_mask", [True, False])
+def test_encoder_over_blocks_of_columns_and_threads(M, K, d_w, layout, tile_rows, with_mask):
+    W = synth.weights(M + K, M, K)
+    mask = synth.mask_bernoulli(M + K, M, K, d_w)
+    if not with_mask:
+        W[mask == 0] = np.float16(-0.0)
+        mask = ((W.view(np.uint16) & 0x7FFF) != 0).astype(np.uint8)
+    m = celty.Matrix(W, mask * np.uint8(200) if with_mask else None, layout=layout, tile_rows=tile_rows)
+    S, R, C = m.row_map()
+    if layout == celty.LAYOUT_LANE_TILE:
+        Wp, mp, rowmap = permute_for_lane_tiles(W, mask, S, R, C)
+        enc = orc.rlc_encode(Wp, mp, 4, tile_rows=R)
+    else:
+        rowmap = np.arange(M)
+        enc = orc.rlc_encode(W, mask, 4)
+    info = m.info()
+    assert info.nnz == int(mask.sum()) and info.n_pad == int(enc.is_pad.sum())
+    for j in range(K):
+        rows, vals, runs, pad = m.decode_host(j)
+        orows, ovals, opad, oruns = orc.column_entries(enc, j)
+        assert np.array_equal(rows, rowmap[orows]) and np.array_equal(vals, ovals)
+        assert np.array_equal(runs, oruns) and np.array_equal(pad, opad)
+
+
 def test_null_mask_keeps_nonzero_weights():
     W = synth.weights(3, 100, 11)
     W[::3] = 0
