@@ -277,7 +277,8 @@ __device__ __noinline__ uint4 ragged_group(const uint16_t *x, int K, int q)
 //   kind 1  out = y rounded to FP16;
 //   kind 2  y holds a stacked [gate; up] product of 2I rows: out_i = SiLU(y_i) * y_{I+i} rounded to FP16, and the (i,
 //           out_i) with |out_i| > tau appended to a list that the next product takes as its survivors (the product's
-//           kernel has set the count to zero).
+//           kernel has set the count to zero);
+//   kind 3  y_host = y, in page-locked host memory.
 // As a programmatic dependent launch its few small blocks sit beside the product's while that runs, and what is left
 // of the step is one trip to L2 for y after the product's last block is gone.  As the end of the product's own launch
 // it needed a second ticket of all blocks, a poll of it and a block barrier on either side, and the larger build of
@@ -286,6 +287,7 @@ __device__ __noinline__ uint4 ragged_group(const uint16_t *x, int K, int q)
 struct EpilogueArgs {
     const float *y;
     int M, kind;
+    float *y_host;
     uint16_t *out;
     float tau;
     int32_t *idx;
@@ -309,6 +311,14 @@ __global__ void __launch_bounds__(kEpilogueThreads) k_epilogue(const EpilogueArg
         } else {
             for (int k = i; k < min(i + 4, p.M); ++k) p.out[k] = __half_as_ushort(__float2half_rn(__ldcg(p.y + k)));
         }
+        return;
+    }
+    if (p.kind == 3) {
+        const int i = (blockIdx.x * kEpilogueThreads + tid) * 4;
+        if (i + 3 < p.M && ((uintptr_t)p.y_host & 15) == 0)
+            *reinterpret_cast<float4 *>(p.y_host + i) = __ldcg(reinterpret_cast<const float4 *>(p.y + i));
+        else
+            for (int k = i; k < min(i + 4, p.M); ++k) p.y_host[k] = __ldcg(p.y + k);
         return;
     }
     __shared__ int warp_tot[kEpilogueThreads / 32], base;

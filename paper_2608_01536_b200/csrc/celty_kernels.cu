@@ -1,5 +1,6 @@
 // CUDA half of the library (sm_100a): activation compaction, the two SpMSpV kernels, the decode
 // kernels used by parity tests, and the C-ABI entry points that launch them.
+#include <cuda.h>
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
@@ -807,17 +808,12 @@ int check_epilogue(const celty_matrix *m, const celty_epilogue *ep)
     return CELTY_OK;
 }
 
-int launch_epilogue(const celty_matrix *m, const celty_epilogue *ep, const float *y, cudaStream_t st)
+int launch_epilogue(const celty_matrix *m, EpilogueArgs a, const float *y, cudaStream_t st)
 {
-    EpilogueArgs a{};
     a.y = y;
     a.M = (int)m->M;
-    a.kind = ep->kind;
-    a.out = static_cast<uint16_t *>(ep->out_fp16);
-    a.tau = ep->tau;
-    a.idx = ep->list_idx; a.val = ep->list_val; a.count = ep->list_count;
-    const int per_block = ep->kind == CELTY_EPILOGUE_FP16 ? 4 * kEpilogueThreads : kEpilogueThreads;
-    const int64_t n = ep->kind == CELTY_EPILOGUE_FP16 ? m->M : m->M / 2;
+    const int per_block = a.kind == CELTY_EPILOGUE_SWIGLU ? kEpilogueThreads : 4 * kEpilogueThreads;
+    const int64_t n = a.kind == CELTY_EPILOGUE_SWIGLU ? m->M / 2 : m->M;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)((n + per_block - 1) / per_block));
     cfg.blockDim = dim3(kEpilogueThreads);
@@ -900,7 +896,13 @@ int run_product(celty_matrix *m, const void *x_dev, float tau, const ListInput *
             rc = plan.lean == 2 ? launch_fused(k_spmspv_fused<false, 0, 2>, g_granted_lean[1], *m, plan, 1, fp, st)
                : plan.lean == 1 ? launch_fused(k_spmspv_fused<false, 0, 1>, g_granted_lean[0], *m, plan, 1, fp, st)
                                 : launch_fused(k_spmspv_fused<false, 0>, g_granted_fused, *m, plan, 1, fp, st);
-        return rc || !after ? rc : launch_epilogue(m, ep, y, st);
+        if (rc || !after) return rc;
+        EpilogueArgs ea{};
+        ea.kind = ep->kind;
+        ea.out = static_cast<uint16_t *>(ep->out_fp16);
+        ea.tau = ep->tau;
+        ea.idx = ep->list_idx; ea.val = ep->list_val; ea.count = ep->list_count;
+        return launch_epilogue(m, ea, y, st);
     }
     // two launches: compaction (which also clears y), then the product.  Sizes are checked and the
     // shared-memory limit is raised before the first launch, so that an error return leaves y untouched.
@@ -1200,15 +1202,60 @@ extern "C" int celty_spmspv_batch(celty_matrix *m, const void *x_dev, int64_t ld
     return CELTY_OK;
 }
 
+namespace {
+
+constexpr int kEpilogueToHost = 3;
+
+// The device address of [p, p + bytes) if all of it is one range of page-locked host memory that the current device
+// can address, else null.
+void *mapped_host(const void *p, size_t bytes)
+{
+    using Query = CUresult (*)(unsigned, CUpointer_attribute *, void **, CUdeviceptr);
+    static const Query query = [] {
+        void *fn = nullptr;
+        cudaDriverEntryPointQueryResult found;
+        if (cudaGetDriverEntryPoint("cuPointerGetAttributes", &fn, cudaEnableDefault, &found) != cudaSuccess ||
+            found != cudaDriverEntryPointSuccess)
+            fn = nullptr;
+        return reinterpret_cast<Query>(fn);
+    }();
+    if (!query) return nullptr;
+    unsigned type = 0, managed = 0;
+    CUdeviceptr device = 0, start = 0;
+    size_t size = 0;
+    CUpointer_attribute what[5] = {CU_POINTER_ATTRIBUTE_MEMORY_TYPE, CU_POINTER_ATTRIBUTE_IS_MANAGED, CU_POINTER_ATTRIBUTE_DEVICE_POINTER,
+                                   CU_POINTER_ATTRIBUTE_RANGE_START_ADDR, CU_POINTER_ATTRIBUTE_RANGE_SIZE};
+    void *into[5] = {&type, &managed, &device, &start, &size};
+    if (query(5, what, into, (CUdeviceptr)(uintptr_t)p) != CUDA_SUCCESS) return nullptr;
+    if (type != CU_MEMORYTYPE_HOST || managed || !device || !start || device < start || size < bytes ||
+        device - start > size - bytes)
+        return nullptr;
+    return reinterpret_cast<void *>((uintptr_t)device);
+}
+
+}  // namespace
+
 extern "C" int celty_spmspv_host(celty_matrix *m, const void *x_host, float tau, void *y_host, void *x_stage_dev,
                                  void *y_stage_dev, celty_stream_t stream)
 {
     if (!m || !x_host || !y_host || !x_stage_dev || !y_stage_dev) return CELTY_EINVAL;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     CELTY_CUDA(cudaMemcpyAsync(x_stage_dev, x_host, (size_t)m->K * 2, cudaMemcpyHostToDevice, st));
-    const int rc = celty_spmspv(m, x_stage_dev, tau, y_stage_dev, stream);
+    int rc = celty_spmspv(m, x_stage_dev, tau, y_stage_dev, stream);
     if (rc) return rc;
-    CELTY_CUDA(cudaMemcpyAsync(y_host, y_stage_dev, (size_t)m->M * 4, cudaMemcpyDeviceToHost, st));
+    // y by a small kernel behind the product, where its place is page-locked: the copy engine takes several
+    // microseconds to take over from a kernel and to be waited for.  5120 x 5120: 29.5 us per call with a copy, 25.2 this
+    // way.  (The same for x pays nothing: fetched over the link by the product's blocks 30.1 us, as the parameters of a
+    // small kernel 27.3.)
+    EpilogueArgs out{};
+    out.kind = kEpilogueToHost;
+    out.y_host = static_cast<float *>(mapped_host(y_host, (size_t)m->M * 4));
+    if (out.y_host) {
+        rc = launch_epilogue(m, out, static_cast<const float *>(y_stage_dev), st);
+        if (rc) return rc;
+    } else {
+        CELTY_CUDA(cudaMemcpyAsync(y_host, y_stage_dev, (size_t)m->M * 4, cudaMemcpyDeviceToHost, st));
+    }
     CELTY_CUDA(cudaStreamSynchronize(st));
     return CELTY_OK;
 }

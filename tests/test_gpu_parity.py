@@ -605,3 +605,30 @@ def test_column_kernel_over_its_range(M, K, d_w, d_a, grid):
         assert np.array_equal(y.cpu().numpy().astype(np.float64), y_ref)
         idx, val = m.last_compaction()
         assert np.array_equal(idx.cpu().numpy(), oi) and np.array_equal(val.cpu().numpy().view(np.uint16), ov)
+
+
+@pytest.mark.parametrize("M,K,kw", [(1, 1, {}), (1000, 33, {}), (1026, 4099, {}), (28672, 72, {}),
+                                    (17, 131080, {}), (900, 200, dict(layout=celty.LAYOUT_COLUMN))])
+def test_host_vectors_pinned_and_pageable(M, K, kw):
+    """Integer data, so every sum is exact: vectors in page-locked memory (y stored there by a kernel, at an odd
+    place in a wider buffer too), in ordinary memory (copied) and one of each."""
+    W = synth.integer_weights(31, M, K)
+    mask = synth.mask_bernoulli(31, M, K, 0.5)
+    m = celty.Matrix(W, mask, device="cuda", **kw)
+    stage_x, stage_y = torch.empty(K, dtype=torch.float16, device="cuda"), torch.empty(M, device="cuda")
+    wide_x, wide_y = torch.zeros(K + 9, dtype=torch.float16).pin_memory(), torch.zeros(M + 7).pin_memory()
+    plain_x, plain_y = torch.zeros(K, dtype=torch.float16), torch.zeros(M)
+    for call, (xb, yb) in enumerate([(wide_x[:K], wide_y[:M]), (wide_x[3:K + 3], wide_y[1:M + 1]), (plain_x, plain_y),
+                                     (wide_x[:K], plain_y), (plain_x, wide_y[:M]), (wide_x[8:K + 8], wide_y[4:M + 4])]):
+        x = synth.integer_activations(32 + call, K)
+        y_ref, _ = orc.masked_gemv(W, mask, x, 1.0, threads=8)
+        xb.copy_(torch.from_numpy(x))
+        wide_y.fill_(-3.0)
+        m.spmspv_host(xb, 1.0, yb, stage_x, stage_y)
+        assert np.array_equal(yb.numpy().astype(np.float64), y_ref), call
+        assert np.array_equal(stage_x.cpu().numpy(), x) and np.array_equal(stage_y.cpu().numpy(), yb.numpy())
+        if yb.data_ptr() != plain_y.data_ptr():
+            assert int((wide_y == -3.0).sum()) >= 7                # nothing written beside the result
+        assert m.last_status() == 0
+        idx, _ = m.last_compaction()
+        assert np.array_equal(idx.cpu().numpy(), orc.compact(x, 1.0)[0])
