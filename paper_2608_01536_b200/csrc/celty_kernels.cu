@@ -1065,6 +1065,9 @@ extern "C" int celty_spmspv_static(const celty_matrix *m, const void *image_dev,
         fp.idx = idx; fp.val = val; fp.count = count;
         fp.status = reinterpret_cast<uint32_t *>(scratch);
         fp.tickets = fp.status + 2;
+        // nothing of the image is read before the previous kernel of the stream is complete: it may be the one that
+        // puts it there (0.1 us)
+        fp.win_cols = 0;
         return plan.lean == 2 ? launch_fused(k_spmspv_fused<false, 0, 2>, g_granted_lean[1], knobs, plan, 1, fp, st)
                               : launch_fused(k_spmspv_fused<false, 0, 1>, g_granted_lean[0], knobs, plan, 1, fp, st);
     }

@@ -123,3 +123,22 @@ def test_static_scratch_entry_point_rejects_what_it_cannot_hold():
     ok = celty.Matrix(np.ones((4, 4), np.float16))
     assert lib.celty_spmspv_static(ok._h, p16, p16, -1.0, p16, None) == -1
     assert lib.celty_spmspv_static(ok._h, None, p16, 0.0, p16, None) == -1
+
+
+def test_static_entry_point_behind_the_kernel_that_writes_the_image():
+    """The image need not come from a copy: here the kernel right before the call in the stream writes it."""
+    build.build()
+    M, K = 4096, 4096
+    W = synth.integer_weights(6, M, K)
+    mask = synth.mask_bernoulli(6, M, K, 0.5)
+    x = synth.integer_activations(7, K)
+    m = celty.Matrix(W, mask, device="cuda")
+    y_ref, _ = orc.masked_gemv(W, mask, x, 1.0, threads=8)
+    xd = torch.from_numpy(x).cuda()
+    scrambled = m._image ^ 0x5A
+    key = torch.full_like(scrambled, 0x5A)
+    for _ in range(5):
+        m._image.zero_()
+        torch.bitwise_xor(scrambled, key, out=m._image)
+        y = m.spmspv_static(xd, 1.0)
+        assert np.array_equal(y.cpu().numpy().astype(np.float64), y_ref)
