@@ -13,7 +13,7 @@
 // What bounds it: shared memory.  The rows of the 32 lanes fall on the banks as good as at random (8 entries, or
 // some 16 rows at 50 % density, lie between two lanes), so a load or store takes 3 to 4 wavefronts where the lane
 // tiles' takes one; entries per SM / 32 x 7 wavefronts is 3.2 us at 4096 x 4096, 50 % / 50 %.  Measured there:
-// 16.0 us against 41.6 us for warps that each took whole columns and added with shared-memory atomics, behind a
+// 11.7 us against 41.6 us for warps that each took whole columns and added with shared-memory atomics, behind a
 // one-block compaction kernel.
 //
 // a0 and a1 as in the fused kernel: every block clears its share of y and takes a ticket, and thresholds all of x.
@@ -40,15 +40,19 @@ struct ColumnParams {
 
 constexpr int kColumnThreads = 1024;
 
-struct ColumnSmem { uint32_t acc, spans, items, imeta, warps, keep, rank, total; };
+constexpr int kColumnWindow = 256;     // columns of the offset table a block fetches while the previous kernel ends
+
+struct ColumnSmem { uint32_t acc, dump, spans, items, imeta, window, warps, keep, rank, total; };
 
 __host__ __device__ inline ColumnSmem column_smem_layout(int M, int K, int groups, int cap, int own_list)
 {
     ColumnSmem l;
     uint32_t off = 0;
     l.acc = off;    off += (uint32_t)groups * ((M + 3) & ~3) * 4u;    // one accumulator per group
+    l.dump = off;   off += 32u * 4u;                                 // where the lanes of a column's last chunk put what is no entry
     l.items = off;  off += (uint32_t)cap * 8u;                       // {column, x bits}
     l.imeta = off;  off += (uint32_t)cap * 8u;                       // {offset/16, entries}
+    l.window = off; off += own_list ? (uint32_t)kColumnWindow * 8u : 0u;
     l.spans = off;  off += 2u * 32u * 4u;                            // rows spanned by each warp's chunk, two columns deep
     l.warps = off;  off += 33u * 4u;                                 // survivors before each warp's words, and of all
     l.keep = off;   off += own_list ? (uint32_t)((K + 31) / 32) * 4u : 0u;
@@ -100,6 +104,11 @@ __global__ void __launch_bounds__(kColumnThreads, 1) k_spmspv_column(const Colum
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     for (int i = tid; i < p.groups * Mp / 4; i += kColumnThreads)
         reinterpret_cast<float4 *>(acc)[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+    // The block's columns lie around the same fraction of K as the block in the grid: their offsets are fetched now.
+    // (The table is part of the image, which no kernel writes.)
+    uint2 *const window = reinterpret_cast<uint2 *>(smem + lay.window);
+    const int win0 = max(0, min(p.K - kColumnWindow, (int)((float)(2 * blockIdx.x + 1) * (float)p.K / (float)(2 * gridDim.x)) - kColumnWindow / 2));
+    if (p.own_list && tid < kColumnWindow && win0 + tid < p.K) window[tid] = __ldg(p.meta + win0 + tid);
     asm volatile("griddepcontrol.wait;" ::: "memory");
 
     uint32_t y_ticket = 0;
@@ -142,11 +151,14 @@ __global__ void __launch_bounds__(kColumnThreads, 1) k_spmspv_column(const Colum
         n = __ldcg(p.count);
     }
 
-    const int p0 = (int)((int64_t)blockIdx.x * n / gridDim.x), p1 = (int)((int64_t)(blockIdx.x + 1) * n / gridDim.x);
-    const int g = warp / p.W, w = warp - g * p.W;
+    // n / blocks columns each, the first n mod blocks one more
+    const int share = n / (int)gridDim.x, extra = n - share * (int)gridDim.x, b = (int)blockIdx.x;
+    const int p0 = b * share + min(b, extra), p1 = p0 + share + (b < extra ? 1 : 0);
+    const int g = idiv_small(warp, p.W), w = warp - g * p.W;
     const bool works = g < p.groups;
     float *const a = acc + (size_t)(works ? g : 0) * Mp;
     volatile uint32_t *const spans = reinterpret_cast<uint32_t *>(smem + lay.spans) + (works ? g * p.W : 0);
+    const uint32_t acc0 = smem_u32(a), dump = smem_u32(smem + lay.dump) + 4u * lane;
     uint32_t parity = 0;
     bool out_of_range = false;
     for (int b0 = p0; b0 < p1; b0 += p.cap) {
@@ -154,21 +166,25 @@ __global__ void __launch_bounds__(kColumnThreads, 1) k_spmspv_column(const Colum
         const int cnt = min(p.cap, p1 - b0);
         if (p.own_list) {
             const int nwords = (p.K + 31) >> 5;
-            for (int i = tid; i < nwords; i += kColumnThreads) {
-                uint32_t word = keep[i];
-                int r = rank[i] - b0;
-                if (r >= cnt || r + __popc(word) <= 0) continue;
-                for (; word; word &= word - 1, ++r)
-                    if (r >= 0 && r < cnt) items[r].x = 32 * i + __ffs(word) - 1;
-            }
-            __syncthreads();
             for (int i = tid; i < cnt; i += kColumnThreads) {
-                const int j = items[i].x;
+                // the last word with rank[] <= r, then the bit: halve the word, keep the half with the wanted set bit
+                const int r = b0 + i;
+                int at = 0;
+                for (int step = 1 << (31 - __clz(nwords)); step; step >>= 1)
+                    if (at + step < nwords && rank[at + step] <= r) at += step;
+                int k = r - rank[at], pos = 0;
+                const uint32_t word = keep[at];
+#pragma unroll
+                for (int sh = 16; sh; sh >>= 1) {
+                    const int c = __popc((word >> pos) & ((1u << sh) - 1u));
+                    if (k >= c) { k -= c; pos += sh; }
+                }
+                const int j = 32 * at + pos;
                 const uint16_t xb = __ldg(p.x + j);
-                items[i].y = (int)xb;
-                imeta[i] = __ldg(p.meta + j);
-                p.idx[b0 + i] = j;
-                p.val[b0 + i] = xb;
+                items[i] = make_int2(j, (int)xb);
+                imeta[i] = j >= win0 && j < win0 + kColumnWindow ? window[j - win0] : __ldg(p.meta + j);
+                p.idx[r] = j;
+                p.val[r] = xb;
             }
         } else {
             for (int i = tid; i < cnt; i += kColumnThreads) {
@@ -180,8 +196,8 @@ __global__ void __launch_bounds__(kColumnThreads, 1) k_spmspv_column(const Colum
         __syncthreads();
         // ---- a2 - a4: this group's columns of the batch
         if (works) {
-            const int i1 = (int)((int64_t)(g + 1) * cnt / p.groups);
-            int li = (int)((int64_t)g * cnt / p.groups), lc = 0;       // what is loaded next: column, first chunk
+            const int i1 = idiv_small((g + 1) * cnt, p.groups);          // cnt <= 1024
+            int li = idiv_small(g * cnt, p.groups), lc = 0;            // what is loaded next: column, first chunk
             int pi = li, pc = 0;                                       // what is scattered next
             struct Chunk { uint4 v; uint32_t runs; };
             auto next = [&](int &i, int &c) {                          // the group's next W chunks
@@ -231,21 +247,37 @@ __global__ void __launch_bounds__(kColumnThreads, 1) k_spmspv_column(const Colum
                     carry += mine;
                     __syncwarp();                                      // the lanes' stores of the column before this one
                 }
-                const float xj = __half2float(__ushort_as_half((uint16_t)items[pi].y));
+                const uint16_t xj = (uint16_t)items[pi].y;
                 const uint32_t have = nent > e0 ? min(nent - e0, (uint32_t)kGroup) : 0u;
-                uint32_t row[kGroup];
-                float sumv[kGroup];
+                // A lane's rows grow, so its last one tells whether all are in range.
+                const uint32_t last = row0 + entry_offset(even, odd, kGroup - 1);
+                uint32_t cell[kGroup];
+                const uint32_t cell0 = acc0 + 4u * row0;
+                cell[0] = __dp4a(even, 0x00000004u, cell0);
+                cell[1] = __dp4a(odd, 0x00000004u, cell0);
+                cell[2] = __dp4a(even, 0x00000400u, cell0);
+                cell[3] = __dp4a(odd, 0x00000400u, cell0);
+                cell[4] = __dp4a(even, 0x00040000u, cell0);
+                cell[5] = __dp4a(odd, 0x00040000u, cell0);
+                cell[6] = __dp4a(even, 0x04000000u, cell0);
+                cell[7] = __dp4a(odd, 0x04000000u, cell0);
+                if (!__all_sync(kFull, have == kGroup && last < (uint32_t)p.M)) {   // the end of a column, or of the image
 #pragma unroll
-                for (int e = 0; e < kGroup; ++e) {
-                    row[e] = row0 + entry_offset(even, odd, e);
-                    const bool ok = (uint32_t)e < have;
-                    if (ok && row[e] >= (uint32_t)p.M) out_of_range = true;
-                    if (!ok || row[e] >= (uint32_t)p.M) row[e] = 0xFFFFFFFFu;
-                    sumv[e] = row[e] != 0xFFFFFFFFu ? a[row[e]] : 0.f;
+                    for (int e = 0; e < kGroup; ++e) {
+                        const bool in = cell[e] < acc0 + 4u * (uint32_t)p.M && row0 < (uint32_t)p.M;
+                        if ((uint32_t)e < have && !in) out_of_range = true;
+                        if ((uint32_t)e >= have || !in) cell[e] = dump;
+                    }
                 }
+                float c[kGroup], d[kGroup];
 #pragma unroll
-                for (int e = 0; e < kGroup; ++e)
-                    if (row[e] != 0xFFFFFFFFu) a[row[e]] = fmaf(entry_value(c0.v, e), xj, sumv[e]);
+                for (int e = 0; e < kGroup; ++e) c[e] = lds_f32(cell[e]);
+                fma_pair(c0.v.x, xj, c[0], c[1], d[0], d[1]);
+                fma_pair(c0.v.y, xj, c[2], c[3], d[2], d[3]);
+                fma_pair(c0.v.z, xj, c[4], c[5], d[4], d[5]);
+                fma_pair(c0.v.w, xj, c[6], c[7], d[6], d[7]);
+#pragma unroll
+                for (int e = 0; e < kGroup; ++e) sts_f32(cell[e], d[e]);
                 const int before = pi;
                 next(pi, pc);
                 if (pi != before) carry = 0;
