@@ -275,8 +275,8 @@ int celty_shard_columns(int64_t K, int32_t world, int32_t rank, int64_t *k_begin
  * FP32 result of the stacked [gate; up] product (gate_up_dev: 2K values, the K gate results first), and step a1
  * works on  x_j = SiLU(gate_j) * up_j  evaluated in FP32 and rounded once to FP16 -- the same values
  * CELTY_EPILOGUE_SWIGLU stores -- thresholding them with `tau` and listing the survivors as celty_spmspv does
- * (celty_last_compaction then reports that list, ascending).  No launch and no pass over memory sits between the
- * two products.  h_out_dev (may be NULL) receives the K FP16 values of x.  `ep` as in celty_spmspv_ex.
+ * (celty_last_compaction then reports that list, ascending).  A small kernel ahead of the product's makes them, in the
+ * handle's workspace.  h_out_dev (may be NULL) receives the K FP16 values of x.  `ep` as in celty_spmspv_ex.
  * Errors: as celty_spmspv_ex.
  */
 int celty_spmspv_swiglu(celty_matrix *m, const float *gate_up_dev, float tau, void *y_dev, void *h_out_dev,

@@ -290,7 +290,7 @@ class Matrix:
         return y
 
     def spmspv_ex(self, x, tau: float, y=None, fp16_out=None, swiglu: "SwigluOut | None" = None, stream=None):
-        """spmspv followed in the same launch by an FP16 copy of y (fp16_out: M float16) or by the SiLU(gate) * up
+        """spmspv followed in the same call by an FP16 copy of y (fp16_out: M float16) or by the SiLU(gate) * up
         step of a stacked [gate; up] matrix (swiglu: a SwigluOut)."""
         import torch
         if y is None:

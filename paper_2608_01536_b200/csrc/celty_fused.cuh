@@ -3,8 +3,6 @@
 //
 // One launch does the whole call (Sections 3.1-3.3):
 //   a0  the last warp of every block clears its share of y and takes a ticket (the merge at the end adds into y);
-//   (with swiglu_in: x = SiLU(gate) * up is made here, every block a share of it, and the ticket of a0 tells when all
-//       of it is there)
 //   a1  every block thresholds all of x (K <= a few 10k values, served by L2) into one keep bit per
 //       activation and ranks the survivors (popcounts + warp scans); each warp team then looks up the
 //       columns whose ranks belong to it -- the list is balanced over all teams by count -- and their
@@ -142,21 +140,6 @@ __device__ __forceinline__ bool ticket_wait(const uint32_t *ticket, uint32_t min
     return ok;
 }
 
-// Loads of values that other blocks of this launch may have written (not through the read-only path).
-__device__ __forceinline__ uint4 ld_plain_v4(const uint16_t *p)
-{
-    uint4 v;
-    asm volatile("ld.global.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p) : "memory");
-    return v;
-}
-
-__device__ __forceinline__ uint16_t ld_plain_u16(const uint16_t *p)
-{
-    uint16_t v;
-    asm volatile("ld.global.u16 %0, [%1];" : "=h"(v) : "l"(p) : "memory");
-    return v;
-}
-
 // One lane's work on the steps of a sub-block, as a three-stage software pipeline (a step =
 // one group of 8 entries of every lane that still has one):
 //   fetch(q+2)   128-bit value vector + 32-bit run word from the ring slot
@@ -273,6 +256,21 @@ __device__ __noinline__ uint4 ragged_group(const uint16_t *x, int K, int q)
     return make_uint4(h[0], h[1], h[2], h[3]);
 }
 
+// x = SiLU(gate) * up from the FP32 result of a stacked [gate; up] product (2K values, gate first), rounded to FP16, for
+// the down projection: a kernel of its own ahead of the product's.  Bound by the change of kernels, which the dependent
+// launches hide but for the trip to L2; 4096 x 11008 14.6 us against 16.3 for shares evaluated by the product's blocks
+// behind a ticket that all of them wait for, 18.6 for every block evaluating all of x (plain product 12.9).
+__global__ void __launch_bounds__(256) k_swiglu(const float *__restrict__ gate_up, uint16_t *__restrict__ x, uint16_t *x_copy, int K)
+{
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    const int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x;
+    if (i >= K) return;
+    const uint16_t h = (uint16_t)swiglu_half_bits(__ldcg(gate_up + i), __ldcg(gate_up + K + i));
+    x[i] = h;
+    if (x_copy) x_copy[i] = h;
+}
+
 // Work on the finished y (celty_epilogue), a kernel of its own behind the product:
 //   kind 1  out = y rounded to FP16;
 //   kind 2  y holds a stacked [gate; up] product of 2I rows: out_i = SiLU(y_i) * y_{I+i} rounded to FP16, and the (i,
@@ -346,7 +344,7 @@ __global__ void __launch_bounds__(kEpilogueThreads) k_epilogue(const EpilogueArg
     }
 }
 
-// kExtras = false compiles the list input and the making of x from gate and up out: the plain product keeps its
+// kExtras = false compiles the list input out: the plain product keeps its
 // register budget, which the streaming loop's scheduling depends on.
 // kRegRows > 0 is the software analogue of register-file accumulation (Section 4.1, the register / shared-memory
 // split of Section 6.4): the first kRegRows local rows of every lane are summed in registers across the team's
@@ -365,7 +363,7 @@ __global__ void __launch_bounds__(kRegRows > 0 ? 256 : 512, 1) k_spmspv_fused(co
     const int pp = kLean ? (kLean == 2 ? 1 : 0) : p.pp;
     const int merge = kLean ? 1 : p.merge;
     const int cl = kLean ? 1 : p.cl;
-    const uint16_t *const x = kBatch ? p.x + (size_t)blockIdx.y * p.ldx : kExtras && p.swiglu_in ? p.h_ws : p.x;
+    const uint16_t *const x = kBatch ? p.x + (size_t)blockIdx.y * p.ldx : p.x;
     float *const y = kBatch ? p.y + (size_t)blockIdx.y * p.ldy : p.y;
     uint32_t *const tickets = kBatch ? p.tickets + blockIdx.y : p.tickets;
     const bool lists = !kBatch || blockIdx.y + 1 == gridDim.y;    // the survivor list reported is the last vector's
@@ -466,19 +464,6 @@ __global__ void __launch_bounds__(kRegRows > 0 ? 256 : 512, 1) k_spmspv_fused(co
     }
     asm volatile("griddepcontrol.wait;" ::: "memory");
     uint32_t y_ticket = 0;
-    // x made from the FP32 gate / up result: every block evaluates a share (32 values per warp, dealt to the blocks in
-    // turn) into the workspace, and takes its ticket once the share is stored.  The alternative, every block
-    // evaluating all of x for itself, cost 18.6 us at 4096 x 11008 (each thread 32 SiLUs in a row, 148 times
-    // the expf work); this is one block barrier and one trip to L2 and back: 16.3 us.
-    if (kExtras && p.swiglu_in) {
-#pragma unroll 1
-        for (uint32_t i = ((uint32_t)warp * gridDim.x + blockIdx.x) * 32u + lane; i < (uint32_t)p.K; i += nthreads * gridDim.x) {
-            const uint16_t h = (uint16_t)swiglu_half_bits(__ldg(p.swiglu_in + i), __ldg(p.swiglu_in + p.K + i));
-            p.h_ws[i] = h;
-            if (p.h_out) p.h_out[i] = h;
-        }
-        __syncthreads();
-    }
     // Bulk reduce-add merge: the adds at the end need a cleared y.  The last warp clears this block's share
     // and announces it right away, so that the fence and the ticket overlap the loads of a1.
     if (merge == 1 && warp == nwarps - 1) {
@@ -493,10 +478,8 @@ __global__ void __launch_bounds__(kRegRows > 0 ? 256 : 512, 1) k_spmspv_fused(co
             // The ticket counts modulo 2 * gridDim.x, so it never has to be reset: calls alternate between
             // waiting for the lower and for the upper half.
             y_ticket = atomicInc(&tickets[0], 2u * gridDim.x - 1u);
-            if (kExtras && p.swiglu_in && !ticket_wait(tickets, y_ticket, p.spin_limit)) atomicOr(p.status, kStatusTimeout);
         }
     }
-    if (kExtras && p.swiglu_in) __syncthreads();
     // ---- a1: threshold all of x.  A thread takes 32 activations (four 128-bit loads) and makes one keep word,
     // and the warp scans the survivor counts of its block of 32 words:
     //   kbw[w]  keep bits of activations 32w .. 32w+31,
@@ -518,7 +501,7 @@ __global__ void __launch_bounds__(kRegRows > 0 ? 256 : 512, 1) k_spmspv_fused(co
                     const int q = 4 * w + c;
                     h[c][0] = h[c][1] = h[c][2] = h[c][3] = 0u;        // zero past the end of x: never kept (tau >= 0)
                     if (8 * q + 8 <= p.K) {
-                        const uint4 v = kExtras ? ld_plain_v4(x + 8 * q) : __ldg(reinterpret_cast<const uint4 *>(x + 8 * q));
+                        const uint4 v = __ldg(reinterpret_cast<const uint4 *>(x + 8 * q));
                         h[c][0] = v.x; h[c][1] = v.y; h[c][2] = v.z; h[c][3] = v.w;
                     } else if (__builtin_expect(q < ngroups, 0)) {
                         const uint4 v = ragged_group(x, p.K, q);     // the one group that K cuts short
@@ -660,7 +643,7 @@ __global__ void __launch_bounds__(kRegRows > 0 ? 256 : 512, 1) k_spmspv_fused(co
                     if (k >= c) { k -= c; pos += sh; }
                 }
                 j = 32 * w + pos;
-                xb = kExtras ? ld_plain_u16(x + j) : __ldg(x + j);   // x went through L1 in the thresholding pass
+                xb = __ldg(x + j);                                   // x went through L1 in the thresholding pass
                 }
                 items[i] = make_int2(j, (int)xb);
                 if (!from_list && lists && part == 0 && sl == 0) {

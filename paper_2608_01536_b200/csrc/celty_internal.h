@@ -155,11 +155,6 @@ struct FusedParams {
     const int32_t *list_idx;
     const uint16_t *list_val;
     const int32_t *list_count;
-    // The activations are not given but made from the FP32 result of a stacked [gate; up] product (2K values, gate
-    // first): x_j = SiLU(g_j) * u_j rounded to FP16, for the down projection, into the workspace (h_ws, K values).
-    // h_out (may be null) receives a copy.
-    const float *swiglu_in;
-    uint16_t *h_ws, *h_out;
     int32_t *ep_count;         // not null: set to zero for the list that k_epilogue appends to after this kernel
 };
 

@@ -820,23 +820,30 @@ int check_epilogue(const celty_matrix *m, const celty_epilogue *ep)
     return CELTY_OK;
 }
 
+// A small kernel of 256 threads per block, launched like the product's (programmatic dependent launch).
+template <typename... Params, typename... Args>
+int launch_dependent(void (*kernel)(Params...), int64_t blocks, const LaunchKnobs &knobs, cudaStream_t st, Args... args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)blocks);
+    cfg.blockDim = dim3(256);
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = knobs.no_overlap ? 0 : 1;
+    CELTY_CUDA(cudaLaunchKernelEx(&cfg, kernel, args...));
+    return CELTY_OK;
+}
+
 int launch_epilogue(const celty_matrix *m, EpilogueArgs a, const float *y, cudaStream_t st)
 {
     a.y = y;
     a.M = (int)m->M;
     const int per_block = a.kind == CELTY_EPILOGUE_SWIGLU ? kEpilogueThreads : 4 * kEpilogueThreads;
     const int64_t n = a.kind == CELTY_EPILOGUE_SWIGLU ? m->M / 2 : m->M;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)((n + per_block - 1) / per_block));
-    cfg.blockDim = dim3(kEpilogueThreads);
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = m->no_overlap ? 0 : 1;
-    CELTY_CUDA(cudaLaunchKernelEx(&cfg, k_epilogue, a));
-    return CELTY_OK;
+    return launch_dependent(k_epilogue, (n + per_block - 1) / per_block, *m, st, a);
 }
 
 // The product for every entry point: x thresholded by the kernel (list == nullptr) or the survivors given as a
@@ -876,14 +883,15 @@ int run_product(celty_matrix *m, const void *x_dev, float tau, const ListInput *
             fp.list_val = list->val;
             fp.list_count = list->count;
         }
-        if (sw) {
-            fp.swiglu_in = sw->gate_up;
-            fp.h_ws = reinterpret_cast<uint16_t *>(m->d_ws + m->ws.partial_off);
-            fp.h_out = sw->h_out;
-        }
         const bool after = ep && ep->kind != CELTY_EPILOGUE_NONE;
         if (after && ep->kind == CELTY_EPILOGUE_SWIGLU) fp.ep_count = ep->list_count;
         fp.x = static_cast<const uint16_t *>(x_dev);           // not looked at when the survivors come as a list
+        if (sw) {
+            uint16_t *made = reinterpret_cast<uint16_t *>(m->d_ws + m->ws.partial_off);
+            rc = launch_dependent(k_swiglu, (m->K + 255) / 256, *m, st, sw->gate_up, made, sw->h_out, (int)m->K);
+            if (rc) return rc;
+            fp.x = made;
+        }
         fp.tau = tau;
         fp.y = y;
         fp.idx = idx; fp.val = val; fp.count = count; fp.status = status; fp.tickets = status + 2;
@@ -894,8 +902,7 @@ int run_product(celty_matrix *m, const void *x_dev, float tau, const ListInput *
             m->last_grid = plan.grid;
             m->last_merge = plan.merge;
         }
-        // the list input and the making of x from gate and up have builds of their own
-        if (list || sw)
+        if (list)                                                // the list input has builds of its own
             rc = plan.lean == 2 ? launch_fused(k_spmspv_fused<true, 0, 2>, g_granted_lean_extras[1], *m, plan, 1, fp, st)
                : plan.lean == 1 ? launch_fused(k_spmspv_fused<true, 0, 1>, g_granted_lean_extras[0], *m, plan, 1, fp, st)
                                 : launch_fused(k_spmspv_fused<true, 0>, g_granted_fused_extras, *m, plan, 1, fp, st);
