@@ -358,7 +358,7 @@ __global__ void __launch_bounds__(kEpilogueThreads) k_epilogue(const EpilogueArg
 // nothing.
 // kBatch: one launch for several activation vectors, the blocks dealt out among them (FusedParams::ldx).
 template <bool kExtras, int kRegRows, int kLean = 0, bool kBatch = false>
-__global__ void __launch_bounds__(kRegRows > 0 ? 256 : 512, 1) k_spmspv_fused(const FusedParams p)
+__global__ void __launch_bounds__(kRegRows > 0 ? 256 : 544, 1) k_spmspv_fused(const FusedParams p)
 {
     const int pp = kLean ? (kLean == 2 ? 1 : 0) : p.pp;
     const int merge = kLean ? 1 : p.merge;
@@ -382,7 +382,7 @@ __global__ void __launch_bounds__(kRegRows > 0 ? 256 : 512, 1) k_spmspv_fused(co
     const int teams = p.G * p.Sc;
     // (The partner of warp t is warp t + 8: the two sit on the same warp scheduler, which suits them, since only
     // one of them is in its step loop at any time.)
-    const bool streams = pp ? (warp & 7) < teams : warp < teams;
+    const bool streams = pp ? (warp & 7) < teams && warp < 16 : warp < teams;
     const int team = streams ? (pp ? (warp & 7) : warp) : 0;
     const int half = streams && pp ? warp >> 3 : 0;               // which of the team's two warps (0 without pp)
     const int stride = 1 + pp, Dw = p.D / stride;                 // columns between a warp's own, ring slots per warp
@@ -783,31 +783,31 @@ __global__ void __launch_bounds__(kRegRows > 0 ? 256 : 512, 1) k_spmspv_fused(co
             if (lane == 0) atomicOr(p.status, kStatusTimeout);
         }
     }
+    // Every block's share of y is cleared by the time the reduce-adds start.  The last warp does not stream (with pairs
+    // it is a 17th warp), so it asks now, under the streaming: the poll and the two fences, the second of which also
+    // puts the other blocks' clearing stores (generic proxy) before this block's reduce-adds (asynchronous proxy),
+    // were 700 cycles of every block's end when they came after it.
+    if (merge == 1 && warp == nwarps - 1 && lane == 0) {
+        if (__builtin_expect(!ticket_wait(tickets, y_ticket, p.spin_limit), 0)) atomicOr(p.status, kStatusTimeout);
+        asm volatile("fence.proxy.async.global;" ::: "memory");
+    }
     __syncthreads();
 
     if (merge == 1) {
         // ---- a5 by bulk reduce-add.  The block adds its G accumulators; the row segments of its slabs (32*C rows
         // of y each, see the row map) are then dealt to the blocks of the cluster, a block adds its peers' sums
         // for its segments (through distributed shared memory), and the copy engine adds the result into y
-        // (cp.reduce.async.bulk, FP32 add at L2).  y was cleared by all blocks at the start; the ticket makes
-        // sure of it.
-        if (warp == nwarps - 1 && lane == 0) {                      // every block's share of y is cleared by now
-            const bool ok = ticket_wait(tickets, y_ticket, p.spin_limit);
-            // the clearing stores of the other blocks (generic proxy) come before this block's reduce-adds
-            // (asynchronous proxy) to the same addresses
-            asm volatile("fence.proxy.async.global;" ::: "memory");
-            if (__builtin_expect(!ok, 0)) atomicOr(p.status, kStatusTimeout);
-        }
-        __syncwarp();
+        // (cp.reduce.async.bulk, FP32 add at L2).
         // add the G accumulators of every slab into the first one
         const int group_words = Sc * slab_words;
         if (G > 1) {
             float4 *acc4 = reinterpret_cast<float4 *>(acc);
-            const int group4 = group_words / 4;
+            // (with one slab, without its spare rows: R = 64 then is one round of 512 threads)
+            const int group4 = group_words / 4, sum4 = Sc == 1 ? p.R * 8 : group4;
 #pragma unroll 1
-            for (int q4 = tid; q4 < group4; q4 += nthreads) {
+            for (int q4 = tid; q4 < sum4; q4 += nthreads) {
                 float4 v = acc4[q4];
-#pragma unroll 2
+#pragma unroll 4
                 for (int gg = 1; gg < G; ++gg) {
                     const float4 t = acc4[(size_t)gg * group4 + q4];
                     v.x += t.x; v.y += t.y; v.z += t.z; v.w += t.w;

@@ -565,7 +565,7 @@ int plan_fused(const celty_matrix *m, const LaunchKnobs &knobs, const DeviceInfo
         pl.pp = 0;
     }
     if (pl.G == 0) return CELTY_EINVAL;
-    pl.threads = reg_rows > 0 ? 256 : 512;
+    pl.threads = reg_rows > 0 ? 256 : pl.pp || pl.G * pl.Sc > 15 ? 544 : 512;   // the last warp does not stream
     pl.smem = fused_smem_bytes(m->R, (int)m->K, pl.G, pl.Sc, pl.D, pl.slot_bytes, pl.cap);
     pl.merge = (knobs.merge >= 0 ? knobs.merge : 1);
     // Clusters (bulk reduce-add merge only, on request): as long as the grid is made of whole clusters, every row
