@@ -61,6 +61,20 @@ __host__ __device__ inline ColumnSmem column_smem_layout(int M, int K, int group
     return l;
 }
 
+// The group of 8 activations that the end of x cuts short (K not a multiple of 8), zero-filled.  Out of line: one
+// thread of a block needs it, if any, and the thresholding pass is unrolled four times around the call.
+__device__ __noinline__ uint4 ragged_group(const uint16_t *x, int K, int q)
+{
+    uint32_t h[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const uint32_t lo = (8 * q + 2 * k < K) ? x[8 * q + 2 * k] : 0u;
+        const uint32_t hi = (8 * q + 2 * k + 1 < K) ? x[8 * q + 2 * k + 1] : 0u;
+        h[k] = lo | (hi << 16);
+    }
+    return make_uint4(h[0], h[1], h[2], h[3]);
+}
+
 // One keep bit per activation of x[32w .. 32w+31] (zero past the end of x).
 __device__ __forceinline__ uint32_t keep_word(const uint16_t *x, int K, int w, __half2 tau2)
 {

@@ -242,18 +242,22 @@ __device__ __forceinline__ uint32_t swiglu_half_bits(float gate, float up)
     return (uint32_t)__half_as_ushort(__float2half_rn(gate / (1.f + expf(-gate)) * up));
 }
 
-// The group of 8 activations that the end of x cuts short (K not a multiple of 8), zero-filled.  Out of line: one
-// thread of a block needs it, if any, and the thresholding pass is unrolled four times around the call.
-__device__ __noinline__ uint4 ragged_group(const uint16_t *x, int K, int q)
+// Keep bits of 8 activations, bit k for activation k: not(|x| <= tau), NaN kept.  The comparisons give 0xFFFF or 0 per
+// half; a byte of each is picked, masked to its bit, and a multiplication adds the four bytes of a word up.
+__device__ __forceinline__ uint32_t keep_byte(const uint4 v, __half2 tau2)
 {
-    uint32_t h[4];
+    auto le = [&](uint32_t h) { return __hle2_mask(__habs2(*reinterpret_cast<const __half2 *>(&h)), tau2); };
+    const uint32_t lo = __byte_perm(le(v.x), le(v.y), 0x6420), hi = __byte_perm(le(v.z), le(v.w), 0x6420);
+    return ~((((lo & 0x08040201u) | (hi & 0x80402010u)) * 0x01010101u) >> 24) & 0xFFu;
+}
+
+// Keep bits of 32 activations (x 16-byte aligned): four independent 128-bit loads.
+__device__ __forceinline__ uint32_t keep_word32(const uint16_t *x, __half2 tau2)
+{
+    uint4 h[4];
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        const uint32_t lo = (8 * q + 2 * k < K) ? x[8 * q + 2 * k] : 0u;
-        const uint32_t hi = (8 * q + 2 * k + 1 < K) ? x[8 * q + 2 * k + 1] : 0u;
-        h[k] = lo | (hi << 16);
-    }
-    return make_uint4(h[0], h[1], h[2], h[3]);
+    for (int c = 0; c < 4; ++c) h[c] = __ldg(reinterpret_cast<const uint4 *>(x) + c);
+    return keep_byte(h[0], tau2) | keep_byte(h[1], tau2) << 8 | keep_byte(h[2], tau2) << 16 | keep_byte(h[3], tau2) << 24;
 }
 
 // x = SiLU(gate) * up from the FP32 result of a stacked [gate; up] product (2K values, gate first), rounded to FP16, for
@@ -464,8 +468,52 @@ __global__ void __launch_bounds__(kRegRows > 0 ? 256 : 544, 1) k_spmspv_fused(co
     }
     asm volatile("griddepcontrol.wait;" ::: "memory");
     uint32_t y_ticket = 0;
-    // Bulk reduce-add merge: the adds at the end need a cleared y.  The last warp clears this block's share
-    // and announces it right away, so that the fence and the ticket overlap the loads of a1.
+    // ---- a1: threshold all of x.  A thread takes 32 activations (four 128-bit loads) and makes one keep word,
+    // and the warp scans the survivor counts of its block of 32 words:
+    //   kbw[w]  keep bits of activations 32w .. 32w+31,
+    //   wrel[w] survivors in the words before w of the same block of 32 words,
+    //   blk[e]  survivors in block e (turned into survivors before block e by the scan below).
+    // |x| > tau in FP32 is the same decision as |x| > (tau rounded down to FP16) in FP16; NaN is kept.
+    const int nfull = p.K >> 5, nwords = (p.K + 31) >> 5, nblk = (nwords + 31) >> 5;
+    const bool from_list = kExtras && p.list_count != nullptr;    // a1 was done by whoever produced the activations
+    if (!from_list) {
+        const __half2 tau2 = __half2half2(__float2half_rd(p.tau));
+#pragma unroll 1
+        for (int w0 = 0; w0 < nwords; w0 += nthreads) {             // the same trip count for every thread
+            const int w = w0 + tid;
+            const uint32_t word = w < nfull ? keep_word32(x + 32 * w, tau2) : 0u;
+            const int cnt = __popc(word);
+            int incl = cnt;
+#pragma unroll
+            for (int d = 1; d < 32; d <<= 1) {                         // scan within the block of 32 words
+                const int up = __shfl_up_sync(kFull, incl, d);
+                if (lane >= d) incl += up;
+            }
+            if (w < nfull) kbw[w] = word;
+            if (w < nwords) wrel[w] = incl - cnt;
+            if (lane == 31 && (w >> 5) < nblk) const_cast<int *>(blk)[w >> 5] = incl;
+        }
+    }
+    // The window has had the whole thresholding pass to arrive; nobody may clear an accumulator before it has.  The last
+    // warp also takes the word that the end of x cuts short, one activation per lane, and waits for it, for everybody: a wait for a phase that is long complete takes 300 to 600 cycles here.
+    int *const win_failed = reinterpret_cast<int *>(smem + lay.flag) + teams, *const tail_cnt = win_failed + 1;
+    if (warp == nwarps - 1) {
+        const int j = 32 * nfull + lane;
+        const bool kept = !from_list && j < p.K && !(fabsf(__half2float(__ushort_as_half(x[j]))) <= p.tau);
+        const uint32_t word = __ballot_sync(kFull, kept);
+        if (lane == 0) {
+            if (nfull < nwords) kbw[nfull] = word;
+            *tail_cnt = __popc(word);
+        }
+        const bool late = p.win_cols > 0 && !mbar_wait_bounded(win_bar, 0, p.spin_limit);
+        if (lane == 0) *win_failed = late;
+    }
+    __syncthreads();
+    bool failed = *win_failed != 0;
+    if (failed) win_n = 0;
+    // Bulk reduce-add merge: the adds at the end need a cleared y.  The last warp, which does not
+    // stream, clears this block's share and announces it while the others look their columns up (its fence would
+    // hold the barrier above up).
     if (merge == 1 && warp == nwarps - 1) {
         const int b = (int)blockIdx.x;
         const int r0 = b * p.clear_rows + min(b, p.clear_extra), r1 = r0 + p.clear_rows + (b < p.clear_extra ? 1 : 0);
@@ -480,64 +528,6 @@ __global__ void __launch_bounds__(kRegRows > 0 ? 256 : 544, 1) k_spmspv_fused(co
             y_ticket = atomicInc(&tickets[0], 2u * gridDim.x - 1u);
         }
     }
-    // ---- a1: threshold all of x.  A thread takes 32 activations (four 128-bit loads) and makes one keep word,
-    // and the warp scans the survivor counts of its block of 32 words:
-    //   kbw[w]  keep bits of activations 32w .. 32w+31,
-    //   wrel[w] survivors in the words before w of the same block of 32 words,
-    //   blk[e]  survivors in block e (turned into survivors before block e by the scan below).
-    // |x| > tau in FP32 is the same decision as |x| > (tau rounded down to FP16) in FP16; NaN is kept.
-    const int ngroups = (p.K + 7) >> 3, nwords = (p.K + 31) >> 5, nblk = (nwords + 31) >> 5;
-    const bool from_list = kExtras && p.list_count != nullptr;    // a1 was done by whoever produced the activations
-    if (!from_list) {
-        const __half2 tau2 = __half2half2(__float2half_rd(p.tau));
-#pragma unroll 1
-        for (int w0 = 0; w0 < nwords; w0 += nthreads) {             // the same trip count for every thread
-            const int w = w0 + tid;
-            uint32_t word = 0;
-            if (w < nwords) {
-                uint32_t h[4][4];
-#pragma unroll
-                for (int c = 0; c < 4; ++c) {                          // four independent 128-bit loads per thread
-                    const int q = 4 * w + c;
-                    h[c][0] = h[c][1] = h[c][2] = h[c][3] = 0u;        // zero past the end of x: never kept (tau >= 0)
-                    if (8 * q + 8 <= p.K) {
-                        const uint4 v = __ldg(reinterpret_cast<const uint4 *>(x + 8 * q));
-                        h[c][0] = v.x; h[c][1] = v.y; h[c][2] = v.z; h[c][3] = v.w;
-                    } else if (__builtin_expect(q < ngroups, 0)) {
-                        const uint4 v = ragged_group(x, p.K, q);     // the one group that K cuts short
-                        h[c][0] = v.x; h[c][1] = v.y; h[c][2] = v.z; h[c][3] = v.w;
-                    }
-                }
-#pragma unroll
-                for (int c = 0; c < 4; ++c)
-#pragma unroll
-                    for (int k = 0; k < 4; ++k) {
-                        // 0xFFFF in a half where |x| <= tau (false for NaN); the keep bits are the complement
-                        const uint32_t le = __hle2_mask(__habs2(*reinterpret_cast<const __half2 *>(&h[c][k])), tau2);
-                        word |= ((~le & 1u) | ((~le >> 15) & 2u)) << (8 * c + 2 * k);
-                    }
-                if (32 * w + 32 > p.K) word &= (32 * w < p.K) ? (0xFFFFFFFFu >> (32 * w + 32 - p.K)) : 0u;
-            }
-            const int cnt = __popc(word);
-            int incl = cnt;
-#pragma unroll
-            for (int d = 1; d < 32; d <<= 1) {                         // scan within the block of 32 words
-                const int up = __shfl_up_sync(kFull, incl, d);
-                if (lane >= d) incl += up;
-            }
-            if (w < nwords) {
-                kbw[w] = word;
-                wrel[w] = incl - cnt;
-            }
-            if (lane == 31 && (w >> 5) < nblk) const_cast<int *>(blk)[w >> 5] = incl;
-        }
-    }
-    __syncthreads();
-    bool failed = false;
-    // the window has had the whole thresholding pass to arrive; nobody may clear an accumulator before it has
-    if (p.win_cols > 0 && !mbar_wait_bounded(win_bar, 0, p.spin_limit)) failed = true;
-    if (pp) failed = __syncthreads_or(failed);                  // the two warps of a team must agree on what follows
-    if (failed) win_n = 0;
     // ---- ranks: every streaming warp turns the block counts into survivors before each block for itself, 32
     // blocks at a time (a copy per warp costs a few hundred bytes and saves a block-wide barrier behind a single
     // warp); the list is then cut into equal shares for the groups that work on different columns.
@@ -545,11 +535,25 @@ __global__ void __launch_bounds__(kRegRows > 0 ? 256 : 544, 1) k_spmspv_fused(co
     if (from_list) {
         n_surv = max(0, min(p.K, __ldcg(p.list_count)));
         if (blockIdx.x == 0 && tid == 0) *p.count = n_surv;
+    } else if (nblk <= 8) {
+        if (streams) {
+            const int cnt = lane < nblk ? blk[lane] + (lane == nblk - 1 ? *tail_cnt : 0) : 0;
+            int incl = cnt;
+#pragma unroll
+            for (int d = 1; d < 8; d <<= 1) {
+                const int up = __shfl_up_sync(kFull, incl, d);
+                if (lane >= d) incl += up;
+            }
+            if (lane < nblk) myblk[lane] = incl - cnt;
+            n_surv = __shfl_sync(kFull, incl, 7);
+            __syncwarp();
+            if (lists && blockIdx.x == 0 && tid == 0) *p.count = n_surv;
+        }
     } else if (streams) {
         int carry = 0;
 #pragma unroll 1
         for (int e0 = 0; e0 < nblk; e0 += 32) {
-            const int e = e0 + lane, cnt = e < nblk ? blk[e] : 0;
+            const int e = e0 + lane, cnt = e < nblk ? blk[e] + (e == nblk - 1 ? *tail_cnt : 0) : 0;
             int incl = cnt;
             const int nscan = min(32, nblk - e0);                     // no more steps than there are blocks
 #pragma unroll

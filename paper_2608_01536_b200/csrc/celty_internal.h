@@ -101,7 +101,7 @@ CELTY_HD inline FusedSmem fused_smem_layout(int R, int K, int teams, int D, int 
     l.acc = off;       off += (uint32_t)teams * (R + kTileSlack) * 32 * 4;   // FP32 accumulators, one slab per team
     l.ring = off;      off += (uint32_t)teams * D * slot_bytes;              // bulk-copy ring slots (multiples of 128 bytes)
     l.bars = off;      off += (uint32_t)teams * D * 8 + 8;                   // one "full" mbarrier per slot, one for the offset window
-    l.flag = off;      off += (uint32_t)teams * 4;                           // per team: a wait of one of its warps ran out
+    l.flag = off;      off += (uint32_t)teams * 4 + 8;                       // per team: a wait of one of its warps ran out; the window's; survivors in the last, short word
     off = (off + 15) / 16 * 16;
     l.items = off;     off += (uint32_t)teams * cap * 8;                     // {column, x bits} per looked-up item
     l.imeta = off;     off += (uint32_t)teams * cap * 8;                     // {offset/16, bytes} of its sub-block
