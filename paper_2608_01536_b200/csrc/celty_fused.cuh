@@ -494,8 +494,9 @@ __global__ void __launch_bounds__(kRegRows > 0 ? 256 : 544, 1) k_spmspv_fused(co
             if (lane == 31 && (w >> 5) < nblk) const_cast<int *>(blk)[w >> 5] = incl;
         }
     }
-    // The window has had the whole thresholding pass to arrive; nobody may clear an accumulator before it has.  The last
-    // warp also takes the word that the end of x cuts short, one activation per lane, and waits for it, for everybody: a wait for a phase that is long complete takes 300 to 600 cycles here.
+    // The last warp takes the word that the end of x cuts short, one activation per lane.  And it waits for the window,
+    // for everybody: that has had the whole thresholding pass to arrive, but a wait for a phase that is long complete
+    // takes 300 to 600 cycles here.  (Nobody may clear an accumulator before the window is there.)
     int *const win_failed = reinterpret_cast<int *>(smem + lay.flag) + teams, *const tail_cnt = win_failed + 1;
     if (warp == nwarps - 1) {
         const int j = 32 * nfull + lane;

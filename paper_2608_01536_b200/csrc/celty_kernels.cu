@@ -547,13 +547,17 @@ int plan_fused(const celty_matrix *m, const LaunchKnobs &knobs, const DeviceInfo
     };
     fit(0);
     // Pairs pay where a team has many columns to stream (the hand-over hides the latencies at the head of every
-    // sub-block) and cost a little where it has few: measured +7-8 % at 28672 x 8192 and 8192 x 28672, +2 % at
-    // 11008 x 4096 and 13824 x 5120, -1 % at 5120 x 5120, -5 % at 4096 x 4096; and they must not cost teams (5120 x 13824
-    // runs 11 teams of one warp faster than 8 pairs).  The number of survivors is not known here, so the rule goes
-    // by the columns: a dozen or more per team, and no more than eight teams to begin with.
+    // sub-block) and cost a little where it has few.  The number of survivors is not known here, so the rule goes by the
+    // columns per team, measured with 10, 30, 50 and 70 % of the activations kept:
+    //   9 or more columns:  2 to 4 % faster from 30 % on (2048 x 5504, 11008 x 4096, 4096 x 11008, 8192 x 8192), level at 10 %;
+    //   6 to 9, at most 7 teams:  1 to 3 % faster from 30 % on (11008 x 2048, 16384 x 2048), level at 10 %;
+    //   6 to 9, 8 teams:  1 to 3 % slower at 10 %, level at 50 % (4096 x 4096, 1024 x 4096): not taken;
+    //   9 teams, of which pairs leave 8:  5 to 8 % faster (13824 x 5120 with 30 % of the weights, 3000 x 28672);
+    //   11 teams or more:  6 % slower at 70 % (5120 x 13824): not taken.
     if (reg_rows == 0 && knobs.pairs != 0 && pl.G > 0 && pl.Sc <= 8) {             // a pair is warps t and t + 8
         const int teams_per_part = std::max(1, pl.grid / pl.P) * pl.G;
-        if (knobs.pairs > 0 || (pl.G * pl.Sc <= 8 && m->K / teams_per_part >= 12)) {
+        const int64_t columns = m->K / teams_per_part;
+        if (knobs.pairs > 0 || (pl.G * pl.Sc <= 9 && columns >= (pl.G * pl.Sc <= 7 ? 6 : 9))) {
             const FusedPlan keep = pl;
             fit(1);
             if (pl.G == 0) pl = keep;
