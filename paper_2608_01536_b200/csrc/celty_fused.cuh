@@ -88,6 +88,15 @@ __device__ __forceinline__ void bulk_load_elected(uint32_t dst, const void *src,
         : "memory");
 }
 
+// The same from one thread.
+__device__ __forceinline__ void bulk_load(uint32_t dst, const void *src, uint32_t bytes, uint32_t bar)
+{
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst), "l"(src),
+                 "r"(bytes), "r"(bar)
+                 : "memory");
+}
+
 // Barrier across the thread blocks of the cluster (release / acquire: shared-memory writes made before it
 // are visible to the other blocks' distributed-shared-memory reads after it).
 __device__ __forceinline__ void cluster_sync()
@@ -620,8 +629,10 @@ __global__ void __launch_bounds__(kRegRows > 0 ? 256 : 544, 1) k_spmspv_fused(co
                 // round, the 32 words of a block in two -- quarters, then the eight words of the quarter)
                 int e = 0;
                 if (nblk <= 8) {
+                    const int4 b0 = *reinterpret_cast<const int4 *>(myblk), b1 = *reinterpret_cast<const int4 *>(myblk + 4);
+                    const int before[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
 #pragma unroll
-                    for (int u = 1; u < 8; ++u) e += (u < nblk && myblk[u] <= r) ? 1 : 0;
+                    for (int u = 1; u < 8; ++u) e += (u < nblk && before[u] <= r) ? 1 : 0;
                 } else {
 #pragma unroll 1
                     for (int step = 1 << (31 - __clz(nblk - 1)); step; step >>= 1)
@@ -633,9 +644,11 @@ __global__ void __launch_bounds__(kRegRows > 0 ? 256 : 544, 1) k_spmspv_fused(co
 #pragma unroll
                     for (int u = 8; u < 32; u += 8) quarter += (w + u < nwords && wrel[w + u] <= k) ? 1 : 0;
                     w += 8 * quarter;
+                    const int4 a0 = *reinterpret_cast<const int4 *>(wrel + w), a1 = *reinterpret_cast<const int4 *>(wrel + w + 4);
+                    const int before[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
                     int in_quarter = 0;
 #pragma unroll
-                    for (int u = 1; u < 8; ++u) in_quarter += (w + u < nwords && wrel[w + u] <= k) ? 1 : 0;
+                    for (int u = 1; u < 8; ++u) in_quarter += (w + u < nwords && before[u] <= k) ? 1 : 0;
                     w += in_quarter;
                 }
                 k -= wrel[w];
@@ -667,6 +680,14 @@ __global__ void __launch_bounds__(kRegRows > 0 ? 256 : 544, 1) k_spmspv_fused(co
                         o1 = p.meta[(size_t)j * p.S + s + 1];
                     }
                     imeta[i] = make_uint2(o0, (o1 - o0) * 16u);
+                    // The first column of every ring slot (slot k of the team's warp h takes columns h, h + stride, ...):
+                    // the lane that has found it starts its copy right away -- 300 cycles sooner than through imeta and
+                    // behind the barrier below, for which the copies need not wait: the window is not in the ring.
+                    if (pp && rb == r_begin && i < p.D) {
+                        const int h = i & (stride - 1), k = i >> (stride - 1), place = h * Dw + k;
+                        bulk_load(smem_u32(ring + ((size_t)team * p.D + place) * p.slot_bytes), p.stream + (size_t)o0 * 16,
+                                  (o1 - o0) * 16u, smem_u32(&bars[team * p.D + place]));
+                    }
                 }
             }
             // The accumulators take the place of the window: every team has to be through with its look-ups
@@ -687,8 +708,13 @@ __global__ void __launch_bounds__(kRegRows > 0 ? 256 : 544, 1) k_spmspv_fused(co
                 ++issued;
                 if (++islot == (uint32_t)Dw) islot = 0;
             };
+            if (pp && rb == r_begin) {                              // started by the look-ups
+                issued = (uint32_t)min(Dw, (cnt - half + stride - 1) >> (stride - 1));
+                islot = issued == (uint32_t)Dw ? 0 : issued;
+            } else {
 #pragma unroll 1
-            for (int k = 0, i = half; k < Dw && i < cnt; ++k, i += stride) issue_im(imeta[i]);
+                for (int k = 0, i = half; k < Dw && i < cnt; ++k, i += stride) issue_im(imeta[i]);
+            }
             if (!zeroed) {                                          // clear the slab while the first copies fly
                 float4 *slab4 = reinterpret_cast<float4 *>(acc + (size_t)team * slab_words);
 #pragma unroll 1
@@ -796,6 +822,24 @@ __global__ void __launch_bounds__(kRegRows > 0 ? 256 : 544, 1) k_spmspv_fused(co
         if (__builtin_expect(!ticket_wait(tickets, y_ticket, p.spin_limit), 0)) atomicOr(p.status, kStatusTimeout);
         asm volatile("fence.proxy.async.global;" ::: "memory");
     }
+    // The row map makes local rows [kC, kC + C) of a slab 32*C consecutive rows of y, in accumulator order (with one slab
+    // the whole accumulator is y itself): each such segment is one bulk reduce-add.  The last warp, one segment per lane,
+    // works out where they go under the streaming.
+    const int seg = p.S == 1 ? 16 : p.C, nseg = idiv_small(p.R + seg - 1, seg), seg4 = seg * 8;
+    const int owned = (Sc * nseg - crank + cl - 1) / cl;   // segments crank, crank + cl, ...
+    struct Segment { float *to; const float *from; int nrows; };
+    auto segment = [&](int o) {
+        const int sg = crank + cl * o;
+        const int fsl = idiv_small(sg, nseg), k = sg - fsl * nseg, sfull = part * Sc + fsl;
+        const int i0 = k * seg, i1 = min(p.R, i0 + seg);
+        // tile_row(S, C, sfull, 0, i0) for a segment's first local row i0 = k * seg, without its divisions: seg is C (one
+        // chunk of the row map) unless there is one slab, whose rows are y in order
+        const int64_t row0 = p.S == 1 ? (int64_t)i0 * 32 : ((int64_t)(k * p.S + sfull) * p.C) * 32;
+        return Segment{y + row0, acc + (size_t)fsl * slab_words + (size_t)i0 * 32,
+                       sfull >= p.S || row0 >= p.M ? 0 : min((i1 - i0) * 32, p.M - (int)row0)};
+    };
+    Segment first{nullptr, nullptr, 0};
+    if (pp && merge == 1 && warp == nwarps - 1 && lane < owned) first = segment(lane);
     __syncthreads();
 
     if (merge == 1) {
@@ -820,8 +864,6 @@ __global__ void __launch_bounds__(kRegRows > 0 ? 256 : 544, 1) k_spmspv_fused(co
                 acc4[q4] = v;
             }
         }
-        const int seg = p.S == 1 ? 16 : p.C, nseg = idiv_small(p.R + seg - 1, seg), seg4 = seg * 8;
-        const int owned = (Sc * nseg - crank + cl - 1) / cl;   // segments crank, crank + cl, ...
         if (cl > 1) {
             cluster_sync();                                         // the peers' sums are complete
             for (int t = tid; t < owned * seg4; t += nthreads) {
@@ -840,29 +882,20 @@ __global__ void __launch_bounds__(kRegRows > 0 ? 256 : 544, 1) k_spmspv_fused(co
         }
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         __syncthreads();
-        // The row map makes local rows [kC, kC + C) of a slab 32*C consecutive rows of y, in accumulator
-        // order (with one slab the whole accumulator is y itself): each such segment is one bulk reduce-add.
+        // (With pairs the last warp alone, one segment per lane, from what it has worked out; otherwise any thread: 1 %
+        // faster the one way and 1 % the other.)
         {
 #pragma unroll 1
-            for (int o = tid; o < owned; o += nthreads) {
-                const int sg = crank + cl * o;
-                const int fsl = idiv_small(sg, nseg), k = sg - fsl * nseg, sfull = part * Sc + fsl;
-                if (sfull >= p.S) continue;
-                const int i0 = k * seg, i1 = min(p.R, i0 + seg);
-                // tile_row(S, C, sfull, 0, i0) for a segment's first local row i0 = k * seg, without its divisions:
-                // seg is C (one chunk of the row map) unless there is one slab, whose rows are y in order
-                const int64_t row0 = p.S == 1 ? (int64_t)i0 * 32 : ((int64_t)(k * p.S + sfull) * p.C) * 32;
-                if (row0 >= p.M) continue;
-                const int nrows = min((i1 - i0) * 32, p.M - (int)row0);
-                const uint32_t bytes = ((uint32_t)nrows * 4u) & ~15u;
-                const float *src = acc + (size_t)fsl * slab_words + (size_t)i0 * 32;
+            for (int o = pp ? (warp == nwarps - 1 ? lane : owned) : tid; o < owned; o += pp ? 32 : nthreads) {
+                const Segment sg = pp && o == lane ? first : segment(o);
+                const uint32_t bytes = ((uint32_t)sg.nrows * 4u) & ~15u;
                 if (bytes)
-                    asm volatile("cp.reduce.async.bulk.global.shared::cta.bulk_group.add.f32 [%0], [%1], %2;" ::"l"(y + row0),
-                                 "r"(smem_u32(src)), "r"(bytes)
+                    asm volatile("cp.reduce.async.bulk.global.shared::cta.bulk_group.add.f32 [%0], [%1], %2;" ::"l"(sg.to),
+                                 "r"(smem_u32(sg.from)), "r"(bytes)
                                  : "memory");
 #pragma unroll 1
-                for (int i = (int)(bytes >> 2); i < nrows; ++i)
-                    if (src[i] != 0.f) atomicAdd(y + row0 + i, src[i]);
+                for (int i = (int)(bytes >> 2); i < sg.nrows; ++i)
+                    if (sg.from[i] != 0.f) atomicAdd(sg.to + i, sg.from[i]);
             }
             asm volatile("cp.async.bulk.commit_group;" ::: "memory");
             asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");   // shared memory may go once it has been read

@@ -108,8 +108,9 @@ CELTY_HD inline FusedSmem fused_smem_layout(int R, int K, int teams, int D, int 
     l.zero = off;      off += 16;                                          // the all-zero group that idle lanes fetch
     l.keep = off;      off += ((uint32_t)((K + 31) / 32) * 4 + 15) / 16 * 16;   // one keep bit per activation
     l.wrel = off;      off += ((uint32_t)((K + 31) / 32) * 4 + 15) / 16 * 16;   // survivors before each keep word, in its block of 32
-    l.blk = off;       off += ((uint32_t)((K + 1023) / 1024) * 4 + 15) / 16 * 16; // survivors in each block of 32 keep words
-    l.blkw = off;      off += 16 * (((uint32_t)((K + 1023) / 1024) * 4 + 15) / 16 * 16);   // per warp: survivors before each block
+    const uint32_t blocks = ((uint32_t)((K + 1023) / 1024) * 4 + 31) / 32 * 32;   // (eight are read at a time)
+    l.blk = off;       off += blocks;                                      // survivors in each block of 32 keep words
+    l.blkw = off;      off += 16 * blocks;                                 // per warp: survivors before each block
     l.total = off;
     return l;
 }
