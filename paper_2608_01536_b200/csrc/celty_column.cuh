@@ -75,7 +75,8 @@ __device__ __noinline__ uint4 ragged_group(const uint16_t *x, int K, int q)
     return make_uint4(h[0], h[1], h[2], h[3]);
 }
 
-// One keep bit per activation of x[32w .. 32w+31] (zero past the end of x).
+// One keep bit per activation of x[32w .. 32w+31] (zero past the end of x).  Plain loads, as in the fused kernel: x may be
+// the work of a kernel that has not ended when this one starts.
 __device__ __forceinline__ uint32_t keep_word(const uint16_t *x, int K, int w, __half2 tau2)
 {
     const int ngroups = (K + 7) >> 3;
@@ -85,7 +86,7 @@ __device__ __forceinline__ uint32_t keep_word(const uint16_t *x, int K, int w, _
     for (int c = 0; c < 4; ++c) {
         const int q = 4 * w + c;
         h[c] = make_uint4(0u, 0u, 0u, 0u);                          // never kept (tau >= 0)
-        if (8 * q + 8 <= K) h[c] = __ldg(reinterpret_cast<const uint4 *>(x + 8 * q));
+        if (8 * q + 8 <= K) h[c] = *reinterpret_cast<const uint4 *>(x + 8 * q);
         else if (q < ngroups) h[c] = ragged_group(x, K, q);
     }
 #pragma unroll
@@ -194,7 +195,7 @@ __global__ void __launch_bounds__(kColumnThreads, 1) k_spmspv_column(const Colum
                     if (k >= c) { k -= c; pos += sh; }
                 }
                 const int j = 32 * at + pos;
-                const uint16_t xb = __ldg(p.x + j);
+                const uint16_t xb = p.x[j];
                 items[i] = make_int2(j, (int)xb);
                 imeta[i] = j >= win0 && j < win0 + kColumnWindow ? window[j - win0] : __ldg(p.meta + j);
                 p.idx[r] = j;

@@ -260,12 +260,14 @@ __device__ __forceinline__ uint32_t keep_byte(const uint4 v, __half2 tau2)
     return ~((((lo & 0x08040201u) | (hi & 0x80402010u)) * 0x01010101u) >> 24) & 0xFFu;
 }
 
-// Keep bits of 32 activations (x 16-byte aligned): four independent 128-bit loads.
+// Keep bits of 32 activations (x 16-byte aligned): four independent 128-bit loads.  Plain ones, here and wherever x is
+// read: the kernel that writes x (k_swiglu, k_epilogue) may still run when this block starts, and a non-coherent load
+// (__ldg) is defined only for memory that nobody writes while the kernel runs.
 __device__ __forceinline__ uint32_t keep_word32(const uint16_t *x, __half2 tau2)
 {
     uint4 h[4];
 #pragma unroll
-    for (int c = 0; c < 4; ++c) h[c] = __ldg(reinterpret_cast<const uint4 *>(x) + c);
+    for (int c = 0; c < 4; ++c) h[c] = reinterpret_cast<const uint4 *>(x)[c];
     return keep_byte(h[0], tau2) | keep_byte(h[1], tau2) << 8 | keep_byte(h[2], tau2) << 16 | keep_byte(h[3], tau2) << 24;
 }
 
@@ -661,7 +663,7 @@ __global__ void __launch_bounds__(kRegRows > 0 ? 256 : 544, 1) k_spmspv_fused(co
                     if (k >= c) { k -= c; pos += sh; }
                 }
                 j = 32 * w + pos;
-                xb = __ldg(x + j);                                   // x went through L1 in the thresholding pass
+                xb = x[j];                                           // x went through L1 in the thresholding pass
                 }
                 items[i] = make_int2(j, (int)xb);
                 if (!from_list && lists && part == 0 && sl == 0) {

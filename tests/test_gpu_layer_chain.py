@@ -165,6 +165,43 @@ def test_swiglu_made_inside_the_down_projection(I, K, d_a, d_h):
         assert np.all(err <= ref["tol_yd"]), (call, float((err - ref["tol_yd"]).max()))
 
 
+@pytest.mark.parametrize("M,K", [(256, 512), (700, 1333), (4096, 2048), (3000, 9000)])
+def test_activations_are_read_as_the_kernel_before_left_them(M, K):
+    """Calls enqueued back to back, whose activations another kernel of the chain writes into the same place every time
+    while the product's blocks may already be on the GPU: SiLU(gate) * up in the workspace (another gate_up in every
+    call), and the FP16 copy of one product as the next one's x, for both layouts.  Every value is exact: SiLU(32) is
+    32 in FP32, the rest are small integers."""
+    Wd, md = synth.integer_weights(51, M, K), synth.mask_bernoulli(51, M, K, 0.3)
+    down = celty.Matrix(Wd, md, device="cuda")
+    calls = 12
+    hs = [(32.0 * synth.integer_activations(60 + c, K)).astype(np.float16) for c in range(calls)]
+    gate_up = [_dev(np.concatenate([np.full(K, 32.0), h.astype(np.float64) / 32.0]).astype(np.float32)) for h in hs]
+    h_out = [torch.zeros(K, dtype=torch.float16, device="cuda") for _ in range(calls)]
+    ys = [torch.full((M,), -1.0, device="cuda") for _ in range(calls)]
+    for c in range(calls):
+        down.spmspv_swiglu(gate_up[c], 40.0, y=ys[c], h_out=h_out[c])
+    torch.cuda.synchronize()
+    assert down.last_status() == 0
+    for c in range(calls):
+        assert np.array_equal(h_out[c].cpu().numpy(), hs[c]), c
+        assert np.array_equal(ys[c].cpu().numpy().astype(np.float64), orc.masked_gemv(Wd, md, hs[c], 40.0, threads=8)[0]), c
+    # first: K x 64, its FP16 result is x of the second, always in the same place
+    Wf = synth.integer_weights(52, K, 64)
+    first = celty.Matrix(Wf, None, device="cuda")
+    xs = [synth.integer_activations(80 + c, 64) for c in range(calls)]
+    xd = [_dev(x) for x in xs]
+    between, y_first = torch.zeros(K, dtype=torch.float16, device="cuda"), torch.empty(K, device="cuda")
+    for second in (down, celty.Matrix(Wd, md, layout=celty.LAYOUT_COLUMN, device="cuda")):
+        for c in range(calls):
+            first.spmspv_ex(xd[c], 1.0, y=y_first, fp16_out=between)
+            second.spmspv(between, 2.0, y=ys[c])
+        torch.cuda.synchronize()
+        assert first.last_status() == 0 and second.last_status() == 0
+        for c in range(calls):
+            mid = orc.masked_gemv(Wf, np.ones_like(Wf, dtype=np.uint8), xs[c], 1.0)[0].astype(np.float16)
+            assert np.array_equal(ys[c].cpu().numpy().astype(np.float64), orc.masked_gemv(Wd, md, mid, 2.0, threads=8)[0]), c
+
+
 def test_list_input_matches_thresholded_input():
     """A list made by the oracle's compaction (shuffled: any order is allowed) gives the product that thresholding x
     inside the call gives."""
