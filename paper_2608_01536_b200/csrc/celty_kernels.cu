@@ -1232,10 +1232,12 @@ namespace {
 
 constexpr int kEpilogueToHost = 3;
 
-// The device address of [p, p + bytes) if all of it is one range of page-locked host memory that the current device
-// can address, else null.
+// The device address of the floats at [p, p + bytes) if all of it is one range of page-locked host memory that the
+// current device can address, else null; also null where the floats do not start on 4 bytes, which a copy can take and
+// a kernel's stores cannot.
 void *mapped_host(const void *p, size_t bytes)
 {
+    if ((uintptr_t)p & 3) return nullptr;
     using Query = CUresult (*)(unsigned, CUpointer_attribute *, void **, CUdeviceptr);
     static const Query query = [] {
         void *fn = nullptr;
@@ -1254,7 +1256,7 @@ void *mapped_host(const void *p, size_t bytes)
     void *into[5] = {&type, &managed, &device, &start, &size};
     if (query(5, what, into, (CUdeviceptr)(uintptr_t)p) != CUDA_SUCCESS) return nullptr;
     if (type != CU_MEMORYTYPE_HOST || managed || !device || !start || device < start || size < bytes ||
-        device - start > size - bytes)
+        device - start > size - bytes || (device & 3))
         return nullptr;
     return reinterpret_cast<void *>((uintptr_t)device);
 }

@@ -632,3 +632,23 @@ def test_host_vectors_pinned_and_pageable(M, K, kw):
         assert m.last_status() == 0
         idx, _ = m.last_compaction()
         assert np.array_equal(idx.cpu().numpy(), orc.compact(x, 1.0)[0])
+
+
+@pytest.mark.parametrize("shift", [0, 1, 2, 3, 4, 6])
+def test_host_result_at_any_byte_of_page_locked_memory(shift):
+    """The C entry point takes y_host anywhere: places that do not start on 4 bytes are copied to, not stored to."""
+    M, K = 515, 260
+    W = synth.integer_weights(35, M, K)
+    mask = synth.mask_bernoulli(35, M, K, 0.5)
+    x = synth.integer_activations(36, K)
+    m = celty.Matrix(W, mask, device="cuda")
+    xh = torch.from_numpy(x).pin_memory()
+    raw = torch.full((4 * M + 16,), 0x55, dtype=torch.uint8).pin_memory()
+    stage_x, stage_y = torch.empty(K, dtype=torch.float16, device="cuda"), torch.empty(M, device="cuda")
+    stream = torch.cuda.current_stream().cuda_stream
+    assert celty.load().celty_spmspv_host(m._h, xh.data_ptr(), 1.0, raw.data_ptr() + shift, stage_x.data_ptr(),
+                                          stage_y.data_ptr(), stream) == 0
+    got = raw.numpy()
+    y = np.frombuffer(got[shift:shift + 4 * M].tobytes(), np.float32)
+    assert np.array_equal(y.astype(np.float64), orc.masked_gemv(W, mask, x, 1.0, threads=4)[0])
+    assert np.all(got[:shift] == 0x55) and np.all(got[shift + 4 * M:] == 0x55)
