@@ -305,16 +305,18 @@ int celty_spmspv_host(celty_matrix *m, const void *x_host, float tau, void *y_ho
  *              copied celty_host_image there, or it is the buffer given to celty_bind_device)
  *   x_dev      K FP16 (device, 16-byte aligned), not modified
  *   y_dev      M FP32 (device, 16-byte aligned), overwritten
- * It runs the kernel of celty_spmspv (with the library's own launch choices) and calls no cudaMalloc,
- * cudaFree or other allocating routine.  (Slabs per block and tile heights that leave no room for that
- * kernel's rings: the two-launch path of celty_set_launch variant 1.)
+ * It runs a kernel that clears y and then the kernel of celty_spmspv (with the library's own launch choices) and
+ * calls no cudaMalloc, cudaFree or other allocating routine.  (Slabs per block and tile heights that leave no room
+ * for that kernel's rings: the two-launch path of celty_set_launch variant 1.)  No thread block of the call waits
+ * for another one, so it may share the GPU with whatever else runs.  There is no status word to read after it: should
+ * a block's wait for its own copies from the image run out (celty_set_wait_limit), the rows concerned are NaN.
  * Limit: K <= 32768 (the scratch array holds 196 864 bytes: a header, int32 indices and FP16 values
  * for that many columns; every GPU that loads the library carries it until the process exits);
  * larger K returns CELTY_ELIMIT.
  * The first call on each device looks up the array's device address (cudaGetSymbolAddress, with that
  * device current); make that first call before any stream capture.
- * All calls on a device share the one array, which keeps the previous call's contents (count and list are
- * rewritten by every call, a ticket of the thread blocks counts on), and two calls that overlap on
+ * All calls on a device share the one array, which keeps the previous call's contents; nothing in it
+ * has to start at zero (count and list are rewritten by every call), but two calls that overlap on
  * the GPU (different streams, or one stream of another thread) race on it: serialise them.
  * Errors: CELTY_EINVAL (null, misaligned, tau < 0 or not finite, COLUMN-layout handle), CELTY_ELIMIT,
  * CELTY_ECUDA.

@@ -2,7 +2,8 @@
 // anonymous namespace, after decode_group).
 //
 // One launch does the whole call (Sections 3.1-3.3):
-//   a0  the last warp of every block clears its share of y and takes a ticket (the merge at the end adds into y);
+//   a0  the last warp of every block clears its share of y and takes a ticket (the merge at the end adds into y; without
+//       tickets y was cleared by a kernel before this one, and no block waits for another);
 //   a1  every block thresholds all of x (K <= a few 10k values, served by L2) into one keep bit per
 //       activation and ranks the survivors (popcounts + warp scans); each warp team then looks up the
 //       columns whose ranks belong to it -- the list is balanced over all teams by count -- and their
@@ -26,9 +27,9 @@
 // Rows are split over P parts of Sc slabs each, columns over the blocks of a part and, inside a block, over
 // G teams per slab; a team = one warp (or, with pp, two warps that take turns) with its own accumulator slab.
 // Blocks that are left over when the grid does not divide by P may serve several parts each with fewer teams per
-// part (FusedParams::mix).  Every block must be resident at once (grid <= SM count) because of the tickets.  All
+// part (FusedParams::mix).  With tickets every block must be resident at once (grid <= SM count).  All
 // waits are bounded: when one runs out the kernel sets kStatusTimeout in the status word and carries on to a clean
-// exit.
+// exit; what a team that gave up was to add to y is NaN.
 
 constexpr uint32_t kSpinLimit = 1u << 21;   // default for FusedParams::spin_limit
 
@@ -529,11 +530,13 @@ __global__ void __launch_bounds__(kRegRows > 0 ? 256 : 544, 1) k_spmspv_fused(co
     if (merge == 1 && warp == nwarps - 1) {
         const int b = (int)blockIdx.x;
         const int r0 = b * p.clear_rows + min(b, p.clear_extra), r1 = r0 + p.clear_rows + (b < p.clear_extra ? 1 : 0);
+        if (p.tickets) {
 #pragma unroll 1
-        for (int i = r0 + lane; i < r1; i += 32) y[i] = 0.f;
+            for (int i = r0 + lane; i < r1; i += 32) y[i] = 0.f;
+        }
         if (!kBatch && blockIdx.x == 0 && lane == 0 && p.ep_count) *p.ep_count = 0;      // k_epilogue appends to it
         __syncwarp();
-        if (lane == 0) {
+        if (lane == 0 && p.tickets) {
             __threadfence();
             // The ticket counts modulo 2 * gridDim.x, so it never has to be reset: calls alternate between
             // waiting for the lower and for the upper half.
@@ -813,6 +816,10 @@ __global__ void __launch_bounds__(kRegRows > 0 ? 256 : 544, 1) k_spmspv_fused(co
                 mbar_wait_bounded(bar0 + 8u * slot, parity, p.spin_limit);
                 if (++slot == (uint32_t)Dw) { slot = 0; parity ^= 1u; }
             }
+            // the rows of this slab are NaN then: celty_spmspv_static has no status word that its caller could read
+            if (s < p.S)
+#pragma unroll 1
+                for (int i = lane; i < slab_words; i += 32) acc[(size_t)team * slab_words + i] = __int_as_float(0x7FC00000);
             if (lane == 0) atomicOr(p.status, kStatusTimeout);
         }
     }
@@ -821,7 +828,7 @@ __global__ void __launch_bounds__(kRegRows > 0 ? 256 : 544, 1) k_spmspv_fused(co
     // puts the other blocks' clearing stores (generic proxy) before this block's reduce-adds (asynchronous proxy),
     // were 700 cycles of every block's end when they came after it.
     if (merge == 1 && warp == nwarps - 1 && lane == 0) {
-        if (__builtin_expect(!ticket_wait(tickets, y_ticket, p.spin_limit), 0)) atomicOr(p.status, kStatusTimeout);
+        if (__builtin_expect(p.tickets && !ticket_wait(tickets, y_ticket, p.spin_limit), 0)) atomicOr(p.status, kStatusTimeout);
         asm volatile("fence.proxy.async.global;" ::: "memory");
     }
     // The row map makes local rows [kC, kC + C) of a slab 32*C consecutive rows of y, in accumulator order (with one slab

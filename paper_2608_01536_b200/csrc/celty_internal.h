@@ -125,7 +125,8 @@ struct FusedParams {
     uint16_t *val;
     int32_t *count;
     uint32_t *status;
-    uint32_t *tickets;         // [0] y cleared / partial stored, [1] departed (ordered merge)
+    uint32_t *tickets;         // [0] y cleared / partial stored, [1] departed (ordered merge); null (bulk reduce-add merge):
+                               // a kernel before this one has cleared y
     float *partials;           // gridDim.x vectors of Sc * R * 32 floats (accumulator layout)
     int M, K, R, S, C;         // rows, columns, local rows per tile, slabs, chunk of the row map (tile_row)
     int G, Sc, P, D;           // teams per slab, slabs per block, row parts, ring depth

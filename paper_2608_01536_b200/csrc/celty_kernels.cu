@@ -1016,7 +1016,7 @@ extern "C" int celty_spmspv_list(celty_matrix *m, const int32_t *idx_dev, const 
 
 // ------------------------------------------------------------------------------------------------
 // celty_spmspv_static: scratch in a file-scope device array instead of a caller-provided workspace,
-// for callers that cannot allocate device memory.  Layout of the array: [256 B header: status, count]
+// for callers that cannot allocate device memory.  Layout of the array: [256 B header: status (not read), count]
 // [int32 idx[kStaticMaxK]][uint16 val[kStaticMaxK]].
 // ------------------------------------------------------------------------------------------------
 namespace {
@@ -1073,24 +1073,31 @@ extern "C" int celty_spmspv_static(const celty_matrix *m, const void *image_dev,
     uint16_t *val = reinterpret_cast<uint16_t *>(scratch + 256 + (size_t)kStaticMaxK * 4);
     float *y = static_cast<float *>(y_dev);
     const uint8_t *image = static_cast<const uint8_t *>(image_dev);
-    // The single-launch kernel with its ticket in the shared array.  Every block of every call takes the ticket exactly
-    // once and all calls have one block per SM, so the count is back at a multiple of that after any call, also after
-    // calls that overlapped in spite of the rule above.  4096 x 4096, 50 % / 50 %: 28.7 us with the two kernels below,
-    // 8.4 us this way.  The handle's launch choices are for its workspace's calls and are not looked at.
+    // The kernel of celty_spmspv behind one that clears y.  With a ticket in the shared array instead, as the workspace's
+    // calls have it, blocks would wait for one another: next to a kernel of another stream that keeps some of the SMs
+    // they could give up, and a caller without a workspace has no status word to find out by.  4096 x 4096, 50 % / 50 %:
+    // 28.7 us with the two kernels below, 9.4 us this way (7.8 with a ticket).  The handle's launch choices are for its
+    // workspace's calls and are not looked at, but for the limit of the waits.
     FusedPlan plan;
-    const LaunchKnobs knobs;
+    LaunchKnobs knobs;
+    knobs.spin_limit = m->spin_limit;
     rc = plan_launch(m, knobs, di, 1, &plan);
-    if (rc == CELTY_OK && plan.lean && plan.grid == std::min(di.sms, kMaxBlocks)) {
+    if (rc == CELTY_OK && plan.lean) {
         FusedParams fp = plan_params(m, knobs, plan, image);
         fp.x = static_cast<const uint16_t *>(x_dev);
         fp.tau = tau;
         fp.y = y;
         fp.idx = idx; fp.val = val; fp.count = count;
         fp.status = reinterpret_cast<uint32_t *>(scratch);
-        fp.tickets = fp.status + 2;
+        fp.tickets = nullptr;
         // nothing of the image is read before the previous kernel of the stream is complete: it may be the one that
         // puts it there (0.1 us)
         fp.win_cols = 0;
+        // (the limit is raised before the first launch: an error return leaves y untouched)
+        rc = plan.lean == 2 ? ensure_smem(k_spmspv_fused<false, 0, 2>, plan.smem, g_granted_lean[1])
+                            : ensure_smem(k_spmspv_fused<false, 0, 1>, plan.smem, g_granted_lean[0]);
+        if (rc == CELTY_OK) rc = launch_clear(y, m->M, st);
+        if (rc) return rc;
         return plan.lean == 2 ? launch_fused(k_spmspv_fused<false, 0, 2>, g_granted_lean[1], knobs, plan, 1, fp, st)
                               : launch_fused(k_spmspv_fused<false, 0, 1>, g_granted_lean[0], knobs, plan, 1, fp, st);
     }

@@ -60,3 +60,29 @@ def permute_for_lane_tiles(W, mask, S, R, C):
     Wp[live] = W[rows[live]]
     mp[live] = mask[rows[live]]
     return Wp, mp, rows
+
+
+def hold_some_sms(celty, synth, stream, blocks=40, polls=400_000):
+    """Enqueues on `stream` a product that keeps `blocks - 1` SMs to itself for some tenths of a second, by a bounded
+    wait that runs out: its ticket is moved so that all blocks but one wait for a count that never comes.  Returns the
+    handle (whose next last_status() is CELTY_ETIMEOUT) and an event behind the call."""
+    import time
+
+    import torch
+    holder = celty.Matrix(synth.weights(70, 4096, 1024), None, device="cuda")
+    holder.set_launch(grid=blocks)
+    plan = holder.launch_plan()
+    assert plan["grid"] == blocks and plan["smem_bytes"] > 120 * 1024        # no block of the products fits beside one
+    x = torch.from_numpy(synth.activations(71, 1024, "laplace")).cuda()
+    holder.spmspv(x, 0.5)
+    torch.cuda.synchronize()
+    assert holder.last_status() == 0
+    ticket = holder._ws[8:12].view(torch.int32)
+    ticket[0] = blocks - 1
+    holder.set_wait_limit(polls)
+    torch.cuda.synchronize()
+    done = torch.cuda.Event()
+    holder.spmspv(x, 0.5, stream=stream)
+    done.record(stream)
+    time.sleep(0.01)                                                         # it is on the SMs now
+    return holder, done

@@ -12,6 +12,7 @@ import numpy as np
 import pytest
 import torch
 
+from conftest import hold_some_sms
 from oracle import celty_oracle as orc
 from paper_2608_01536_b200 import build, celty, synth
 
@@ -142,3 +143,27 @@ def test_static_entry_point_behind_the_kernel_that_writes_the_image():
         torch.bitwise_xor(scrambled, key, out=m._image)
         y = m.spmspv_static(xd, 1.0)
         assert np.array_equal(y.cpu().numpy().astype(np.float64), y_ref)
+
+
+def test_static_call_needs_only_the_sms_that_are_free():
+    """No block of the call waits for another: while a kernel of another stream keeps 39 SMs, the call's blocks run on
+    the others, one after another where they have to, and the call is over before that kernel is."""
+    build.build()
+    M, K = 4096, 2048
+    W = synth.integer_weights(8, M, K)
+    mask = synth.mask_bernoulli(8, M, K, 0.5)
+    x = synth.integer_activations(9, K)
+    m = celty.Matrix(W, mask, device="cuda")
+    y_ref, _ = orc.masked_gemv(W, mask, x, 1.0, threads=8)
+    xd = torch.from_numpy(x).cuda()
+    y = torch.full((M,), 7.0, device="cuda")
+    m.spmspv_static(xd, 1.0, y=torch.empty_like(y))            # everything loaded
+    torch.cuda.synchronize()
+    other, mine = torch.cuda.Stream(), torch.cuda.Stream()
+    holder, held = hold_some_sms(celty, synth, other)
+    m.spmspv_static(xd, 1.0, y=y, stream=mine)
+    mine.synchronize()
+    assert not held.query()
+    held.synchronize()
+    assert holder.last_status() == -5
+    assert np.array_equal(y.cpu().numpy().astype(np.float64), y_ref)
