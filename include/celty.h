@@ -177,10 +177,14 @@ int celty_compact(const void *x_dev, int64_t K, float tau, int32_t *idx_dev, uin
  * the surviving columns, decodes their runs to rows, accumulates value * x_j in shared memory in
  * FP32 (one rounding per multiply-add) and merges the thread blocks' results into y (FP32 adds in L2
  * by bulk reduce-add copies; celty_set_launch can select a sum in a fixed order instead); the COLUMN
- * layout has one kernel of the same outline, behind a compaction kernel where K is so large that its keep bits leave
- * no room in shared memory.  On a stream of calls the kernel's
+ * layout has one kernel of the same outline behind a small one that clears y (a compaction kernel where K is so large
+ * that its keep bits leave no room in shared memory).  On a stream of calls the kernel's
  * set-up overlaps the end of the previous kernel (programmatic dependent launch); it waits for that
  * kernel before it reads x or touches y or the workspace.
+ * The thread blocks of the fused kernel wait (with a limit) for one another before they add into y, so all of them have
+ * to find an SM: beside a kernel of another stream that keeps some of the SMs, the call takes until they are free, and
+ * past the limit it ends with CELTY_ETIMEOUT from celty_last_status.  (Not so: COLUMN handles, the two-launch variant,
+ * celty_spmspv_static.)
  *   x_dev  K FP16 (device, 16-byte aligned), not modified
  *   y_dev  M FP32 (device, 16-byte aligned), overwritten
  * The order of FP32 additions is not fixed (Section 4.2: scatter-accumulation is order-

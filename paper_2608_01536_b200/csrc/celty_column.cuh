@@ -13,12 +13,12 @@
 // What bounds it: shared memory.  The rows of the 32 lanes fall on the banks as good as at random (8 entries, or
 // some 16 rows at 50 % density, lie between two lanes), so a load or store takes 3 to 4 wavefronts where the lane
 // tiles' takes one; entries per SM / 32 x 7 wavefronts is 3.2 us at 4096 x 4096, 50 % / 50 %.  Measured there:
-// 11.7 us against 41.6 us for warps that each took whole columns and added with shared-memory atomics, behind a
+// 11.8 us against 41.6 us for warps that each took whole columns and added with shared-memory atomics, behind a
 // one-block compaction kernel.
 //
-// a0 and a1 as in the fused kernel: every block clears its share of y and takes a ticket, and thresholds all of x.
-// Where K's keep words leave no room the list comes from k_compact, which also clears y; more blocks than fit the
-// device at once cannot wait for one another's tickets, and k_clear comes before them.
+// a0: k_clear clears y ahead of this kernel (11.4 us where every block cleared its share and all waited for one
+// another's ticket, but a call must not need all SMs at once).  a1 as in the fused kernel: every block thresholds all of
+// x; where K's keep words leave no room the list comes from k_compact, which also clears y.
 
 struct ColumnParams {
     const uint2 *meta;          // [K] {offset/16, entries}
@@ -28,10 +28,8 @@ struct ColumnParams {
     int32_t *idx;               // the compacted list: written here, or read when own_list is 0
     uint16_t *val;
     int32_t *count;
-    float *y;
+    float *y;                   // zero: the kernel before this one cleared it
     uint32_t *status;
-    uint32_t *ticket;           // null: the kernel before this one cleared y
-    uint32_t spin_limit;
     int M, K;
     int W, groups;              // warps per column, columns in flight per block (W * groups <= 32, groups <= 15 if W > 1)
     int cap;                    // columns a block looks up at a time
@@ -126,15 +124,6 @@ __global__ void __launch_bounds__(kColumnThreads, 1) k_spmspv_column(const Colum
     if (p.own_list && tid < kColumnWindow && win0 + tid < p.K) window[tid] = __ldg(p.meta + win0 + tid);
     asm volatile("griddepcontrol.wait;" ::: "memory");
 
-    uint32_t y_ticket = 0;
-    if (p.ticket && warp == kColumnThreads / 32 - 1) {
-        for (int i = blockIdx.x * 32 + lane; i < p.M; i += gridDim.x * 32) p.y[i] = 0.f;
-        __syncwarp();
-        if (lane == 0) {
-            __threadfence();
-            y_ticket = atomicInc(p.ticket, 2u * gridDim.x - 1u);
-        }
-    }
     // ---- a1: keep words and the survivors before each of them
     int n = 0;
     if (p.own_list) {
@@ -304,10 +293,6 @@ __global__ void __launch_bounds__(kColumnThreads, 1) k_spmspv_column(const Colum
     }
     if (out_of_range) atomicOr(p.status, kStatusBounds);
     if (p0 >= p1) return;                                              // (the same for the whole block)
-    if (p.ticket && warp == kColumnThreads / 32 - 1) {
-        if (lane == 0 && !ticket_wait(p.ticket, y_ticket, p.spin_limit)) atomicOr(p.status, kStatusTimeout);
-        __syncwarp();
-    }
     // ---- a5: the groups' accumulators, then one bulk reduce-add per 512 rows of y
     if (p.groups > 1) {
         float4 *acc4 = reinterpret_cast<float4 *>(acc);
@@ -323,7 +308,7 @@ __global__ void __launch_bounds__(kColumnThreads, 1) k_spmspv_column(const Colum
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     __syncthreads();
     for (int r0 = tid * 512; r0 < p.M; r0 += kColumnThreads * 512) {
-        // the clearing of y by other blocks or another kernel (generic proxy) comes before these adds (asynchronous proxy)
+        // the clearing of y (generic proxy) comes before these adds (asynchronous proxy)
         asm volatile("fence.proxy.async.global;" ::: "memory");
         const int nrows = min(512, p.M - r0);
         const uint32_t bytes = ((uint32_t)nrows * 4u) & ~15u;

@@ -461,7 +461,7 @@ int ensure_smem(Kernel kernel, size_t bytes, int *granted /* [64], per device */
 #include "celty_fused.cuh"
 #include "celty_column.cuh"
 
-// y = 0, for the products whose blocks do not clear y themselves.  Bound by its launch: it may be scheduled while the
+// y = 0, for the products whose blocks do not clear y themselves (COLUMN, celty_spmspv_static).  Bound by its launch: it may be scheduled while the
 // previous kernel of the stream drains and lets the next one do the same.
 __global__ void __launch_bounds__(256) k_clear(float *__restrict__ y, int M)
 {
@@ -927,8 +927,9 @@ int run_product(celty_matrix *m, const void *x_dev, float tau, const ListInput *
         ea.idx = ep->list_idx; ea.val = ep->list_val; ea.count = ep->list_count;
         return launch_epilogue(m, ea, y, st);
     }
-    // two launches: compaction (which also clears y), then the product.  Sizes are checked and the
-    // shared-memory limit is raised before the first launch, so that an error return leaves y untouched.
+    // two launches: one that clears y (COLUMN: k_clear; lane tiles, and a very long x: the compaction), then the product.
+    // Sizes are checked and the shared-memory limit is raised before the first launch, so that an error return leaves y
+    // untouched.
     if (m->layout == CELTY_LAYOUT_COLUMN) {
         const int grid = m->grid > 0 ? m->grid : di.sms;
         const ColumnShape shape = column_shape(m, di, grid);
@@ -940,20 +941,11 @@ int run_product(celty_matrix *m, const void *x_dev, float tau, const ListInput *
         cp.tau = tau;
         cp.idx = idx; cp.val = val; cp.count = count; cp.status = status;
         cp.y = y;
-        cp.spin_limit = m->spin_limit ? m->spin_limit : kSpinLimit;
-        if (shape.own_list && grid <= di.sms) {
-            cp.ticket = status + 2;
-            if (m->last_grid != grid || m->last_merge != 1) {   // the ticket counts blocks of one launch shape
-                CELTY_CUDA(cudaMemsetAsync(cp.ticket, 0, 4, st));
-                m->last_grid = grid;
-                m->last_merge = 1;
-            }
-        }
         cp.M = (int)m->M; cp.K = (int)m->K;
         cp.W = shape.W; cp.groups = shape.groups; cp.cap = shape.cap; cp.own_list = shape.own_list;
         rc = ensure_smem(k_spmspv_column, shape.smem, g_granted_column);
         if (rc) return rc;
-        if (!cp.ticket) rc = shape.own_list ? launch_clear(y, m->M, st) : launch_compact(x_dev, m->K, tau, idx, val, count, y, m->M, st);
+        rc = shape.own_list ? launch_clear(y, m->M, st) : launch_compact(x_dev, m->K, tau, idx, val, count, y, m->M, st);
         if (rc) return rc;
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3((unsigned)grid);

@@ -10,7 +10,7 @@ import numpy as np
 import pytest
 import torch
 
-from conftest import permute_for_lane_tiles
+from conftest import hold_some_sms, permute_for_lane_tiles
 from oracle import celty_oracle as orc
 from paper_2608_01536_b200 import build, celty, synth
 
@@ -652,3 +652,27 @@ def test_host_result_at_any_byte_of_page_locked_memory(shift):
     y = np.frombuffer(got[shift:shift + 4 * M].tobytes(), np.float32)
     assert np.array_equal(y.astype(np.float64), orc.masked_gemv(W, mask, x, 1.0, threads=4)[0])
     assert np.all(got[:shift] == 0x55) and np.all(got[shift + 4 * M:] == 0x55)
+
+
+@pytest.mark.parametrize("M,K", [(4096, 2048), (7000, 300)])
+def test_column_call_needs_only_the_sms_that_are_free(M, K):
+    """No block of the call waits for another, and none for a count in the workspace: while a kernel of another stream
+    keeps 39 SMs the call runs on the others and is over before that kernel is."""
+    W = synth.integer_weights(37, M, K)
+    mask = synth.mask_bernoulli(37, M, K, 0.5)
+    x = synth.integer_activations(38, K)
+    m = celty.Matrix(W, mask, layout=celty.LAYOUT_COLUMN, device="cuda")
+    y_ref, _ = orc.masked_gemv(W, mask, x, 1.0, threads=8)
+    xd, y = _dev(x), torch.full((M,), 7.0, device="cuda")
+    m.spmspv(xd, 1.0)                                            # everything loaded
+    torch.cuda.synchronize()
+    m._ws[8:16] = 17
+    other, mine = torch.cuda.Stream(), torch.cuda.Stream()
+    holder, held = hold_some_sms(celty, synth, other)
+    m.spmspv(xd, 1.0, y=y, stream=mine)
+    mine.synchronize()
+    assert not held.query()
+    assert m.last_status(stream=mine) == 0
+    held.synchronize()
+    assert holder.last_status() == -5
+    assert np.array_equal(y.cpu().numpy().astype(np.float64), y_ref)
