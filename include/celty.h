@@ -452,7 +452,8 @@ int celty_launch_plan(const celty_matrix *m, int32_t *out, int32_t n);
  * thread blocks' tickets) makes before it gives up, sets the status word and lets the kernel finish; 0 = the
  * library's limit (about two million polls, far beyond any real wait).  The kernels never spin without a
  * limit: a wait that runs out shows up as CELTY_ETIMEOUT from celty_last_status, the call's y is then
- * undefined, and the handle is usable again after that call to celty_last_status.
+ * undefined, and the handle is usable again after that call to celty_last_status.  Copies into shared memory that
+ * were given up are still waited for, with the library's limit, before a thread block ends.
  * Errors: CELTY_EINVAL.
  */
 int celty_set_wait_limit(celty_matrix *m, uint32_t polls);

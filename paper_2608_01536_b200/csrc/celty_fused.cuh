@@ -519,6 +519,7 @@ __global__ void __launch_bounds__(kRegRows > 0 ? 256 : 544, 1) k_spmspv_fused(co
             *tail_cnt = __popc(word);
         }
         const bool late = p.win_cols > 0 && !mbar_wait_bounded(win_bar, 0, p.spin_limit);
+        if (__builtin_expect(late, 0)) mbar_wait_bounded(win_bar, 0, kSpinLimit);        // given up, but not left in flight
         if (lane == 0) *win_failed = late;
     }
     __syncthreads();
@@ -810,10 +811,11 @@ __global__ void __launch_bounds__(kRegRows > 0 ? 256 : 544, 1) k_spmspv_fused(co
             for (int i = lane; i < slab_words / 4; i += 32) slab4[i] = make_float4(0.f, 0.f, 0.f, 0.f);
         }
         if (__builtin_expect(failed, 0)) {
-            // give the copies that are still in flight a last (bounded) chance to land before the block goes on
+            // The copies that are still in flight have to land before the block goes on: after it their place is another
+            // block's.  With the library's limit, whatever the call's is.
 #pragma unroll 1
             for (; consumed < issued; ++consumed) {
-                mbar_wait_bounded(bar0 + 8u * slot, parity, p.spin_limit);
+                mbar_wait_bounded(bar0 + 8u * slot, parity, kSpinLimit);
                 if (++slot == (uint32_t)Dw) { slot = 0; parity ^= 1u; }
             }
             // the rows of this slab are NaN then: celty_spmspv_static has no status word that its caller could read

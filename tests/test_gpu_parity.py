@@ -676,3 +676,36 @@ def test_column_call_needs_only_the_sms_that_are_free(M, K):
     held.synchronize()
     assert holder.last_status() == -5
     assert np.array_equal(y.cpu().numpy().astype(np.float64), y_ref)
+
+
+@pytest.mark.parametrize("M,K,depth", [(4096, 2048, 0), (11008, 4096, 0), (11008, 4096, 4), (300, 257, 0)])
+def test_the_shortest_wait_limit_leaves_nothing_behind(M, K, depth):
+    """One poll per wait: most of them run out.  The kernels come back, what they asked for has landed before their
+    blocks end (so the call after them is not disturbed), and the handle is right again after last_status.  In the
+    call without a status word every row is right or NaN."""
+    W = synth.integer_weights(41, M, K)
+    mask = synth.mask_bernoulli(41, M, K, 0.5)
+    x = synth.integer_activations(42, K)
+    y_ref, _ = orc.masked_gemv(W, mask, x, 1.0, threads=8)
+    m, beside = celty.Matrix(W, mask, device="cuda"), celty.Matrix(W, mask, device="cuda")
+    m.set_launch(depth=depth)
+    oi, ov, _ = orc.compact(x, 1.0)
+    xd, idx, val, n = _dev(x), _dev(oi), _dev(ov.view(np.int16)), _dev(np.array([oi.size], np.int32))
+    xb, yb = xd.repeat(4, 1).contiguous() if K % 8 == 0 else None, torch.empty(4, M, device="cuda")
+    cold = torch.empty(1 << 26, dtype=torch.float32, device="cuda")
+    for _ in range(3):
+        cold.zero_()                                             # the first copies come from memory, not from L2
+        m.set_wait_limit(1)
+        m.spmspv(xd, 1.0)
+        m.spmspv_list(idx, val, n)
+        if xb is not None:
+            m.spmspv_batch(xb, 1.0, y=yb)
+        y = beside.spmspv(xd, 1.0)
+        assert m.last_status() in (0, -5)
+        assert beside.last_status() == 0 and np.array_equal(y.cpu().numpy().astype(np.float64), y_ref)
+        cold.zero_()
+        ys = m.spmspv_static(xd, 1.0).cpu().numpy().astype(np.float64)
+        assert np.all(np.isnan(ys) | (ys == y_ref))
+        m.set_wait_limit(0)
+        assert np.array_equal(_run(m, x, 1.0).astype(np.float64), y_ref)
+        assert np.array_equal(m.spmspv_static(xd, 1.0).cpu().numpy().astype(np.float64), y_ref)
