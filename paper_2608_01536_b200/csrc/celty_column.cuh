@@ -38,27 +38,6 @@ struct ColumnParams {
 
 constexpr int kColumnThreads = 1024;
 
-constexpr int kColumnWindow = 256;     // columns of the offset table a block fetches while the previous kernel ends
-
-struct ColumnSmem { uint32_t acc, dump, spans, items, imeta, window, warps, keep, rank, total; };
-
-__host__ __device__ inline ColumnSmem column_smem_layout(int M, int K, int groups, int cap, int own_list)
-{
-    ColumnSmem l;
-    uint32_t off = 0;
-    l.acc = off;    off += (uint32_t)groups * ((M + 3) & ~3) * 4u;    // one accumulator per group
-    l.dump = off;   off += 32u * 4u;                                 // where the lanes of a column's last chunk put what is no entry
-    l.items = off;  off += (uint32_t)cap * 8u;                       // {column, x bits}
-    l.imeta = off;  off += (uint32_t)cap * 8u;                       // {offset/16, entries}
-    l.window = off; off += own_list ? (uint32_t)kColumnWindow * 8u : 0u;
-    l.spans = off;  off += 2u * 32u * 4u;                            // rows spanned by each warp's chunk, two columns deep
-    l.warps = off;  off += 33u * 4u;                                 // survivors before each warp's words, and of all
-    l.keep = off;   off += own_list ? (uint32_t)((K + 31) / 32) * 4u : 0u;
-    l.rank = off;   off += own_list ? (uint32_t)((K + 31) / 32) * 4u : 0u;   // survivors before each keep word
-    l.total = (off + 15u) & ~15u;
-    return l;
-}
-
 // The group of 8 activations that the end of x cuts short (K not a multiple of 8), zero-filled.  Out of line: one
 // thread of a block needs it, if any, and the thresholding pass is unrolled four times around the call.
 __device__ __noinline__ uint4 ragged_group(const uint16_t *x, int K, int q)

@@ -1,5 +1,7 @@
 // Internal definitions shared by the host encoder and the CUDA translation unit.
 #pragma once
+#include <algorithm>
+#include <cmath>
 #include <cstddef>
 #include <cstdint>
 #include <cstring>
@@ -170,6 +172,66 @@ struct FusedPlan {
 inline size_t fused_smem_bytes(int R, int K, int G, int Sc, int D, int slot_bytes, int cap)
 {
     return fused_smem_layout(R, K, G * Sc, D, slot_bytes, cap).total;
+}
+
+// Shared memory of the COLUMN kernel.
+constexpr int kColumnWindow = 256;     // columns of the offset table a block fetches while the previous kernel ends
+
+struct ColumnSmem { uint32_t acc, dump, spans, items, imeta, window, warps, keep, rank, total; };
+
+CELTY_HD inline ColumnSmem column_smem_layout(int M, int K, int groups, int cap, int own_list)
+{
+    ColumnSmem l;
+    uint32_t off = 0;
+    l.acc = off;    off += (uint32_t)groups * ((M + 3) & ~3) * 4u;    // one accumulator per group
+    l.dump = off;   off += 32u * 4u;                                 // where the lanes of a column's last chunk put what is no entry
+    l.items = off;  off += (uint32_t)cap * 8u;                       // {column, x bits}
+    l.imeta = off;  off += (uint32_t)cap * 8u;                       // {offset/16, entries}
+    l.window = off; off += own_list ? (uint32_t)kColumnWindow * 8u : 0u;
+    l.spans = off;  off += 2u * 32u * 4u;                            // rows spanned by each warp's chunk, two columns deep
+    l.warps = off;  off += 33u * 4u;                                 // survivors before each warp's words, and of all
+    l.keep = off;   off += own_list ? (uint32_t)((K + 31) / 32) * 4u : 0u;
+    l.rank = off;   off += own_list ? (uint32_t)((K + 31) / 32) * 4u : 0u;   // survivors before each keep word
+    l.total = (off + 15u) & ~15u;
+    return l;
+}
+
+// Warps per column and columns in flight of the COLUMN kernel.
+struct ColumnShape { int W, groups, cap, own_list; size_t smem; };
+
+inline ColumnShape column_shape(int64_t M, int64_t K, size_t stream_bytes, size_t budget, int grid)
+{
+    ColumnShape s{};
+    const int64_t columns = (K + grid - 1) / grid;                     // a block has, at most
+    s.cap = (int)std::min<int64_t>(1024, columns + 1);
+    // W warps take ceil(chunks / W) passes over a column, and 32 / W columns are in flight: the split with the fewest
+    // passes for a block's share of the columns (taken as half of them; a tenth of a chunk more than the average, so
+    // that columns a little longer than that need no pass of their own).  4096 x 4096, 50 %: 12.4 us with
+    // the 9 warps for each of 3 columns that this gives, 12.6 with 4 for 8, 13.2 with 6 for 5, 14.4 with 8 for 3; 7000 x
+    // 2300: 14.5 with 6 for 5, 16.3 with 4 for 8, 19.5 with 16 for 2
+    const double chunks = (double)stream_bytes / 20.0 / (double)K / kChunkGroups + 0.1;
+    const int64_t share = std::max<int64_t>(1, (K / 2 + grid - 1) / grid);
+    int64_t best = 0;
+    const int64_t room = std::max<int64_t>(1, ((int64_t)budget - 24576) / (4 * ((M + 3) & ~3)));
+    for (int w = 1; w <= 32; ++w) {
+        const int64_t groups = std::min(std::min(columns, room), (int64_t)(w > 1 ? std::min(15, 32 / w) : 32));   // 15: named barriers
+        const int64_t passes = ((share + groups - 1) / groups) * (int64_t)std::ceil(chunks / w);
+        if (w == 1 || passes < best) {
+            best = passes;
+            s.W = w;
+            s.groups = (int)groups;
+        }
+    }
+    for (s.own_list = 1; s.own_list >= 0; --s.own_list) {
+        // thresholding in the blocks needs 8 bytes per 32 activations; where they leave no room: k_compact
+        if (s.own_list && K > 262144) continue;
+        for (int g = s.groups; g >= 1; --g) {
+            s.smem = column_smem_layout((int)M, (int)K, g, s.cap, s.own_list).total;
+            if (s.smem <= budget) { s.groups = g; return s; }
+        }
+    }
+    s.groups = 0;
+    return s;
 }
 
 // Launch choices of a handle (celty_set_launch and its neighbours); a default-constructed one is the library's.

@@ -581,45 +581,6 @@ int plan_fused(const celty_matrix *m, const LaunchKnobs &knobs, const DeviceInfo
     return CELTY_OK;
 }
 
-// Warps per column and columns in flight of the COLUMN kernel.
-struct ColumnShape { int W, groups, cap, own_list; size_t smem; };
-
-ColumnShape column_shape(const celty_matrix *m, const DeviceInfo &di, int grid)
-{
-    ColumnShape s{};
-    const size_t budget = (size_t)di.max_smem_optin;
-    const int64_t columns = (m->K + grid - 1) / grid;                     // a block has, at most
-    s.cap = (int)std::min<int64_t>(1024, columns + 1);
-    // W warps take ceil(chunks / W) passes over a column, and 32 / W columns are in flight: the split with the fewest
-    // passes for a block's share of the columns (taken as half of them; a tenth of a chunk more than the average, so
-    // that columns a little longer than that need no pass of their own).  4096 x 4096, 50 %: 12.4 us with
-    // the 9 warps for each of 3 columns that this gives, 12.6 with 4 for 8, 13.2 with 6 for 5, 14.4 with 8 for 3; 7000 x
-    // 2300: 14.5 with 6 for 5, 16.3 with 4 for 8, 19.5 with 16 for 2
-    const double chunks = (double)m->stream_bytes / 20.0 / (double)m->K / kChunkGroups + 0.1;
-    const int64_t share = std::max<int64_t>(1, (m->K / 2 + grid - 1) / grid);
-    int64_t best = 0;
-    const int64_t room = std::max<int64_t>(1, ((int64_t)budget - 24576) / (4 * ((m->M + 3) & ~3)));
-    for (int w = 1; w <= 32; ++w) {
-        const int64_t groups = std::min(std::min(columns, room), (int64_t)(w > 1 ? std::min(15, 32 / w) : 32));   // 15: named barriers
-        const int64_t passes = ((share + groups - 1) / groups) * (int64_t)std::ceil(chunks / w);
-        if (w == 1 || passes < best) {
-            best = passes;
-            s.W = w;
-            s.groups = (int)groups;
-        }
-    }
-    for (s.own_list = 1; s.own_list >= 0; --s.own_list) {
-        // thresholding in the blocks needs 8 bytes per 32 activations; where they leave no room: k_compact
-        if (s.own_list && m->K > 262144) continue;
-        for (int g = s.groups; g >= 1; --g) {
-            s.smem = column_smem_layout((int)m->M, (int)m->K, g, s.cap, s.own_list).total;
-            if (s.smem <= budget) { s.groups = g; return s; }
-        }
-    }
-    s.groups = 0;
-    return s;
-}
-
 // How many clusters of `cl` blocks of the fused kernel (with `smem` bytes of dynamic shared memory each) the
 // current device holds at once; asked of the runtime once per (device, cluster size, shared-memory KB).
 int max_active_clusters(int cl, size_t smem, int threads, int *out)
@@ -932,7 +893,7 @@ int run_product(celty_matrix *m, const void *x_dev, float tau, const ListInput *
     // untouched.
     if (m->layout == CELTY_LAYOUT_COLUMN) {
         const int grid = m->grid > 0 ? m->grid : di.sms;
-        const ColumnShape shape = column_shape(m, di, grid);
+        const ColumnShape shape = column_shape(m->M, m->K, m->stream_bytes, (size_t)di.max_smem_optin, grid);
         if (shape.groups == 0) return CELTY_EINVAL;
         ColumnParams cp{};
         cp.meta = reinterpret_cast<const uint2 *>(m->d_image);

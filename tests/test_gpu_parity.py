@@ -13,6 +13,7 @@ import torch
 from conftest import hold_some_sms, permute_for_lane_tiles
 from oracle import celty_oracle as orc
 from paper_2608_01536_b200 import build, celty, synth
+from test_column_shape import COLUMN_EDGES, SMEM, SMS
 
 pytestmark = pytest.mark.gpu
 
@@ -572,20 +573,13 @@ def test_host_buffer_entry_point():
     _check_y(yh.numpy(), Wo, mo, xo, tau)
 
 
-@pytest.mark.parametrize("M,K,d_w,d_a,grid", [
-    (256, 150, 1.0, 1.0, 0),          # every column exactly one chunk of 256 entries, one warp per column
-    (257, 40, 1.0, 1.0, 0),           # ... and one entry more
-    (511, 2000, 0.9, 0.9, 3),         # more columns per block than it looks up at a time (three blocks)
-    (3, 5000, 0.5, 0.5, 1),           # one block, tiny columns
-    (8192, 64, 1.0, 1.0, 0),          # 32 warps per column
-    (8200, 64, 1.0, 1.0, 0),          # a second pass over the column for one group of entries
-    (49152, 37, 0.4, 1.0, 0),         # the tallest accumulator
-    (40001, 300, 0.02, 0.7, 0),       # padding entries; M not a multiple of 4
-    (2, 262145, 0.5, 0.001, 0),       # the list comes from the compaction kernel
-])
+@pytest.mark.parametrize("M,K,d_w,d_a,grid", [case for case, _ in COLUMN_EDGES])
 def test_column_kernel_over_its_range(M, K, d_w, d_a, grid):
     """Integer data, so every sum is exact: the edges of a chunk and of a pass over a column, warps per column from
-    one to 32, batches of columns, both ways to the list (which is compared as well)."""
+    one to 32, batches of columns, both ways to the list (which is compared as well).  test_column_shape.py checks
+    that the cases reach these edges on a device like this one."""
+    device = torch.cuda.get_device_properties(0)
+    assert (device.multi_processor_count, device.shared_memory_per_block_optin) == (SMS, SMEM)
     W = synth.integer_weights(21, M, K)
     mask = synth.mask_bernoulli(21, M, K, d_w) if d_w < 1 else np.ones((M, K), np.uint8)
     x = synth.integer_activations(22, K)
