@@ -21,7 +21,7 @@ def _dev(a):
     return torch.from_numpy(np.ascontiguousarray(a)).cuda()
 
 
-@pytest.mark.parametrize("variant", [0, 1])          # N launches of the single-vector kernel / the widened kernels
+@pytest.mark.parametrize("variant", [0, 1])          # launches of the fused kernel / the widened kernels
 @pytest.mark.parametrize("N", [1, 2, 3, 4, 5, 8])
 @pytest.mark.parametrize("M,K,d_w,d_a", [(1000, 520, 0.5, 0.5), (4096, 1024, 0.3, 0.2), (11008, 300, 0.5, 0.9),
                                          (28672, 96, 0.5, 0.5)])
@@ -87,6 +87,39 @@ def test_batches_of_changing_size_on_one_handle(M, K, tile_rows):
         assert np.array_equal(idx.cpu().numpy(), oi) and np.array_equal(val.cpu().numpy().view(np.uint16), ov), N
         y1 = m.spmspv(wide[N % 8, :K].contiguous(), 1.0)
         assert np.array_equal(y1.cpu().numpy().astype(np.float64), ref[N % 8]), N
+
+
+@pytest.mark.parametrize("M,N,stuck", [(4096, 2, 1), (4096, 8, 0), (9000, 3, 2)])
+def test_a_batch_wait_that_runs_out_is_reported_and_the_handle_recovers(M, N, stuck):
+    """One vector's ticket is moved ahead by hand, so that some of its blocks wait for a count that never comes: the
+    launch comes back by itself, last_status says CELTY_ETIMEOUT once and repairs the tickets, the other vectors of
+    the launch are right, and so is the next batch."""
+    K = 512
+    W = synth.integer_weights(6, M, K)
+    mask = synth.mask_bernoulli(6, M, K, 0.5)
+    X = np.stack([synth.integer_activations(60 + n, K) for n in range(N)])
+    ref = np.stack([orc.masked_gemv(W, mask, X[n], 1.0, threads=8)[0] for n in range(N)])
+    m = celty.Matrix(W, mask, device="cuda")
+    xd, y = _dev(X), torch.empty(N, M, device="cuda")
+    m.spmspv_batch(xd, 1.0, y=y)
+    torch.cuda.synchronize()
+    assert m.last_status() == 0
+    words = m._ws[:256].view(torch.int32)
+    used = torch.nonzero(words[16:52]).flatten().tolist()        # tickets of batch launches stand at their block counts
+    assert len(used) == N                                        # one launch served all of them
+    grid = int(words[16 + used[stuck]].item())
+    words[16 + used[stuck]] = grid + 5                           # five blocks will land in the other half
+    m.set_wait_limit(2000)
+    m.spmspv_batch(xd, 1.0, y=y)
+    torch.cuda.synchronize()
+    assert m.last_status() == -5 and m.last_status() == 0
+    others = [n for n in range(N) if n != stuck]
+    assert np.array_equal(y.cpu().numpy().astype(np.float64)[others], ref[others])
+    m.set_wait_limit(0)
+    for _ in range(2):
+        m.spmspv_batch(xd, 1.0, y=y)
+        assert m.last_status() == 0
+        assert np.array_equal(y.cpu().numpy().astype(np.float64), ref)
 
 
 def test_batch_argument_errors():

@@ -97,7 +97,7 @@ def test_fp16_output(M, K, d_a):
 @pytest.mark.parametrize("I,K,d_a,d_h", [(1536, 1024, 0.4, 0.4), (700, 333, 0.9, 0.1), (4000, 512, 0.5, 1.0),
                                          (13824, 5120, 0.4, 0.4)])
 def test_swiglu_step_list_and_down_projection(I, K, d_a, d_h):
-    """[gate; up] product -> SiLU(gate) * up -> FP16 -> list, in one launch; then the down projection from that
+    """[gate; up] product -> SiLU(gate) * up -> FP16 -> list, in one call; then the down projection from that
     list.  (13824, 5120) is the Llama-2-13B layer of the bench's chain, at full size.)"""
     Wgu, mgu, Wd, md = _layer(I + K, I, K)
     x = synth.activations(I + K, K, "laplace")
@@ -106,7 +106,7 @@ def test_swiglu_step_list_and_down_projection(I, K, d_a, d_h):
     mg = celty.Matrix(Wgu, mgu, device="cuda")
     mdn = celty.Matrix(Wd, md, device="cuda")
     out = celty.SwigluOut(I, ref["tau2"], "cuda")
-    for call in range(2):                                        # twice: the second ticket wraps around too
+    for call in range(2):                                        # twice: the list's count starts over
         out.count.fill_(12345)
         y = mg.spmspv_ex(_dev(x), tau, swiglu=out)
         yd = mdn.spmspv_list(out.idx, out.val, out.count)
@@ -138,7 +138,7 @@ def test_swiglu_step_list_and_down_projection(I, K, d_a, d_h):
 @pytest.mark.parametrize("I,K,d_a,d_h", [(1536, 1024, 0.4, 0.4), (701, 333, 0.9, 0.1), (13824, 5120, 0.4, 0.4)])
 def test_swiglu_made_inside_the_down_projection(I, K, d_a, d_h):
     """The other way to fuse the step: the gate/up product is a plain call, and the down projection makes
-    SiLU(gate) * up itself while it thresholds (no launch, no pass over memory in between)."""
+    SiLU(gate) * up itself, by a small kernel ahead of its own."""
     Wgu, mgu, Wd, md = _layer(I + K + 1, I, K)
     x = synth.activations(I + K + 1, K, "laplace")
     tau = synth.threshold_for_density(x, d_a)

@@ -68,23 +68,27 @@ def test_static_scratch_entry_point_leaves_device_memory_alone():
 
 
 def test_static_and_two_launch_entry_points_share_one_kernel_attribute():
-    """Both entry points launch the same lane-tile kernel with different amounts of dynamic shared memory
-    (a 4096-row handle asks for more than a 12288-row one).  Interleaving them must not leave either with
-    a stale idea of what the runtime currently allows."""
+    """Entry points that launch one kernel with different amounts of dynamic shared memory: the lane-tile kernel of two
+    launches, which the third handle's static call falls back to as well, and the fused kernel of the other static
+    calls and of a handle without variant 1.  Interleaving them must not leave any with a stale idea of what the
+    runtime currently allows."""
     build.build()
     K = 256
     mats = []
-    for M in (4096, 12288):
+    for M, kw in ((4096, {}), (12288, {}), (40000, dict(tile_rows=240, slabs_per_block=6)), (1000, {})):
         W = synth.weights(80 + M, M, K)
         mask = synth.mask_bernoulli(80 + M, M, K, 0.5)
-        m = celty.Matrix(W, mask, device="cuda")
-        m.set_launch(variant=1)
+        m = celty.Matrix(W, mask, device="cuda", **kw)
+        m.set_launch(variant=0 if M == 1000 else 1)
         mats.append((m, W, mask))
+    with pytest.raises(celty.CeltyError):
+        mats[2][0].launch_plan()                              # no room for the fused kernel: the static call's other route
     x = synth.activations(5, K, "laplace")
     tau = synth.threshold_for_density(x, 0.5)
     xd = torch.from_numpy(x).cuda()
-    small, big = 0, 1
-    for which, static in ((small, False), (big, True), (small, False), (small, True), (big, False)):
+    small, big, tall, fused = 0, 1, 2, 3
+    for which, static in ((small, False), (tall, True), (big, False), (fused, False), (big, True), (small, False),
+                          (small, True), (tall, False), (fused, True), (big, False), (tall, True), (fused, False)):
         m, W, mask = mats[which]
         y = m.spmspv_static(xd, tau) if static else m.spmspv(xd, tau)
         torch.cuda.synchronize()
@@ -167,3 +171,35 @@ def test_static_call_needs_only_the_sms_that_are_free():
     held.synchronize()
     assert holder.last_status() == -5
     assert np.array_equal(y.cpu().numpy().astype(np.float64), y_ref)
+
+
+@pytest.mark.parametrize("layout", [celty.LAYOUT_LANE_TILE, celty.LAYOUT_COLUMN])
+def test_calls_behind_a_clearing_kernel_in_a_captured_graph(layout):
+    """The calls that clear y by a kernel of their own, captured after one call each and replayed with other activations
+    in the same place; other y contents before every replay."""
+    build.build()
+    M, K = 3000, 1111
+    W = synth.integer_weights(12, M, K)
+    mask = synth.mask_bernoulli(12, M, K, 0.5)
+    m = celty.Matrix(W, mask, layout=layout, device="cuda")
+    call = m.spmspv if layout == celty.LAYOUT_COLUMN else m.spmspv_static
+    xd = torch.zeros(K, dtype=torch.float16, device="cuda")
+    ys = [torch.full((M,), 3.0, device="cuda") for _ in range(3)]
+    side = torch.cuda.Stream()
+    with torch.cuda.stream(side):
+        call(xd, 1.0, y=ys[0])
+    side.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        for y in ys:
+            call(xd, 1.0, y=y)
+    for seed in range(4):
+        x = synth.integer_activations(90 + seed, K)
+        xd.copy_(torch.from_numpy(x))
+        for y in ys:
+            y.fill_(float(seed - 7))
+        graph.replay()
+        torch.cuda.synchronize()
+        y_ref, _ = orc.masked_gemv(W, mask, x, 1.0, threads=4)
+        for y in ys:
+            assert np.array_equal(y.cpu().numpy().astype(np.float64), y_ref)
