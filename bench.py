@@ -433,9 +433,9 @@ def run_sweep(args):
                     "roofline_frac": tot_bytes / 2 / us / 1e3 / peak, "cublas_gemv_us_per_layer": dus,
                     "speedup_vs_cublas": dus / us,
                     "note": ("plain products and a separate element-wise kernel (PyTorch) between gate/up and down"
-                             if consumer_side == "kernel" else "plain products; the down projection makes SiLU(gate)*up from the FP32 gate/up result while it "
-                             "thresholds" if consumer_side else
-                             "FP16 outputs, SiLU(gate)*up and its list inside the gate/up launch, down projection from "
+                             if consumer_side == "kernel" else "plain products; the down projection makes SiLU(gate)*up from the FP32 gate/up result in a "
+                             "kernel ahead of its own" if consumer_side else
+                             "FP16 outputs, SiLU(gate)*up and its list inside the gate/up call, down projection from "
                              "the list") + "; the dense side adds the element-wise step as a kernel of its own"}
         extra["chain_stacked_fused"] = chain_fused(False)
         extra["chain_stacked_separate_step"] = chain_fused("kernel")
@@ -970,7 +970,8 @@ def run_celty(args):
                      "frac_of_nominal_8000": wl.total_bytes / sec_per_call / 1e9 / 8000.0,
                      "peak_source": peak_src,
                      "kernel": "k_spmspv_fused" if launches_per_step == 1 else "all kernels of the call",
-                     "note": "one launch per call: algorithmic bytes per call / CUDA-event time per call",
+                     "note": f"{launches_per_step} launch{'es' if launches_per_step > 1 else ''} per call: algorithmic bytes per call "
+                             "/ CUDA-event time per call",
                      "us_per_call": us_per_call, "us_per_call_fastest_region": min(regions) * 1e3 / calls_per_region,
                      "dense_gemv_us": dense_us, "dense_gemv_us_by_layout": dense_both,
                      "speedup_vs_dense_gemv": (dense_us / us_per_call) if dense_us else None,

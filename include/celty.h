@@ -86,6 +86,8 @@ typedef struct {
  * Nothing is emitted after the last kept row.  The caller keeps ownership of W_host and mask_host;
  * the handle copies what it needs.  Limits: 1 <= M <= 49152 (one thread block's FP32 accumulators
  * must fit shared memory), 1 <= K < 2^31, at most 2^32 - 1 stored entries, at most 1024 tiles.
+ * From 2^18 weights on the packing is shared with up to 15 host threads that the call starts and joins (as many as the
+ * host has cores; fewer, or none, where the system gives no more).  The result does not depend on their number.
  * Errors: CELTY_EINVAL, CELTY_ENOMEM.
  */
 int celty_encode(const uint16_t *W_host, int64_t ldw, const uint8_t *mask_host, int64_t M, int64_t K,
@@ -177,8 +179,8 @@ int celty_compact(const void *x_dev, int64_t K, float tau, int32_t *idx_dev, uin
  * the surviving columns, decodes their runs to rows, accumulates value * x_j in shared memory in
  * FP32 (one rounding per multiply-add) and merges the thread blocks' results into y (FP32 adds in L2
  * by bulk reduce-add copies; celty_set_launch can select a sum in a fixed order instead); the COLUMN
- * layout has one kernel of the same outline behind a small one that clears y (a compaction kernel where K is so large
- * that its keep bits leave no room in shared memory).  On a stream of calls the kernel's
+ * layout has one kernel of the same outline behind a small one that clears y (a compaction kernel where K is so
+ * large that its keep bits leave no room in shared memory).  On a stream of calls the kernel's
  * set-up overlaps the end of the previous kernel (programmatic dependent launch); it waits for that
  * kernel before it reads x or touches y or the workspace.
  * The thread blocks of the fused kernel wait (with a limit) for one another before they add into y, so all of them have
@@ -199,8 +201,8 @@ int celty_compact(const void *x_dev, int64_t K, float tau, int32_t *idx_dev, uin
 int celty_spmspv(celty_matrix *m, const void *x_dev, float tau, void *y_dev, celty_stream_t stream);
 
 /*
- * Work on y after the merge, by a small kernel enqueued behind the product's in the same call (LANE_TILE handles, single-launch kernel, bulk reduce-add
- * merge).  Section 6.2 times the seven products of a decode layer; between the gate/up and the down projection of
+ * Work on y after the merge, by a small kernel enqueued behind the product's in the same call (LANE_TILE handles,
+ * single-launch kernel, bulk reduce-add merge).  Section 6.2 times the seven products of a decode layer; between the gate/up and the down projection of
  * its MLP sits SiLU(gate) * up, and every product's output feeds FP16 consumers.
  *   CELTY_EPILOGUE_FP16    out_fp16[i] = y[i] rounded to FP16 (nearest even), i < M; y keeps the FP32 values.
  *   CELTY_EPILOGUE_SWIGLU  the handle holds the gate projection's rows stacked on the up projection's
@@ -402,7 +404,8 @@ int celty_last_status(celty_matrix *m, celty_stream_t stream);
  *            launch (with which the kernel's set-up overlaps the tail of the previous kernel of the stream),
  *            16 = always / 32 = never run warp pairs: two warps per team that take turns at the team's
  *            accumulator, one waiting for its next sub-block and reading its header while the other runs its
- *            steps (by default the library pairs warps where a team has a dozen or more columns to stream),
+ *            steps (by default the library pairs warps where a team has nine or more columns to stream, or six with at most
+ *            seven teams to a block, and in place of nine teams),
  *            64 = never / 128 = wherever possible share a thread block between row parts.  (With the bulk
  *            reduce-add merge and no clusters: when the blocks do not divide by the row parts and the blocks left
  *            over can be shared evenly, each of them can serve several parts with correspondingly fewer teams per

@@ -88,7 +88,7 @@ inline uint64_t kept_word(const uint16_t *W, int64_t ldw, const uint8_t *mask, i
     return word;
 }
 
-// 64 x 64 bits: bit c of a[k] goes to bit k of a[c] (halves swapped recursively).
+// 64 x 64 bits: bit c of a[k] goes to bit k of a[c] (halves swapped recursively: H. S. Warren, Hacker's Delight, 7-3).
 inline void transpose64(uint64_t *a)
 {
     uint64_t m = 0x00000000FFFFFFFFull;

@@ -206,9 +206,10 @@ inline ColumnShape column_shape(int64_t M, int64_t K, size_t stream_bytes, size_
     s.cap = (int)std::min<int64_t>(1024, columns + 1);
     // W warps take ceil(chunks / W) passes over a column, and 32 / W columns are in flight: the split with the fewest
     // passes for a block's share of the columns (taken as half of them; a tenth of a chunk more than the average, so
-    // that columns a little longer than that need no pass of their own).  4096 x 4096, 50 %: 12.4 us with
-    // the 9 warps for each of 3 columns that this gives, 12.6 with 4 for 8, 13.2 with 6 for 5, 14.4 with 8 for 3; 7000 x
-    // 2300: 14.5 with 6 for 5, 16.3 with 4 for 8, 19.5 with 16 for 2
+    // that columns a little longer than that need no pass of their own).  4096 x 4096, 50 %: 11.5 us of
+    // device time with the 9 warps for each of 3 columns that this gives, 11.8 with 4 for 8, 12.3 with 6 for 5, 13.2 with 8
+    // for 4; 7000 x 2300: 11.4 with the 7 for 4, 11.9 with 16 for 2, 13.3 with 4 for 8; 28672 x 8192, one column at a
+    // time: 92.9 with the 29, 94.0 with 32, 110.5 with 16
     const double chunks = (double)stream_bytes / 20.0 / (double)K / kChunkGroups + 0.1;
     const int64_t share = std::max<int64_t>(1, (K / 2 + grid - 1) / grid);
     int64_t best = 0;

@@ -1071,9 +1071,9 @@ namespace {
 // A batch through the single-launch kernel.  One launch serves several vectors at once, each with its share of the
 // blocks: a vector's product streams no faster than before on as much of the chip as it has, but the part of a call
 // that does not stream -- thresholding, look-ups, the latency of the first copies, the merge, the change of kernels,
-// some 5 us -- is paid once for all of them (4096 x 4096, 50 % / 50 %, four vectors: 33.1 us in four launches,
-// 15.6 us in one; 8192 x 4096, eight vectors: 84.4 -> 41.0).  How many vectors share a launch is chosen by that trade: fixed time against what the division
-// of the blocks loses when they do not divide by vectors and row parts (5 vectors of a layer of 8 row parts: 29
+// some 5 us -- is paid once for all of them (4096 x 4096, 50 % / 50 %, four vectors: 30.0 us in four launches,
+// 14.9 us in one; 8192 x 4096, eight vectors: 80.9 and 38.9).  How many vectors share a launch is chosen by that trade:
+// fixed time against what the division of the blocks loses when they do not divide by vectors and row parts (5 vectors of a layer of 8 row parts: 29
 // blocks for 8 parts leaves five parts with one block more than the other three).
 int run_batch(celty_matrix *m, const uint16_t *x, int64_t ldx, int N, float tau, float *y, int64_t ldy,
               celty_stream_t stream)
@@ -1149,10 +1149,10 @@ extern "C" int celty_spmspv_batch(celty_matrix *m, const void *x_dev, int64_t ld
     const size_t need = 256 + round_up((size_t)m->K * 4, 256) + (size_t)8 * m->K * 2;
     if (scratch_bytes < need || ((uintptr_t)list_scratch_dev & 255)) return CELTY_ENOMEM;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    // Measured, the widened kernels below lose to the single-vector kernel called N times at every N (N accumulators
-    // per warp leave room for fewer warps, and the union of N activation patterns is nearly every column from N = 4
-    // on): unless the two-launch variant is asked for, the batch is N launches of the single-launch kernel, where the
-    // handle has its workspace and every row of x and y starts on a 16-byte boundary.
+    // Measured, the widened kernels below lose to the single-vector kernel at every N (N accumulators per warp leave room
+    // for fewer warps, and the union of N activation patterns is nearly every column from N = 4 on; 4096 x 4096, N = 2 / 4 /
+    // 8: 41 / 93 / 251 us against 10.4 / 15.6 / 25.4): unless the two-launch variant is asked for, the batch goes to
+    // run_batch where the handle has its workspace and every row of x and y starts on a 16-byte boundary.
     if (m->variant == 0 && m->d_ws && !(((uintptr_t)x_dev | (uintptr_t)(ldx * 2) | (uintptr_t)y_dev | (uintptr_t)(ldy * 4)) & 15)) {
         return run_batch(m, static_cast<const uint16_t *>(x_dev), ldx, N, tau, static_cast<float *>(y_dev), ldy, stream);
     }
@@ -1232,9 +1232,9 @@ extern "C" int celty_spmspv_host(celty_matrix *m, const void *x_host, float tau,
     int rc = celty_spmspv(m, x_stage_dev, tau, y_stage_dev, stream);
     if (rc) return rc;
     // y by a small kernel behind the product, where its place is page-locked: the copy engine takes several
-    // microseconds to take over from a kernel and to be waited for.  5120 x 5120: 29.5 us per call with a copy, 25.2 this
-    // way.  (The same for x pays nothing: fetched over the link by the product's blocks 30.1 us, as the parameters of a
-    // small kernel 27.3.)
+    // microseconds to take over from a kernel and to be waited for.  5120 x 5120: 30.3 us per call with a copy, 25.4 this
+    // way.  (The same for x pays nothing: fetched over the link by the product's blocks 4.9 us more than with a copy, as
+    // the parameters of a small kernel 2.1 more.)
     EpilogueArgs out{};
     out.kind = kEpilogueToHost;
     out.y_host = static_cast<float *>(mapped_host(y_host, (size_t)m->M * 4));
