@@ -965,7 +965,7 @@ def run_celty(args):
                                "mean_groups_per_lane": wl.layout_stats[2] / 32.0 / max(1, wl.layout_stats[0]),
                                "step_slots_per_group": 32.0 * wl.layout_stats[1] / max(1, wl.layout_stats[2])}},
         "roofline": {"bound": "hbm", "achieved": wl.total_bytes / sec_per_call / 1e9, "peak": peak, "unit": "GB/s",
-                     "frac": wl.total_bytes / sec_per_call / 1e9 / peak, "traffic": dram_traffic_per_launch(name),
+                     "frac": wl.total_bytes / sec_per_call / 1e9 / peak, "traffic": dram_traffic_per_launch(name) if args.layout != "column" else None,
                      "frac_on_bare_format_bytes": wl.bare_bytes / sec_per_call / 1e9 / peak,
                      "frac_of_nominal_8000": wl.total_bytes / sec_per_call / 1e9 / 8000.0,
                      "peak_source": peak_src,
