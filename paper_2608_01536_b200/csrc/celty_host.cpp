@@ -469,6 +469,7 @@ extern "C" int celty_clone(const celty_matrix *m, celty_matrix **out)
         copy->last_grid = 0;
         copy->last_merge = -1;
         for (int32_t &g : copy->last_batch_grid) g = 0;
+        copy->forget_launches();
         *out = copy.release();
         return CELTY_OK;
     } catch (const std::exception &) {
@@ -697,6 +698,7 @@ extern "C" int celty_set_launch(celty_matrix *m, int32_t grid, int32_t variant, 
     m->groups = groups;
     m->depth = depth;
     m->cluster = cluster;
+    m->forget_launches();
     return CELTY_OK;
 }
 
@@ -704,6 +706,7 @@ extern "C" int celty_set_register_rows(celty_matrix *m, int32_t rows)
 {
     if (!m || !(rows == 0 || rows == 32 || rows == 64 || rows == 96 || rows == 128)) return CELTY_EINVAL;
     m->reg_rows = rows;
+    m->forget_launches();
     return CELTY_OK;
 }
 
@@ -711,6 +714,7 @@ extern "C" int celty_set_wait_limit(celty_matrix *m, uint32_t polls)
 {
     if (!m) return CELTY_EINVAL;
     m->spin_limit = polls;
+    m->forget_launches();
     return CELTY_OK;
 }
 

@@ -169,6 +169,15 @@ struct FusedPlan {
     size_t smem;
 };
 
+// A launch worked out once for a handle, a device and a kind of call (prepared_launch): its shape and what of its
+// parameters follows from it.
+struct PreparedLaunch {
+    int device = -1;           // -1: not worked out
+    int status = 0;            // what working it out came to
+    FusedPlan plan{};
+    FusedParams params{};
+};
+
 inline size_t fused_smem_bytes(int R, int K, int G, int Sc, int D, int slot_bytes, int cap)
 {
     return fused_smem_layout(R, K, G * Sc, D, slot_bytes, cap).total;
@@ -277,4 +286,6 @@ struct celty_matrix : celty::LaunchKnobs {
     celty::WorkspaceLayout ws{};
     int32_t last_grid = 0, last_merge = -1;   // what the tickets in the workspace were last used with
     int32_t last_batch_grid[9] = {};          // the same for the tickets of launches that serve 2 .. 8 vectors
+    celty::PreparedLaunch prepared[9];        // [0] one vector, [v] launches that serve v = 2 .. 8
+    void forget_launches() { for (celty::PreparedLaunch &p : prepared) p.device = -1; }   // the handle has changed
 };

@@ -29,7 +29,7 @@ thread_local int g_last_cuda = 0;
 constexpr unsigned kFull = 0xFFFFFFFFu;
 enum : uint32_t { kStatusTimeout = 1u, kStatusBounds = 2u };
 
-struct DeviceInfo { int sms = 0; int max_smem_optin = 0; };
+struct DeviceInfo { int sms = 0; int max_smem_optin = 0; int device = 0; };
 
 int device_info(DeviceInfo *out)
 {
@@ -44,6 +44,7 @@ int device_info(DeviceInfo *out)
         CELTY_CUDA(cudaDeviceGetAttribute(&cache[dev].max_smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
     }
     *out = cache[dev];
+    out->device = dev;
     return CELTY_OK;
 }
 
@@ -689,6 +690,20 @@ FusedParams plan_params(const celty_matrix *m, const LaunchKnobs &knobs, const F
     return fp;
 }
 
+// Plan and parameters of the handle's launches that serve `vectors` vectors, worked out by the first such call after the
+// handle was bound or its choices changed: 0.45 us of host time that every call paid otherwise, and a call on a small
+// layer is bound by the host.
+const PreparedLaunch &prepared_launch(celty_matrix *m, const DeviceInfo &di, int vectors)
+{
+    PreparedLaunch &p = m->prepared[vectors > 1 ? vectors : 0];
+    if (p.device != di.device) {
+        p.status = plan_launch(m, *m, di, vectors, &p.plan);
+        if (p.status == CELTY_OK) p.params = plan_params(m, *m, p.plan, m->d_image);
+        p.device = p.status == CELTY_ECUDA ? -1 : di.device;
+    }
+    return p;
+}
+
 // Programmatic dependent launch: the kernel may be scheduled while the previous kernel of the stream drains; it
 // waits for that kernel (griddepcontrol.wait) before it reads or writes anything of the call.
 int launch_fused(void (*kernel)(FusedParams), int *granted, const LaunchKnobs &knobs, const FusedPlan &plan, int vectors,
@@ -758,6 +773,7 @@ extern "C" int celty_bind_device(celty_matrix *m, void *image_dev, size_t image_
     CELTY_CUDA(cudaMemsetAsync(workspace_dev, 0, m->ws.total, st));
     m->d_image = static_cast<uint8_t *>(image_dev);
     m->d_ws = static_cast<uint8_t *>(workspace_dev);
+    m->forget_launches();
     return CELTY_OK;
 }
 
@@ -838,11 +854,11 @@ int run_product(celty_matrix *m, const void *x_dev, float tau, const ListInput *
     float *y = static_cast<float *>(y_dev);
     const uint8_t *stream_base = m->d_image + m->meta_bytes;
     if (m->layout == CELTY_LAYOUT_LANE_TILE && m->variant == 0) {
-        FusedPlan plan;
-        rc = plan_launch(m, *m, di, 1, &plan);
-        if (rc) return rc;
+        const PreparedLaunch &prepared = prepared_launch(m, di, 1);
+        if (prepared.status) return prepared.status;
         if (extras && m->reg_rows) return CELTY_EINVAL;
-        FusedParams fp = plan_params(m, *m, plan, m->d_image);
+        const FusedPlan &plan = prepared.plan;
+        FusedParams fp = prepared.params;
         if (list) {
             fp.list_idx = list->idx;
             fp.list_val = list->val;
@@ -1082,14 +1098,14 @@ int run_batch(celty_matrix *m, const uint16_t *x, int64_t ldx, int N, float tau,
     DeviceInfo di;
     int rc = device_info(&di);
     if (rc) return rc;
-    FusedPlan plans[9];
     double cost[9] = {};
     // streaming time of one vector on the whole chip: half of the columns at 5 TB/s
     const double stream_us = 0.5 * 2.5 * (double)(m->nnz + m->n_pad) / 5e6, fixed_us = 5.0;
     int most = 1;
     for (int v = 1; v <= N; ++v) {
-        if (plan_launch(m, *m, di, v, &plans[v]) != CELTY_OK || (v > 1 && plans[v].lean == 0)) break;
-        const FusedPlan &pl = plans[v];
+        const PreparedLaunch &prepared = prepared_launch(m, di, v);
+        if (prepared.status != CELTY_OK || (v > 1 && prepared.plan.lean == 0)) break;
+        const FusedPlan &pl = prepared.plan;
         // teams that share a part's columns, in blocks of G teams
         const double per_part = pl.grid / pl.P + (pl.mix >= 2 ? 1.0 / pl.mix : 0.0);
         cost[v] = fixed_us + stream_us * di.sms / (per_part * pl.P);
@@ -1113,9 +1129,9 @@ int run_batch(celty_matrix *m, const uint16_t *x, int64_t ldx, int N, float tau,
             if (rc) return rc;
             continue;
         }
-        const FusedPlan &plan = plans[v];
+        const FusedPlan &plan = m->prepared[v].plan;
         uint32_t *status = reinterpret_cast<uint32_t *>(m->d_ws + m->ws.status_off);
-        FusedParams fp = plan_params(m, *m, plan, m->d_image);
+        FusedParams fp = m->prepared[v].params;
         fp.x = xv; fp.ldx = ldx;
         fp.y = yv; fp.ldy = ldy;
         fp.tau = tau;
