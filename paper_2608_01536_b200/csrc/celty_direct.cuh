@@ -1,0 +1,357 @@
+// The single-launch kernel for layers whose blocks own few columns, and for products from a list (included by
+// celty_kernels.cu inside its anonymous namespace, after celty_fused.cuh, whose streaming steps, waits and copies it uses):
+// LANE_TILE layout, one slab per block, bulk reduce-add merge, no clusters.
+//
+// What bounds a call on such a layer is a chain of dependent steps, and in k_spmspv_fused the longest part of it is the way
+// from x to the first copy: threshold all of x, rank the survivors, cut the list into equal shares, look the shares up,
+// 4 100 cycles.  Here columns are dealt to blocks whatever x is: x is cut into as many intervals as a block has chunks of
+// 32 columns, and of each interval a block has its share, a run of up to 32 neighbouring columns (so that survivors
+// that cluster in x are shared by all blocks to some degree, and a warp's loads stay coalesced).  Every streaming
+// warp loads the activations of all the block's columns, one column per lane and chunk; ballots tell each lane the place
+// of its column among the block's survivors, and survivor i goes to team i mod G.  The lane that holds one of its team's
+// columns notes it, and starts the copy itself if it is one of the first; the sub-block offsets were loaded while the
+// previous kernel drained.  Neither a barrier nor a look-up lies between x and the first copy, 1 400 cycles.  The
+// accumulators, which no offset window needs before the first copies here, are cleared while the previous kernel drains as
+// well (a tenth of a call's time at 4096 x 4096: cleared under the first copies they held these up).
+//
+// What it costs is balance: the survivors per block differ as they fall, sqrt((1 - d) / (d n)) of n columns at density d,
+// where the ranked list is even to one column.  Device time with 50 % of the weights, in us, ranked -> this kernel, by
+// columns per block:   7 (1024 x 1024, d = 0.5) 3.80 -> 3.37;   56 (4096 x 4096, d = 0.1 / 0.5 / 0.7) 4.84 -> 4.11, 7.23 -> 6.09,
+// 8.08 -> 7.22;   70 (5120 x 5120, 0.4) 7.96 -> 7.41;   75 (4096 x 11008, 0.5) 12.02 -> 10.80;   84 (11008 x 4096, 0.5) 11.16 ->
+// 10.57;   111 (8192 x 8192, 0.1 / 0.3 / 0.7) 7.34 -> 6.43, 10.58 -> 10.03, 18.04 -> 17.90;   139 (13824 x 5120, 0.4) 12.84 ->
+// 13.3 (older version): the line is at 128.  Groups of 2 to 32 blocks that share their columns' survivors evenly, ranked
+// shares of the columns beyond a fixed core under the streaming: both slower (more code and loads on the way to the first
+// copy, or a streaming loop that the compiler schedules worse).  A list is shared evenly whatever its length; the second
+// product of the 5504 x 2048 MLP chain gains 1.9 of 15.4 us from this kernel.
+//
+// Roles of a block's warps: the first ones stream (a2 - a4; with pairs warps t and t + 8 for team t), the next make the
+// survivor list that the API reports, in a few blocks; the last clears the block's share of y, takes its ticket, waits
+// for the others' and works out where the block's row segments go.
+constexpr int kDirectChunks = 4;         // columns of a block, in chunks of 32
+constexpr int kDirectHelpers = 3;        // at least; 20 warps leave a thread 96 registers
+constexpr int kDirectThreads = 32 * (16 + kDirectHelpers + 1);
+
+// kPairs: two warps per team that take turns at its accumulator; kBatch: one launch for several vectors
+// (FusedParams::ldx); kChunks: chunks of 32 columns that the block's columns fit in, 2 or 4; 0: the
+// survivors come as a list (FusedParams::list_count), in equal shares for all teams.
+template <bool kPairs, bool kBatch, int kChunks>
+__global__ void __launch_bounds__(kDirectThreads, 1) k_spmspv_direct(const FusedParams p)
+{
+    constexpr bool kList = kChunks == 0;
+    const uint16_t *const x = kBatch ? p.x + (size_t)blockIdx.y * p.ldx : p.x;
+    float *const y = kBatch ? p.y + (size_t)blockIdx.y * p.ldy : p.y;
+    uint32_t *const tickets = kBatch ? p.tickets + blockIdx.y : p.tickets;
+    const bool lists = !kList && (!kBatch || blockIdx.y + 1 == gridDim.y);    // the survivor list reported is the last vector's
+    extern __shared__ __align__(128) uint8_t smem[];
+    const int tid = threadIdx.x, lane = tid & 31, nthreads = blockDim.x, nwarps = nthreads >> 5;
+    const int warp = __shfl_sync(kFull, tid >> 5, 0);             // the same for all lanes, and the compiler knows it
+    const int slab_words = (p.R + kTileSlack) * 32;
+    const int G = p.G;
+    constexpr int pp = kPairs ? 1 : 0, stride = 1 + pp;
+    const bool streams = kPairs ? (warp & 7) < G && warp < 16 : warp < G;
+    const int first_helper = kPairs ? 16 : G, helpers = nwarps - 1 - first_helper;
+    const int g = streams ? (kPairs ? (warp & 7) : warp) : 0;     // the team
+    const int half = streams && kPairs ? warp >> 3 : 0;           // which of its two warps
+    const int Dw = p.D / stride;                                  // ring slots per warp
+    const DirectSmem &lay = p.direct;
+    float *acc = reinterpret_cast<float *>(smem + lay.acc);
+    uint8_t *ring = smem + lay.ring;
+    uint64_t *bars = reinterpret_cast<uint64_t *>(smem + lay.bars);
+    uint2 *items = reinterpret_cast<uint2 *>(smem + lay.items);   // [team][cap] {offset/16, units of 16 bytes << 16 | x bits}
+    int *zero_group = reinterpret_cast<int *>(smem + lay.zero);
+    uint32_t *kbw = reinterpret_cast<uint32_t *>(smem + lay.keep), *wrel = reinterpret_cast<uint32_t *>(smem + lay.wrel);
+    uint32_t *blk = reinterpret_cast<uint32_t *>(smem + lay.blk);
+    volatile int *flags = reinterpret_cast<volatile int *>(smem + lay.flag);     // [G] a warp of the team gave up
+
+    // Row part s (one slab) and place of this block in it.
+    const int per_part = idiv_small(gridDim.x, p.P), kslice = idiv_small(blockIdx.x, p.P), s = blockIdx.x - kslice * p.P;
+    const bool long_part = s < (int)gridDim.x - per_part * p.P;
+    const int nK = per_part + (long_part ? 1 : 0);
+    const uint32_t g_inv = (uint32_t)idiv_small(65535 + G, G);    // i / G = i * g_inv >> 16 for i < 4096
+    // The block's columns: from every interval of p.interval columns its share, at most 32 (one per lane).
+    int first[kChunks + 1], there[kChunks + 1];               // column of the lane, or of no lane; bit: it has one
+#pragma unroll
+    for (int c = 0; c < kChunks; ++c) {
+        const int c0 = c * p.interval, length = max(0, min(p.interval, p.K - c0));
+        const int base = idiv_small(length, nK), extra = length - base * nK;
+        first[c] = c0 + kslice * base + min(kslice, extra) + lane;
+        there[c] = lane < base + (kslice < extra ? 1 : 0);
+    }
+
+    // Programmatic dependent launch: see k_spmspv_fused.
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    uint2 at[kChunks + 1];                                      // {offset/16, units of 16 bytes} of the lane's columns' sub-blocks
+    auto load_offsets = [&]() {
+#pragma unroll
+        for (int c = 0; c < kChunks; ++c)
+            if (there[c]) {
+                at[c].x = p.meta[(size_t)first[c] * p.S + s];
+                at[c].y = p.meta[(size_t)first[c] * p.S + s + 1] - at[c].x;
+            }
+    };
+    if (streams && p.image_early) load_offsets();
+    if (tid < 4) zero_group[tid] = 0;
+    if (tid < G) const_cast<int *>(flags)[tid] = 0;
+    if (streams && lane == 0) {
+#pragma unroll 1
+        for (int d = 0; d < Dw; ++d) mbar_init(smem_u32(&bars[g * p.D + half * Dw + d]), 1);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    }
+    if (streams) {
+            float4 *slab4 = reinterpret_cast<float4 *>(acc + (size_t)g * slab_words);
+#pragma unroll 1
+            for (int i = half * 32 + lane; i < slab_words / 4; i += 32 * stride) slab4[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+    __syncthreads();
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+
+    // the list that the API reports is made by a few blocks
+    const int nfull = p.K >> 5, nwords = (p.K + 31) >> 5, nblk = (nwords + 31) >> 5;
+    const int list_blocks = min((int)gridDim.x, (nwords + 15) >> 4);
+    const bool listing = lists && (int)blockIdx.x < list_blocks;
+    if (streams) {
+        const uint32_t slab0 = smem_u32(acc + (size_t)g * slab_words);
+        const uint32_t cell0 = slab0 + 4u * lane;
+        const uint32_t ring0 = smem_u32(ring + ((size_t)g * p.D + (size_t)half * Dw) * p.slot_bytes);
+        const uint32_t bar0 = smem_u32(&bars[g * p.D + half * Dw]);
+        uint2 *const mine = items + (size_t)g * p.cap;
+        auto team_sync = [&]() {                                  // the warp alone, or the two warps of the team
+            if (kPairs) asm volatile("bar.sync %0, 64;" ::"r"(2 + g) : "memory");
+            else __syncwarp();
+        };
+        // The lane has found item k of the team: it notes it, and starts its copy if it is one of the first.  (Copies that an
+        // elected lane starts when all chunks are through: 0.2 us slower at 4096 x 4096.)
+        auto found = [&](int k, const uint2 at, uint32_t xb) {
+            if (kPairs && (k & 1) != half) return;
+            mine[k] = make_uint2(at.x, at.y << 16 | xb);
+            const int place = k >> pp;
+            if (place < Dw) bulk_load(ring0 + (uint32_t)(place * p.slot_bytes), p.stream + (size_t)at.x * 16, at.y * 16u, bar0 + 8u * place);
+        };
+        const uint32_t lt_mask = (1u << lane) - 1u;
+        int cnt = 0;
+        if (kList) {
+            const int n = __shfl_sync(kFull, max(0, min(p.K, __ldcg(p.list_count))), 0);
+            if (blockIdx.x == 0 && tid == 0) *p.count = n;
+            const int units = nK * G, u = kslice * G + g;
+            const uint32_t units_inv = long_part ? p.units_inv_long : p.units_inv;
+            uint32_t each = __umulhi((uint32_t)n, units_inv), extra = (uint32_t)n - each * (uint32_t)units;
+            if (extra >= (uint32_t)units) { ++each; extra -= (uint32_t)units; }
+            const int r0 = u * (int)each + min(u, (int)extra);
+            cnt = (int)each + (u < (int)extra ? 1 : 0);
+            for (int k = half + stride * lane; k < cnt; k += stride * 32) {
+                const int j = min(max(__ldcg(p.list_idx + r0 + k), 0), p.K - 1);
+                const uint32_t xb = __ldcg(p.list_val + r0 + k);
+                const uint32_t at = p.meta[(size_t)j * p.S + s];
+                found(k, make_uint2(at, p.meta[(size_t)j * p.S + s + 1] - at), xb);
+            }
+        } else {
+            if (!p.image_early) load_offsets();
+            uint32_t xb[kChunks + 1];
+#pragma unroll
+            for (int c = 0; c < kChunks; ++c) xb[c] = there[c] ? x[first[c]] : 0u;
+            uint32_t n = 0;
+#pragma unroll
+            for (int c = 0; c < kChunks; ++c) {
+                const bool keep = there[c] && !(fabsf(__half2float(__ushort_as_half((uint16_t)xb[c]))) <= p.tau);
+                const uint32_t kept = __ballot_sync(kFull, keep), i = n + __popc(kept & lt_mask), k = i * g_inv >> 16;
+                if (keep && (int)(i - k * G) == g) found((int)k, at[c], xb[c]);
+                n += __popc(kept);
+            }
+            cnt = (int)n > g ? idiv_small((int)n - g + G - 1, G) : 0;
+        }
+        uint32_t slot = 0, parity = 0, consumed = 0;              // of this warp's Dw slots
+        uint32_t issued = (uint32_t)min(Dw, (cnt - half + pp) >> pp), islot = issued == (uint32_t)Dw ? 0 : issued;   // (cnt >= 0, half <= 1)
+        auto issue = [&](const uint2 it) {
+            bulk_load_elected(ring0 + islot * (uint32_t)p.slot_bytes, p.stream + (size_t)it.x * 16, (it.y >> 16) * 16u, bar0 + 8u * islot);
+            ++issued;
+            if (++islot == (uint32_t)Dw) islot = 0;
+        };
+        team_sync();
+        bool failed = false;
+        const uint32_t zeros = smem_u32(zero_group), spare_cell = cell0 + (uint32_t)p.R * 128u;
+        StepBuf b0, b1;                                           // pipeline registers, live across items
+#pragma unroll 1
+        for (int i = half; i < cnt; i += stride) {
+            uint32_t xbits;                                       // the column's activation: asked for before the wait
+            asm volatile("ld.shared.u32 %0, [%1];" : "=r"(xbits) : "r"(smem_u32(&mine[i].y)));
+            if (!failed && !mbar_wait_bounded(bar0 + 8u * slot, parity, p.spin_limit)) failed = true;
+            failed = __any_sync(kFull, failed);
+            if (__builtin_expect(failed, 0)) {
+                // The copies still in flight are awaited below.  A warp that gave up keeps meeting its partner at the
+                // hand-overs, so that nobody waits for it in vain.
+                if (!kPairs) break;
+                if (lane == 0) flags[g] = 1;
+                if (i > 0) team_sync();
+                if (i + 1 < cnt) team_sync();
+                continue;
+            }
+            const uint32_t sub = ring0 + slot * (uint32_t)p.slot_bytes;
+            // what the refill at the end of this sub-block will need, read now so that it does not wait then
+            const bool refill = i + stride * Dw < cnt;
+            const uint2 next = refill ? mine[i + stride * Dw] : make_uint2(0u, 0u);
+            const uint16_t xj = (uint16_t)xbits;
+            // ---- a3 + a4.  Header: groups per lane, vectors and steps (see kSubHeader).
+            uint32_t gl, hw;
+            asm volatile("ld.shared.u8 %0, [%1];" : "=r"(gl) : "r"(sub + lane));
+            asm volatile("ld.shared.u32 %0, [%1];" : "=r"(hw) : "r"(sub + 32));       // vectors | steps << 16
+            const uint32_t steps = hw >> 16, Gs = hw & 0xFFFFu;
+            const uint32_t vbase = sub + kSubHeader, rbase = vbase + 16 * Gs;
+            uint32_t cum = 0, cell = cell0;
+            step_fetch(b0, gl, 0, steps, cum, lt_mask, vbase, rbase, zeros);
+            step_fetch(b1, gl, 1, steps, cum, lt_mask, vbase, rbase, zeros);
+            // nothing above touches the accumulator: here the partner hands it over (it has finished the column
+            // before this one)
+            if (kPairs && i > 0) team_sync();
+            step_decode<0>(b0, cell, spare_cell, 0);                                    // step 0
+            step_fetch(b0, gl, 2, steps, cum, lt_mask, vbase, rbase, zeros);
+            uint32_t q = 1;
+#pragma unroll 2
+            for (; q + 1 < steps; q += 2) {                                            // two real steps per pass
+                step_decode<0>(b1, cell, spare_cell, 0);                                // step q
+                step_finish(b0, xj);                                                   // step q-1
+                step_fetch(b1, gl, q + 2, steps, cum, lt_mask, vbase, rbase, zeros);
+                step_decode<0>(b0, cell, spare_cell, 0);                                // step q+1
+                step_finish(b1, xj);                                                   // step q
+                step_fetch(b0, gl, q + 3, steps, cum, lt_mask, vbase, rbase, zeros);
+            }
+            if (q < steps) {                                                           // one real step left
+                step_decode<0>(b1, cell, spare_cell, 0);
+                step_finish(b0, xj);
+                step_finish(b1, xj);
+            } else {                                                                   // only the last one to finish
+                step_finish(b0, xj);
+            }
+            // The slot's contents were consumed by loads whose values have been used, and the barrier orders
+            // every lane's reads before this point: the copy may overwrite it.
+            __syncwarp();
+            if (refill) issue(next);
+            if (kPairs && i + 1 < cnt) team_sync();               // the accumulator goes to the partner
+            ++consumed;
+            if (++slot == (uint32_t)Dw) { slot = 0; parity ^= 1u; }
+        }
+        if (kPairs) team_sync();                                  // both warps are through with the accumulator
+        if (__builtin_expect(failed || (kPairs && flags[g]), 0)) {
+            // The copies that are still in flight have to land before the block goes on: after it their place is another
+            // block's.  With the library's limit, whatever the call's is.
+#pragma unroll 1
+            for (; consumed < issued; ++consumed) {
+                mbar_wait_bounded(bar0 + 8u * slot, parity, kSpinLimit);
+                if (++slot == (uint32_t)Dw) { slot = 0; parity ^= 1u; }
+            }
+            // the rows of this slab are NaN then: celty_spmspv_static has no status word that its caller could read
+#pragma unroll 1
+            for (int w = lane; w < slab_words; w += 32) acc[(size_t)g * slab_words + w] = __int_as_float(0x7FC00000);
+            if (lane == 0) atomicOr(p.status, kStatusTimeout);
+        }
+    } else if (warp == nwarps - 1) {
+        // The adds at the end need a cleared y: this warp clears the block's share and announces it.
+        const int b = (int)blockIdx.x;
+        const int r0 = b * p.clear_rows + min(b, p.clear_extra), r1 = r0 + p.clear_rows + (b < p.clear_extra ? 1 : 0);
+        uint32_t ticket = 0;
+        if (p.tickets) {
+#pragma unroll 1
+            for (int i = r0 + lane; i < r1; i += 32) y[i] = 0.f;
+            __syncwarp();
+            if (lane == 0) {
+                asm volatile("fence.acq_rel.gpu;" ::: "memory");
+                // The ticket counts modulo 2 * gridDim.x, so it never has to be reset: calls alternate between
+                // waiting for the lower and for the upper half.
+                ticket = atomicInc(&tickets[0], 2u * gridDim.x - 1u);
+            }
+        }
+        if (listing) {                                            // the word that the end of x cuts short
+            const int j = 32 * nfull + lane;
+            const bool kept = j < p.K && !(fabsf(__half2float(__ushort_as_half(x[j]))) <= p.tau);
+            const uint32_t word = __ballot_sync(kFull, kept);
+            if (lane == 0 && nfull < nwords) kbw[nfull] = word;
+            __syncwarp();
+            asm volatile("bar.arrive 1, %0;" ::"r"(32 * helpers + 32) : "memory");
+        }
+        if (!kBatch && blockIdx.x == 0 && lane == 0 && p.ep_count) *p.ep_count = 0;      // k_epilogue appends to it
+        if (lane == 0) {
+            if (__builtin_expect(p.tickets && !ticket_wait(tickets, ticket, p.spin_limit), 0)) atomicOr(p.status, kStatusTimeout);
+            // the others' clearing stores (generic proxy) come before this block's reduce-adds (asynchronous proxy)
+            asm volatile("fence.proxy.async.global;" ::: "memory");
+        }
+    } else if (listing && warp >= first_helper) {
+        // ---- a1 for all of x.  A thread makes one keep word of 32 activations, the warp scans the counts of its block of
+        // 32 words.
+        const int ht = tid - 32 * first_helper, hthreads = 32 * helpers;
+        const __half2 tau2 = __half2half2(__float2half_rd(p.tau));   // |x| > tau decided in FP16, as in k_spmspv_fused
+#pragma unroll 1
+        for (int w0 = 0; w0 < nwords; w0 += hthreads) {             // the same trip count for every thread
+            const int w = w0 + ht;
+            const uint32_t word = w < nfull ? keep_word32(x + 32 * w, tau2) : 0u;
+            const uint32_t cnt = (uint32_t)__popc(word);
+            uint32_t incl = cnt;
+#pragma unroll
+            for (int d = 1; d < 32; d <<= 1) {
+                const uint32_t up = __shfl_up_sync(kFull, incl, d);
+                if (lane >= d) incl += up;
+            }
+            if (w < nfull) kbw[w] = word;
+            if (w < nwords) wrel[w] = incl - cnt;
+            if (lane == 31 && (w >> 5) < nblk) blk[w >> 5] = incl;
+        }
+        asm volatile("bar.sync 1, %0;" ::"r"(hthreads + 32) : "memory");       // with the last warp, for the short word
+        // the list, a few words per block and warp
+#pragma unroll 1
+        for (int w = (int)blockIdx.x + list_blocks * (warp - first_helper); w < nwords; w += list_blocks * helpers) {
+            uint32_t before = 0;
+            for (int e = lane; e < w >> 5; e += 32) before += blk[e];
+            before = __reduce_add_sync(kFull, before) + wrel[w];
+            const uint32_t word = kbw[w];
+            if (word >> lane & 1u) {
+                const int pos = (int)before + __popc(word & ((1u << lane) - 1u)), j = 32 * w + lane;
+                p.idx[pos] = j;
+                p.val[pos] = x[j];
+            }
+            if (w == nwords - 1 && lane == 0) *p.count = (int)before + __popc(word);
+        }
+    }
+    // Row segments, see k_spmspv_fused.  The last warp, one segment per lane, works out where they go under the streaming.
+    const int seg = p.S == 1 ? 16 : p.C, nseg = idiv_small(p.R + seg - 1, seg);
+    struct Segment { float *to; const float *from; int nrows; };
+    auto segment = [&](int k) {
+        const int i0 = k * seg, i1 = min(p.R, i0 + seg);
+        const int64_t row0 = p.S == 1 ? (int64_t)i0 * 32 : ((int64_t)(k * p.S + s) * p.C) * 32;
+        return Segment{y + row0, acc + (size_t)i0 * 32, row0 >= p.M ? 0 : min((i1 - i0) * 32, p.M - (int)row0)};
+    };
+    Segment early{nullptr, nullptr, 0};
+    if (kPairs && warp == nwarps - 1 && lane < nseg) early = segment(lane);
+    __syncthreads();
+
+    // ---- a5: the G accumulators are added into the first one, and each row segment goes to y as one bulk reduce-add.
+    if (G > 1) {
+        float4 *acc4 = reinterpret_cast<float4 *>(acc);
+        const int team4 = slab_words / 4;
+#pragma unroll 1
+        for (int q4 = tid; q4 < p.R * 8; q4 += nthreads) {
+            float4 v = acc4[q4];
+#pragma unroll 4
+            for (int t = 1; t < G; ++t) {
+                const float4 u = acc4[(size_t)t * team4 + q4];
+                v.x += u.x; v.y += u.y; v.z += u.z; v.w += u.w;
+            }
+            acc4[q4] = v;
+        }
+    }
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    __syncthreads();
+#pragma unroll 1
+    for (int o = kPairs ? (warp == nwarps - 1 ? lane : nseg) : tid; o < nseg; o += kPairs ? 32 : nthreads) {
+        const Segment sg = kPairs && o == lane ? early : segment(o);
+        const uint32_t bytes = ((uint32_t)sg.nrows * 4u) & ~15u;
+        if (sg.nrows <= 0) continue;
+        if (bytes)
+            asm volatile("cp.reduce.async.bulk.global.shared::cta.bulk_group.add.f32 [%0], [%1], %2;" ::"l"(sg.to),
+                         "r"(smem_u32(sg.from)), "r"(bytes)
+                         : "memory");
+#pragma unroll 1
+        for (int i = (int)(bytes >> 2); i < sg.nrows; ++i)
+            if (sg.from[i] != 0.f) atomicAdd(sg.to + i, sg.from[i]);
+    }
+    asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+    asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");   // shared memory may go once it has been read
+}

@@ -144,9 +144,9 @@ __device__ __forceinline__ bool ticket_wait(const uint32_t *ticket, uint32_t min
     for (uint32_t it = 0; it < limit; ++it) {
         const uint32_t cur = ld_relaxed_u32(ticket);
         if (low_half ? (cur >= gridDim.x) : (cur < gridDim.x)) { ok = true; break; }
-        __nanosleep(it < 64 ? 20 : 64);
+        if (it >= 32) __nanosleep(64);
     }
-    __threadfence();
+    asm volatile("fence.acq_rel.gpu;" ::: "memory");
     return ok;
 }
 

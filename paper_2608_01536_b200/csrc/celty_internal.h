@@ -93,7 +93,7 @@ inline WorkspaceLayout workspace_layout(int64_t K, int64_t T, int64_t part_words
 // Shared-memory carve-up of the fused kernel, computed by ONE function for the kernel and for the host
 // (which sizes the launch with .total), so that the two can never disagree.
 struct FusedSmem {
-    size_t acc, ring, bars, flag, items, imeta, zero, keep, wrel, blk, blkw, total;
+    uint32_t acc, ring, bars, flag, items, imeta, zero, keep, wrel, blk, blkw, total;
 };
 
 CELTY_HD inline FusedSmem fused_smem_layout(int R, int K, int teams, int D, int slot_bytes, int cap)
@@ -114,6 +114,29 @@ CELTY_HD inline FusedSmem fused_smem_layout(int R, int K, int teams, int D, int 
     l.blk = off;       off += blocks;                                      // survivors in each block of 32 keep words
     l.blkw = off;      off += 16 * blocks;                                 // per warp: survivors before each block
     l.total = off;
+    return l;
+}
+
+// The same for k_spmspv_direct.
+struct DirectSmem {
+    uint32_t acc, ring, bars, flag, items, zero, keep, wrel, blk, total;
+};
+
+inline DirectSmem direct_smem_layout(int R, int K, int G, int D, int slot_bytes, int cap)
+{
+    DirectSmem l;
+    uint32_t off = 0;
+    l.acc = off;       off += (uint32_t)G * (R + kTileSlack) * 32 * 4;       // FP32 accumulators, one slab per team
+    l.ring = off;      off += (uint32_t)G * D * slot_bytes;                  // bulk-copy ring slots (multiples of 128 bytes)
+    l.bars = off;      off += (uint32_t)G * D * 8;                           // one "full" mbarrier per slot
+    l.flag = off;      off += (uint32_t)G * 4;                               // per team: a warp gave up
+    off = (off + 15) / 16 * 16;
+    l.zero = off;      off += 16;                                            // the all-zero group that idle lanes fetch
+    l.items = off;     off += (uint32_t)G * cap * 8;                         // {offset/16, bytes/16 and x} per column of a team
+    l.keep = off;      off += (uint32_t)((K + 31) / 32) * 4;                 // one keep bit per activation
+    l.wrel = off;      off += (uint32_t)((K + 31) / 32) * 4;                 // survivors before each keep word, in its block of 32
+    l.blk = off;       off += (uint32_t)((K + 1023) / 1024) * 4;             // survivors in each block of 32 keep words
+    l.total = (off + 15) / 16 * 16;
     return l;
 }
 
@@ -144,6 +167,10 @@ struct FusedParams {
     int cap;                   // columns a team looks up per batch
     int win_cols;              // columns of the offset table a block copies into shared memory at its start
     FusedSmem lay;             // the block's shared memory, worked out once on the host (fused_smem_layout)
+    // k_spmspv_direct
+    DirectSmem direct;         // its shared memory
+    int interval;              // columns of each of the intervals of x of which every block has up to 32 columns
+    int image_early;           // 0: the kernel before this one may be writing the image
     int clear_rows, clear_extra;   // M / gridDim.x and M mod gridDim.x: block b clears clear_rows (+ 1 if b < clear_extra) rows of y
     // teams that share the survivor list of a row part: units = (column slices of the part) * G;
     // units_inv = floor(2^32 / units) for parts with gridDim / cl / P clusters, units_inv_long for those with
@@ -166,6 +193,8 @@ struct FusedParams {
 struct FusedPlan {
     int G, Sc, P, D, cl, pp, mix, slot_bytes, cap, threads, grid, merge;
     int lean;                  // 0: every option compiled in; 1 / 2: the builds for the default launch (without / with warp pairs)
+    int direct;                // 1: k_spmspv_direct
+    int chunks, interval;      // k_spmspv_direct: intervals of x, and their columns (FusedParams)
     size_t smem;
 };
 
@@ -286,6 +315,6 @@ struct celty_matrix : celty::LaunchKnobs {
     celty::WorkspaceLayout ws{};
     int32_t last_grid = 0, last_merge = -1;   // what the tickets in the workspace were last used with
     int32_t last_batch_grid[9] = {};          // the same for the tickets of launches that serve 2 .. 8 vectors
-    celty::PreparedLaunch prepared[9];        // [0] one vector, [v] launches that serve v = 2 .. 8
+    celty::PreparedLaunch prepared[9];        // [0] one vector, [1] one from a list, [v] launches that serve v = 2 .. 8
     void forget_launches() { for (celty::PreparedLaunch &p : prepared) p.device = -1; }   // the handle has changed
 };

@@ -445,7 +445,7 @@ __global__ void k_decode_lane(const uint32_t *__restrict__ meta, const uint8_t *
 // asked for), so that steady-state calls make no attribute calls.  The attribute belongs to the kernel,
 // so every entry point that launches a kernel shares that kernel's cache (g_granted_*): two caches for
 // one kernel could disagree about what the runtime currently allows.
-int g_granted_fused[64], g_granted_lean[2][64], g_granted_fused_extras[64], g_granted_lean_extras[2][64], g_granted_batch[2][64], g_granted_column[64], g_granted_lane[64], g_granted_reg[4][64];
+int g_granted_fused[64], g_granted_lean[2][64], g_granted_fused_extras[64], g_granted_lean_extras[2][64], g_granted_batch[2][64], g_granted_direct[7][64], g_granted_column[64], g_granted_lane[64], g_granted_reg[4][64];
 
 template <typename Kernel>
 int ensure_smem(Kernel kernel, size_t bytes, int *granted /* [64], per device */)
@@ -460,6 +460,7 @@ int ensure_smem(Kernel kernel, size_t bytes, int *granted /* [64], per device */
 }
 
 #include "celty_fused.cuh"
+#include "celty_direct.cuh"
 #include "celty_column.cuh"
 
 // y = 0, for the products whose blocks do not clear y themselves (COLUMN, celty_spmspv_static).  Bound by its launch: it may be scheduled while the
@@ -497,10 +498,18 @@ int launch_compact(const void *x, int64_t K, float tau, int32_t *idx, uint16_t *
     return CELTY_OK;
 }
 
+constexpr int kMostToMix = 48;           // left-over blocks are shared between row parts up to this (fit_clusters)
+
+// Columns that a team of k_spmspv_direct may get: of the block's, or of an even split of a list over the teams of a row part.
+int direct_cap(int64_t K, int blocks_per_part, int G, bool list)
+{
+    return list ? (int)(K / ((int64_t)blocks_per_part * G) + 1) : (32 * kDirectChunks + G - 1) / G;
+}
+
 // Shape of the fused launch: P row parts of Sc slabs, G teams per slab (teams = G * Sc warps, one accumulator
 // slab and one ring of D slots each), clusters of cl thread blocks that add their accumulators on chip.  The launch
 // serves `vectors` activation vectors, each with an equal share of the device's blocks.
-int plan_fused(const celty_matrix *m, const LaunchKnobs &knobs, const DeviceInfo &di, int vectors, FusedPlan *out)
+int plan_fused(const celty_matrix *m, const LaunchKnobs &knobs, const DeviceInfo &di, int vectors, bool list, FusedPlan *out)
 {
     FusedPlan pl{};
     pl.P = m->P;
@@ -517,6 +526,21 @@ int plan_fused(const celty_matrix *m, const LaunchKnobs &knobs, const DeviceInfo
     // Teams first (each needs its own accumulator), then as many ring slots as still fit (at least two, to
     // keep a copy in flight).  With warp pairs (two warps take turns at a team's accumulator, each with ring slots
     // of its own) there are eight teams at most and an even number of slots.
+    // Layers whose blocks own few columns have a kernel of their own (see there for what decides the line), and so has the
+    // product from a list, but where left-over blocks are shared between row parts, and where a team's items would take
+    // much of the shared memory.
+    const int per_part = pl.grid / pl.P;
+    const int64_t chunks = ((m->K + per_part - 1) / per_part + 31) / 32;
+    const int left = pl.grid % pl.P;
+    const bool mixes = left > 0 && pl.P % left == 0 && (int64_t)(pl.P / left) * per_part <= kMostToMix;    // see fit_clusters
+    pl.direct = reg_rows == 0 && knobs.merge != 0 && knobs.cluster <= 1 && knobs.lean != 0 && knobs.mix <= 0 && pl.Sc == 1 &&
+                (list ? !mixes && m->K / per_part < 4096 : chunks <= kDirectChunks);
+    pl.chunks = (int)chunks;
+    pl.interval = (int)((m->K + chunks - 1) / chunks);
+    auto smem_bytes = [&](int G, int D) {
+        if (!pl.direct) return fused_smem_bytes(m->R, (int)m->K, G, pl.Sc, D, pl.slot_bytes, pl.cap);
+        return (size_t)direct_smem_layout(m->R, (int)m->K, G, D, pl.slot_bytes, direct_cap(m->K, per_part, G, list)).total;
+    };
     auto fit = [&](int pairs) {
         pl.pp = pairs;
         // no more teams than a block can have columns (a tiny layer then leaves half the shared memory free, and
@@ -540,13 +564,17 @@ int plan_fused(const celty_matrix *m, const LaunchKnobs &knobs, const DeviceInfo
         for (int g = g_max; g >= 1 && pl.G == 0; --g)
             for (int d = d_max; d >= d_min; --d)
                 if ((!pairs || (d & 1) == 0) &&
-                    fused_smem_bytes(m->R, (int)m->K, g, pl.Sc, d, pl.slot_bytes, pl.cap) <= budget) {
+                    smem_bytes(g, d) <= budget) {
                     pl.G = g;
                     pl.D = d;
                     break;
                 }
     };
     fit(0);
+    if (pl.G == 0 && pl.direct) {                 // no room for its tables
+        pl.direct = 0;
+        fit(0);
+    }
     // Pairs pay where a team has many columns to stream (the hand-over hides the latencies at the head of every
     // sub-block) and cost a little where it has few.  The number of survivors is not known here, so the rule goes by the
     // columns per team, measured with 10, 30, 50 and 70 % of the activations kept:
@@ -564,14 +592,16 @@ int plan_fused(const celty_matrix *m, const LaunchKnobs &knobs, const DeviceInfo
             if (pl.G == 0) pl = keep;
         }
     }
-    if (pl.G == 0 && knobs.depth == 0 && fused_smem_bytes(m->R, (int)m->K, 1, pl.Sc, 1, pl.slot_bytes, pl.cap) <= budget) {
+    if (pl.G == 0 && knobs.depth == 0 && smem_bytes(1, 1) <= budget) {
         pl.G = 1;
         pl.D = 1;
         pl.pp = 0;
     }
     if (pl.G == 0) return CELTY_EINVAL;
     pl.threads = reg_rows > 0 ? 256 : pl.pp || pl.G * pl.Sc > 15 ? 544 : 512;   // the last warp does not stream
-    pl.smem = fused_smem_bytes(m->R, (int)m->K, pl.G, pl.Sc, pl.D, pl.slot_bytes, pl.cap);
+    if (pl.direct) pl.threads = 32 * (pl.pp ? 16 + kDirectHelpers + 1 : std::max(16, pl.G + kDirectHelpers + 1));
+    pl.smem = smem_bytes(pl.G, pl.D);
+    if (pl.direct) pl.cap = direct_cap(m->K, per_part, pl.G, list);
     pl.merge = (knobs.merge >= 0 ? knobs.merge : 1);
     // Clusters (bulk reduce-add merge only, on request): as long as the grid is made of whole clusters, every row
     // part gets at least one, and the device can hold them all at once.
@@ -642,12 +672,12 @@ int fit_clusters(const LaunchKnobs &knobs, FusedPlan *plan)
     }
     plan->mix = 1;
     const int left = plan->grid % plan->P;
-    if (rc == CELTY_OK && plan->cl == 1 && plan->merge == 1 && knobs.mix != 0 && left > 0 && plan->P % left == 0) {
+    if (rc == CELTY_OK && !plan->direct && plan->cl == 1 && plan->merge == 1 && knobs.mix != 0 && left > 0 && plan->P % left == 0) {
         const int mix = plan->P / left;
         // Sharing evens the parts out by 1 / (mix * blocks per part) of the streaming time, and a shared block adds
         // mix times the bytes into y at the end, which takes it mix times as long (the adders in L2 are shared by
         // all blocks): measured 2.2 % faster at 1 / 36 (28672 x 8192), 3 % slower at 1 / 147 (three parts)
-        const bool pays = knobs.mix > 0 || (int64_t)mix * (plan->grid / plan->P) <= 48;
+        const bool pays = knobs.mix > 0 || (int64_t)mix * (plan->grid / plan->P) <= kMostToMix;
         if (pays && plan->G % mix == 0 && plan->Sc * mix <= 16) plan->mix = mix;
     }
     // the library's default launch has builds of its own (k_spmspv_fused, kLean)
@@ -655,9 +685,9 @@ int fit_clusters(const LaunchKnobs &knobs, FusedPlan *plan)
     return rc;
 }
 
-int plan_launch(const celty_matrix *m, const LaunchKnobs &knobs, const DeviceInfo &di, int vectors, FusedPlan *out)
+int plan_launch(const celty_matrix *m, const LaunchKnobs &knobs, const DeviceInfo &di, int vectors, FusedPlan *out, bool list = false)
 {
-    const int rc = plan_fused(m, knobs, di, vectors, out);
+    const int rc = plan_fused(m, knobs, di, vectors, list, out);
     return rc ? rc : fit_clusters(knobs, out);
 }
 
@@ -678,7 +708,12 @@ FusedParams plan_params(const celty_matrix *m, const LaunchKnobs &knobs, const F
         fp.win_cols = (int)std::min<int64_t>(m->K, words >= 8 ? (int64_t)((words - 8) / m->S) : 0);
     }
     fp.merge = plan.merge;
-    fp.lay = fused_smem_layout(m->R, (int)m->K, plan.G * plan.Sc, plan.D, plan.slot_bytes, plan.cap);
+    fp.image_early = 1;
+    if (plan.direct) {
+        fp.direct = direct_smem_layout(m->R, (int)m->K, plan.G, plan.D, plan.slot_bytes, plan.cap);
+        fp.interval = plan.interval;
+    } else
+        fp.lay = fused_smem_layout(m->R, (int)m->K, plan.G * plan.Sc, plan.D, plan.slot_bytes, plan.cap);
     fp.clear_rows = (int)(m->M / plan.grid);
     fp.clear_extra = (int)(m->M % plan.grid);
     fp.spin_limit = knobs.spin_limit ? knobs.spin_limit : kSpinLimit;
@@ -693,11 +728,11 @@ FusedParams plan_params(const celty_matrix *m, const LaunchKnobs &knobs, const F
 // Plan and parameters of the handle's launches that serve `vectors` vectors, worked out by the first such call after the
 // handle was bound or its choices changed: 0.45 us of host time that every call paid otherwise, and a call on a small
 // layer is bound by the host.
-const PreparedLaunch &prepared_launch(celty_matrix *m, const DeviceInfo &di, int vectors)
+const PreparedLaunch &prepared_launch(celty_matrix *m, const DeviceInfo &di, int vectors, bool list = false)
 {
-    PreparedLaunch &p = m->prepared[vectors > 1 ? vectors : 0];
+    PreparedLaunch &p = m->prepared[vectors > 1 ? vectors : list ? 1 : 0];
     if (p.device != di.device) {
-        p.status = plan_launch(m, *m, di, vectors, &p.plan);
+        p.status = plan_launch(m, *m, di, vectors, &p.plan, list);
         if (p.status == CELTY_OK) p.params = plan_params(m, *m, p.plan, m->d_image);
         p.device = p.status == CELTY_ECUDA ? -1 : di.device;
     }
@@ -734,6 +769,23 @@ int launch_fused(void (*kernel)(FusedParams), int *granted, const LaunchKnobs &k
     cfg.numAttrs = na;
     CELTY_CUDA(cudaLaunchKernelEx(&cfg, kernel, fp));
     return CELTY_OK;
+}
+
+// The build of k_spmspv_direct for a plan, and its shared-memory limit.
+struct DirectBuild { void (*kernel)(FusedParams); int *granted; };
+
+DirectBuild direct_build(const FusedPlan &plan, bool batch, bool list)
+{
+    if (list) return plan.pp ? DirectBuild{k_spmspv_direct<true, false, 0>, g_granted_direct[0]} : DirectBuild{k_spmspv_direct<false, false, 0>, g_granted_direct[1]};
+    if (batch) return plan.pp ? DirectBuild{k_spmspv_direct<true, true, 4>, g_granted_direct[2]} : DirectBuild{k_spmspv_direct<false, true, 4>, g_granted_direct[3]};
+    if (plan.pp) return DirectBuild{k_spmspv_direct<true, false, 4>, g_granted_direct[4]};
+    return plan.chunks > 2 ? DirectBuild{k_spmspv_direct<false, false, 4>, g_granted_direct[5]} : DirectBuild{k_spmspv_direct<false, false, 2>, g_granted_direct[6]};
+}
+
+int launch_direct(const LaunchKnobs &knobs, const FusedPlan &plan, int vectors, bool list, const FusedParams &fp, cudaStream_t st)
+{
+    const DirectBuild b = direct_build(plan, vectors > 1, list);
+    return launch_fused(b.kernel, b.granted, knobs, plan, vectors, fp, st);
 }
 
 // The tickets of launches that serve `vectors` vectors each (one ticket per vector) in the status words.
@@ -854,7 +906,7 @@ int run_product(celty_matrix *m, const void *x_dev, float tau, const ListInput *
     float *y = static_cast<float *>(y_dev);
     const uint8_t *stream_base = m->d_image + m->meta_bytes;
     if (m->layout == CELTY_LAYOUT_LANE_TILE && m->variant == 0) {
-        const PreparedLaunch &prepared = prepared_launch(m, di, 1);
+        const PreparedLaunch &prepared = prepared_launch(m, di, 1, list != nullptr);
         if (prepared.status) return prepared.status;
         if (extras && m->reg_rows) return CELTY_EINVAL;
         const FusedPlan &plan = prepared.plan;
@@ -883,7 +935,9 @@ int run_product(celty_matrix *m, const void *x_dev, float tau, const ListInput *
             m->last_grid = plan.grid;
             m->last_merge = plan.merge;
         }
-        if (list)                                                // the list input has builds of its own
+        if (plan.direct)
+            rc = launch_direct(*m, plan, 1, list != nullptr, fp, st);
+        else if (list)                                           // the list input has builds of its own
             rc = plan.lean == 2 ? launch_fused(k_spmspv_fused<true, 0, 2>, g_granted_lean_extras[1], *m, plan, 1, fp, st)
                : plan.lean == 1 ? launch_fused(k_spmspv_fused<true, 0, 1>, g_granted_lean_extras[0], *m, plan, 1, fp, st)
                                 : launch_fused(k_spmspv_fused<true, 0>, g_granted_fused_extras, *m, plan, 1, fp, st);
@@ -1063,10 +1117,14 @@ extern "C" int celty_spmspv_static(const celty_matrix *m, const void *image_dev,
         // puts it there (0.1 us)
         fp.win_cols = 0;
         // (the limit is raised before the first launch: an error return leaves y untouched)
-        rc = plan.lean == 2 ? ensure_smem(k_spmspv_fused<false, 0, 2>, plan.smem, g_granted_lean[1])
+        fp.image_early = 0;
+        const DirectBuild direct = direct_build(plan, false, false);
+        rc = plan.direct ? ensure_smem(direct.kernel, plan.smem, direct.granted)
+           : plan.lean == 2 ? ensure_smem(k_spmspv_fused<false, 0, 2>, plan.smem, g_granted_lean[1])
                             : ensure_smem(k_spmspv_fused<false, 0, 1>, plan.smem, g_granted_lean[0]);
         if (rc == CELTY_OK) rc = launch_clear(y, m->M, st);
         if (rc) return rc;
+        if (plan.direct) return launch_direct(knobs, plan, 1, false, fp, st);
         return plan.lean == 2 ? launch_fused(k_spmspv_fused<false, 0, 2>, g_granted_lean[1], knobs, plan, 1, fp, st)
                               : launch_fused(k_spmspv_fused<false, 0, 1>, g_granted_lean[0], knobs, plan, 1, fp, st);
     }
@@ -1144,7 +1202,10 @@ int run_batch(celty_matrix *m, const uint16_t *x, int64_t ldx, int N, float tau,
             CELTY_CUDA(cudaMemsetAsync(fp.tickets, 0, (size_t)v * 4, st));
             m->last_batch_grid[v] = plan.grid;
         }
-        rc = plan.lean == 2 ? launch_fused(k_spmspv_fused<false, 0, 2, true>, g_granted_batch[1], *m, plan, v, fp, st)
+        if (plan.direct)
+            rc = launch_direct(*m, plan, v, false, fp, st);
+        else
+            rc = plan.lean == 2 ? launch_fused(k_spmspv_fused<false, 0, 2, true>, g_granted_batch[1], *m, plan, v, fp, st)
                             : launch_fused(k_spmspv_fused<false, 0, 1, true>, g_granted_batch[0], *m, plan, v, fp, st);
         if (rc) return rc;
     }
