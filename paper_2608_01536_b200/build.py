@@ -1,4 +1,5 @@
-"""Builds the C-ABI CUDA library in-tree: csrc/*.cpp, csrc/*.cu -> libcelty.so (sm_100a only)."""
+"""Builds the C-ABI CUDA library in-tree, csrc/celty_host.cpp and csrc/*.cu -> libcelty.so (sm_100a only), and the module
+behind the Python binding, csrc/celty_torch.cpp -> _celty_torch.so."""
 from __future__ import annotations
 
 import os
@@ -14,23 +15,48 @@ HEADERS = [os.path.join(CSRC, "celty_internal.h"), os.path.join(CSRC, "celty_fus
            os.path.join(ROOT, "include", "celty.h")]
 
 
-def needs_build() -> bool:
-    if not os.path.exists(LIB):
+# the binding's per-call functions, a CPython module that takes torch tensors
+BINDING = os.path.join(HERE, "_celty_torch.so")
+BINDING_SOURCE = os.path.join(CSRC, "celty_torch.cpp")
+
+
+def _older(target, sources) -> bool:
+    if not os.path.exists(target):
         return True
-    t = os.path.getmtime(LIB)
-    return any(os.path.getmtime(f) > t for f in SOURCES + HEADERS)
+    t = os.path.getmtime(target)
+    return any(os.path.getmtime(f) > t for f in sources)
+
+
+def needs_build() -> bool:
+    return _older(LIB, SOURCES + HEADERS) or _older(BINDING, [BINDING_SOURCE, os.path.join(ROOT, "include", "celty.h")])
+
+
+def _build_binding() -> None:
+    import sysconfig
+
+    import torch
+    base = os.path.join(os.path.dirname(torch.__file__))
+    nvcc = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
+    cuda = os.path.join(os.path.dirname(os.path.dirname(nvcc)), "include")
+    subprocess.check_call(
+        ["g++", "-O2", "-std=c++17", "-fPIC", "-shared", "-D_GLIBCXX_USE_CXX11_ABI=%d" % torch._C._GLIBCXX_USE_CXX11_ABI,
+         "-I", os.path.join(ROOT, "include"), "-I", sysconfig.get_paths()["include"], "-I", cuda,
+         "-isystem", os.path.join(base, "include"), "-isystem", os.path.join(base, "include", "torch", "csrc", "api", "include"),
+         BINDING_SOURCE, "-o", BINDING, "-L", HERE, "-l:libcelty.so", "-L", os.path.join(base, "lib"),
+         "-lc10", "-lc10_cuda", "-ltorch_cpu", "-ltorch_python", "-Wl,-rpath,$ORIGIN"])
 
 
 def build(force: bool = False, verbose: bool = False) -> str:
-    if not (force or needs_build()):
-        return LIB
-    nvcc = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
-    cmd = [nvcc, "-O3", "-std=c++17", "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo",
-           "-Xcompiler", "-fPIC", "-shared", "-I", os.path.join(ROOT, "include"), "-I", CSRC,
-           "-o", LIB] + SOURCES
-    if verbose:
-        cmd.insert(1, "-Xptxas=-v")
-    subprocess.check_call(cmd)
+    if force or _older(LIB, SOURCES + HEADERS):
+        nvcc = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
+        cmd = [nvcc, "-O3", "-std=c++17", "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo",
+               "-Xcompiler", "-fPIC", "-shared", "-I", os.path.join(ROOT, "include"), "-I", CSRC,
+               "-o", LIB] + SOURCES
+        if verbose:
+            cmd.insert(1, "-Xptxas=-v")
+        subprocess.check_call(cmd)
+    if force or _older(BINDING, [BINDING_SOURCE, os.path.join(ROOT, "include", "celty.h")]):
+        _build_binding()
     return LIB
 
 

@@ -1,4 +1,5 @@
-"""Thin ctypes binding over the C-ABI library declared in include/celty.h.
+"""Thin binding over the C-ABI library declared in include/celty.h: ctypes, and for the calls that a decoder makes per
+token a small native module over the same library (csrc/celty_torch.cpp), because those calls are bound by the host.
 
 Argument marshalling only: every step of the path (packing, thresholding/compaction, run-length
 decode, accumulation, reduction) runs inside the library.  PyTorch provides device memory and
@@ -85,6 +86,25 @@ def load():
     return _lib
 
 
+_native = None
+
+
+def _calls():
+    """The module with the calls that take torch tensors (csrc/celty_torch.cpp).  Raises if it is not there."""
+    global _native
+    if _native is None:
+        load()
+        import torch
+        torch.cuda.current_stream()                             # initialises CUDA where nothing has yet
+        try:
+            from . import _celty_torch
+        except ImportError as e:
+            raise RuntimeError("_celty_torch.so is missing or does not load: run `python -m paper_2608_01536_b200.build`.  "
+                               "There is no fallback for this path.") from e
+        _native = _celty_torch
+    return _native
+
+
 def _check(status: int, where: str):
     if status != 0:
         raise CeltyError(status, where)
@@ -98,8 +118,8 @@ _current_stream = None      # () -> handle of the current device's current strea
 
 
 def _stream_ptr(stream):
-    """Handle of `stream`, or of the current stream.  A call's time on the host is mostly this binding's, and making a
-    Stream object just to read its handle took 3.5 of 10.5 us; torch hands the bare handle out as well."""
+    """Handle of `stream`, or of the current stream (making a Stream object just to read its handle takes 3.5 us; torch
+    hands the bare handle out as well)."""
     global _current_stream
     if stream is not None:
         return stream.cuda_stream
@@ -118,11 +138,6 @@ class _Opts(ctypes.Structure):
     _fields_ = [("run_bits", _i32), ("layout", _i32), ("tile_rows", _i32), ("slabs_per_block", _i32)]
 
 
-class _Epilogue(ctypes.Structure):
-    _fields_ = [("kind", _i32), ("out_fp16", _vp), ("tau", _f32), ("list_idx", _vp), ("list_val", _vp),
-                ("list_count", _vp)]
-
-
 class SwigluOut:
     """Device buffers the SiLU(gate) * up epilogue of a stacked [gate; up] product fills: h (FP16, I values) and the
     thresholded list (idx, val, count) that `Matrix.spmspv_list` of the down projection consumes."""
@@ -134,10 +149,6 @@ class SwigluOut:
         self.idx = torch.empty(I, dtype=torch.int32, device=device)
         self.val = torch.empty(I, dtype=torch.int16, device=device)
         self.count = torch.zeros(1, dtype=torch.int32, device=device)
-
-    def _struct(self):
-        return _Epilogue(2, self.h.data_ptr(), self.tau, self.idx.data_ptr(), self.val.data_ptr(),
-                         self.count.data_ptr())
 
 
 class Matrix:
@@ -162,8 +173,9 @@ class Matrix:
         opts = _Opts(4, layout, tile_rows, slabs_per_block)
         h = _vp()
         _check(lib.celty_encode(_np_ptr(W), K, mptr, M, K, ctypes.byref(opts), ctypes.byref(h)), "celty_encode")
-        self._h = h
+        self._h, self._n = h, h.value
         self.M, self.K = M, K
+        self._batch_scratch = None
         self._image = self._ws = None
         if device is not None:
             self.to(device)
@@ -173,7 +185,8 @@ class Matrix:
         h = _vp()
         _check(load().celty_clone(self._h, ctypes.byref(h)), "celty_clone")
         other = object.__new__(Matrix)
-        other._h, other.M, other.K = h, self.M, self.K
+        other._h, other._n, other.M, other.K = h, h.value, self.M, self.K
+        other._batch_scratch = None
         other._image = other._ws = None
         if device is not None:
             other.to(device)
@@ -281,90 +294,54 @@ class Matrix:
 
     def spmspv(self, x, tau: float, y=None, stream=None):
         """y = W . threshold(x, tau); x: K float16 CUDA tensor, y: M float32 CUDA tensor (overwritten)."""
-        import torch
-        if y is None:
-            y = torch.empty(self.M, dtype=torch.float32, device=x.device)
-        assert x.dtype == torch.float16 and x.numel() == self.K and x.is_contiguous()
-        assert y.dtype == torch.float32 and y.numel() == self.M and y.is_contiguous()
-        _check(load().celty_spmspv(self._h, x.data_ptr(), tau, y.data_ptr(), _stream_ptr(stream)), "celty_spmspv")
-        return y
+        r = (_native or _calls()).spmspv(self._n, self.M, self.K, x, tau, y, stream)
+        if r.__class__ is int:
+            _check(r, "celty_spmspv")
+        return r
 
     def spmspv_ex(self, x, tau: float, y=None, fp16_out=None, swiglu: "SwigluOut | None" = None, stream=None):
         """spmspv followed in the same call by an FP16 copy of y (fp16_out: M float16) or by the SiLU(gate) * up
         step of a stacked [gate; up] matrix (swiglu: a SwigluOut)."""
-        import torch
-        if y is None:
-            y = torch.empty(self.M, dtype=torch.float32, device=x.device)
-        assert x.dtype == torch.float16 and x.numel() == self.K and x.is_contiguous()
-        assert y.dtype == torch.float32 and y.numel() == self.M and y.is_contiguous()
-        ep = None
-        if swiglu is not None:
-            ep = swiglu._struct()
-        elif fp16_out is not None:
-            assert fp16_out.dtype == torch.float16 and fp16_out.numel() == self.M
-            ep = _Epilogue(1, fp16_out.data_ptr(), 0.0, None, None, None)
-        _check(load().celty_spmspv_ex(self._h, x.data_ptr(), tau, y.data_ptr(), ctypes.byref(ep) if ep else None,
-                                      _stream_ptr(stream)), "celty_spmspv_ex")
-        return y
+        r = (_native or _calls()).spmspv_ex(self._n, self.M, self.K, x, tau, y, stream, fp16_out, swiglu)
+        if r.__class__ is int:
+            _check(r, "celty_spmspv_ex")
+        return r
 
     def spmspv_swiglu(self, gate_up, tau: float, y=None, h_out=None, fp16_out=None, stream=None):
         """Down projection whose activations SiLU(gate) * up are made inside the call from the FP32 result of the
         stacked [gate; up] product (gate_up: 2K float32); h_out (K float16, optional) receives them."""
-        import torch
-        if y is None:
-            y = torch.empty(self.M, dtype=torch.float32, device=gate_up.device)
-        assert gate_up.dtype == torch.float32 and gate_up.numel() == 2 * self.K and gate_up.is_contiguous()
-        ep = None
-        if fp16_out is not None:
-            ep = _Epilogue(1, fp16_out.data_ptr(), 0.0, None, None, None)
-        _check(load().celty_spmspv_swiglu(self._h, gate_up.data_ptr(), tau, y.data_ptr(),
-                                          h_out.data_ptr() if h_out is not None else None,
-                                          ctypes.byref(ep) if ep else None, _stream_ptr(stream)), "celty_spmspv_swiglu")
-        return y
+        r = (_native or _calls()).spmspv_swiglu(self._n, self.M, self.K, gate_up, tau, y, stream, h_out, fp16_out)
+        if r.__class__ is int:
+            _check(r, "celty_spmspv_swiglu")
+        return r
 
     def spmspv_list(self, idx, val, count, y=None, fp16_out=None, stream=None):
         """The product from a ready-made survivor list (device tensors: int32 columns, FP16 bit patterns, int32[1]
         count), e.g. the one a SwigluOut holds."""
-        import torch
-        if y is None:
-            y = torch.empty(self.M, dtype=torch.float32, device=idx.device)
-        assert idx.dtype == torch.int32 and val.dtype in (torch.int16, torch.float16) and count.dtype == torch.int32
-        ep = None
-        if fp16_out is not None:
-            assert fp16_out.dtype == torch.float16 and fp16_out.numel() == self.M
-            ep = _Epilogue(1, fp16_out.data_ptr(), 0.0, None, None, None)
-        _check(load().celty_spmspv_list(self._h, idx.data_ptr(), val.data_ptr(), count.data_ptr(), y.data_ptr(),
-                                        ctypes.byref(ep) if ep else None, _stream_ptr(stream)), "celty_spmspv_list")
-        return y
+        r = (_native or _calls()).spmspv_list(self._n, self.M, idx, val, count, y, stream, fp16_out)
+        if r.__class__ is int:
+            _check(r, "celty_spmspv_list")
+        return r
 
     def spmspv_batch(self, x, tau: float, y=None, stream=None):
         """y[n] = W . threshold(x[n], tau) for a batch x of shape (N, K), N <= 8; y: (N, M) float32."""
-        import torch
-        assert x.dtype == torch.float16 and x.dim() == 2 and x.shape[1] == self.K and x.stride(1) == 1
-        N = x.shape[0]
-        if y is None:
-            y = torch.empty(N, self.M, dtype=torch.float32, device=x.device)
-        assert y.dtype == torch.float32 and y.shape == (N, self.M) and y.stride(1) == 1
-        need = 256 + (4 * self.K + 255) // 256 * 256 + 16 * self.K
-        if getattr(self, "_batch_scratch", None) is None or self._batch_scratch.numel() < need:
+        if self._batch_scratch is None:
+            import torch
+            need = 256 + (4 * self.K + 255) // 256 * 256 + 16 * self.K
             self._batch_scratch = torch.empty(need, dtype=torch.uint8, device=x.device)
-        _check(load().celty_spmspv_batch(self._h, x.data_ptr(), x.stride(0), N, tau, y.data_ptr(), y.stride(0),
-                                         self._batch_scratch.data_ptr(), self._batch_scratch.numel(),
-                                         _stream_ptr(stream)), "celty_spmspv_batch")
-        return y
+        r = (_native or _calls()).spmspv_batch(self._n, self.M, self.K, x, tau, y, stream, self._batch_scratch)
+        if r.__class__ is int:
+            _check(r, "celty_spmspv_batch")
+        return r
 
     def spmspv_static(self, x, tau: float, y=None, stream=None):
         """Same product through the entry point that needs no workspace: its scratch is a fixed array inside
         the library, for callers that cannot allocate device memory.  K <= 32768; calls that overlap on the
         GPU race on that array.  The matrix's packed image must be on the device (`to()`)."""
-        import torch
-        if y is None:
-            y = torch.empty(self.M, dtype=torch.float32, device=x.device)
-        assert x.dtype == torch.float16 and x.numel() == self.K and x.is_contiguous()
-        assert y.dtype == torch.float32 and y.numel() == self.M and y.is_contiguous()
-        _check(load().celty_spmspv_static(self._h, self._image.data_ptr(), x.data_ptr(), tau, y.data_ptr(),
-                                          _stream_ptr(stream)), "celty_spmspv_static")
-        return y
+        r = (_native or _calls()).spmspv_static(self._n, self.M, self.K, x, tau, y, stream, self._image)
+        if r.__class__ is int:
+            _check(r, "celty_spmspv_static")
+        return r
 
     def spmspv_host(self, x_host, tau: float, y_host, x_stage, y_stage, stream=None):
         """Same product for host tensors (pinned for speed); copies run inside the library call."""
