@@ -270,7 +270,7 @@ __global__ void __launch_bounds__(kDirectThreads, 1) k_spmspv_direct(const Fused
         }
         if (!kBatch && blockIdx.x == 0 && lane == 0 && p.ep_count) *p.ep_count = 0;      // k_epilogue appends to it
         if (lane == 0) {
-            if (__builtin_expect(p.tickets && !ticket_wait(tickets, ticket, p.spin_limit), 0)) atomicOr(p.status, kStatusTimeout);
+            if (__builtin_expect(p.tickets && !ticket_wait<true>(tickets, ticket, p.spin_limit), 0)) atomicOr(p.status, kStatusTimeout);
             // the others' clearing stores (generic proxy) come before this block's reduce-adds (asynchronous proxy)
             asm volatile("fence.proxy.async.global;" ::: "memory");
         }

@@ -93,10 +93,11 @@ inline WorkspaceLayout workspace_layout(int64_t K, int64_t T, int64_t part_words
 // Shared-memory carve-up of the fused kernel, computed by ONE function for the kernel and for the host
 // (which sizes the launch with .total), so that the two can never disagree.
 struct FusedSmem {
-    uint32_t acc, ring, bars, flag, items, imeta, zero, keep, wrel, blk, blkw, total;
+    size_t acc, ring, bars, flag, items, imeta, zero, keep, wrel, blk, blkw, win, total;   // (32 bits each: 0.5 % slower)
 };
 
-CELTY_HD inline FusedSmem fused_smem_layout(int R, int K, int teams, int D, int slot_bytes, int cap)
+// window: bytes of a place of its own for the window of the offset table (launches for several vectors)
+CELTY_HD inline FusedSmem fused_smem_layout(int R, int K, int teams, int D, int slot_bytes, int cap, int window = 0)
 {
     FusedSmem l;
     uint32_t off = 0;
@@ -113,6 +114,8 @@ CELTY_HD inline FusedSmem fused_smem_layout(int R, int K, int teams, int D, int 
     const uint32_t blocks = ((uint32_t)((K + 1023) / 1024) * 4 + 31) / 32 * 32;   // (eight are read at a time)
     l.blk = off;       off += blocks;                                      // survivors in each block of 32 keep words
     l.blkw = off;      off += 16 * blocks;                                 // per warp: survivors before each block
+    l.win = off;
+    off += (uint32_t)window;
     l.total = off;
     return l;
 }
@@ -167,10 +170,6 @@ struct FusedParams {
     int cap;                   // columns a team looks up per batch
     int win_cols;              // columns of the offset table a block copies into shared memory at its start
     FusedSmem lay;             // the block's shared memory, worked out once on the host (fused_smem_layout)
-    // k_spmspv_direct
-    DirectSmem direct;         // its shared memory
-    int interval;              // columns of each of the intervals of x of which every block has up to 32 columns
-    int image_early;           // 0: the kernel before this one may be writing the image
     int clear_rows, clear_extra;   // M / gridDim.x and M mod gridDim.x: block b clears clear_rows (+ 1 if b < clear_extra) rows of y
     // teams that share the survivor list of a row part: units = (column slices of the part) * G;
     // units_inv = floor(2^32 / units) for parts with gridDim / cl / P clusters, units_inv_long for those with
@@ -187,11 +186,16 @@ struct FusedParams {
     const uint16_t *list_val;
     const int32_t *list_count;
     int32_t *ep_count;         // not null: set to zero for the list that k_epilogue appends to after this kernel
+    // k_spmspv_direct
+    DirectSmem direct;         // its shared memory
+    int interval;              // columns of each of the intervals of x of which every block has up to 32 columns
+    int image_early;           // 0: the kernel before this one may be writing the image
 };
 
 // Shape of a fused launch (plan_fused).
 struct FusedPlan {
     int G, Sc, P, D, cl, pp, mix, slot_bytes, cap, threads, grid, merge;
+    int window;                // bytes of the offset window where it has a place of its own (several vectors), else -1
     int lean;                  // 0: every option compiled in; 1 / 2: the builds for the default launch (without / with warp pairs)
     int direct;                // 1: k_spmspv_direct
     int chunks, interval;      // k_spmspv_direct: intervals of x, and their columns (FusedParams)

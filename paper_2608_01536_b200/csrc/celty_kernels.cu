@@ -601,6 +601,13 @@ int plan_fused(const celty_matrix *m, const LaunchKnobs &knobs, const DeviceInfo
     pl.threads = reg_rows > 0 ? 256 : pl.pp || pl.G * pl.Sc > 15 ? 544 : 512;   // the last warp does not stream
     if (pl.direct) pl.threads = 32 * (pl.pp ? 16 + kDirectHelpers + 1 : std::max(16, pl.G + kDirectHelpers + 1));
     pl.smem = smem_bytes(pl.G, pl.D);
+    pl.window = -1;
+    if (vectors > 1 && !pl.direct) {
+        // the offset window: a quarter more columns than the block has, as far as there is room
+        const size_t wanted = std::min<size_t>(32768, (size_t)((m->K / per_part * 5 / 4 + 64) * m->S * 4 + 32));
+        pl.window = (int)(std::min(wanted, budget - pl.smem) / 128 * 128);
+        pl.smem += (size_t)pl.window;
+    }
     if (pl.direct) pl.cap = direct_cap(m->K, per_part, pl.G, list);
     pl.merge = (knobs.merge >= 0 ? knobs.merge : 1);
     // Clusters (bulk reduce-add merge only, on request): as long as the grid is made of whole clusters, every row
@@ -704,7 +711,7 @@ FusedParams plan_params(const celty_matrix *m, const LaunchKnobs &knobs, const F
     {
         // offset window: as many columns as 32 KB (or the accumulator area, or the table) hold
         const size_t acc_bytes = (size_t)plan.G * plan.Sc * (m->R + kTileSlack) * 128;
-        const size_t words = std::min<size_t>(std::min<size_t>(acc_bytes, 32768) / 4, (size_t)m->K * m->S + 4);
+        const size_t words = std::min<size_t>((plan.window >= 0 ? (size_t)plan.window : std::min<size_t>(acc_bytes, 32768)) / 4, (size_t)m->K * m->S + 4);
         fp.win_cols = (int)std::min<int64_t>(m->K, words >= 8 ? (int64_t)((words - 8) / m->S) : 0);
     }
     fp.merge = plan.merge;
@@ -713,7 +720,7 @@ FusedParams plan_params(const celty_matrix *m, const LaunchKnobs &knobs, const F
         fp.direct = direct_smem_layout(m->R, (int)m->K, plan.G, plan.D, plan.slot_bytes, plan.cap);
         fp.interval = plan.interval;
     } else
-        fp.lay = fused_smem_layout(m->R, (int)m->K, plan.G * plan.Sc, plan.D, plan.slot_bytes, plan.cap);
+        fp.lay = fused_smem_layout(m->R, (int)m->K, plan.G * plan.Sc, plan.D, plan.slot_bytes, plan.cap, std::max(0, plan.window));
     fp.clear_rows = (int)(m->M / plan.grid);
     fp.clear_extra = (int)(m->M % plan.grid);
     fp.spin_limit = knobs.spin_limit ? knobs.spin_limit : kSpinLimit;
