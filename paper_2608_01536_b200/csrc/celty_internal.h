@@ -122,7 +122,7 @@ CELTY_HD inline FusedSmem fused_smem_layout(int R, int K, int teams, int D, int 
 
 // The same for k_spmspv_direct.
 struct DirectSmem {
-    uint32_t acc, ring, bars, flag, items, zero, keep, wrel, blk, total;
+    uint32_t acc, ring, bars, flag, items, zero, keep, total;
 };
 
 inline DirectSmem direct_smem_layout(int R, int K, int G, int D, int slot_bytes, int cap)
@@ -137,8 +137,6 @@ inline DirectSmem direct_smem_layout(int R, int K, int G, int D, int slot_bytes,
     l.zero = off;      off += 16;                                            // the all-zero group that idle lanes fetch
     l.items = off;     off += (uint32_t)G * cap * 8;                         // {offset/16, bytes/16 and x} per column of a team
     l.keep = off;      off += (uint32_t)((K + 31) / 32) * 4;                 // one keep bit per activation
-    l.wrel = off;      off += (uint32_t)((K + 31) / 32) * 4;                 // survivors before each keep word, in its block of 32
-    l.blk = off;       off += (uint32_t)((K + 1023) / 1024) * 4;             // survivors in each block of 32 keep words
     l.total = (off + 15) / 16 * 16;
     return l;
 }

@@ -56,3 +56,41 @@ def test_columns_dealt_to_blocks(M, tile_rows, K):
             assert m.last_status() == 0
         y = m.spmspv_static(xd, 0.5, y=torch.full((M,), 7.0, device="cuda"))
         assert np.array_equal(y.cpu().numpy().astype(np.float64), y_ref)
+
+
+def test_the_binding_takes_and_refuses_what_it_should():
+    """Calls through the native module: the caller's y comes back itself, a made one is new; wrong types, sizes and strides
+    are refused before anything is launched, and the library's own refusals carry its status."""
+    M, K = 64, 48
+    W = synth.integer_weights(3, M, K)
+    m = celty.Matrix(W, None, device="cuda")
+    x = torch.from_numpy(synth.integer_activations(4, K)).cuda()
+    y = torch.full((M,), 9.0, device="cuda")
+    y_ref, _ = orc.masked_gemv(W, np.ones((M, K), np.uint8), x.cpu().numpy(), 1.0, threads=1)
+    assert m.spmspv(x, 1, y=y) is y and m.spmspv(x, np.float32(1.0)) is not y
+    assert np.array_equal(y.cpu().numpy().astype(np.float64), y_ref)
+    side = torch.cuda.Stream()
+    side.wait_stream(torch.cuda.current_stream())
+    z = m.spmspv(x, 1.0, y=torch.zeros(M, device="cuda"), stream=side)
+    side.synchronize()
+    assert torch.equal(z, y)
+    for bad in (x.float(), x[:-1], torch.zeros(2 * K, dtype=torch.float16, device="cuda")[::2]):
+        for call in (m.spmspv, m.spmspv_ex, m.spmspv_static):
+            with pytest.raises(AssertionError):
+                call(bad, 1.0)
+    for bad in (y.half(), y[:-1], torch.zeros(2 * M, device="cuda")[::2]):
+        with pytest.raises(AssertionError):
+            m.spmspv(x, 1.0, y=bad)
+    with pytest.raises(AssertionError):
+        m.spmspv_ex(x, 1.0, fp16_out=torch.zeros(M, device="cuda"))
+    with pytest.raises(AssertionError):
+        m.spmspv_list(x, x, x)
+    with pytest.raises(AssertionError):
+        m.spmspv_batch(x, 1.0)
+    with pytest.raises(TypeError):
+        m.spmspv(x.cpu().numpy(), 1.0)
+    for tau in (-1.0, float("nan"), 1e300):
+        with pytest.raises(celty.CeltyError) as e:
+            m.spmspv(x, tau)
+        assert e.value.status == -1
+    torch.cuda.synchronize()
