@@ -98,10 +98,10 @@ __global__ void __launch_bounds__(kDirectThreads, 1) k_spmspv_direct(const Fused
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
     if (streams) {
-            float4 *slab4 = reinterpret_cast<float4 *>(acc + (size_t)g * slab_words);
+        float4 *slab4 = reinterpret_cast<float4 *>(acc + (size_t)g * slab_words);
 #pragma unroll 1
-            for (int i = half * 32 + lane; i < slab_words / 4; i += 32 * stride) slab4[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-        }
+        for (int i = half * 32 + lane; i < slab_words / 4; i += 32 * stride) slab4[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+    }
     __syncthreads();
     asm volatile("griddepcontrol.wait;" ::: "memory");
 
