@@ -4,10 +4,9 @@
 //
 // What bounds a call on such a layer is a chain of dependent steps, and in k_spmspv_fused the longest part of it is the way
 // from x to the first copy: threshold all of x, rank the survivors, cut the list into equal shares, look the shares up,
-// 4 100 cycles.  Here columns are dealt to blocks whatever x is: x is cut into as many intervals as a block has chunks of
-// 32 columns, and of each interval a block has its share, a run of up to 32 neighbouring columns (so that survivors
-// that cluster in x are shared by all blocks to some degree, and a warp's loads stay coalesced).  Every streaming
-// warp loads the activations of all the block's columns, one column per lane and chunk; ballots tell each lane the place
+// 4 100 cycles.  Here columns are dealt to blocks whatever x is (direct_column): runs of two neighbouring columns go round
+// the blocks of a row part, and every round starts three blocks further on.  Every streaming
+// warp loads the activations of all the block's columns, one column per lane and chunk of 32; ballots tell each lane the place
 // of its column among the block's survivors, and survivor i goes to team i mod G.  The lane that holds one of its team's
 // columns notes it, and starts the copy itself if it is one of the first; the sub-block offsets were loaded while the
 // previous kernel drained.  Neither a barrier nor a look-up lies between x and the first copy, 1 400 cycles.  The
@@ -15,11 +14,27 @@
 // well (a tenth of a call's time at 4096 x 4096: cleared under the first copies they held these up).
 //
 // What it costs is balance: the survivors per block differ as they fall, sqrt((1 - d) / (d n)) of n columns at density d,
-// where the ranked list is even to one column.  Device time with 50 % of the weights, in us, ranked -> this kernel, by
-// columns per block:   7 (1024 x 1024, d = 0.5) 3.80 -> 3.37;   56 (4096 x 4096, d = 0.1 / 0.5 / 0.7) 4.84 -> 4.11, 7.23 -> 6.09,
-// 8.08 -> 7.22;   70 (5120 x 5120, 0.4) 7.96 -> 7.41;   75 (4096 x 11008, 0.5) 12.02 -> 10.80;   84 (11008 x 4096, 0.5) 11.16 ->
-// 10.57;   111 (8192 x 8192, 0.1 / 0.3 / 0.7) 7.34 -> 6.43, 10.58 -> 10.03, 18.04 -> 17.90;   139 (13824 x 5120, 0.4) 12.84 ->
-// 13.3 (older version): the line is at 128.  Groups of 2 to 32 blocks that share their columns' survivors evenly, ranked
+// where the ranked list is even to one column.  Device time with 50 % of the weights, in us, mean over 16 draws of
+// independent survivors, ranked -> this kernel, by columns per block:
+//    14 (1024 x 1024, d = 0.1 / 0.5)              3.74 -> 3.34, 3.78 -> 3.34
+//    56 (4096 x 4096, 0.1 / 0.3 / 0.5 / 0.7)      4.81 -> 3.99, 6.34 -> 5.35, 7.78 -> 6.95, 8.64 -> 8.01
+//    70 (5120 x 5120, 0.3 / 0.5)                  7.27 -> 6.69, 9.30 -> 8.65
+//    75 (4096 x 11008, 0.1 / 0.5 / 0.7)           7.66 -> 5.91, 12.25 -> 11.62, 14.34 -> 13.61
+//    84 (11008 x 4096, 0.1 / 0.5 / 0.7)           6.92 -> 5.64, 11.59 -> 11.32, 14.17 -> 13.32
+//   111 (14336 x 4096, 0.1 / 0.3 / 0.5 / 0.7)     7.01 -> 5.93, 9.88 -> 9.38, 12.83 -> 12.82, 15.61 -> 15.45
+//   111 (8192 x 8192, 0.1 / 0.3 / 0.5 / 0.7)      7.66 -> 6.46, 10.79 -> 10.89, 14.24 -> 14.62, 17.60 -> 17.56
+// and with a build for six chunks
+//   138 (8192 x 10240, 0.1 / 0.3 / 0.5 / 0.7)     8.06 -> 7.20, 12.59 -> 12.77, 16.40 -> 16.77, 20.54 -> 20.66
+//   139 (13824 x 5120, 0.1 / 0.5 / 0.7)           7.09 -> 6.61, 14.60 -> 14.60, 18.18 -> 17.87
+//   187 (5120 x 13824, 0.1 / 0.5 / 0.7)           7.29 -> 6.41, 15.42 -> 14.39, 18.62 -> 17.77
+// so the line, four chunks, lies where the first layer is slower from 30 % on; it gives away what other shapes would gain beyond.
+// Survivors that lie together in x are shared about as evenly as independent ones.  Half of the 128-column heads zeroed,
+// ranked / runs of 32 columns / of 8 / of 4 / of two:   4096 x 4096 7.7 / 8.5 / 7.2 / 7.0 / 6.7;   4096 x 11008 12.2 / 15.2 / 15.7 /
+// 12.3 / 11.4;   8192 x 8192 14.2 / 18.6 / 15.8 / 14.9 / 13.9.  Single columns are no more even, and loads of x that touch a
+// sector per column cost 1 to 6 %; with runs of two independent survivors take 0 to 2 % more than with runs of 32 from 84 columns per
+// block on (8192 x 8192 at 10 %: 4 %), below that the offsets' new place (load_places) gains more.  One warp per chunk that
+// shares its ballot and its activations with the others through shared memory behind a barrier: 0 to 2 % slower.
+// Groups of 2 to 32 blocks that share their columns' survivors evenly, ranked
 // shares of the columns beyond a fixed core under the streaming: both slower (more code and loads on the way to the first
 // copy, or a streaming loop that the compiler schedules worse).  A list is shared evenly whatever its length; the second
 // product of the 5504 x 2048 MLP chain gains 1.9 of 15.4 us from this kernel.
@@ -27,9 +42,9 @@
 // Roles of a block's warps: the first ones stream (a2 - a4; with pairs warps t and t + 8 for team t), the next make the
 // survivor list that the API reports, in a few blocks; the last clears the block's share of y, takes its ticket, waits
 // for the others' and works out where the block's row segments go.
-constexpr int kDirectChunks = 4;         // columns of a block, in chunks of 32
 constexpr int kDirectHelpers = 3;        // at least; 20 warps leave a thread 96 registers
 constexpr int kDirectThreads = 32 * (16 + kDirectHelpers + 1);
+static_assert(kDirectChunks <= kDirectHelpers + 1, "a thread of the warps that do not stream for each of a block's columns");
 
 // kPairs: two warps per team that take turns at its accumulator; kBatch: one launch for several vectors
 // (FusedParams::ldx); kChunks: chunks of 32 columns that the block's columns fit in, 2 or 4; 0: the
@@ -59,6 +74,7 @@ __global__ void __launch_bounds__(kDirectThreads, 1) k_spmspv_direct(const Fused
     uint64_t *bars = reinterpret_cast<uint64_t *>(smem + lay.bars);
     uint2 *items = reinterpret_cast<uint2 *>(smem + lay.items);   // [team][cap] {offset/16, units of 16 bytes << 16 | x bits}
     int *zero_group = reinterpret_cast<int *>(smem + lay.zero);
+    uint2 *place = reinterpret_cast<uint2 *>(smem + lay.place);
     uint32_t *kbw = reinterpret_cast<uint32_t *>(smem + lay.keep);
     volatile int *flags = reinterpret_cast<volatile int *>(smem + lay.flag);     // [G] a warp of the team gave up
 
@@ -67,28 +83,23 @@ __global__ void __launch_bounds__(kDirectThreads, 1) k_spmspv_direct(const Fused
     const bool long_part = s < (int)gridDim.x - per_part * p.P;
     const int nK = per_part + (long_part ? 1 : 0);
     const uint32_t g_inv = (uint32_t)idiv_small(65535 + G, G);    // i / G = i * g_inv >> 16 for i < 4096
-    // The block's columns: from every interval of p.interval columns its share, at most 32 (one per lane).
-    int first[kChunks + 1], there[kChunks + 1];               // column of the lane, or of no lane; bit: it has one
+    const float nK_inv = __fdividef(1.f, (float)nK);
+    int column[kChunks + 1];                                  // the lane's columns of the block's (K or more: none)
 #pragma unroll
-    for (int c = 0; c < kChunks; ++c) {
-        const int c0 = c * p.interval, length = max(0, min(p.interval, p.K - c0));
-        const int base = idiv_small(length, nK), extra = length - base * nK;
-        first[c] = c0 + kslice * base + min(kslice, extra) + lane;
-        there[c] = lane < base + (kslice < extra ? 1 : 0);
-    }
+    for (int c = 0; c < kChunks; ++c) column[c] = direct_column(32 * c + lane, kslice, nK, nK_inv);
 
     // Programmatic dependent launch: see k_spmspv_fused.
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    uint2 at[kChunks + 1];                                      // {offset/16, units of 16 bytes} of the lane's columns' sub-blocks
-    auto load_offsets = [&]() {
-#pragma unroll
-        for (int c = 0; c < kChunks; ++c)
-            if (there[c]) {
-                at[c].x = p.meta[(size_t)first[c] * p.S + s];
-                at[c].y = p.meta[(size_t)first[c] * p.S + s + 1] - at[c].x;
-            }
+    // {offset/16, units of 16 bytes} of the block's columns' sub-blocks: once per block, by the last warps, which do not stream
+    // (each streaming warp for itself, in registers: 0.05 to 0.3 us slower, their loads touch a sector per run of columns)
+    auto load_places = [&]() {
+        const int i = tid - (nthreads - 32 * kDirectChunks), j = direct_column(max(i, 0), kslice, nK, nK_inv);
+        if (i >= 0 && i < 32 * kChunks && j < p.K) {
+            const uint32_t at = p.meta[(size_t)j * p.S + s];
+            place[i] = make_uint2(at, p.meta[(size_t)j * p.S + s + 1] - at);
+        }
     };
-    if (streams && p.image_early) load_offsets();
+    if (!kList && p.image_early) load_places();
     if (tid < 4) zero_group[tid] = 0;
     if (tid < G) const_cast<int *>(flags)[tid] = 0;
     if (streams && lane == 0) {
@@ -104,6 +115,10 @@ __global__ void __launch_bounds__(kDirectThreads, 1) k_spmspv_direct(const Fused
     }
     __syncthreads();
     asm volatile("griddepcontrol.wait;" ::: "memory");
+    if (!kList && !p.image_early && !streams) {
+        load_places();
+        asm volatile("bar.arrive 15, %0;" ::"r"(nthreads) : "memory");
+    }
 
     // The list that the API reports is made by a few blocks, eight words of x each (2048 x 5504 with 16 each: 0.3 us slower).
     const int nfull = p.K >> 5, nwords = (p.K + 31) >> 5;
@@ -124,8 +139,8 @@ __global__ void __launch_bounds__(kDirectThreads, 1) k_spmspv_direct(const Fused
         auto found = [&](int k, const uint2 at, uint32_t xb) {
             if (kPairs && (k & 1) != half) return;
             mine[k] = make_uint2(at.x, at.y << 16 | xb);
-            const int place = k >> pp;
-            if (place < Dw) bulk_load(ring0 + (uint32_t)(place * p.slot_bytes), p.stream + (size_t)at.x * 16, at.y * 16u, bar0 + 8u * place);
+            const int slot = k >> pp;
+            if (slot < Dw) bulk_load(ring0 + (uint32_t)(slot * p.slot_bytes), p.stream + (size_t)at.x * 16, at.y * 16u, bar0 + 8u * slot);
         };
         const uint32_t lt_mask = (1u << lane) - 1u;
         int cnt = 0;
@@ -145,16 +160,16 @@ __global__ void __launch_bounds__(kDirectThreads, 1) k_spmspv_direct(const Fused
                 found(k, make_uint2(at, p.meta[(size_t)j * p.S + s + 1] - at), xb);
             }
         } else {
-            if (!p.image_early) load_offsets();
             uint32_t xb[kChunks + 1];
 #pragma unroll
-            for (int c = 0; c < kChunks; ++c) xb[c] = there[c] ? x[first[c]] : 0u;
+            for (int c = 0; c < kChunks; ++c) xb[c] = column[c] < p.K ? x[column[c]] : 0u;
+            if (!p.image_early) asm volatile("bar.sync 15, %0;" ::"r"(nthreads) : "memory");   // the places, under x's way here
             uint32_t n = 0;
 #pragma unroll
             for (int c = 0; c < kChunks; ++c) {
-                const bool keep = there[c] && !(fabsf(__half2float(__ushort_as_half((uint16_t)xb[c]))) <= p.tau);
+                const bool keep = column[c] < p.K && !(fabsf(__half2float(__ushort_as_half((uint16_t)xb[c]))) <= p.tau);
                 const uint32_t kept = __ballot_sync(kFull, keep), i = n + __popc(kept & lt_mask), k = i * g_inv >> 16;
-                if (keep && (int)(i - k * G) == g) found((int)k, at[c], xb[c]);
+                if (keep && (int)(i - k * G) == g) found((int)k, place[32 * c + lane], xb[c]);
                 n += __popc(kept);
             }
             cnt = (int)n > g ? idiv_small((int)n - g + G - 1, G) : 0;

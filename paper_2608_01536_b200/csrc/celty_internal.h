@@ -121,11 +121,14 @@ CELTY_HD inline FusedSmem fused_smem_layout(int R, int K, int teams, int D, int 
 }
 
 // The same for k_spmspv_direct.
+constexpr int kDirectChunks = 4;         // columns of a block, in chunks of 32
+
 struct DirectSmem {
-    uint32_t acc, ring, bars, flag, items, zero, keep, total;
+    uint32_t acc, ring, bars, flag, items, zero, place, keep, total;
 };
 
-inline DirectSmem direct_smem_layout(int R, int K, int G, int D, int slot_bytes, int cap)
+// chunks: of 32 columns that a block owns; 0: the survivors come as a list
+inline DirectSmem direct_smem_layout(int R, int K, int G, int D, int slot_bytes, int cap, int chunks)
 {
     DirectSmem l;
     uint32_t off = 0;
@@ -136,9 +139,21 @@ inline DirectSmem direct_smem_layout(int R, int K, int G, int D, int slot_bytes,
     off = (off + 15) / 16 * 16;
     l.zero = off;      off += 16;                                            // the all-zero group that idle lanes fetch
     l.items = off;     off += (uint32_t)G * cap * 8;                         // {offset/16, bytes/16 and x} per column of a team
+    l.place = off;     off += 32 * (uint32_t)chunks * 8;                     // {offset/16, bytes/16} of the block's columns
     l.keep = off;      off += (uint32_t)((K + 31) / 32) * 4;                 // one keep bit per activation
     l.total = (off + 15) / 16 * 16;
     return l;
+}
+
+// k_spmspv_direct: column of x that is the i-th of block b's, where nK blocks share the columns (K or more: block b has no
+// i-th column).  Runs of kDirectRun columns go round the blocks, and each round starts kDirectTurn blocks further on.
+constexpr int kDirectRun = 2, kDirectTurn = 3;
+
+CELTY_HD inline int direct_column(int i, int b, int nK, float nK_inv)   // nK_inv: 1 / nK to a few units in the last place
+{
+    const int round = i / kDirectRun, turned = b + round * kDirectTurn;
+    const int place = turned - (int)(((float)turned + 0.5f) * nK_inv) * nK;      // modulo nK, exact for turned < 2^14
+    return (round * nK + place) * kDirectRun + i % kDirectRun;
 }
 
 struct FusedParams {
@@ -186,7 +201,6 @@ struct FusedParams {
     int32_t *ep_count;         // not null: set to zero for the list that k_epilogue appends to after this kernel
     // k_spmspv_direct
     DirectSmem direct;         // its shared memory
-    int interval;              // columns of each of the intervals of x of which every block has up to 32 columns
     int image_early;           // 0: the kernel before this one may be writing the image
 };
 
@@ -196,7 +210,7 @@ struct FusedPlan {
     int window;                // bytes of the offset window where it has a place of its own (several vectors), else -1
     int lean;                  // 0: every option compiled in; 1 / 2: the builds for the default launch (without / with warp pairs)
     int direct;                // 1: k_spmspv_direct
-    int chunks, interval;      // k_spmspv_direct: intervals of x, and their columns (FusedParams)
+    int chunks;                // k_spmspv_direct: columns of a block, in chunks of 32
     size_t smem;
 };
 

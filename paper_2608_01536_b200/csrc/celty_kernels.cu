@@ -535,11 +535,10 @@ int plan_fused(const celty_matrix *m, const LaunchKnobs &knobs, const DeviceInfo
     const bool mixes = left > 0 && pl.P % left == 0 && (int64_t)(pl.P / left) * per_part <= kMostToMix;    // see fit_clusters
     pl.direct = reg_rows == 0 && knobs.merge != 0 && knobs.cluster <= 1 && knobs.lean != 0 && knobs.mix <= 0 && pl.Sc == 1 &&
                 (list ? !mixes && m->K / per_part < 4096 : chunks <= kDirectChunks);
-    pl.chunks = (int)chunks;
-    pl.interval = (int)((m->K + chunks - 1) / chunks);
+    pl.chunks = list ? 0 : (int)chunks;
     auto smem_bytes = [&](int G, int D) {
         if (!pl.direct) return fused_smem_bytes(m->R, (int)m->K, G, pl.Sc, D, pl.slot_bytes, pl.cap);
-        return (size_t)direct_smem_layout(m->R, (int)m->K, G, D, pl.slot_bytes, direct_cap(m->K, per_part, G, list)).total;
+        return (size_t)direct_smem_layout(m->R, (int)m->K, G, D, pl.slot_bytes, direct_cap(m->K, per_part, G, list), pl.chunks).total;
     };
     auto fit = [&](int pairs) {
         pl.pp = pairs;
@@ -716,10 +715,9 @@ FusedParams plan_params(const celty_matrix *m, const LaunchKnobs &knobs, const F
     }
     fp.merge = plan.merge;
     fp.image_early = 1;
-    if (plan.direct) {
-        fp.direct = direct_smem_layout(m->R, (int)m->K, plan.G, plan.D, plan.slot_bytes, plan.cap);
-        fp.interval = plan.interval;
-    } else
+    if (plan.direct)
+        fp.direct = direct_smem_layout(m->R, (int)m->K, plan.G, plan.D, plan.slot_bytes, plan.cap, plan.chunks);
+    else
         fp.lay = fused_smem_layout(m->R, (int)m->K, plan.G * plan.Sc, plan.D, plan.slot_bytes, plan.cap, std::max(0, plan.window));
     fp.clear_rows = (int)(m->M / plan.grid);
     fp.clear_extra = (int)(m->M % plan.grid);

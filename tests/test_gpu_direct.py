@@ -94,3 +94,27 @@ def test_the_binding_takes_and_refuses_what_it_should():
             m.spmspv(x, tau)
         assert e.value.status == -1
     torch.cuda.synchronize()
+
+
+# 4096 columns in two row parts of 74 blocks (56 columns each), 8192 (111 each)
+@pytest.mark.parametrize("M,K", [(4096, 4096), (3000, 8192)])
+def test_survivors_that_lie_together_in_x(M, K):
+    """Zeroed heads of 64 and 128 activations, half of every head, and one stretch of x: such survivors are dealt to blocks
+    as unevenly as the rule allows (a call's values do not depend on it)."""
+    W = synth.integer_weights(7, M, K)
+    mask = synth.mask_bernoulli(7, M, K, 0.5)
+    m = celty.Matrix(W, mask, tile_rows=64 if M == 4096 else 0, device="cuda")
+    rng = np.random.default_rng(K)
+    i = np.arange(K)
+    heads = rng.random(K // 128) < 0.5
+    for keep in (heads[i // 128], (i // 64) % 2 == 0, i % 128 < 64, i < K // 8, i >= K - 40, i % 148 < 2):
+        x = np.where(keep, rng.integers(1, 4, K) * rng.choice([-1, 1], K), 0).astype(np.float16)
+        y_ref, _ = orc.masked_gemv(W, mask, x, 0.5, threads=8)
+        xd = torch.from_numpy(x).cuda()
+        for y in (m.spmspv(xd, 0.5, y=torch.full((M,), 5.0, device="cuda")), m.spmspv_static(xd, 0.5)):
+            assert np.array_equal(y.cpu().numpy().astype(np.float64), y_ref)
+        m.spmspv(xd, 0.5)
+        gi, gv = m.last_compaction()
+        oi, ov, _ = orc.compact(x, 0.5)
+        assert np.array_equal(gi.cpu().numpy(), oi) and np.array_equal(gv.cpu().numpy().view(np.uint16), ov)
+        assert m.last_status() == 0
