@@ -284,6 +284,7 @@ class Matrix:
         import torch
         ib, wb = self.device_bytes()
         dev = torch.device(device)
+        self._batch_scratch = None
         with torch.cuda.device(dev):
             self._image = torch.empty(ib, dtype=torch.uint8, device=dev)
             self._ws = torch.empty(wb, dtype=torch.uint8, device=dev)
@@ -325,11 +326,15 @@ class Matrix:
 
     def spmspv_batch(self, x, tau: float, y=None, stream=None):
         """y[n] = W . threshold(x[n], tau) for a batch x of shape (N, K), N <= 8; y: (N, M) float32."""
-        if self._batch_scratch is None:
+        scratch = self._batch_scratch
+        if scratch is None:
             import torch
             need = 256 + (4 * self.K + 255) // 256 * 256 + 16 * self.K
-            self._batch_scratch = torch.empty(need, dtype=torch.uint8, device=x.device)
-        r = (_native or _calls()).spmspv_batch(self._n, self.M, self.K, x, tau, y, stream, self._batch_scratch)
+            # beside the image, wherever x lies: it is kept even if this call is refused
+            scratch = torch.empty(need, dtype=torch.uint8, device=x.device if self._image is None else self._image.device)
+            if self._image is not None:
+                self._batch_scratch = scratch
+        r = (_native or _calls()).spmspv_batch(self._n, self.M, self.K, x, tau, y, stream, scratch)
         if r.__class__ is int:
             _check(r, "celty_spmspv_batch")
         return r
