@@ -23,10 +23,10 @@ const at::Tensor &tensor(PyObject *o)
 
 struct Failed {};                                                 // a Python exception is set
 
-void demand(bool ok)
+void demand(bool ok, const char *wanted)
 {
     if (ok) return;
-    PyErr_SetNone(PyExc_AssertionError);
+    PyErr_SetString(PyExc_AssertionError, wanted);
     throw Failed();
 }
 
@@ -73,26 +73,39 @@ celty_stream_t stream_of(PyObject *o)
     return p;
 }
 
-void demand_vector(const at::Tensor &t, at::ScalarType type, int64_t n)
+// The library gets bare pointers and cannot tell how long a vector is or where it lies, so all of that is checked here.
+// A kernel reaches GPU memory, and host memory that is page-locked.
+bool reachable(const at::Tensor &t) { return t.is_cuda() || (t.is_cpu() && t.is_pinned()); }
+
+void *vector(const at::Tensor &t, at::ScalarType type, int64_t n, const char *wanted)
 {
-    demand(t.scalar_type() == type && t.numel() == n && t.is_contiguous());
+    demand(t.scalar_type() == type && t.numel() == n && t.is_contiguous() && reachable(t), wanted);
+    return t.data_ptr();
 }
+
+// The same for one that may be longer than what is read or written.
+void *long_vector(const at::Tensor &t, at::ScalarType type, int64_t n, const char *wanted)
+{
+    demand(t.scalar_type() == type && t.numel() >= n && t.is_contiguous() && reachable(t), wanted);
+    return t.data_ptr();
+}
+
+constexpr char kWantX[] = "x: K float16, contiguous, on the GPU", kWantY[] = "y: M float32, contiguous, on the GPU",
+               kWantFp16[] = "fp16_out: M float16, contiguous, on the GPU";
 
 // The result: the caller's y, checked, or a new vector of M on `like`'s device.
 struct Result {
     at::Tensor made;
     PyObject *given = nullptr;
     void *data = nullptr;
-    Result(PyObject *y, int64_t M, const at::Tensor &like)
+    Result(PyObject *y, int64_t M, const at::Tensor &like, bool may_be_longer = false)
     {
         if (y == Py_None) {
             made = at::empty({M}, at::TensorOptions().dtype(at::kFloat).device(like.device()));
-            data = made.data_ptr();
+            data = vector(made, at::kFloat, M, kWantY);
         } else {
             given = y;
-            const at::Tensor &t = tensor(y);
-            demand_vector(t, at::kFloat, M);
-            data = t.data_ptr();
+            data = (may_be_longer ? long_vector : vector)(tensor(y), at::kFloat, M, kWantY);
         }
     }
     PyObject *give(int status)
@@ -118,15 +131,19 @@ int without_lock(Call call)
 }
 
 // FP16 copy of y (a tensor or None) as an epilogue
-bool fp16_epilogue(PyObject *out, int64_t M, celty_epilogue *ep)
+bool fp16_epilogue(PyObject *out, int64_t M, celty_epilogue *ep, bool may_be_longer = false)
 {
     *ep = celty_epilogue{};
     if (out == Py_None) return false;
-    const at::Tensor &t = tensor(out);
-    if (M >= 0) demand(t.scalar_type() == at::kHalf && t.numel() == M);
     ep->kind = CELTY_EPILOGUE_FP16;
-    ep->out_fp16 = t.data_ptr();
+    ep->out_fp16 = (may_be_longer ? long_vector : vector)(tensor(out), at::kHalf, M, kWantFp16);
     return true;
+}
+
+// FP16 values of a survivor list, as such or as their bit patterns
+uint16_t *list_values(const at::Tensor &t, int64_t n, const char *wanted)
+{
+    return static_cast<uint16_t *>(long_vector(t, t.scalar_type() == at::kHalf ? at::kHalf : at::kShort, n, wanted));
 }
 
 template <PyObject *(*body)(PyObject *const *)>
@@ -155,9 +172,8 @@ PyObject *spmspv(PyObject *const *a)
     const int64_t M = integer(a[1]), K = integer(a[2]);
     const at::Tensor &x = tensor(a[3]);
     const float tau = real(a[4]);
+    const void *xp = vector(x, at::kHalf, K, kWantX);
     Result y(a[5], M, x);
-    demand_vector(x, at::kHalf, K);
-    const void *xp = x.data_ptr();
     const celty_stream_t st = stream_of(a[6]);
     return y.give(without_lock([&] { return celty_spmspv(m, xp, tau, y.data, st); }));
 }
@@ -170,9 +186,11 @@ PyObject *spmspv_static(PyObject *const *a)
     const int64_t M = integer(a[1]), K = integer(a[2]);
     const at::Tensor &x = tensor(a[3]);
     const float tau = real(a[4]);
+    const void *xp = vector(x, at::kHalf, K, kWantX);
     Result y(a[5], M, x);
-    demand_vector(x, at::kHalf, K);
-    const void *xp = x.data_ptr(), *image = tensor(a[7]).data_ptr();
+    const at::Tensor &packed = tensor(a[7]);
+    demand(reachable(packed), "the packed image on the GPU");
+    const void *image = packed.data_ptr();
     const celty_stream_t st = stream_of(a[6]);
     return y.give(without_lock([&] { return celty_spmspv_static(m, image, xp, tau, y.data, st); }));
 }
@@ -185,8 +203,8 @@ PyObject *spmspv_ex(PyObject *const *a)
     const int64_t M = integer(a[1]), K = integer(a[2]);
     const at::Tensor &x = tensor(a[3]);
     const float tau = real(a[4]);
+    const void *xp = vector(x, at::kHalf, K, kWantX);
     Result y(a[5], M, x);
-    demand_vector(x, at::kHalf, K);
     celty_epilogue ep{};
     bool with = false;
     if (a[8] != Py_None) {
@@ -194,15 +212,14 @@ PyObject *spmspv_ex(PyObject *const *a)
                   count = attribute(a[8], "count");
         ep.kind = CELTY_EPILOGUE_SWIGLU;
         ep.tau = real(t.o);
-        ep.out_fp16 = tensor(h.o).data_ptr();
-        ep.list_idx = static_cast<int32_t *>(tensor(idx.o).data_ptr());
-        ep.list_val = static_cast<uint16_t *>(tensor(val.o).data_ptr());
-        ep.list_count = static_cast<int32_t *>(tensor(count.o).data_ptr());
+        ep.out_fp16 = long_vector(tensor(h.o), at::kHalf, M / 2, "swiglu.h: M / 2 float16, contiguous, on the GPU");
+        ep.list_idx = static_cast<int32_t *>(long_vector(tensor(idx.o), at::kInt, M / 2, "swiglu.idx: M / 2 int32, contiguous, on the GPU"));
+        ep.list_val = list_values(tensor(val.o), M / 2, "swiglu.val: M / 2 FP16 values or bit patterns, contiguous, on the GPU");
+        ep.list_count = static_cast<int32_t *>(long_vector(tensor(count.o), at::kInt, 1, "swiglu.count: an int32 on the GPU"));
         with = true;
     } else {
         with = fp16_epilogue(a[7], M, &ep);
     }
-    const void *xp = x.data_ptr();
     const celty_stream_t st = stream_of(a[6]);
     return y.give(without_lock([&] { return celty_spmspv_ex(m, xp, tau, y.data, with ? &ep : nullptr, st); }));
 }
@@ -215,22 +232,13 @@ PyObject *spmspv_swiglu(PyObject *const *a)
     const int64_t M = integer(a[1]), K = integer(a[2]);
     const at::Tensor &gate_up = tensor(a[3]);
     const float tau = real(a[4]);
-    // (y is the library's to check here, as its epilogue's place is)
-    at::Tensor made;
-    PyObject *given = a[5];
-    if (given == Py_None) made = at::empty({M}, at::TensorOptions().dtype(at::kFloat).device(gate_up.device()));
-    void *y = given == Py_None ? made.data_ptr() : tensor(given).data_ptr();
-    demand_vector(gate_up, at::kFloat, 2 * K);
+    const float *in = static_cast<const float *>(vector(gate_up, at::kFloat, 2 * K, "gate_up: 2 K float32, contiguous, on the GPU"));
+    Result y(a[5], M, gate_up, true);
     celty_epilogue ep;
-    const bool with = fp16_epilogue(a[8], -1, &ep);
-    const float *in = static_cast<const float *>(gate_up.data_ptr());
-    void *h = a[7] == Py_None ? nullptr : tensor(a[7]).data_ptr();
+    const bool with = fp16_epilogue(a[8], M, &ep, true);
+    void *h = a[7] == Py_None ? nullptr : long_vector(tensor(a[7]), at::kHalf, K, "h_out: K float16, contiguous, on the GPU");
     const celty_stream_t st = stream_of(a[6]);
-    const int rc = without_lock([&] { return celty_spmspv_swiglu(m, in, tau, y, h, with ? &ep : nullptr, st); });
-    if (rc != CELTY_OK) return PyLong_FromLong(rc);
-    if (given == Py_None) return THPVariable_Wrap(std::move(made));
-    Py_INCREF(given);
-    return given;
+    return y.give(without_lock([&] { return celty_spmspv_swiglu(m, in, tau, y.data, h, with ? &ep : nullptr, st); }));
 }
 CELTY_METHOD(spmspv_swiglu, 9)
 
@@ -239,23 +247,16 @@ PyObject *spmspv_list(PyObject *const *a)
 {
     celty_matrix *m = handle(a[0]);
     const int64_t M = integer(a[1]);
-    const at::Tensor &idx = tensor(a[2]), &val = tensor(a[3]), &count = tensor(a[4]);
-    at::Tensor made;
-    PyObject *given = a[5];
-    if (given == Py_None) made = at::empty({M}, at::TensorOptions().dtype(at::kFloat).device(idx.device()));
-    void *y = given == Py_None ? made.data_ptr() : tensor(given).data_ptr();
-    demand(idx.scalar_type() == at::kInt && (val.scalar_type() == at::kShort || val.scalar_type() == at::kHalf) &&
-           count.scalar_type() == at::kInt);
+    // (how many columns are listed is known on the GPU only: the two vectors have to be as long as the list)
+    const at::Tensor &idx = tensor(a[2]);
+    const int32_t *ip = static_cast<const int32_t *>(long_vector(idx, at::kInt, 0, "idx: int32, contiguous, on the GPU"));
+    const uint16_t *vp = list_values(tensor(a[3]), 0, "val: FP16 values or bit patterns, contiguous, on the GPU");
+    const int32_t *np = static_cast<const int32_t *>(long_vector(tensor(a[4]), at::kInt, 1, "count: an int32 on the GPU"));
+    Result y(a[5], M, idx, true);
     celty_epilogue ep;
     const bool with = fp16_epilogue(a[7], M, &ep);
-    const int32_t *ip = static_cast<const int32_t *>(idx.data_ptr()), *np = static_cast<const int32_t *>(count.data_ptr());
-    const uint16_t *vp = static_cast<const uint16_t *>(val.data_ptr());
     const celty_stream_t st = stream_of(a[6]);
-    const int rc = without_lock([&] { return celty_spmspv_list(m, ip, vp, np, y, with ? &ep : nullptr, st); });
-    if (rc != CELTY_OK) return PyLong_FromLong(rc);
-    if (given == Py_None) return THPVariable_Wrap(std::move(made));
-    Py_INCREF(given);
-    return given;
+    return y.give(without_lock([&] { return celty_spmspv_list(m, ip, vp, np, y.data, with ? &ep : nullptr, st); }));
 }
 CELTY_METHOD(spmspv_list, 8)
 
@@ -266,14 +267,17 @@ PyObject *spmspv_batch(PyObject *const *a)
     const int64_t M = integer(a[1]), K = integer(a[2]);
     const at::Tensor &x = tensor(a[3]);
     const float tau = real(a[4]);
-    demand(x.scalar_type() == at::kHalf && x.dim() == 2 && x.size(1) == K && x.stride(1) == 1);
+    demand(x.scalar_type() == at::kHalf && x.dim() == 2 && x.size(1) == K && x.stride(1) == 1 && reachable(x),
+           "x: N rows of K float16 on the GPU, the values of a row side by side");
     const int64_t N = x.size(0);
     at::Tensor made;
     PyObject *given = a[5];
     if (given == Py_None) made = at::empty({N, M}, at::TensorOptions().dtype(at::kFloat).device(x.device()));
     const at::Tensor &y = given == Py_None ? made : tensor(given);
-    demand(y.scalar_type() == at::kFloat && y.dim() == 2 && y.size(0) == N && y.size(1) == M && y.stride(1) == 1);
+    demand(y.scalar_type() == at::kFloat && y.dim() == 2 && y.size(0) == N && y.size(1) == M && y.stride(1) == 1 && reachable(y),
+           "y: N rows of M float32 on the GPU, the values of a row side by side");
     const at::Tensor &scratch = tensor(a[7]);
+    demand(reachable(scratch), "the scratch on the GPU");
     const void *xp = x.data_ptr();
     void *yp = y.data_ptr(), *sp = scratch.data_ptr();
     const int64_t ldx = x.stride(0), ldy = y.stride(0);

@@ -38,3 +38,22 @@ def test_batch_scratch_lies_beside_the_image(monkeypatch):
     with pytest.raises(AssertionError):
         unbound.spmspv_batch(torch.zeros(2, m.K), 1.0)
     assert unbound._batch_scratch is None
+
+
+def test_vectors_in_pageable_host_memory_are_refused():
+    """A kernel does not reach them.  (The handle has no device memory: what is let through ends with the library's status.)"""
+    from paper_2608_01536_b200 import _celty_torch as calls
+    M, K = 64, 48
+    n, stream = _matrix(M, K)._n, SimpleNamespace(cuda_stream=0)
+    x, y, f = torch.zeros(K, dtype=torch.float16), torch.zeros(M), torch.zeros(M, dtype=torch.float16)
+    gate_up, idx, val, count = torch.zeros(2 * K), torch.zeros(K, dtype=torch.int32), x, torch.zeros(1, dtype=torch.int32)
+    scratch = torch.zeros(1 << 16, dtype=torch.uint8)
+    for out in (y, None):
+        for call, args in ((calls.spmspv, (n, M, K, x, 1.0, out, stream)),
+                           (calls.spmspv_static, (n, M, K, x, 1.0, out, stream, scratch)),
+                           (calls.spmspv_ex, (n, M, K, x, 1.0, out, stream, f, None)),
+                           (calls.spmspv_swiglu, (n, M, K, gate_up, 1.0, out, stream, x, f)),
+                           (calls.spmspv_list, (n, M, idx, val, count, out, stream, None)),
+                           (calls.spmspv_batch, (n, M, K, x[None], 1.0, None if out is None else out[None], stream, scratch))):
+            with pytest.raises(AssertionError):
+                call(*args)

@@ -118,3 +118,65 @@ def test_survivors_that_lie_together_in_x(M, K):
         oi, ov, _ = orc.compact(x, 0.5)
         assert np.array_equal(gi.cpu().numpy(), oi) and np.array_equal(gv.cpu().numpy().view(np.uint16), ov)
         assert m.last_status() == 0
+
+
+def test_no_call_takes_a_vector_that_is_too_short_or_elsewhere():
+    """The library gets bare pointers: sizes, types, strides and memory are the binding's to check, in every call.  Longer
+    vectors are taken where only their beginning is written or read, and so is page-locked host memory."""
+    M, K = 64, 48
+    W = synth.integer_weights(5, M, K)
+    m = celty.Matrix(W, None, device="cuda")
+    half, dev = torch.float16, "cuda"
+    x = torch.from_numpy(synth.integer_activations(6, K)).cuda()
+    gate_up = torch.randn(2 * K, device=dev)
+
+    def short(t):
+        return (t[:-1], t.repeat(2)[::2], t.cpu(), t.double())
+
+    y, f, h = torch.zeros(M, device=dev), torch.zeros(M, dtype=half, device=dev), torch.zeros(K, dtype=half, device=dev)
+    for bad in short(y):
+        for call in (lambda: m.spmspv(x, 1.0, y=bad), lambda: m.spmspv_ex(x, 1.0, y=bad), lambda: m.spmspv_static(x, 1.0, y=bad),
+                     lambda: m.spmspv_swiglu(gate_up, 1.0, y=bad), lambda: m.spmspv_batch(x[None], 1.0, y=bad[None])):
+            with pytest.raises(AssertionError):
+                call()
+    for bad in short(f):
+        for call in (lambda: m.spmspv_ex(x, 1.0, fp16_out=bad), lambda: m.spmspv_swiglu(gate_up, 1.0, fp16_out=bad)):
+            with pytest.raises(AssertionError):
+                call()
+    for bad in short(h):
+        with pytest.raises(AssertionError):
+            m.spmspv_swiglu(gate_up, 1.0, h_out=bad)
+    for bad in short(gate_up):
+        with pytest.raises(AssertionError):
+            m.spmspv_swiglu(bad, 1.0)
+    mid = celty.SwigluOut(M // 2, 0.1, dev)
+    for name in ("h", "idx", "val", "count"):
+        good = getattr(mid, name)
+        for bad in (good[:-1], good.cpu(), good.double()) + ((good.repeat(2)[::2],) if name != "count" else ()):
+            setattr(mid, name, bad)
+            with pytest.raises(AssertionError):
+                m.spmspv_ex(x, 1.0, swiglu=mid)
+        setattr(mid, name, good)
+    idx, val = (x.abs() > 1).nonzero().flatten().int(), x[x.abs() > 1]
+    n = torch.tensor([idx.numel()], dtype=torch.int32, device=dev)
+    for bad in (dict(y=y[:-1]), dict(y=y.cpu()), dict(y=y.half()), dict(idx=idx.cpu()), dict(idx=idx.repeat(2)[::2]), dict(idx=idx.long()),
+                dict(val=val.cpu()), dict(val=val.repeat(2)[::2]), dict(val=val.float()), dict(count=n[:0]), dict(count=n.cpu()),
+                dict(fp16_out=f[:-1]), dict(fp16_out=f.repeat(2)[::2])):
+        with pytest.raises(AssertionError):
+            m.spmspv_list(**{**dict(idx=idx, val=val, count=n), **bad})
+
+    # what is longer than it has to be, or page-locked, is taken
+    want = m.spmspv(x, 1.0)
+    wide, wide_h = torch.full((M + 9,), 3.0, device=dev), torch.full((K + 9,), 3.0, dtype=half, device=dev)
+    assert m.spmspv_list(idx, val.view(torch.int16), n, y=wide) is wide and torch.equal(wide[:M], want) and torch.all(wide[M:] == 3)
+    longer = celty.SwigluOut(M, 0.1, dev)
+    assert torch.equal(m.spmspv_ex(x, 1.0, swiglu=longer), want)
+    plain = m.spmspv_swiglu(gate_up, 1.0)
+    again = m.spmspv_swiglu(gate_up, 1.0, y=wide, h_out=wide_h)[:M]
+    apart = torch.from_numpy(np.abs(W).astype(np.float32)).cuda() @ wide_h[:K].float().abs() * (2 * K * 2.0 ** -24)
+    assert torch.all((again - plain).abs() <= apart) and torch.all(wide_h[K:] == 3)      # K FP32 additions in another order
+    pinned = x.cpu().pin_memory()
+    assert torch.equal(m.spmspv(pinned, 1.0, y=y), want)
+    with pytest.raises(AssertionError):
+        m.spmspv(pinned, 1.0)                                     # y would be made in pageable memory
+    assert m.last_status() == 0
