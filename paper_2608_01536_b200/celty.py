@@ -193,7 +193,7 @@ class Matrix:
         return other
 
     def __del__(self):
-        h, self._h = getattr(self, "_h", None), None
+        h, self._h, self._n = getattr(self, "_h", None), None, None
         if h and _lib is not None:
             _lib.celty_destroy(h)
 

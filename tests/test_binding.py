@@ -57,3 +57,11 @@ def test_vectors_in_pageable_host_memory_are_refused():
                            (calls.spmspv_batch, (n, M, K, x[None], 1.0, None if out is None else out[None], stream, scratch))):
             with pytest.raises(AssertionError):
                 call(*args)
+
+
+def test_a_matrix_that_was_given_back_has_no_handle():
+    """Calls on it reach the library with null, which it refuses, and not with memory that is no longer the matrix's."""
+    m = _matrix()
+    assert m._n == m._h.value
+    m.__del__()
+    assert m._h is None and m._n is None
