@@ -732,16 +732,20 @@ FusedParams plan_params(const celty_matrix *m, const LaunchKnobs &knobs, const F
 
 // Plan and parameters of the handle's launches that serve `vectors` vectors, worked out by the first such call after the
 // handle was bound or its choices changed: 0.45 us of host time that every call paid otherwise, and a call on a small
-// layer is bound by the host.
-const PreparedLaunch &prepared_launch(celty_matrix *m, const DeviceInfo &di, int vectors, bool list = false)
+// layer is bound by the host.  Threads may call on one handle at once (on one stream), so they are copied out under a lock.
+int prepared_launch(celty_matrix *m, const DeviceInfo &di, int vectors, bool list, FusedPlan *plan, FusedParams *params)
 {
+    static std::mutex mu;
+    std::lock_guard<std::mutex> lock(mu);
     PreparedLaunch &p = m->prepared[vectors > 1 ? vectors : list ? 1 : 0];
     if (p.device != di.device) {
         p.status = plan_launch(m, *m, di, vectors, &p.plan, list);
         if (p.status == CELTY_OK) p.params = plan_params(m, *m, p.plan, m->d_image);
         p.device = p.status == CELTY_ECUDA ? -1 : di.device;
     }
-    return p;
+    *plan = p.plan;
+    if (params) *params = p.params;
+    return p.status;
 }
 
 // Programmatic dependent launch: the kernel may be scheduled while the previous kernel of the stream drains; it
@@ -911,11 +915,11 @@ int run_product(celty_matrix *m, const void *x_dev, float tau, const ListInput *
     float *y = static_cast<float *>(y_dev);
     const uint8_t *stream_base = m->d_image + m->meta_bytes;
     if (m->layout == CELTY_LAYOUT_LANE_TILE && m->variant == 0) {
-        const PreparedLaunch &prepared = prepared_launch(m, di, 1, list != nullptr);
-        if (prepared.status) return prepared.status;
+        FusedPlan plan;
+        FusedParams fp;
+        rc = prepared_launch(m, di, 1, list != nullptr, &plan, &fp);
+        if (rc) return rc;
         if (extras && m->reg_rows) return CELTY_EINVAL;
-        const FusedPlan &plan = prepared.plan;
-        FusedParams fp = prepared.params;
         if (list) {
             fp.list_idx = list->idx;
             fp.list_val = list->val;
@@ -1166,9 +1170,8 @@ int run_batch(celty_matrix *m, const uint16_t *x, int64_t ldx, int N, float tau,
     const double stream_us = 0.5 * 2.5 * (double)(m->nnz + m->n_pad) / 5e6, fixed_us = 5.0;
     int most = 1;
     for (int v = 1; v <= N; ++v) {
-        const PreparedLaunch &prepared = prepared_launch(m, di, v);
-        if (prepared.status != CELTY_OK || (v > 1 && prepared.plan.lean == 0)) break;
-        const FusedPlan &pl = prepared.plan;
+        FusedPlan pl;
+        if (prepared_launch(m, di, v, false, &pl, nullptr) != CELTY_OK || (v > 1 && pl.lean == 0)) break;
         // teams that share a part's columns, in blocks of G teams
         const double per_part = pl.grid / pl.P + (pl.mix >= 2 ? 1.0 / pl.mix : 0.0);
         cost[v] = fixed_us + stream_us * di.sms / (per_part * pl.P);
@@ -1192,9 +1195,11 @@ int run_batch(celty_matrix *m, const uint16_t *x, int64_t ldx, int N, float tau,
             if (rc) return rc;
             continue;
         }
-        const FusedPlan &plan = m->prepared[v].plan;
+        FusedPlan plan;
+        FusedParams fp;
+        rc = prepared_launch(m, di, v, false, &plan, &fp);
+        if (rc) return rc;
         uint32_t *status = reinterpret_cast<uint32_t *>(m->d_ws + m->ws.status_off);
-        FusedParams fp = m->prepared[v].params;
         fp.x = xv; fp.ldx = ldx;
         fp.y = yv; fp.ldy = ldy;
         fp.tau = tau;

@@ -1,6 +1,8 @@
 """Products of layers whose thread blocks own few columns, dealt to them whatever x is, against the oracle and against the
 kernel that ranks the survivors (variant 256): the edges of 32, 64, 96 and 128 columns per block, row parts of unequal block
 counts, more blocks than columns, survivors that cluster in x."""
+import threading
+
 import numpy as np
 import pytest
 import torch
@@ -180,3 +182,41 @@ def test_no_call_takes_a_vector_that_is_too_short_or_elsewhere():
     with pytest.raises(AssertionError):
         m.spmspv(pinned, 1.0)                                     # y would be made in pageable memory
     assert m.last_status() == 0
+
+
+def test_first_calls_of_several_threads_on_one_handle():
+    """A handle's launches are worked out by the first call of each kind: threads whose first calls meet (on one stream, which
+    keeps their kernels apart) all launch the finished plan."""
+    M, K, threads = 640, 512, 6
+    W = synth.integer_weights(8, M, K)
+    mask = synth.mask_bernoulli(8, M, K, 0.5)
+    first = celty.Matrix(W, mask, device="cuda")
+    X = np.stack([synth.integer_activations(70 + n, K) for n in range(threads)])
+    ref = np.stack([orc.masked_gemv(W, mask, X[n], 1.0, threads=4)[0] for n in range(threads)])
+    xd = torch.from_numpy(X).cuda()
+    lists = [(torch.from_numpy(i).cuda(), torch.from_numpy(v.view(np.int16)).cuda(), torch.tensor([i.size], dtype=torch.int32, device="cuda"))
+             for i, v, _ in (orc.compact(X[n], 1.0) for n in range(threads))]
+    torch.cuda.synchronize()
+    for _ in range(12):
+        m = first.clone("cuda")
+        ys, failed, start = [None] * threads, [], threading.Barrier(threads)
+
+        def work(n):
+            try:
+                start.wait()
+                calls = [lambda: m.spmspv(xd[n], 1.0), lambda: m.spmspv_list(*lists[n]), lambda: m.spmspv_batch(xd[:2], 1.0)]
+                ys[n] = [calls[(n + k) % 3]() for k in range(3)], [(n + k) % 3 for k in range(3)]
+            except BaseException as e:                            # noqa: BLE001
+                failed.append(e)
+
+        workers = [threading.Thread(target=work, args=(n,)) for n in range(threads)]
+        for w in workers:
+            w.start()
+        for w in workers:
+            w.join()
+        assert not failed
+        assert m.last_status() == 0
+        for n in range(threads):
+            for y, kind in zip(*ys[n]):
+                want = ref[:2] if kind == 2 else ref[n]
+                assert np.array_equal(y.cpu().numpy().astype(np.float64), want), (n, kind)
