@@ -697,13 +697,6 @@ def dense_gemv_us(torch, wl, dev, steps):
     return out
 
 
-def product_kernel(m):
-    """Name of the kernel that a single-launch call on this handle runs (one slab per block, library's choices)."""
-    plan = m.launch_plan()
-    columns = -(-m.K // max(1, plan["grid"] // plan["row_parts"]))
-    return "k_spmspv_direct" if columns <= 128 and plan["slabs_per_block"] == 1 else "k_spmspv_fused"
-
-
 def dram_traffic_per_launch(name):
     """dram__bytes_read.sum + dram__bytes_write.sum of one launch of the fused kernel on this workload, from the
     profiler capture summarised under profiles/ (kept as data next to the summaries); None when there is none."""
@@ -976,7 +969,7 @@ def run_celty(args):
                      "frac_on_bare_format_bytes": wl.bare_bytes / sec_per_call / 1e9 / peak,
                      "frac_of_nominal_8000": wl.total_bytes / sec_per_call / 1e9 / 8000.0,
                      "peak_source": peak_src,
-                     "kernel": product_kernel(wl.mats[0]) if launches_per_step == 1 else "all kernels of the call",
+                     "kernel": wl.mats[0].launch_plan()["kernel"] if launches_per_step == 1 else "all kernels of the call",
                      "note": f"{launches_per_step} launch{'es' if launches_per_step > 1 else ''} per call: algorithmic bytes per call "
                              "/ CUDA-event time per call",
                      "us_per_call": us_per_call, "us_per_call_fastest_region": min(regions) * 1e3 / calls_per_region,

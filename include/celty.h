@@ -444,12 +444,15 @@ int celty_set_launch(celty_matrix *m, int32_t grid, int32_t variant, int32_t gro
 int celty_set_register_rows(celty_matrix *m, int32_t rows);
 
 /*
- * celty_launch_plan -- the shape the fused kernel would be launched with for this handle on the current
+ * celty_launch_plan -- the shape the single-launch kernel would be launched with for this handle on the current
  * device, with the knobs of celty_set_launch applied (LANE_TILE handles; needs a CUDA device):
  *   out[0..9] = thread blocks, threads per block, dynamic shared memory (bytes), warp teams per slab,
  *   ring slots per team, thread blocks per cluster, row parts, slabs per block, ring slot size (bytes),
  *   merge (0 ordered two-stage sum, 1 bulk reduce-add) + 16 if warp pairs are in use + 256 x the number of row
- *   parts a left-over block serves (1 = blocks are not shared between parts).   n = capacity of out (at least 10).
+ *   parts a left-over block serves (1 = blocks are not shared between parts).
+ *   out[10] = which kernel that is: 0 the one that ranks the survivors, 1 the one that deals columns to blocks; out[11] the same
+ *   for celty_spmspv_list, out[12..18] for launches that serve 2 .. 8 vectors of celty_spmspv_batch (-1: there is none).
+ *   n = capacity of out (at least 10; words beyond it are not written).
  * Errors: CELTY_EINVAL, CELTY_ECUDA.
  */
 int celty_launch_plan(const celty_matrix *m, int32_t *out, int32_t n);

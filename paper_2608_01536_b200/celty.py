@@ -261,14 +261,18 @@ class Matrix:
         _check(load().celty_set_launch(self._h, grid, variant, groups, depth, cluster), "celty_set_launch")
 
     def launch_plan(self) -> dict:
-        """Shape of the fused kernel's launch for this handle on the current device."""
-        out = (_i32 * 10)()
-        _check(load().celty_launch_plan(self._h, out, 10), "celty_launch_plan")
+        """Shape of the single-launch kernel's launch for this handle on the current device, and which kernel it is; which
+        one runs from a list, and (index 2 .. 8) in launches that serve so many vectors of a batch (None: there is none)."""
+        out = (_i32 * 19)()
+        _check(load().celty_launch_plan(self._h, out, 19), "celty_launch_plan")
         keys = ("grid", "threads", "smem_bytes", "teams_per_slab", "ring_depth", "cluster", "row_parts",
                 "slabs_per_block", "slot_bytes", "merge")
         plan = dict(zip(keys, [int(v) for v in out]))
         plan["parts_per_spare_block"] = plan["merge"] >> 8
         plan["warp_pairs"], plan["merge"] = (plan["merge"] >> 4) & 1, plan["merge"] & 15
+        name = {-1: None, 0: "k_spmspv_fused", 1: "k_spmspv_direct"}
+        plan["kernel"], plan["list_kernel"] = name[out[10]], name[out[11]]
+        plan["batch_kernels"] = {v: name[out[10 + v]] for v in range(2, 9)}
         return plan
 
     def set_register_rows(self, rows: int = 0):

@@ -819,6 +819,13 @@ extern "C" int celty_launch_plan(const celty_matrix *m, int32_t *out, int32_t n)
     const int32_t v[10] = {plan.grid, plan.threads, (int32_t)plan.smem, plan.G, plan.D, plan.cl, plan.P, plan.Sc,
                            plan.slot_bytes, plan.merge + 16 * plan.pp + 256 * plan.mix};
     for (int i = 0; i < 10; ++i) out[i] = v[i];
+    // which kernel: of this launch, of one from a list, of launches that serve 2 .. 8 vectors
+    if (n > 10) out[10] = plan.direct;
+    for (int i = 11; i < std::min(n, 19); ++i) {
+        rc = plan_launch(m, *m, di, i == 11 ? 1 : i - 10, &plan, i == 11);
+        if (rc == CELTY_ECUDA) return rc;
+        out[i] = rc ? -1 : plan.direct;
+    }
     return CELTY_OK;
 }
 

@@ -105,7 +105,7 @@ def test_survivors_that_lie_together_in_x(M, K):
     as unevenly as the rule allows (a call's values do not depend on it)."""
     W = synth.integer_weights(7, M, K)
     mask = synth.mask_bernoulli(7, M, K, 0.5)
-    m = celty.Matrix(W, mask, tile_rows=64 if M == 4096 else 0, device="cuda")
+    m = celty.Matrix(W, mask, tile_rows=64 if M == 4096 else 48, device="cuda")
     rng = np.random.default_rng(K)
     i = np.arange(K)
     heads = rng.random(K // 128) < 0.5
@@ -220,3 +220,35 @@ def test_first_calls_of_several_threads_on_one_handle():
             for y, kind in zip(*ys[n]):
                 want = ref[:2] if kind == 2 else ref[n]
                 assert np.array_equal(y.cpu().numpy().astype(np.float64), want), (n, kind)
+
+
+def test_the_plan_names_the_kernel():
+    """At most 128 columns per block: dealt; more, several slabs per block, or on request: ranked.  A list is shared by the
+    kernel that deals unless left-over blocks serve several row parts.  A caller of the C entry with room for ten words
+    gets ten."""
+    def plan(M, K, variant=0, **kw):
+        m = celty.Matrix(synth.integer_weights(1, M, K), None, device="cuda", **kw)
+        m.set_launch(variant=variant)
+        p = m.launch_plan()
+        assert 148 // p["row_parts"] == p["grid"] // p["row_parts"]                # one block per SM of a B200
+        return p
+
+    ranked, direct = "k_spmspv_fused", "k_spmspv_direct"
+    for K, kernel in ((148 * 128, direct), (148 * 128 + 1, ranked)):
+        p = plan(40, K)
+        assert (p["kernel"], p["list_kernel"]) == (kernel, direct)
+    for N in range(2, 9):
+        columns = 128 * (148 // N)
+        for K, kernel in ((columns, direct), (columns + 1, ranked)):
+            assert plan(40, K)["batch_kernels"][N] == kernel, (N, K)
+    for variant in (2, 128, 256):
+        p = plan(300, 400, variant)
+        assert p["kernel"] == ranked and p["list_kernel"] in (ranked, None)
+    assert plan(300, 400, tile_rows=2, slabs_per_block=2)["kernel"] == ranked
+    m = celty.Matrix(synth.integer_weights(1, 40, 40), None, device="cuda")
+    import ctypes
+    out = (ctypes.c_int32 * 20)(*[-7] * 20)
+    for n in (10, 11, 12, 18, 19, 20):
+        assert celty.load().celty_launch_plan(m._h, out, n) == 0
+        assert out[min(n, 19):] == [-7] * (20 - min(n, 19)) and out[0] == 148
+    assert celty.load().celty_launch_plan(m._h, out, 9) == -1
