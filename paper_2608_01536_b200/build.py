@@ -27,8 +27,17 @@ def _older(target, sources) -> bool:
     return any(os.path.getmtime(f) > t for f in sources)
 
 
+def _binding_outdated() -> bool:
+    """The module is tied to the torch it was built against, which it names (TORCH_VERSION): file times do not tell."""
+    import torch
+    if _older(BINDING, [BINDING_SOURCE, os.path.join(ROOT, "include", "celty.h")]):
+        return True
+    with open(BINDING, "rb") as f:
+        return b"built with torch %s\0" % torch.__version__.encode() not in f.read()
+
+
 def needs_build() -> bool:
-    return _older(LIB, SOURCES + HEADERS) or _older(BINDING, [BINDING_SOURCE, os.path.join(ROOT, "include", "celty.h")])
+    return _older(LIB, SOURCES + HEADERS) or _binding_outdated()
 
 
 def _build_binding() -> None:
@@ -39,7 +48,7 @@ def _build_binding() -> None:
     nvcc = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
     cuda = os.path.join(os.path.dirname(os.path.dirname(nvcc)), "include")
     subprocess.check_call(
-        ["g++", "-O2", "-std=c++17", "-fPIC", "-shared", "-D_GLIBCXX_USE_CXX11_ABI=%d" % torch._C._GLIBCXX_USE_CXX11_ABI,
+        ["g++", "-O2", "-std=c++17", "-fPIC", "-shared", '-DTORCH_VERSION="%s"' % torch.__version__, "-D_GLIBCXX_USE_CXX11_ABI=%d" % torch._C._GLIBCXX_USE_CXX11_ABI,
          "-I", os.path.join(ROOT, "include"), "-I", sysconfig.get_paths()["include"], "-I", cuda,
          "-isystem", os.path.join(base, "include"), "-isystem", os.path.join(base, "include", "torch", "csrc", "api", "include"),
          BINDING_SOURCE, "-o", BINDING, "-L", HERE, "-l:libcelty.so", "-L", os.path.join(base, "lib"),
@@ -47,6 +56,8 @@ def _build_binding() -> None:
 
 
 def build(force: bool = False, verbose: bool = False) -> str:
+    if not (force or needs_build()):
+        return LIB
     if force or _older(LIB, SOURCES + HEADERS):
         nvcc = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
         cmd = [nvcc, "-O3", "-std=c++17", "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo",
@@ -55,7 +66,7 @@ def build(force: bool = False, verbose: bool = False) -> str:
         if verbose:
             cmd.insert(1, "-Xptxas=-v")
         subprocess.check_call(cmd)
-    if force or _older(BINDING, [BINDING_SOURCE, os.path.join(ROOT, "include", "celty.h")]):
+    if force or _binding_outdated():
         _build_binding()
     return LIB
 

@@ -101,6 +101,9 @@ def _calls():
         except ImportError as e:
             raise RuntimeError("_celty_torch.so is missing or does not load: run `python -m paper_2608_01536_b200.build`.  "
                                "There is no fallback for this path.") from e
+        if _celty_torch.built_with != f"built with torch {torch.__version__}":
+            raise RuntimeError(f"_celty_torch.so was {_celty_torch.built_with}, not {torch.__version__}: "
+                               "run `python -m paper_2608_01536_b200.build`.")
         _native = _celty_torch
     return _native
 

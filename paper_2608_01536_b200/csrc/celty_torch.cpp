@@ -298,4 +298,15 @@ PyModuleDef module = {PyModuleDef_HEAD_INIT, "_celty_torch", nullptr, -1, method
 
 }  // namespace
 
-PyMODINIT_FUNC PyInit__celty_torch(void) { return PyModule_Create(&module); }
+// What the build looks for in the file; the binding compares the version with torch's before the first call.
+const char built_with[] = "built with torch " TORCH_VERSION;
+
+PyMODINIT_FUNC PyInit__celty_torch(void)
+{
+    PyObject *m = PyModule_Create(&module);
+    if (m && PyModule_AddStringConstant(m, "built_with", built_with) < 0) {
+        Py_DECREF(m);
+        return nullptr;
+    }
+    return m;
+}

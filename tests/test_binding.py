@@ -65,3 +65,14 @@ def test_a_matrix_that_was_given_back_has_no_handle():
     assert m._n == m._h.value
     m.__del__()
     assert m._h is None and m._n is None
+
+
+def test_the_module_is_tied_to_its_torch(monkeypatch):
+    """With another torch than the one it was built against it is built again, and is not called."""
+    assert not build.needs_build()
+    monkeypatch.setattr(torch, "__version__", torch.__version__ + ".other")
+    assert build.needs_build()
+    monkeypatch.setattr(celty, "_native", None)
+    monkeypatch.setattr(torch.cuda, "current_stream", lambda: None)
+    with pytest.raises(RuntimeError, match="built with torch"):
+        celty._calls()
