@@ -16,24 +16,25 @@
 // What it costs is balance: the survivors per block differ as they fall, sqrt((1 - d) / (d n)) of n columns at density d,
 // where the ranked list is even to one column.  Device time with 50 % of the weights, in us, mean over 16 draws of
 // independent survivors, ranked -> this kernel, by columns per block:
-//    14 (1024 x 1024, d = 0.1 / 0.5)              3.74 -> 3.34, 3.78 -> 3.34
-//    56 (4096 x 4096, 0.1 / 0.3 / 0.5 / 0.7)      4.81 -> 3.99, 6.34 -> 5.35, 7.78 -> 6.95, 8.64 -> 8.01
-//    70 (5120 x 5120, 0.3 / 0.5)                  7.27 -> 6.69, 9.30 -> 8.65
-//    75 (4096 x 11008, 0.1 / 0.5 / 0.7)           7.66 -> 5.91, 12.25 -> 11.62, 14.34 -> 13.61
-//    84 (11008 x 4096, 0.1 / 0.5 / 0.7)           6.92 -> 5.64, 11.59 -> 11.32, 14.17 -> 13.32
-//   111 (14336 x 4096, 0.1 / 0.3 / 0.5 / 0.7)     7.01 -> 5.93, 9.88 -> 9.38, 12.83 -> 12.82, 15.61 -> 15.45
-//   111 (8192 x 8192, 0.1 / 0.3 / 0.5 / 0.7)      7.66 -> 6.46, 10.79 -> 10.89, 14.24 -> 14.62, 17.60 -> 17.56
+//    14 (1024 x 1024, d = 0.1 / 0.5)              3.74 -> 3.30, 3.80 -> 3.30
+//    56 (4096 x 4096, 0.1 / 0.3 / 0.5 / 0.7)      4.82 -> 3.95, 6.32 -> 5.29, 7.79 -> 6.89, 8.65 -> 7.94
+//    70 (5120 x 5120, 0.3 / 0.5)                  7.27 -> 6.64, 9.29 -> 8.60
+//    75 (4096 x 11008, 0.1 / 0.5 / 0.7)           7.70 -> 5.92, 12.26 -> 11.64, 14.36 -> 13.64
+//    84 (11008 x 4096, 0.1 / 0.5 / 0.7)           6.92 -> 5.64, 11.63 -> 11.39, 14.19 -> 13.37
+//   111 (14336 x 4096, 0.1 / 0.3 / 0.5 / 0.7)     7.01 -> 5.91, 9.87 -> 9.38, 12.86 -> 12.82, 15.64 -> 15.45
+//   111 (8192 x 8192, 0.1 / 0.3 / 0.5 / 0.7)      7.68 -> 6.43, 10.77 -> 10.91, 14.26 -> 14.63, 17.58 -> 17.56
 // and with a build for six chunks
 //   138 (8192 x 10240, 0.1 / 0.3 / 0.5 / 0.7)     8.06 -> 7.20, 12.59 -> 12.77, 16.40 -> 16.77, 20.54 -> 20.66
 //   139 (13824 x 5120, 0.1 / 0.5 / 0.7)           7.09 -> 6.61, 14.60 -> 14.60, 18.18 -> 17.87
 //   187 (5120 x 13824, 0.1 / 0.5 / 0.7)           7.29 -> 6.41, 15.42 -> 14.39, 18.62 -> 17.77
 // so the line, four chunks, lies where the first layer is slower from 30 % on; it gives away what other shapes would gain beyond.
 // Survivors that lie together in x are shared about as evenly as independent ones.  Half of the 128-column heads zeroed,
-// ranked / runs of 32 columns / of 8 / of 4 / of two:   4096 x 4096 7.7 / 8.5 / 7.2 / 7.0 / 6.7;   4096 x 11008 12.2 / 15.2 / 15.7 /
-// 12.3 / 11.4;   8192 x 8192 14.2 / 18.6 / 15.8 / 14.9 / 13.9.  Single columns are no more even, and loads of x that touch a
-// sector per column cost 1 to 6 %; with runs of two independent survivors take 0 to 2 % more than with runs of 32 from 84 columns per
-// block on (8192 x 8192 at 10 %: 4 %), below that the offsets' new place (load_places) gains more.  One warp per chunk that
-// shares its ballot and its activations with the others through shared memory behind a barrier: 0 to 2 % slower.
+// ranked / runs of 32 columns / of 8 / of 4 / of two:   4096 x 4096 7.7 / 8.5 / 7.2 / 6.9 / 6.6;   4096 x 11008 12.2 / 15.2 / 15.7 /
+// 12.2 / 11.5;   8192 x 8192 14.3 / 18.6 / 15.8 / 14.9 / 13.9.  Single columns are no more even, and loads of x that touch a
+// sector per column cost 1 to 6 %.  Independent survivors take 1 to 3 % more with runs of two than with runs of 32 on layers
+// of 84 columns per block and more (8192 x 8192 at 10 %: 4 %), whose blocks now reach over all of a large image, and 2 to 6 % less
+// below.  One warp per chunk that shares its ballot and its activations with the others through shared memory behind a barrier,
+// or the two warps of a pair half of the chunks each: 0 to 2 % slower.
 // Groups of 2 to 32 blocks that share their columns' survivors evenly, ranked
 // shares of the columns beyond a fixed core under the streaming: both slower (more code and loads on the way to the first
 // copy, or a streaming loop that the compiler schedules worse).  A list is shared evenly whatever its length; the second
@@ -91,15 +92,22 @@ __global__ void __launch_bounds__(kDirectThreads, 1) k_spmspv_direct(const Fused
     // Programmatic dependent launch: see k_spmspv_fused.
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     // {offset/16, units of 16 bytes} of the block's columns' sub-blocks: once per block, by the last warps, which do not stream
-    // (each streaming warp for itself, in registers: 0.05 to 0.3 us slower, their loads touch a sector per run of columns)
-    auto load_places = [&]() {
-        const int i = tid - (nthreads - 32 * kDirectChunks), j = direct_column(max(i, 0), kslice, nK, nK_inv);
-        if (i >= 0 && i < 32 * kChunks && j < p.K) {
-            const uint32_t at = p.meta[(size_t)j * p.S + s];
-            place[i] = make_uint2(at, p.meta[(size_t)j * p.S + s + 1] - at);
-        }
+    // (each streaming warp for itself, in registers: 0.05 to 0.3 us slower, their loads touch a sector per run of columns).
+    // The streaming warps meet them at barrier 15, when x is on its way (at the barrier of all warps below, ahead of the wait for
+    // the previous kernel: 1024 x 1024 3.34 us instead of 3.30, 4096 x 4096 6.93 instead of 6.87).
+    const int own = tid - (nthreads - 32 * kDirectChunks), own_column = direct_column(max(own, 0), kslice, nK, nK_inv);
+    const bool owns = own >= 0 && own < 32 * kChunks && own_column < p.K;
+    uint2 own_place = make_uint2(0u, 0u);
+    auto load_place = [&]() {
+        if (!owns) return;
+        own_place.x = p.meta[(size_t)own_column * p.S + s];
+        own_place.y = p.meta[(size_t)own_column * p.S + s + 1];
     };
-    if (!kList && p.image_early) load_places();
+    auto give_place = [&]() {
+        if (owns) place[own] = make_uint2(own_place.x, own_place.y - own_place.x);
+        asm volatile("bar.arrive 15, %0;" ::"r"(nthreads) : "memory");
+    };
+    if (!kList && p.image_early) load_place();
     if (tid < 4) zero_group[tid] = 0;
     if (tid < G) const_cast<int *>(flags)[tid] = 0;
     if (streams && lane == 0) {
@@ -114,10 +122,11 @@ __global__ void __launch_bounds__(kDirectThreads, 1) k_spmspv_direct(const Fused
         for (int i = half * 32 + lane; i < slab_words / 4; i += 32 * stride) slab4[i] = make_float4(0.f, 0.f, 0.f, 0.f);
     }
     __syncthreads();
+    if (!kList && p.image_early && !streams) give_place();
     asm volatile("griddepcontrol.wait;" ::: "memory");
     if (!kList && !p.image_early && !streams) {
-        load_places();
-        asm volatile("bar.arrive 15, %0;" ::"r"(nthreads) : "memory");
+        load_place();
+        give_place();
     }
 
     // The list that the API reports is made by a few blocks, eight words of x each (2048 x 5504 with 16 each: 0.3 us slower).
@@ -163,7 +172,7 @@ __global__ void __launch_bounds__(kDirectThreads, 1) k_spmspv_direct(const Fused
             uint32_t xb[kChunks + 1];
 #pragma unroll
             for (int c = 0; c < kChunks; ++c) xb[c] = column[c] < p.K ? x[column[c]] : 0u;
-            if (!p.image_early) asm volatile("bar.sync 15, %0;" ::"r"(nthreads) : "memory");   // the places, under x's way here
+            asm volatile("bar.sync 15, %0;" ::"r"(nthreads) : "memory");                // the places are there
             uint32_t n = 0;
 #pragma unroll
             for (int c = 0; c < kChunks; ++c) {

@@ -127,8 +127,8 @@ struct DirectSmem {
     uint32_t acc, ring, bars, flag, items, zero, place, keep, total;
 };
 
-// chunks: of 32 columns that a block owns; 0: the survivors come as a list
-inline DirectSmem direct_smem_layout(int R, int K, int G, int D, int slot_bytes, int cap, int chunks)
+// columns: of a block, at most (direct_columns); 0: the survivors come as a list
+inline DirectSmem direct_smem_layout(int R, int K, int G, int D, int slot_bytes, int cap, int columns)
 {
     DirectSmem l;
     uint32_t off = 0;
@@ -139,7 +139,7 @@ inline DirectSmem direct_smem_layout(int R, int K, int G, int D, int slot_bytes,
     off = (off + 15) / 16 * 16;
     l.zero = off;      off += 16;                                            // the all-zero group that idle lanes fetch
     l.items = off;     off += (uint32_t)G * cap * 8;                         // {offset/16, bytes/16 and x} per column of a team
-    l.place = off;     off += 32 * (uint32_t)chunks * 8;                     // {offset/16, bytes/16} of the block's columns
+    l.place = off;     off += (uint32_t)columns * 8;                            // {offset/16, bytes/16} of the block's columns
     l.keep = off;      off += (uint32_t)((K + 31) / 32) * 4;                 // one keep bit per activation
     l.total = (off + 15) / 16 * 16;
     return l;

@@ -500,10 +500,18 @@ int launch_compact(const void *x, int64_t K, float tau, int32_t *idx, uint16_t *
 
 constexpr int kMostToMix = 48;           // left-over blocks are shared between row parts up to this (fit_clusters)
 
+// Columns that a block of k_spmspv_direct may own.  Its tables are sized by them: with 32 per chunk the 4096 x 11008 layer had
+// room for seven teams instead of eight (from gate and up 13.0 us, with eight 12.8).
+int direct_columns(int64_t K, int blocks_per_part)
+{
+    const int64_t round = (int64_t)kDirectRun * blocks_per_part;
+    return (int)((K + round - 1) / round) * kDirectRun;
+}
+
 // Columns that a team of k_spmspv_direct may get: of the block's, or of an even split of a list over the teams of a row part.
 int direct_cap(int64_t K, int blocks_per_part, int G, bool list)
 {
-    return list ? (int)(K / ((int64_t)blocks_per_part * G) + 1) : (32 * kDirectChunks + G - 1) / G;
+    return list ? (int)(K / ((int64_t)blocks_per_part * G) + 1) : (direct_columns(K, blocks_per_part) + G - 1) / G;
 }
 
 // Shape of the fused launch: P row parts of Sc slabs, G teams per slab (teams = G * Sc warps, one accumulator
@@ -538,7 +546,8 @@ int plan_fused(const celty_matrix *m, const LaunchKnobs &knobs, const DeviceInfo
     pl.chunks = list ? 0 : (int)chunks;
     auto smem_bytes = [&](int G, int D) {
         if (!pl.direct) return fused_smem_bytes(m->R, (int)m->K, G, pl.Sc, D, pl.slot_bytes, pl.cap);
-        return (size_t)direct_smem_layout(m->R, (int)m->K, G, D, pl.slot_bytes, direct_cap(m->K, per_part, G, list), pl.chunks).total;
+        return (size_t)direct_smem_layout(m->R, (int)m->K, G, D, pl.slot_bytes, direct_cap(m->K, per_part, G, list),
+                                          list ? 0 : direct_columns(m->K, per_part)).total;
     };
     auto fit = [&](int pairs) {
         pl.pp = pairs;
@@ -716,7 +725,8 @@ FusedParams plan_params(const celty_matrix *m, const LaunchKnobs &knobs, const F
     fp.merge = plan.merge;
     fp.image_early = 1;
     if (plan.direct)
-        fp.direct = direct_smem_layout(m->R, (int)m->K, plan.G, plan.D, plan.slot_bytes, plan.cap, plan.chunks);
+        fp.direct = direct_smem_layout(m->R, (int)m->K, plan.G, plan.D, plan.slot_bytes, plan.cap,
+                                       plan.chunks ? direct_columns(m->K, plan.grid / plan.P) : 0);
     else
         fp.lay = fused_smem_layout(m->R, (int)m->K, plan.G * plan.Sc, plan.D, plan.slot_bytes, plan.cap, std::max(0, plan.window));
     fp.clear_rows = (int)(m->M / plan.grid);

@@ -252,3 +252,13 @@ def test_the_plan_names_the_kernel():
         assert celty.load().celty_launch_plan(m._h, out, n) == 0
         assert out[min(n, 19):] == [-7] * (20 - min(n, 19)) and out[0] == 148
     assert celty.load().celty_launch_plan(m._h, out, 9) == -1
+
+
+def test_the_tables_leave_room_for_eight_teams():
+    """A block's accumulators and ring slots fill shared memory nearly to the brim on this layer (128 rows per lane, one row
+    part): what the kernel keeps per column may not cost it a team."""
+    M, K = 4096, 11008
+    W = synth.weights(9, M, K)
+    plan = celty.Matrix(W, synth.mask_magnitude(W, 0.5), device="cuda").launch_plan()
+    assert plan["kernel"] == "k_spmspv_direct" and plan["row_parts"] == 1
+    assert plan["teams_per_slab"] == 8 and plan["warp_pairs"] == 1
