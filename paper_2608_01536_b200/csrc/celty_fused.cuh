@@ -279,7 +279,7 @@ __device__ __forceinline__ uint32_t keep_word32(const uint16_t *x, __half2 tau2)
 
 // x = SiLU(gate) * up from the FP32 result of a stacked [gate; up] product (2K values, gate first), rounded to FP16, for
 // the down projection: a kernel of its own ahead of the product's.  Bound by the change of kernels, which the dependent
-// launches hide but for the trip to L2: 1.5 us on top of the product's 12.2 at 4096 x 11008, against 3.4 for shares
+// launches hide but for the trip to L2: 1.2 us on top of the product's 11.6 at 4096 x 11008, against 3.4 for shares
 // evaluated by the product's blocks behind a ticket that all of them wait for and 5.7 for every block evaluating all of x.
 __global__ void __launch_bounds__(256) k_swiglu(const float *__restrict__ gate_up, uint16_t *__restrict__ x, uint16_t *x_copy, int K)
 {
@@ -301,8 +301,8 @@ __global__ void __launch_bounds__(256) k_swiglu(const float *__restrict__ gate_u
 // As a programmatic dependent launch its few small blocks sit beside the product's while that runs, and what is left
 // of the step is one trip to L2 for y after the product's last block is gone.  As the end of the product's own launch
 // it needed a second ticket of all blocks, a poll of it and a block barrier on either side, and the larger build of
-// the streaming loop: 4.3 us on top of the product at 11008 x 4096 with the FP16 copy; 1.4 us this way (12.3 us of device
-// time, the plain product 10.9).
+// the streaming loop: 4.3 us on top of the product at 11008 x 4096 with the FP16 copy; 1.1 us this way (12.4 us of device
+// time, the plain product 11.3).
 struct EpilogueArgs {
     const float *y;
     int M, kind;
