@@ -415,9 +415,9 @@ int celty_last_status(celty_matrix *m, celty_stream_t stream);
  *            the default one (bulk reduce-add merge, no clusters), for which the library otherwise uses smaller
  *            builds without the other options' code (same results; the smaller builds are faster).  With 128 or 256 the
  *            blocks always share a ranked list of the survivors; by default a layer of at most 128 columns per block has
- *            its columns dealt to the blocks whatever x is, in runs of two.  That takes 5 to 20 % less time on layers of up
+ *            its columns dealt to the blocks whatever x is, in runs of two.  That takes 5 to 23 % less time on layers of up
  *            to 75 columns per block, whether or not the survivors lie together in x (zeroed heads, one stretch), and
- *            between 16 % less and 3 % more on layers of 84 to 128.
+ *            between 18 % less and 3 % more on layers of 84 to 128.
  *   groups   fused kernel: warp teams per slab working on different columns (each has an accumulator)
  *   depth    fused kernel: bulk copies each team keeps in flight (ring slots)
  *   cluster  fused kernel, bulk reduce-add merge: thread blocks per cluster (1, 2 or 4); the blocks of a
