@@ -5,55 +5,41 @@
 // What bounds a call on such a layer is a chain of dependent steps, and in k_spmspv_fused the longest part of it is the way
 // from x to the first copy: threshold all of x, rank the survivors, cut the list into equal shares, look the shares up,
 // 4 100 cycles.  Here columns are dealt to blocks whatever x is (direct_column): runs of two neighbouring columns go round
-// the blocks of a row part, and every round starts three blocks further on.  Every streaming
-// warp loads the activations of all the block's columns, one column per lane and chunk of 32; ballots tell each lane the place
-// of its column among the block's survivors, and survivor i goes to team i mod G.  The lane that holds one of its team's
-// columns notes it, and starts the copy itself if it is one of the first; the sub-block offsets were loaded while the
-// previous kernel drained.  Neither a barrier nor a look-up lies between x and the first copy, 1 400 cycles.  The
+// the blocks of a row part, and every round starts three blocks further on.  If each block streamed the survivors of its own
+// columns, the busiest block, which sets the time, would have a quarter more than the mean (4096 x 4096 at 50 %: 35 columns, mean
+// 28).  So up to 16 neighbouring blocks form a group (direct_groups), whose warps hold the group's columns, one per lane: every
+// block of a group thresholds the same up to 512 activations, and takes every size-th survivor (direct_taker; busiest block 31
+// columns).  The lane that holds one of the block's columns takes the next place among the block's items, notes the column, and
+// starts its copy itself if it is one of a team's first; the sub-block offset was loaded while the previous kernel drained.
+// Neither a block barrier nor a look-up lies between x and the first copy.  The
 // accumulators, which no offset window needs before the first copies here, are cleared while the previous kernel drains as
 // well (a tenth of a call's time at 4096 x 4096: cleared under the first copies they held these up).
 //
-// What it costs is balance: the survivors per block differ as they fall, sqrt((1 - d) / (d n)) of n columns at density d,
-// where the ranked list is even to one column.  Device time with 50 % of the weights, in us, mean over 16 draws of
-// independent survivors, ranked -> this kernel, by columns per block:
-//    14 (1024 x 1024, d = 0.1 / 0.5)              3.74 -> 3.30, 3.80 -> 3.30
-//    56 (4096 x 4096, 0.1 / 0.3 / 0.5 / 0.7)      4.82 -> 3.95, 6.32 -> 5.29, 7.79 -> 6.89, 8.65 -> 7.94
-//    70 (5120 x 5120, 0.3 / 0.5)                  7.27 -> 6.64, 9.29 -> 8.60
-//    75 (4096 x 11008, 0.1 / 0.5 / 0.7)           7.70 -> 5.92, 12.26 -> 11.64, 14.36 -> 13.64
-//    84 (11008 x 4096, 0.1 / 0.5 / 0.7)           6.92 -> 5.64, 11.63 -> 11.39, 14.19 -> 13.37
-//   111 (14336 x 4096, 0.1 / 0.3 / 0.5 / 0.7)     7.01 -> 5.91, 9.87 -> 9.38, 12.86 -> 12.82, 15.64 -> 15.45
-//   111 (8192 x 8192, 0.1 / 0.3 / 0.5 / 0.7)      7.68 -> 6.43, 10.77 -> 10.91, 14.26 -> 14.63, 17.58 -> 17.56
-// and with a build for six chunks
-//   138 (8192 x 10240, 0.1 / 0.3 / 0.5 / 0.7)     8.06 -> 7.20, 12.59 -> 12.77, 16.40 -> 16.77, 20.54 -> 20.66
-//   139 (13824 x 5120, 0.1 / 0.5 / 0.7)           7.09 -> 6.61, 14.60 -> 14.60, 18.18 -> 17.87
-//   187 (5120 x 13824, 0.1 / 0.5 / 0.7)           7.29 -> 6.41, 15.42 -> 14.39, 18.62 -> 17.77
-// so the line, four chunks, lies where the first layer is slower from 30 % on; it gives away what other shapes would gain beyond.
-// Survivors that lie together in x are shared about as evenly as independent ones.  Half of the 128-column heads zeroed,
-// ranked / runs of 32 columns / of 8 / of 4 / of two:   4096 x 4096 7.7 / 8.5 / 7.2 / 6.9 / 6.6;   4096 x 11008 12.2 / 15.2 / 15.7 /
-// 12.2 / 11.5;   8192 x 8192 14.3 / 18.6 / 15.8 / 14.9 / 13.9.  Single columns are no more even, and loads of x that touch a
-// sector per column cost 1 to 6 %.  Independent survivors take 1 to 3 % more with runs of two than with runs of 32 on layers
-// of 84 columns per block and more (8192 x 8192 at 10 %: 4 %), whose blocks now reach over all of a large image, and 2 to 6 % less
-// below.  One warp per chunk that shares its ballot and its activations with the others through shared memory behind a barrier,
-// or the two warps of a pair half of the chunks each: 0 to 2 % slower.
-// Groups of 2 to 32 blocks that share their columns' survivors evenly, ranked
-// shares of the columns beyond a fixed core under the streaming: both slower (more code and loads on the way to the first
-// copy, or a streaming loop that the compiler schedules worse).  A list is shared evenly whatever its length; the second
+// What is left of imbalance is the difference between groups.  Device time with 50 % of the weights, in us, k_spmspv_fused / blocks with columns of their
+// own / this kernel, by columns per block (mean of 6 draws; the first figure of 16):
+//    14 (1024 x 1024, d = 0.5)              3.80 / 3.29 / 3.30
+//    56 (4096 x 4096, 0.1 / 0.5 / 0.7)      4.82 / 3.94 / 3.86, 7.79 / 6.24 / 5.80, 8.65 / 7.82 / 7.27
+//    70 (5120 x 5120, 0.4)                  7.38 -> 6.58
+//    75 (4096 x 11008, 0.5)                 12.26 / 11.80 / 10.91
+//    84 (11008 x 4096, 0.1 / 0.5)           6.92 / 5.63 / 5.22, 11.63 / 11.43 / 10.68
+//   111 (14336 x 4096, 0.5)                 12.86 / 12.97 / 12.19
+//   111 (8192 x 8192, 0.5)                  14.26 / 14.80 / 13.57
+// The line, 128 columns per block, was drawn before there were groups, where blocks with columns of their own lost to k_spmspv_fused.
+// Runs of two, so that survivors that lie together in x (zeroed heads of an attention output) are shared about as evenly as independent ones.
+// A list is shared evenly whatever its length; the second
 // product of the 5504 x 2048 MLP chain gains 1.9 of 15.4 us from this kernel.
 //
-// Roles of a block's warps: the first ones stream (a2 - a4; with pairs warps t and t + 8 for team t), the next make the
-// survivor list that the API reports, in a few blocks; the last clears the block's share of y, takes its ticket, waits
+// Roles of a block's warps: the first ones threshold the group's columns and stream (a2 - a4; with pairs warps t and t + 8 for team t), the
+// next make the survivor list that the API reports, in a few blocks; the last clears the block's share of y, takes its ticket, waits
 // for the others' and works out where the block's row segments go.
 constexpr int kDirectHelpers = 3;        // at least; 20 warps leave a thread 96 registers
 constexpr int kDirectThreads = 32 * (16 + kDirectHelpers + 1);
-static_assert(kDirectChunks <= kDirectHelpers + 1, "a thread of the warps that do not stream for each of a block's columns");
 
 // kPairs: two warps per team that take turns at its accumulator; kBatch: one launch for several vectors
-// (FusedParams::ldx); kChunks: chunks of 32 columns that the block's columns fit in, 2 or 4; 0: the
-// survivors come as a list (FusedParams::list_count), in equal shares for all teams.
-template <bool kPairs, bool kBatch, int kChunks>
-__global__ void __launch_bounds__(kDirectThreads, 1) k_spmspv_direct(const FusedParams p)
+// (DirectParams::ldx); kList: the survivors come as a list (DirectParams::list), in equal shares for all teams.
+template <bool kPairs, bool kBatch, bool kList>
+__global__ void __launch_bounds__(kDirectThreads, 1) k_spmspv_direct(const DirectParams p)
 {
-    constexpr bool kList = kChunks == 0;
     const uint16_t *const x = kBatch ? p.x + (size_t)blockIdx.y * p.ldx : p.x;
     float *const y = kBatch ? p.y + (size_t)blockIdx.y * p.ldy : p.y;
     uint32_t *const tickets = kBatch ? p.tickets + blockIdx.y : p.tickets;
@@ -65,17 +51,16 @@ __global__ void __launch_bounds__(kDirectThreads, 1) k_spmspv_direct(const Fused
     const int G = p.G;
     constexpr int pp = kPairs ? 1 : 0, stride = 1 + pp;
     const bool streams = kPairs ? (warp & 7) < G && warp < 16 : warp < G;
-    const int first_helper = kPairs ? 16 : G, helpers = nwarps - 1 - first_helper;
     const int g = streams ? (kPairs ? (warp & 7) : warp) : 0;     // the team
     const int half = streams && kPairs ? warp >> 3 : 0;           // which of its two warps
     const int Dw = p.D / stride;                                  // ring slots per warp
-    const DirectSmem &lay = p.direct;
-    float *acc = reinterpret_cast<float *>(smem + lay.acc);
+    const DirectSmem &lay = p.lay;
+    float *acc = reinterpret_cast<float *>(smem);
     uint8_t *ring = smem + lay.ring;
     uint64_t *bars = reinterpret_cast<uint64_t *>(smem + lay.bars);
     uint2 *items = reinterpret_cast<uint2 *>(smem + lay.items);   // [team][cap] {offset/16, units of 16 bytes << 16 | x bits}
     int *zero_group = reinterpret_cast<int *>(smem + lay.zero);
-    uint2 *place = reinterpret_cast<uint2 *>(smem + lay.place);
+    int *taken = reinterpret_cast<int *>(smem + lay.taken);       // survivors that the block has taken
     uint32_t *kbw = reinterpret_cast<uint32_t *>(smem + lay.keep);
     volatile int *flags = reinterpret_cast<volatile int *>(smem + lay.flag);     // [G] a warp of the team gave up
 
@@ -83,32 +68,24 @@ __global__ void __launch_bounds__(kDirectThreads, 1) k_spmspv_direct(const Fused
     const int per_part = idiv_small(gridDim.x, p.P), kslice = idiv_small(blockIdx.x, p.P), s = blockIdx.x - kslice * p.P;
     const bool long_part = s < (int)gridDim.x - per_part * p.P;
     const int nK = per_part + (long_part ? 1 : 0);
-    const uint32_t g_inv = (uint32_t)idiv_small(65535 + G, G);    // i / G = i * g_inv >> 16 for i < 4096
     const float nK_inv = __fdividef(1.f, (float)nK);
-    int column[kChunks + 1];                                  // the lane's columns of the block's (K or more: none)
-#pragma unroll
-    for (int c = 0; c < kChunks; ++c) column[c] = direct_column(32 * c + lane, kslice, nK, nK_inv);
+    const DirectGroup group = kList ? DirectGroup{} : direct_group(kslice, long_part ? p.sizes[1] : p.sizes[0]);
+    const int rankers = kList ? 0 : p.rankers;                    // warps that rank the group's columns
+    const int takers = kPairs ? 16 : max(rankers, G);             // these and those that stream: they meet at barrier 15
+    const int first_helper = takers, helpers = nwarps - 1 - first_helper;
+    const int column = !kList && warp < rankers ? direct_held(tid, group, nK, nK_inv) : p.K;     // (K or more: none)
 
     // Programmatic dependent launch: see k_spmspv_fused.
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    // {offset/16, units of 16 bytes} of the block's columns' sub-blocks: once per block, by the last warps, which do not stream
-    // (each streaming warp for itself, in registers: 0.05 to 0.3 us slower, their loads touch a sector per run of columns).
-    // The streaming warps meet them at barrier 15, when x is on its way (at the barrier of all warps below, ahead of the wait for
-    // the previous kernel: 1024 x 1024 3.34 us instead of 3.30, 4096 x 4096 6.93 instead of 6.87).
-    const int own = tid - (nthreads - 32 * kDirectChunks), own_column = direct_column(max(own, 0), kslice, nK, nK_inv);
-    const bool owns = own >= 0 && own < 32 * kChunks && own_column < p.K;
-    uint2 own_place = make_uint2(0u, 0u);
+    uint32_t place0 = 0, place1 = 0;                              // offset/16 of the column's sub-block, and of the next one
     auto load_place = [&]() {
-        if (!owns) return;
-        own_place.x = p.meta[(size_t)own_column * p.S + s];
-        own_place.y = p.meta[(size_t)own_column * p.S + s + 1];
+        if (column >= p.K) return;
+        place0 = p.meta[(size_t)column * p.S + s];
+        place1 = p.meta[(size_t)column * p.S + s + 1];
     };
-    auto give_place = [&]() {
-        if (owns) place[own] = make_uint2(own_place.x, own_place.y - own_place.x);
-        asm volatile("bar.arrive 15, %0;" ::"r"(nthreads) : "memory");
-    };
-    if (!kList && p.image_early) load_place();
+    if (p.image_early) load_place();
     if (tid < 4) zero_group[tid] = 0;
+    if (tid == 0) *taken = 0;
     if (tid < G) const_cast<int *>(flags)[tid] = 0;
     if (streams && lane == 0) {
 #pragma unroll 1
@@ -122,12 +99,32 @@ __global__ void __launch_bounds__(kDirectThreads, 1) k_spmspv_direct(const Fused
         for (int i = half * 32 + lane; i < slab_words / 4; i += 32 * stride) slab4[i] = make_float4(0.f, 0.f, 0.f, 0.f);
     }
     __syncthreads();
-    if (!kList && p.image_early && !streams) give_place();
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    if (!kList && !p.image_early && !streams) {
-        load_place();
-        give_place();
+    if (!p.image_early) load_place();
+
+    const uint32_t lt_mask = (1u << lane) - 1u;
+    // The lane has found item k of team `to`: it notes it, and starts its copy if it is one of the first.  (Copies that an
+    // elected lane starts when all are found: 0.2 us slower at 4096 x 4096.)
+    auto found = [&](int to, int k, const uint2 at, uint32_t xb) {
+        (items + (size_t)to * p.cap)[k] = make_uint2(at.x, at.y << 16 | xb);
+        if (k >= p.D) return;
+        const int slot = to * p.D + (kPairs ? (k & 1) * Dw + (k >> 1) : k);          // a pair's warps take turns
+        bulk_load(smem_u32(ring + (size_t)slot * p.slot_bytes), p.stream + (size_t)at.x * 16, at.y * 16u, smem_u32(&bars[slot]));
+    };
+    // The group's survivors are dealt to its blocks, a ranking warp's one after the other, beginning with a block of the warp's
+    // own: what a block has differs by one per warp at most, and no warp has to know the others' counts.  In the block they go
+    // to the teams in the order in which they are found.  (Exact ranks through shared memory, a barrier and two reductions:
+    // 4096 x 4096 6.00 us instead of 5.97, 4096 x 11008 11.1 instead of 10.9.)
+    if (warp < rankers) {
+        const uint32_t xb = column < p.K ? x[column] : 0u;
+        const bool keep = column < p.K && !(fabsf(__half2float(__ushort_as_half((uint16_t)xb))) <= p.tau);
+        const uint32_t kept = __ballot_sync(kFull, keep);
+        if (keep && direct_taker(__popc(kept & lt_mask), warp, p.rankers_inv, group) == kslice - group.first) {
+            const int i = atomicAdd(taken, 1), k = i * (int)p.G_inv >> 16;
+            found(i - k * G, k, make_uint2(place0, place1 - place0), xb);
+        }
     }
+    if (!kList && warp < takers) asm volatile("bar.sync 15, %0;" ::"r"(32 * takers) : "memory");       // the items are there
 
     // The list that the API reports is made by a few blocks, eight words of x each (2048 x 5504 with 16 each: 0.3 us slower).
     const int nfull = p.K >> 5, nwords = (p.K + 31) >> 5;
@@ -143,45 +140,25 @@ __global__ void __launch_bounds__(kDirectThreads, 1) k_spmspv_direct(const Fused
             if (kPairs) asm volatile("bar.sync %0, 64;" ::"r"(2 + g) : "memory");
             else __syncwarp();
         };
-        // The lane has found item k of the team: it notes it, and starts its copy if it is one of the first.  (Copies that an
-        // elected lane starts when all chunks are through: 0.2 us slower at 4096 x 4096.)
-        auto found = [&](int k, const uint2 at, uint32_t xb) {
-            if (kPairs && (k & 1) != half) return;
-            mine[k] = make_uint2(at.x, at.y << 16 | xb);
-            const int slot = k >> pp;
-            if (slot < Dw) bulk_load(ring0 + (uint32_t)(slot * p.slot_bytes), p.stream + (size_t)at.x * 16, at.y * 16u, bar0 + 8u * slot);
-        };
-        const uint32_t lt_mask = (1u << lane) - 1u;
         int cnt = 0;
         if (kList) {
             const int n = __shfl_sync(kFull, max(0, min(p.K, __ldcg(p.list_count))), 0);
             if (blockIdx.x == 0 && tid == 0) *p.count = n;
             const int units = nK * G, u = kslice * G + g;
-            const uint32_t units_inv = long_part ? p.units_inv_long : p.units_inv;
+            const uint32_t units_inv = long_part ? p.list.units_inv_long : p.list.units_inv;
             uint32_t each = __umulhi((uint32_t)n, units_inv), extra = (uint32_t)n - each * (uint32_t)units;
             if (extra >= (uint32_t)units) { ++each; extra -= (uint32_t)units; }
             const int r0 = u * (int)each + min(u, (int)extra);
             cnt = (int)each + (u < (int)extra ? 1 : 0);
             for (int k = half + stride * lane; k < cnt; k += stride * 32) {
-                const int j = min(max(__ldcg(p.list_idx + r0 + k), 0), p.K - 1);
-                const uint32_t xb = __ldcg(p.list_val + r0 + k);
+                const int j = min(max(__ldcg(p.list.idx + r0 + k), 0), p.K - 1);
+                const uint32_t xb = __ldcg(p.x + r0 + k);
                 const uint32_t at = p.meta[(size_t)j * p.S + s];
-                found(k, make_uint2(at, p.meta[(size_t)j * p.S + s + 1] - at), xb);
+                found(g, k, make_uint2(at, p.meta[(size_t)j * p.S + s + 1] - at), xb);
             }
         } else {
-            uint32_t xb[kChunks + 1];
-#pragma unroll
-            for (int c = 0; c < kChunks; ++c) xb[c] = column[c] < p.K ? x[column[c]] : 0u;
-            asm volatile("bar.sync 15, %0;" ::"r"(nthreads) : "memory");                // the places are there
-            uint32_t n = 0;
-#pragma unroll
-            for (int c = 0; c < kChunks; ++c) {
-                const bool keep = column[c] < p.K && !(fabsf(__half2float(__ushort_as_half((uint16_t)xb[c]))) <= p.tau);
-                const uint32_t kept = __ballot_sync(kFull, keep), i = n + __popc(kept & lt_mask), k = i * g_inv >> 16;
-                if (keep && (int)(i - k * G) == g) found((int)k, place[32 * c + lane], xb[c]);
-                n += __popc(kept);
-            }
-            cnt = (int)n > g ? idiv_small((int)n - g + G - 1, G) : 0;
+            const int n = *taken;
+            cnt = n > g ? idiv_small(n - g + G - 1, G) : 0;
         }
         uint32_t slot = 0, parity = 0, consumed = 0;              // of this warp's Dw slots
         uint32_t issued = (uint32_t)min(Dw, (cnt - half + pp) >> pp), islot = issued == (uint32_t)Dw ? 0 : issued;   // (cnt >= 0, half <= 1)
@@ -190,7 +167,7 @@ __global__ void __launch_bounds__(kDirectThreads, 1) k_spmspv_direct(const Fused
             ++issued;
             if (++islot == (uint32_t)Dw) islot = 0;
         };
-        team_sync();
+        if (kList) team_sync();
         bool failed = false;
         const uint32_t zeros = smem_u32(zero_group), spare_cell = cell0 + (uint32_t)p.R * 128u;
         StepBuf b0, b1;                                           // pipeline registers, live across items

@@ -121,25 +121,22 @@ CELTY_HD inline FusedSmem fused_smem_layout(int R, int K, int teams, int D, int 
 }
 
 // The same for k_spmspv_direct.
-constexpr int kDirectChunks = 4;         // columns of a block, in chunks of 32
-
 struct DirectSmem {
-    uint32_t acc, ring, bars, flag, items, zero, place, keep, total;
+    uint32_t ring, bars, flag, items, zero, taken, keep, total;              // (the accumulators lie at 0)
 };
 
-// columns: of a block, at most (direct_columns); 0: the survivors come as a list
-inline DirectSmem direct_smem_layout(int R, int K, int G, int D, int slot_bytes, int cap, int columns)
+inline DirectSmem direct_smem_layout(int R, int K, int G, int D, int slot_bytes, int cap)
 {
     DirectSmem l;
     uint32_t off = 0;
-    l.acc = off;       off += (uint32_t)G * (R + kTileSlack) * 32 * 4;       // FP32 accumulators, one slab per team
+    off += (uint32_t)G * (R + kTileSlack) * 32 * 4;                          // FP32 accumulators, one slab per team
     l.ring = off;      off += (uint32_t)G * D * slot_bytes;                  // bulk-copy ring slots (multiples of 128 bytes)
     l.bars = off;      off += (uint32_t)G * D * 8;                           // one "full" mbarrier per slot
     l.flag = off;      off += (uint32_t)G * 4;                               // per team: a warp gave up
     off = (off + 15) / 16 * 16;
     l.zero = off;      off += 16;                                            // the all-zero group that idle lanes fetch
     l.items = off;     off += (uint32_t)G * cap * 8;                         // {offset/16, bytes/16 and x} per column of a team
-    l.place = off;     off += (uint32_t)columns * 8;                            // {offset/16, bytes/16} of the block's columns
+    l.taken = off;     off += 16;                                            // survivors that the block has taken
     l.keep = off;      off += (uint32_t)((K + 31) / 32) * 4;                 // one keep bit per activation
     l.total = (off + 15) / 16 * 16;
     return l;
@@ -154,6 +151,70 @@ CELTY_HD inline int direct_column(int i, int b, int nK, float nK_inv)   // nK_in
     const int round = i / kDirectRun, turned = b + round * kDirectTurn;
     const int place = turned - (int)(((float)turned + 0.5f) * nK_inv) * nK;      // modulo nK, exact for turned < 2^14
     return (round * nK + place) * kDirectRun + i % kDirectRun;
+}
+
+// Most columns of a block.
+inline int direct_columns(int64_t K, int blocks_per_part)
+{
+    const int64_t round = (int64_t)kDirectRun * blocks_per_part;
+    return (int)((K + round - 1) / round) * kDirectRun;
+}
+
+// The blocks of a row part form groups, which share the survivors of their columns.  Blocks [0, larger) are in groups of least + 1
+// neighbouring ones, those behind them in groups of least.
+struct DirectSizes { int32_t least, larger; };
+
+struct DirectGroup { int first, size; float size_inv; };          // blocks [first, first + size)
+
+CELTY_HD inline DirectGroup direct_group(int b, const DirectSizes &z)
+{
+    DirectGroup g;
+    const bool more = b < z.larger;
+    g.size = more ? z.least + 1 : z.least;
+    g.size_inv = 1.f / (float)g.size;
+    const int in = more ? b : b - z.larger;
+    g.first = b - in + (int)(((float)in + 0.5f) * g.size_inv) * g.size;
+    return g;
+}
+
+// Column that a group's ranking lane t (32 * warp + lane) holds (K or more: none): the members' first runs, then their next ones.
+CELTY_HD inline int direct_held(int t, const DirectGroup &g, int nK, float nK_inv)
+{
+    const int run = t / kDirectRun, round = (int)(((float)run + 0.5f) * g.size_inv);
+    return direct_column(round * kDirectRun + t % kDirectRun, g.first + run - round * g.size, nK, nK_inv);
+}
+
+// Block of the group (counted from its first) that takes the i-th survivor of ranking warp w: the warps start at evenly spaced ones.
+CELTY_HD inline int direct_taker(int i, int w, float rankers_inv, const DirectGroup &g)
+{
+    const int r = i + (int)(((float)(w * g.size) + 0.5f) * rankers_inv);
+    return r - (int)(((float)r + 0.5f) * g.size_inv) * g.size;
+}
+
+// Groups for a launch of `grid` blocks and P row parts with `warps` warps that can rank, a column per lane: as few as hold
+// all columns.  They even out what a group's blocks have, and every ranking warp is another 32 columns.  Device time with up to
+// 12 or 16 (pairs) ranking warps / 8 / 5 / 2, in us: 4096 x 4096 5.89 / 5.91 / 6.16 / 6.48;  4096 x 11008 10.8 / 10.9 / 10.9 / 11.3;  8192 x 8192
+// 13.5 / 13.6 / 14.2 / 14.2;  with twice or four times the columns per group, two or four per lane: level to 1 % slower, and
+// 6 % / 12 % slower on small layers.
+struct DirectGroups {
+    int rankers;               // warps that rank
+    int most;                  // columns that a block may take
+    DirectSizes sizes[2];      // in row parts with floor(grid / P) blocks, and in those with one more
+};
+
+inline DirectGroups direct_groups(int64_t K, int grid, int P, int warps)
+{
+    DirectGroups g;
+    const int nK = grid / P, columns = direct_columns(K, nK), most = nK + (grid % P ? 1 : 0);
+    const int members = std::max(1, std::min(most, 32 * warps / columns)), groups = (most + members - 1) / members;
+    const int size = (most + groups - 1) / groups;
+    for (int l = 0; l < 2; ++l) {
+        const int least = (nK + l) / groups;
+        g.sizes[l] = DirectSizes{least, (nK + l - least * groups) * (least + 1)};
+    }
+    g.rankers = (size * columns + 31) / 32;
+    g.most = std::min(size * columns, g.rankers * (32 / std::max(1, nK / groups) + 1));
+    return g;
 }
 
 struct FusedParams {
@@ -199,9 +260,45 @@ struct FusedParams {
     const uint16_t *list_val;
     const int32_t *list_count;
     int32_t *ep_count;         // not null: set to zero for the list that k_epilogue appends to after this kernel
-    // k_spmspv_direct
-    DirectSmem direct;         // its shared memory
     int image_early;           // 0: the kernel before this one may be writing the image
+};
+
+// Parameters of k_spmspv_direct, in the order in which a block looks at them: every 64 bytes of parameters that a kernel
+// touches may be a miss of the constant cache on its way.  (As a part of FusedParams, 430 bytes of which a block read here and
+// there: 0.1 to 0.15 us per call, 4096 x 4096 6.01 instead of 5.89.)
+struct DirectParams {
+    const uint32_t *meta;      // as in FusedParams, where nothing else is said
+    int32_t K, S, P, G;
+    union {
+        DirectSizes sizes[2];  // of the groups
+        struct { const int32_t *idx; uint32_t units_inv, units_inv_long; } list;        // list builds
+    };
+    int32_t R, D;
+    float *y;
+    int32_t clear_rows, clear_extra;
+
+    DirectSmem lay;
+    union {
+        struct { int32_t rankers; float rankers_inv; };
+        const int32_t *list_count;
+    };
+    int32_t image_early;
+    float tau;
+    const uint16_t *x;         // list builds: the list's values
+    uint32_t *tickets;
+
+    const uint8_t *stream;
+    uint32_t G_inv;            // i / G = i * G_inv >> 16 for i < 4096
+    int32_t cap, slot_bytes;
+    uint32_t spin_limit;
+    int32_t M, C;
+    int32_t *ep_count;
+
+    int32_t *idx;
+    uint16_t *val;
+    int32_t *count;
+    uint32_t *status;
+    int64_t ldx, ldy;
 };
 
 // Shape of a fused launch (plan_fused).
@@ -210,7 +307,6 @@ struct FusedPlan {
     int window;                // bytes of the offset window where it has a place of its own (several vectors), else -1
     int lean;                  // 0: every option compiled in; 1 / 2: the builds for the default launch (without / with warp pairs)
     int direct;                // 1: k_spmspv_direct
-    int chunks;                // k_spmspv_direct: columns of a block, in chunks of 32
     size_t smem;
 };
 

@@ -445,7 +445,7 @@ __global__ void k_decode_lane(const uint32_t *__restrict__ meta, const uint8_t *
 // asked for), so that steady-state calls make no attribute calls.  The attribute belongs to the kernel,
 // so every entry point that launches a kernel shares that kernel's cache (g_granted_*): two caches for
 // one kernel could disagree about what the runtime currently allows.
-int g_granted_fused[64], g_granted_lean[2][64], g_granted_fused_extras[64], g_granted_lean_extras[2][64], g_granted_batch[2][64], g_granted_direct[7][64], g_granted_column[64], g_granted_lane[64], g_granted_reg[4][64];
+int g_granted_fused[64], g_granted_lean[2][64], g_granted_fused_extras[64], g_granted_lean_extras[2][64], g_granted_batch[2][64], g_granted_direct[6][64], g_granted_column[64], g_granted_lane[64], g_granted_reg[4][64];
 
 template <typename Kernel>
 int ensure_smem(Kernel kernel, size_t bytes, int *granted /* [64], per device */)
@@ -500,18 +500,19 @@ int launch_compact(const void *x, int64_t K, float tau, int32_t *idx, uint16_t *
 
 constexpr int kMostToMix = 48;           // left-over blocks are shared between row parts up to this (fit_clusters)
 
-// Columns that a block of k_spmspv_direct may own.  Its tables are sized by them: with 32 per chunk the 4096 x 11008 layer had
-// room for seven teams instead of eight (from gate and up 13.0 us, with eight 12.8).
-int direct_columns(int64_t K, int blocks_per_part)
+constexpr int kDirectMost = 128;         // columns of a block of k_spmspv_direct (see there)
+
+int direct_threads(int G, int pairs) { return 32 * (pairs ? 16 + kDirectHelpers + 1 : std::max(16, G + kDirectHelpers + 1)); }
+
+DirectGroups direct_groups(const celty_matrix *m, int grid, int P, int threads)
 {
-    const int64_t round = (int64_t)kDirectRun * blocks_per_part;
-    return (int)((K + round - 1) / round) * kDirectRun;
+    return celty::direct_groups(m->K, grid, P, threads / 32 - 1 - kDirectHelpers);
 }
 
 // Columns that a team of k_spmspv_direct may get: of the block's, or of an even split of a list over the teams of a row part.
-int direct_cap(int64_t K, int blocks_per_part, int G, bool list)
+int direct_cap(const celty_matrix *m, int grid, int P, int G, int pairs, bool list)
 {
-    return list ? (int)(K / ((int64_t)blocks_per_part * G) + 1) : (direct_columns(K, blocks_per_part) + G - 1) / G;
+    return list ? (int)(m->K / ((int64_t)(grid / P) * G) + 1) : (direct_groups(m, grid, P, direct_threads(G, pairs)).most + G - 1) / G;
 }
 
 // Shape of the fused launch: P row parts of Sc slabs, G teams per slab (teams = G * Sc warps, one accumulator
@@ -538,16 +539,13 @@ int plan_fused(const celty_matrix *m, const LaunchKnobs &knobs, const DeviceInfo
     // product from a list, but where left-over blocks are shared between row parts, and where a team's items would take
     // much of the shared memory.
     const int per_part = pl.grid / pl.P;
-    const int64_t chunks = ((m->K + per_part - 1) / per_part + 31) / 32;
     const int left = pl.grid % pl.P;
     const bool mixes = left > 0 && pl.P % left == 0 && (int64_t)(pl.P / left) * per_part <= kMostToMix;    // see fit_clusters
     pl.direct = reg_rows == 0 && knobs.merge != 0 && knobs.cluster <= 1 && knobs.lean != 0 && knobs.mix <= 0 && pl.Sc == 1 &&
-                (list ? !mixes && m->K / per_part < 4096 : chunks <= kDirectChunks);
-    pl.chunks = list ? 0 : (int)chunks;
+                (list ? !mixes && m->K / per_part < 4096 : (m->K + per_part - 1) / per_part <= kDirectMost);
     auto smem_bytes = [&](int G, int D) {
         if (!pl.direct) return fused_smem_bytes(m->R, (int)m->K, G, pl.Sc, D, pl.slot_bytes, pl.cap);
-        return (size_t)direct_smem_layout(m->R, (int)m->K, G, D, pl.slot_bytes, direct_cap(m->K, per_part, G, list),
-                                          list ? 0 : direct_columns(m->K, per_part)).total;
+        return (size_t)direct_smem_layout(m->R, (int)m->K, G, D, pl.slot_bytes, direct_cap(m, pl.grid, pl.P, G, pl.pp, list)).total;
     };
     auto fit = [&](int pairs) {
         pl.pp = pairs;
@@ -607,7 +605,7 @@ int plan_fused(const celty_matrix *m, const LaunchKnobs &knobs, const DeviceInfo
     }
     if (pl.G == 0) return CELTY_EINVAL;
     pl.threads = reg_rows > 0 ? 256 : pl.pp || pl.G * pl.Sc > 15 ? 544 : 512;   // the last warp does not stream
-    if (pl.direct) pl.threads = 32 * (pl.pp ? 16 + kDirectHelpers + 1 : std::max(16, pl.G + kDirectHelpers + 1));
+    if (pl.direct) pl.threads = direct_threads(pl.G, pl.pp);
     pl.smem = smem_bytes(pl.G, pl.D);
     pl.window = -1;
     if (vectors > 1 && !pl.direct) {
@@ -616,7 +614,7 @@ int plan_fused(const celty_matrix *m, const LaunchKnobs &knobs, const DeviceInfo
         pl.window = (int)(std::min(wanted, budget - pl.smem) / 128 * 128);
         pl.smem += (size_t)pl.window;
     }
-    if (pl.direct) pl.cap = direct_cap(m->K, per_part, pl.G, list);
+    if (pl.direct) pl.cap = direct_cap(m, pl.grid, pl.P, pl.G, pl.pp, list);
     pl.merge = (knobs.merge >= 0 ? knobs.merge : 1);
     // Clusters (bulk reduce-add merge only, on request): as long as the grid is made of whole clusters, every row
     // part gets at least one, and the device can hold them all at once.
@@ -724,10 +722,7 @@ FusedParams plan_params(const celty_matrix *m, const LaunchKnobs &knobs, const F
     }
     fp.merge = plan.merge;
     fp.image_early = 1;
-    if (plan.direct)
-        fp.direct = direct_smem_layout(m->R, (int)m->K, plan.G, plan.D, plan.slot_bytes, plan.cap,
-                                       plan.chunks ? direct_columns(m->K, plan.grid / plan.P) : 0);
-    else
+    if (!plan.direct)
         fp.lay = fused_smem_layout(m->R, (int)m->K, plan.G * plan.Sc, plan.D, plan.slot_bytes, plan.cap, std::max(0, plan.window));
     fp.clear_rows = (int)(m->M / plan.grid);
     fp.clear_extra = (int)(m->M % plan.grid);
@@ -760,8 +755,9 @@ int prepared_launch(celty_matrix *m, const DeviceInfo &di, int vectors, bool lis
 
 // Programmatic dependent launch: the kernel may be scheduled while the previous kernel of the stream drains; it
 // waits for that kernel (griddepcontrol.wait) before it reads or writes anything of the call.
-int launch_fused(void (*kernel)(FusedParams), int *granted, const LaunchKnobs &knobs, const FusedPlan &plan, int vectors,
-                 const FusedParams &fp, cudaStream_t st)
+template <typename Params>
+int launch_fused(void (*kernel)(Params), int *granted, const LaunchKnobs &knobs, const FusedPlan &plan, int vectors,
+                 const Params &fp, cudaStream_t st)
 {
     const int rc = ensure_smem(kernel, plan.smem, granted);
     if (rc) return rc;
@@ -791,20 +787,40 @@ int launch_fused(void (*kernel)(FusedParams), int *granted, const LaunchKnobs &k
 }
 
 // The build of k_spmspv_direct for a plan, and its shared-memory limit.
-struct DirectBuild { void (*kernel)(FusedParams); int *granted; };
+struct DirectBuild { void (*kernel)(DirectParams); int *granted; };
 
 DirectBuild direct_build(const FusedPlan &plan, bool batch, bool list)
 {
-    if (list) return plan.pp ? DirectBuild{k_spmspv_direct<true, false, 0>, g_granted_direct[0]} : DirectBuild{k_spmspv_direct<false, false, 0>, g_granted_direct[1]};
-    if (batch) return plan.pp ? DirectBuild{k_spmspv_direct<true, true, 4>, g_granted_direct[2]} : DirectBuild{k_spmspv_direct<false, true, 4>, g_granted_direct[3]};
-    if (plan.pp) return DirectBuild{k_spmspv_direct<true, false, 4>, g_granted_direct[4]};
-    return plan.chunks > 2 ? DirectBuild{k_spmspv_direct<false, false, 4>, g_granted_direct[5]} : DirectBuild{k_spmspv_direct<false, false, 2>, g_granted_direct[6]};
+    if (list) return plan.pp ? DirectBuild{k_spmspv_direct<true, false, true>, g_granted_direct[0]} : DirectBuild{k_spmspv_direct<false, false, true>, g_granted_direct[1]};
+    if (batch) return plan.pp ? DirectBuild{k_spmspv_direct<true, true, false>, g_granted_direct[2]} : DirectBuild{k_spmspv_direct<false, true, false>, g_granted_direct[3]};
+    return plan.pp ? DirectBuild{k_spmspv_direct<true, false, false>, g_granted_direct[4]} : DirectBuild{k_spmspv_direct<false, false, false>, g_granted_direct[5]};
 }
 
-int launch_direct(const LaunchKnobs &knobs, const FusedPlan &plan, int vectors, bool list, const FusedParams &fp, cudaStream_t st)
+int launch_direct(const celty_matrix *m, const LaunchKnobs &knobs, const FusedPlan &plan, int vectors, bool list, const FusedParams &fp, cudaStream_t st)
 {
     const DirectBuild b = direct_build(plan, vectors > 1, list);
-    return launch_fused(b.kernel, b.granted, knobs, plan, vectors, fp, st);
+    DirectParams p{};
+    p.meta = fp.meta; p.stream = fp.stream;
+    p.K = fp.K; p.S = fp.S; p.P = fp.P; p.G = fp.G; p.R = fp.R; p.D = fp.D; p.M = fp.M; p.C = fp.C;
+    p.lay = direct_smem_layout(fp.R, fp.K, plan.G, plan.D, plan.slot_bytes, plan.cap);
+    p.image_early = fp.image_early;
+    p.x = fp.x; p.ldx = fp.ldx; p.tau = fp.tau;
+    p.G_inv = (65535u + plan.G) / plan.G;
+    p.cap = plan.cap; p.slot_bytes = plan.slot_bytes;
+    p.y = fp.y; p.ldy = fp.ldy; p.tickets = fp.tickets;
+    p.clear_rows = fp.clear_rows; p.clear_extra = fp.clear_extra; p.spin_limit = fp.spin_limit;
+    p.ep_count = fp.ep_count;
+    p.idx = fp.idx; p.val = fp.val; p.count = fp.count; p.status = fp.status;
+    if (list) {
+        p.list.idx = fp.list_idx; p.x = fp.list_val; p.list_count = fp.list_count;
+        p.list.units_inv = fp.units_inv; p.list.units_inv_long = fp.units_inv_long;
+    } else {
+        const DirectGroups g = direct_groups(m, plan.grid, plan.P, plan.threads);
+        p.sizes[0] = g.sizes[0]; p.sizes[1] = g.sizes[1];
+        p.rankers = g.rankers;
+        p.rankers_inv = 1.f / (float)g.rankers;
+    }
+    return launch_fused(b.kernel, b.granted, knobs, plan, vectors, p, st);
 }
 
 // The tickets of launches that serve `vectors` vectors each (one ticket per vector) in the status words.
@@ -962,7 +978,7 @@ int run_product(celty_matrix *m, const void *x_dev, float tau, const ListInput *
             m->last_merge = plan.merge;
         }
         if (plan.direct)
-            rc = launch_direct(*m, plan, 1, list != nullptr, fp, st);
+            rc = launch_direct(m, *m, plan, 1, list != nullptr, fp, st);
         else if (list)                                           // the list input has builds of its own
             rc = plan.lean == 2 ? launch_fused(k_spmspv_fused<true, 0, 2>, g_granted_lean_extras[1], *m, plan, 1, fp, st)
                : plan.lean == 1 ? launch_fused(k_spmspv_fused<true, 0, 1>, g_granted_lean_extras[0], *m, plan, 1, fp, st)
@@ -1150,7 +1166,7 @@ extern "C" int celty_spmspv_static(const celty_matrix *m, const void *image_dev,
                             : ensure_smem(k_spmspv_fused<false, 0, 1>, plan.smem, g_granted_lean[0]);
         if (rc == CELTY_OK) rc = launch_clear(y, m->M, st);
         if (rc) return rc;
-        if (plan.direct) return launch_direct(knobs, plan, 1, false, fp, st);
+        if (plan.direct) return launch_direct(m, knobs, plan, 1, false, fp, st);
         return plan.lean == 2 ? launch_fused(k_spmspv_fused<false, 0, 2>, g_granted_lean[1], knobs, plan, 1, fp, st)
                               : launch_fused(k_spmspv_fused<false, 0, 1>, g_granted_lean[0], knobs, plan, 1, fp, st);
     }
@@ -1230,7 +1246,7 @@ int run_batch(celty_matrix *m, const uint16_t *x, int64_t ldx, int N, float tau,
             m->last_batch_grid[v] = plan.grid;
         }
         if (plan.direct)
-            rc = launch_direct(*m, plan, v, false, fp, st);
+            rc = launch_direct(m, *m, plan, v, false, fp, st);
         else
             rc = plan.lean == 2 ? launch_fused(k_spmspv_fused<false, 0, 2, true>, g_granted_batch[1], *m, plan, v, fp, st)
                             : launch_fused(k_spmspv_fused<false, 0, 1, true>, g_granted_batch[0], *m, plan, v, fp, st);
