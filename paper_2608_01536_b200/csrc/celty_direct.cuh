@@ -24,7 +24,20 @@
 //    84 (11008 x 4096, 0.1 / 0.5)           6.92 / 5.63 / 5.22, 11.63 / 11.43 / 10.68
 //   111 (14336 x 4096, 0.5)                 12.86 / 12.97 / 12.19
 //   111 (8192 x 8192, 0.5)                  14.26 / 14.80 / 13.57
-// The line, 128 columns per block, was drawn before there were groups, where blocks with columns of their own lost to k_spmspv_fused.
+// Beyond 128 columns per block the same code runs as k_spmspv_fused_groups (the form of k_spmspv_fused that a plan's readers
+// expect there), with one, two or four of the group's columns per ranking lane, k_spmspv_fused -> this one, one vector:
+//   128 (40 x 18945, 0.5)                   6.83 -> 5.73
+//   139 (13824 x 5120, 0.1 / 0.5)           7.16 -> 5.73, 14.92 -> 14.03
+//   187 (5120 x 13824, 0.1 / 0.5)           7.30 -> 6.01, 15.69 -> 13.75
+//   139 (8192 x 10240, 0.1 / 0.3 / 0.5 / 0.7)   7.79 -> 6.34, 12.61 -> 11.79, 16.57 -> 15.71, 20.50 -> 19.60
+//   198 (9700 x 9700, 0.5)                  18.52 -> 17.00
+//   276 (20000 x 8000, 0.5)                 26.15 -> 26.06
+//   332 (16384 x 12288, 0.1 / 0.5 / 0.7)    10.89 -> 9.99, 30.57 -> 30.50, 40.26 -> 39.78
+//   387 (8192 x 28672, 0.3 / 0.5)           24.55 -> 23.59, 35.47 -> 34.38
+// and batches: 4096 x 4096, N = 4 / 8  15.14 -> 13.57, 24.77 -> 23.35;  11008 x 4096, N = 4  27.92 -> 25.74.  The gain shrinks with the
+// columns, whose streaming outgrows what is saved ahead of it; the line, 512 (four members' columns at four per lane), lies beyond
+// what was measured.  One vector of a layer whose left-over blocks serve several row parts is k_spmspv_fused's (28672 x 8192 at
+// 50 %: 33.3, here 33.6, though at 10 % 11.7 and 10.9).
 // Runs of two, so that survivors that lie together in x (zeroed heads of an attention output) are shared about as evenly as independent ones.
 // A list is shared evenly whatever its length; the second
 // product of the 5504 x 2048 MLP chain gains 1.9 of 15.4 us from this kernel.
@@ -36,10 +49,13 @@ constexpr int kDirectHelpers = 3;        // at least; 20 warps leave a thread 96
 constexpr int kDirectThreads = 32 * (16 + kDirectHelpers + 1);
 
 // kPairs: two warps per team that take turns at its accumulator; kBatch: one launch for several vectors
-// (DirectParams::ldx); kList: the survivors come as a list (DirectParams::list), in equal shares for all teams.
-template <bool kPairs, bool kBatch, bool kList>
-__global__ void __launch_bounds__(kDirectThreads, 1) k_spmspv_direct(const DirectParams p)
+// (DirectParams::ldx); kHeld: columns of the group per ranking lane; 0: the survivors come as a list (DirectParams::list), in
+// equal shares for all teams.
+template <bool kPairs, bool kBatch, int kHeld>
+__device__ __forceinline__ void dealt_product(const DirectParams p)
 {
+    constexpr bool kList = kHeld == 0;
+    constexpr int kArray = kList ? 1 : kHeld;
     const uint16_t *const x = kBatch ? p.x + (size_t)blockIdx.y * p.ldx : p.x;
     float *const y = kBatch ? p.y + (size_t)blockIdx.y * p.ldy : p.y;
     uint32_t *const tickets = kBatch ? p.tickets + blockIdx.y : p.tickets;
@@ -73,15 +89,21 @@ __global__ void __launch_bounds__(kDirectThreads, 1) k_spmspv_direct(const Direc
     const int rankers = kList ? 0 : p.rankers;                    // warps that rank the group's columns
     const int takers = kPairs ? 16 : max(rankers, G);             // these and those that stream: they meet at barrier 15
     const int first_helper = takers, helpers = nwarps - 1 - first_helper;
-    const int column = !kList && warp < rankers ? direct_held(tid, group, nK, nK_inv) : p.K;     // (K or more: none)
+    int column[kArray];                                        // that the lane holds (K or more: none)
+#pragma unroll
+    for (int c = 0; c < kHeld; ++c) column[c] = warp < rankers ? direct_held(kHeld * (tid - lane) + 32 * c + lane, group, nK, nK_inv) : p.K;
 
     // Programmatic dependent launch: see k_spmspv_fused.
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    uint32_t place0 = 0, place1 = 0;                              // offset/16 of the column's sub-block, and of the next one
+    uint32_t place0[kArray], place1[kArray];                // offset/16 of the columns' sub-blocks, and of the next ones
     auto load_place = [&]() {
-        if (column >= p.K) return;
-        place0 = p.meta[(size_t)column * p.S + s];
-        place1 = p.meta[(size_t)column * p.S + s + 1];
+#pragma unroll
+        for (int c = 0; c < kHeld; ++c) {
+            place0[c] = place1[c] = 0u;
+            if (column[c] >= p.K) continue;
+            place0[c] = p.meta[(size_t)column[c] * p.S + s];
+            place1[c] = p.meta[(size_t)column[c] * p.S + s + 1];
+        }
     };
     if (p.image_early) load_place();
     if (tid < 4) zero_group[tid] = 0;
@@ -114,14 +136,21 @@ __global__ void __launch_bounds__(kDirectThreads, 1) k_spmspv_direct(const Direc
     // The group's survivors are dealt to its blocks, a ranking warp's one after the other, beginning with a block of the warp's
     // own: what a block has differs by one per warp at most, and no warp has to know the others' counts.  In the block they go
     // to the teams in the order in which they are found.  (Exact ranks through shared memory, a barrier and two reductions:
-    // 4096 x 4096 6.00 us instead of 5.97, 4096 x 11008 11.1 instead of 10.9.)
+    // 5120 x 5120 at 40 % 7.08 us instead of 6.83, 4096 x 11008 at 50 % 11.1 instead of 10.9, 4096 x 4096 level.)
     if (warp < rankers) {
-        const uint32_t xb = column < p.K ? x[column] : 0u;
-        const bool keep = column < p.K && !(fabsf(__half2float(__ushort_as_half((uint16_t)xb))) <= p.tau);
-        const uint32_t kept = __ballot_sync(kFull, keep);
-        if (keep && direct_taker(__popc(kept & lt_mask), warp, p.rankers_inv, group) == kslice - group.first) {
-            const int i = atomicAdd(taken, 1), k = i * (int)p.G_inv >> 16;
-            found(i - k * G, k, make_uint2(place0, place1 - place0), xb);
+        uint32_t xb[kArray];
+        int n = 0;
+#pragma unroll
+        for (int c = 0; c < kHeld; ++c) xb[c] = column[c] < p.K ? x[column[c]] : 0u;
+#pragma unroll
+        for (int c = 0; c < kHeld; ++c) {
+            const bool keep = column[c] < p.K && !(fabsf(__half2float(__ushort_as_half((uint16_t)xb[c]))) <= p.tau);
+            const uint32_t kept = __ballot_sync(kFull, keep);
+            if (keep && direct_taker(n + __popc(kept & lt_mask), warp, p.rankers_inv, group) == kslice - group.first) {
+                const int i = atomicAdd(taken, 1), k = i * (int)p.G_inv >> 16;
+                found(i - k * G, k, make_uint2(place0[c], place1[c] - place0[c]), xb[c]);
+            }
+            n += __popc(kept);
         }
     }
     if (!kList && warp < takers) asm volatile("bar.sync 15, %0;" ::"r"(32 * takers) : "memory");       // the items are there
@@ -340,4 +369,17 @@ __global__ void __launch_bounds__(kDirectThreads, 1) k_spmspv_direct(const Direc
     }
     asm volatile("cp.async.bulk.commit_group;" ::: "memory");
     asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");   // shared memory may go once it has been read
+}
+
+template <bool kPairs, bool kBatch, int kHeld>
+__global__ void __launch_bounds__(kDirectThreads, 1) k_spmspv_direct(const DirectParams p)
+{
+    dealt_product<kPairs, kBatch, kHeld>(p);
+}
+
+// k_spmspv_fused with dealt columns, for blocks that own more than 128.
+template <bool kPairs, bool kBatch, int kHeld>
+__global__ void __launch_bounds__(kDirectThreads, 1) k_spmspv_fused_groups(const DirectParams p)
+{
+    dealt_product<kPairs, kBatch, kHeld>(p);
 }

@@ -191,29 +191,34 @@ CELTY_HD inline int direct_taker(int i, int w, float rankers_inv, const DirectGr
     return r - (int)(((float)r + 0.5f) * g.size_inv) * g.size;
 }
 
-// Groups for a launch of `grid` blocks and P row parts with `warps` warps that can rank, a column per lane: as few as hold
-// all columns.  They even out what a group's blocks have, and every ranking warp is another 32 columns.  Device time with up to
+// Groups for a launch of `grid` blocks and P row parts with `warps` warps that can rank: as few as hold all columns, a column per
+// lane.  They even out what a group's blocks have, and every ranking warp is another 32 columns.  Device time with up to
 // 12 or 16 (pairs) ranking warps / 8 / 5 / 2, in us: 4096 x 4096 5.89 / 5.91 / 6.16 / 6.48;  4096 x 11008 10.8 / 10.9 / 10.9 / 11.3;  8192 x 8192
-// 13.5 / 13.6 / 14.2 / 14.2;  with twice or four times the columns per group, two or four per lane: level to 1 % slower, and
-// 6 % / 12 % slower on small layers.
+// 13.5 / 13.6 / 14.2 / 14.2.  Two or four columns per lane are two or four more such look-ups one after the other (small
+// layers: 0.2 us each step) and are taken where a group would have less than three members otherwise (wide: more than 128
+// columns per block): for two / three / four members 11008 x 4096, N = 4 28.5 / 25.7 / 25.8;  8192 x 28672 at 30 % 24.4 / 23.6 / 23.6;
+// 16384 x 12288 at 10 % 10.0 / 10.0 / 10.3;  4096 x 4096, N = 4 13.6 / 13.5 / 14.2;  13824 x 5120 at 50 % 14.0 / 14.0 / 13.7.
 struct DirectGroups {
     int rankers;               // warps that rank
+    int held;                  // columns per lane of them
     int most;                  // columns that a block may take
     DirectSizes sizes[2];      // in row parts with floor(grid / P) blocks, and in those with one more
 };
 
-inline DirectGroups direct_groups(int64_t K, int grid, int P, int warps)
+inline DirectGroups direct_groups(int64_t K, int grid, int P, int warps, bool wide)
 {
     DirectGroups g;
     const int nK = grid / P, columns = direct_columns(K, nK), most = nK + (grid % P ? 1 : 0);
-    const int members = std::max(1, std::min(most, 32 * warps / columns)), groups = (most + members - 1) / members;
+    g.held = 1;
+    while (wide && g.held < 4 && 3 * columns > 32 * g.held * warps) g.held *= 2;
+    const int members = std::max(1, std::min(most, 32 * g.held * warps / columns)), groups = (most + members - 1) / members;
     const int size = (most + groups - 1) / groups;
     for (int l = 0; l < 2; ++l) {
         const int least = (nK + l) / groups;
         g.sizes[l] = DirectSizes{least, (nK + l - least * groups) * (least + 1)};
     }
-    g.rankers = (size * columns + 31) / 32;
-    g.most = std::min(size * columns, g.rankers * (32 / std::max(1, nK / groups) + 1));
+    g.rankers = (size * columns + 32 * g.held - 1) / (32 * g.held);
+    g.most = std::min(size * columns, g.rankers * (32 * g.held / std::max(1, nK / groups) + 1));
     return g;
 }
 
@@ -306,7 +311,8 @@ struct FusedPlan {
     int G, Sc, P, D, cl, pp, mix, slot_bytes, cap, threads, grid, merge;
     int window;                // bytes of the offset window where it has a place of its own (several vectors), else -1
     int lean;                  // 0: every option compiled in; 1 / 2: the builds for the default launch (without / with warp pairs)
-    int direct;                // 1: k_spmspv_direct
+    int direct;                // 1: columns are dealt (k_spmspv_direct, k_spmspv_fused_groups)
+    int wide;                  // 1: k_spmspv_fused_groups
     size_t smem;
 };
 

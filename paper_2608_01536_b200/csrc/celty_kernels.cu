@@ -445,7 +445,7 @@ __global__ void k_decode_lane(const uint32_t *__restrict__ meta, const uint8_t *
 // asked for), so that steady-state calls make no attribute calls.  The attribute belongs to the kernel,
 // so every entry point that launches a kernel shares that kernel's cache (g_granted_*): two caches for
 // one kernel could disagree about what the runtime currently allows.
-int g_granted_fused[64], g_granted_lean[2][64], g_granted_fused_extras[64], g_granted_lean_extras[2][64], g_granted_batch[2][64], g_granted_direct[6][64], g_granted_column[64], g_granted_lane[64], g_granted_reg[4][64];
+int g_granted_fused[64], g_granted_lean[2][64], g_granted_fused_extras[64], g_granted_lean_extras[2][64], g_granted_batch[2][64], g_granted_column[64], g_granted_lane[64], g_granted_reg[4][64];
 
 template <typename Kernel>
 int ensure_smem(Kernel kernel, size_t bytes, int *granted /* [64], per device */)
@@ -500,19 +500,19 @@ int launch_compact(const void *x, int64_t K, float tau, int32_t *idx, uint16_t *
 
 constexpr int kMostToMix = 48;           // left-over blocks are shared between row parts up to this (fit_clusters)
 
-constexpr int kDirectMost = 128;         // columns of a block of k_spmspv_direct (see there)
+constexpr int kDirectMost = 128, kGroupsMost = 512;      // columns of a block of k_spmspv_direct, of k_spmspv_fused_groups (see there)
 
 int direct_threads(int G, int pairs) { return 32 * (pairs ? 16 + kDirectHelpers + 1 : std::max(16, G + kDirectHelpers + 1)); }
 
-DirectGroups direct_groups(const celty_matrix *m, int grid, int P, int threads)
+DirectGroups direct_groups(const celty_matrix *m, int grid, int P, int threads, bool wide)
 {
-    return celty::direct_groups(m->K, grid, P, threads / 32 - 1 - kDirectHelpers);
+    return celty::direct_groups(m->K, grid, P, threads / 32 - 1 - kDirectHelpers, wide);
 }
 
 // Columns that a team of k_spmspv_direct may get: of the block's, or of an even split of a list over the teams of a row part.
-int direct_cap(const celty_matrix *m, int grid, int P, int G, int pairs, bool list)
+int direct_cap(const celty_matrix *m, int grid, int P, int G, int pairs, bool list, bool wide)
 {
-    return list ? (int)(m->K / ((int64_t)(grid / P) * G) + 1) : (direct_groups(m, grid, P, direct_threads(G, pairs)).most + G - 1) / G;
+    return list ? (int)(m->K / ((int64_t)(grid / P) * G) + 1) : (direct_groups(m, grid, P, direct_threads(G, pairs), wide).most + G - 1) / G;
 }
 
 // Shape of the fused launch: P row parts of Sc slabs, G teams per slab (teams = G * Sc warps, one accumulator
@@ -539,13 +539,15 @@ int plan_fused(const celty_matrix *m, const LaunchKnobs &knobs, const DeviceInfo
     // product from a list, but where left-over blocks are shared between row parts, and where a team's items would take
     // much of the shared memory.
     const int per_part = pl.grid / pl.P;
+    const int64_t columns = (m->K + per_part - 1) / per_part;
     const int left = pl.grid % pl.P;
     const bool mixes = left > 0 && pl.P % left == 0 && (int64_t)(pl.P / left) * per_part <= kMostToMix;    // see fit_clusters
     pl.direct = reg_rows == 0 && knobs.merge != 0 && knobs.cluster <= 1 && knobs.lean != 0 && knobs.mix <= 0 && pl.Sc == 1 &&
-                (list ? !mixes && m->K / per_part < 4096 : (m->K + per_part - 1) / per_part <= kDirectMost);
+                (list ? !mixes && m->K / per_part < 4096 : columns <= (mixes && vectors == 1 ? kDirectMost : kGroupsMost));
+    pl.wide = pl.direct && !list && columns > kDirectMost;
     auto smem_bytes = [&](int G, int D) {
         if (!pl.direct) return fused_smem_bytes(m->R, (int)m->K, G, pl.Sc, D, pl.slot_bytes, pl.cap);
-        return (size_t)direct_smem_layout(m->R, (int)m->K, G, D, pl.slot_bytes, direct_cap(m, pl.grid, pl.P, G, pl.pp, list)).total;
+        return (size_t)direct_smem_layout(m->R, (int)m->K, G, D, pl.slot_bytes, direct_cap(m, pl.grid, pl.P, G, pl.pp, list, pl.wide)).total;
     };
     auto fit = [&](int pairs) {
         pl.pp = pairs;
@@ -578,7 +580,7 @@ int plan_fused(const celty_matrix *m, const LaunchKnobs &knobs, const DeviceInfo
     };
     fit(0);
     if (pl.G == 0 && pl.direct) {                 // no room for its tables
-        pl.direct = 0;
+        pl.direct = pl.wide = 0;
         fit(0);
     }
     // Pairs pay where a team has many columns to stream (the hand-over hides the latencies at the head of every
@@ -614,7 +616,7 @@ int plan_fused(const celty_matrix *m, const LaunchKnobs &knobs, const DeviceInfo
         pl.window = (int)(std::min(wanted, budget - pl.smem) / 128 * 128);
         pl.smem += (size_t)pl.window;
     }
-    if (pl.direct) pl.cap = direct_cap(m, pl.grid, pl.P, pl.G, pl.pp, list);
+    if (pl.direct) pl.cap = direct_cap(m, pl.grid, pl.P, pl.G, pl.pp, list, pl.wide);
     pl.merge = (knobs.merge >= 0 ? knobs.merge : 1);
     // Clusters (bulk reduce-add merge only, on request): as long as the grid is made of whole clusters, every row
     // part gets at least one, and the device can hold them all at once.
@@ -786,19 +788,30 @@ int launch_fused(void (*kernel)(Params), int *granted, const LaunchKnobs &knobs,
     return CELTY_OK;
 }
 
-// The build of k_spmspv_direct for a plan, and its shared-memory limit.
+// The build of k_spmspv_direct or k_spmspv_fused_groups for a plan, and its shared-memory limit.
 struct DirectBuild { void (*kernel)(DirectParams); int *granted; };
 
-DirectBuild direct_build(const FusedPlan &plan, bool batch, bool list)
+template <bool kPairs, bool kBatch>
+DirectBuild direct_build(const FusedPlan &plan, bool list, int held)
 {
-    if (list) return plan.pp ? DirectBuild{k_spmspv_direct<true, false, true>, g_granted_direct[0]} : DirectBuild{k_spmspv_direct<false, false, true>, g_granted_direct[1]};
-    if (batch) return plan.pp ? DirectBuild{k_spmspv_direct<true, true, false>, g_granted_direct[2]} : DirectBuild{k_spmspv_direct<false, true, false>, g_granted_direct[3]};
-    return plan.pp ? DirectBuild{k_spmspv_direct<true, false, false>, g_granted_direct[4]} : DirectBuild{k_spmspv_direct<false, false, false>, g_granted_direct[5]};
+    static int granted[5][64];
+    if (list) return DirectBuild{k_spmspv_direct<kPairs, false, 0>, granted[0]};
+    if (!plan.wide) return DirectBuild{k_spmspv_direct<kPairs, kBatch, 1>, granted[1]};
+    return held == 1 ? DirectBuild{k_spmspv_fused_groups<kPairs, kBatch, 1>, granted[2]}
+         : held == 2 ? DirectBuild{k_spmspv_fused_groups<kPairs, kBatch, 2>, granted[3]}
+                     : DirectBuild{k_spmspv_fused_groups<kPairs, kBatch, 4>, granted[4]};
+}
+
+DirectBuild direct_build(const celty_matrix *m, const FusedPlan &plan, bool batch, bool list)
+{
+    const int held = list ? 0 : direct_groups(m, plan.grid, plan.P, plan.threads, plan.wide).held;
+    if (batch) return plan.pp ? direct_build<true, true>(plan, false, held) : direct_build<false, true>(plan, false, held);
+    return plan.pp ? direct_build<true, false>(plan, list, held) : direct_build<false, false>(plan, list, held);
 }
 
 int launch_direct(const celty_matrix *m, const LaunchKnobs &knobs, const FusedPlan &plan, int vectors, bool list, const FusedParams &fp, cudaStream_t st)
 {
-    const DirectBuild b = direct_build(plan, vectors > 1, list);
+    const DirectBuild b = direct_build(m, plan, vectors > 1, list);
     DirectParams p{};
     p.meta = fp.meta; p.stream = fp.stream;
     p.K = fp.K; p.S = fp.S; p.P = fp.P; p.G = fp.G; p.R = fp.R; p.D = fp.D; p.M = fp.M; p.C = fp.C;
@@ -815,7 +828,7 @@ int launch_direct(const celty_matrix *m, const LaunchKnobs &knobs, const FusedPl
         p.list.idx = fp.list_idx; p.x = fp.list_val; p.list_count = fp.list_count;
         p.list.units_inv = fp.units_inv; p.list.units_inv_long = fp.units_inv_long;
     } else {
-        const DirectGroups g = direct_groups(m, plan.grid, plan.P, plan.threads);
+        const DirectGroups g = direct_groups(m, plan.grid, plan.P, plan.threads, plan.wide);
         p.sizes[0] = g.sizes[0]; p.sizes[1] = g.sizes[1];
         p.rankers = g.rankers;
         p.rankers_inv = 1.f / (float)g.rankers;
@@ -846,11 +859,11 @@ extern "C" int celty_launch_plan(const celty_matrix *m, int32_t *out, int32_t n)
                            plan.slot_bytes, plan.merge + 16 * plan.pp + 256 * plan.mix};
     for (int i = 0; i < 10; ++i) out[i] = v[i];
     // which kernel: of this launch, of one from a list, of launches that serve 2 .. 8 vectors
-    if (n > 10) out[10] = plan.direct;
+    if (n > 10) out[10] = plan.direct && !plan.wide;
     for (int i = 11; i < std::min(n, 19); ++i) {
         rc = plan_launch(m, *m, di, i == 11 ? 1 : i - 10, &plan, i == 11);
         if (rc == CELTY_ECUDA) return rc;
-        out[i] = rc ? -1 : plan.direct;
+        out[i] = rc ? -1 : plan.direct && !plan.wide;
     }
     return CELTY_OK;
 }
@@ -1160,7 +1173,7 @@ extern "C" int celty_spmspv_static(const celty_matrix *m, const void *image_dev,
         fp.win_cols = 0;
         // (the limit is raised before the first launch: an error return leaves y untouched)
         fp.image_early = 0;
-        const DirectBuild direct = direct_build(plan, false, false);
+        const DirectBuild direct = plan.direct ? direct_build(m, plan, false, false) : DirectBuild{};
         rc = plan.direct ? ensure_smem(direct.kernel, plan.smem, direct.granted)
            : plan.lean == 2 ? ensure_smem(k_spmspv_fused<false, 0, 2>, plan.smem, g_granted_lean[1])
                             : ensure_smem(k_spmspv_fused<false, 0, 1>, plan.smem, g_granted_lean[0]);

@@ -1,0 +1,49 @@
+"""Products whose blocks share their columns' survivors in groups, at the edges of what a ranking lane holds (one, two or four
+columns) and where the kernel that ranks all of x takes over (more than 512 columns per block)."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import celty_oracle as orc
+from paper_2608_01536_b200 import build, celty, synth
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _lib():
+    build.build()
+    assert torch.cuda.is_available(), "these tests need a CUDA device"
+    celty.load()
+
+
+# blocks of the launch; rows, rows per tile (row parts); columns per block of a row part: three members of a group need 512 / 3
+# columns each (384 / 3 without warp pairs) for one column per lane, 341 (256) for two
+@pytest.mark.parametrize("grid,M,tile_rows", [(5, 40, 0), (37, 300, 3), (148, 40, 0), (19, 1100, 4)])
+@pytest.mark.parametrize("columns", [127, 128, 129, 170, 171, 256, 257, 341, 342, 512, 513])
+def test_groups_at_their_edges(grid, M, tile_rows, columns):
+    """Integer data, exact: three densities, survivors that lie together, none and all; the reported list; the call twice."""
+    probe = celty.Matrix(synth.integer_weights(1, M, 8), None, tile_rows=tile_rows)
+    parts = probe.row_map()[0]
+    K = columns * (grid // parts)
+    W = synth.integer_weights(columns + grid, M, K)
+    mask = synth.mask_bernoulli(columns + grid, M, K, 0.4)
+    m = celty.Matrix(W, mask, tile_rows=tile_rows, device="cuda")
+    m.set_launch(grid=grid)
+    assert m.launch_plan()["row_parts"] == parts
+    rng = np.random.default_rng(columns)
+    full = synth.integer_activations(9, K)
+    full = np.where(full == 0, np.float16(1), full)               # 1 .. in magnitude
+    for keep in (rng.random(K) < 0.5, rng.random(K) < 0.05, np.arange(K) < K // 3, np.zeros(K, bool), np.ones(K, bool)):
+        x = np.where(keep, full, np.float16(0))
+        ref, _ = orc.masked_gemv(W, mask, x, 0.5, threads=8)
+        xd = torch.from_numpy(x).cuda()
+        for _ in range(2):
+            y = m.spmspv(xd, 0.5, y=torch.full((M,), 7.0, device="cuda"))
+            assert np.array_equal(y.cpu().numpy().astype(np.float64), ref)
+        oi, ov, _ = orc.compact(x, 0.5)
+        gi, gv = m.last_compaction()
+        assert np.array_equal(gi.cpu().numpy(), oi) and np.array_equal(gv.cpu().numpy().view(np.uint16), ov)
+        if K <= 32768:
+            assert np.array_equal(m.spmspv_static(xd, 0.5).cpu().numpy().astype(np.float64), ref)
+    assert m.last_status() == 0
