@@ -34,6 +34,7 @@ SIGNATURES = {
     "celty_host_image": (ctypes.c_int, [_vp, ctypes.POINTER(_vp), ctypes.POINTER(_sz), ctypes.POINTER(_sz)]),
     "celty_device_bytes": (ctypes.c_int, [_vp, ctypes.POINTER(_sz), ctypes.POINTER(_sz)]),
     "celty_bind_device": (ctypes.c_int, [_vp, _vp, _sz, _vp, _sz, _vp]),
+    "celty_release_staging": (ctypes.c_int, []),
     "celty_compact": (ctypes.c_int, [_vp, _i64, _f32, _vp, _vp, _vp, _vp]),
     "celty_spmspv": (ctypes.c_int, [_vp, _vp, _f32, _vp, _vp]),
     "celty_spmspv_ex": (ctypes.c_int, [_vp, _vp, _f32, _vp, _vp, _vp]),
@@ -139,6 +140,11 @@ def _stream_ptr(stream):
 
 class _Opts(ctypes.Structure):
     _fields_ = [("run_bits", _i32), ("layout", _i32), ("tile_rows", _i32), ("slabs_per_block", _i32)]
+
+
+def release_staging():
+    """Gives back the 8 MB of page-locked memory that the uploads of large matrices go through."""
+    _check(load().celty_release_staging(), "celty_release_staging")
 
 
 class SwigluOut:

@@ -9,7 +9,7 @@
 #include <new>
 #include <thread>
 #ifdef __SSE2__
-#include <emmintrin.h>
+#include <immintrin.h>
 #endif
 
 #include "celty_internal.h"
@@ -22,40 +22,82 @@ namespace {
 // columns: one row of a block is a cache line or two of W and of the mask, its kept positions one 64-bit word.  The
 // words of 64 rows, transposed, are the kept rows of 64 columns, and entries, gaps and padding follow from bit scans.
 // Blocks are independent but for the places their entries go to, which the counts of a first pass give; host threads
-// share them.  2048 x 4096, half kept: 88 ms for sweeps over whole rows with per-entry temporaries, 2.6 ms this way
-// on 16 threads (27 ms on one).
+// share them.  A row of W or of the mask is another page than the one before it, so what the passes read next is prefetched.
+// 2048 x 4096, half kept, 16 threads: 1.6 to 2.1 ms (2.1 to 2.4 with threads started for each pass, weights gathered entry by entry
+// and pages first touched where they are filled); 27 ms on one.  Bound by the rows of W, 128 bytes of a page each (0.6 ms), the mask
+// (0.3), first touches (0.2) and the start and end of the threads (0.25).
 constexpr int kBlockCols = 64;
 
 // What a thread keeps from one block to the next (fresh large vectors would be fresh pages every time).
+struct SubBlock {
+    uint8_t *at;
+    uint32_t vectors;
+    uint16_t slot[(kMaxTileRows + kGroup - 1) / kGroup + 2];      // [q]: next free one of step q
+};
+
 struct Scratch {
     std::vector<uint64_t> row_word;
+    std::vector<SubBlock> subs;
     std::vector<uint16_t> values;
     std::vector<int32_t> pos;
 };
+
+int64_t host_threads(int64_t n, bool worth_threads)
+{
+    return worth_threads ? std::min<int64_t>({n, 16, (int64_t)std::thread::hardware_concurrency()}) : 1;
+}
+
+// Phases of work that several host threads go through together: work(phase, scratch) on each of them, then between(phase) on one
+// while the others wait.  The threads are started once (starting 15 takes 0.2 ms).  false = memory ran out in one.
+template <typename Work, typename Between>
+bool in_phases(int64_t want, int phases, Work work, Between between)
+{
+    std::atomic<bool> failed(false);
+    std::atomic<int64_t> arrived(0);
+    std::atomic<int> open(0);                                     // the phase that may run
+    auto phase = [&](int p, Scratch &scratch) {
+        try {
+            if (!failed) work(p, scratch);
+        } catch (const std::exception &) {
+            failed = true;
+        }
+    };
+    std::vector<std::thread> threads;
+    try {
+        threads.reserve((size_t)want);
+        for (int64_t t = 1; t < want; ++t)
+            threads.emplace_back([&]() {
+                Scratch scratch;
+                for (int p = 0; p < phases; ++p) {
+                    while (open < p) std::this_thread::yield();
+                    phase(p, scratch);
+                    ++arrived;
+                }
+            });
+    } catch (const std::exception &) {                            // no (more) threads to be had: those there are do it
+    }
+    Scratch scratch;
+    for (int p = 0; p < phases; ++p) {
+        phase(p, scratch);
+        while (arrived < (int64_t)threads.size() * (p + 1)) std::this_thread::yield();
+        try {
+            if (!failed) between(p);
+        } catch (const std::exception &) {
+            failed = true;
+        }
+        open = p + 1;
+    }
+    for (std::thread &t : threads) t.join();
+    return !failed;
+}
 
 // f(i, scratch) for i = 0 .. n - 1, on several host threads where there is work for them; false = memory ran out in one.
 template <typename F>
 bool for_blocks(int64_t n, bool worth_threads, F f)
 {
     std::atomic<int64_t> next(0);
-    std::atomic<bool> failed(false);
-    auto work = [&]() {
-        try {
-            Scratch scratch;
-            for (int64_t i; !failed && (i = next.fetch_add(1)) < n;) f(i, scratch);
-        } catch (const std::exception &) {
-            failed = true;
-        }
-    };
-    const int64_t want = worth_threads ? std::min<int64_t>({n, 16, (int64_t)std::thread::hardware_concurrency()}) : 1;
-    std::vector<std::thread> threads;
-    try {
-        for (int64_t t = 1; t < want; ++t) threads.emplace_back(work);
-    } catch (const std::exception &) {                            // no (more) threads to be had: those there are do it
-    }
-    work();
-    for (std::thread &t : threads) t.join();
-    return !failed;
+    return in_phases(host_threads(n, worth_threads), 1,
+                     [&](int, Scratch &scratch) { for (int64_t i; (i = next.fetch_add(1)) < n;) f(i, scratch); }, [](int) {});
 }
 
 // Kept positions of columns j0 .. j0 + n - 1 of row r, n <= 64.
@@ -65,7 +107,7 @@ inline uint64_t kept_word(const uint16_t *W, int64_t ldw, const uint8_t *mask, i
     int c = 0;
     if (mask) {
         const uint8_t *m = mask + r * K + j0;
-#ifdef __SSE2__
+#if defined(__SSE2__) && !defined(CELTY_PLAIN_ENCODER)
         for (; c + 16 <= n; c += 16) {
             const __m128i v = _mm_loadu_si128(reinterpret_cast<const __m128i *>(m + c));
             word |= (uint64_t)(~_mm_movemask_epi8(_mm_cmpeq_epi8(v, _mm_setzero_si128())) & 0xFFFF) << c;
@@ -74,7 +116,7 @@ inline uint64_t kept_word(const uint16_t *W, int64_t ldw, const uint8_t *mask, i
         for (; c < n; ++c) word |= (uint64_t)(m[c] != 0) << c;
     } else {
         const uint16_t *w = W + r * ldw + j0;
-#ifdef __SSE2__
+#if defined(__SSE2__) && !defined(CELTY_PLAIN_ENCODER)
         const __m128i magnitude = _mm_set1_epi16(0x7FFF);
         for (; c + 16 <= n; c += 16) {
             const __m128i a = _mm_and_si128(_mm_loadu_si128(reinterpret_cast<const __m128i *>(w + c)), magnitude);
@@ -114,7 +156,7 @@ struct TileRows {
     }
     // tile t's local row i is row rows(t)[i] + (t mod 32); >= M: does not exist (a tile's rows grow with i)
     const int32_t *rows(int64_t t) const { return row0.data() + t / 32 * m->R; }
-    void bits_of_block(const std::vector<uint64_t> &row_word, uint64_t *bits) const
+    void bits_of_block(const uint64_t *row_word, uint64_t *bits) const
     {
         for (int64_t t = 0; t < m->T; ++t)
             for (int64_t w = 0; w < words; ++w, bits += kBlockCols) {
@@ -154,15 +196,70 @@ inline void count_entries(const uint64_t *bits, int64_t words, uint32_t *kept, u
     *pads = p;
 }
 
-// Writes the entries of one column of one tile: group by group into places that `place(q)` gives (16 bytes of values,
-// one run word each, zeroed beforehand), entry e of a group in bits 4e .. 4e+3 of its run word.
-template <typename Place>
-void emit_entries(celty_matrix *m, const TileRows &tr, const uint64_t *bits, int64_t t, const uint16_t *values /* [M][64] */,
-                  uint64_t logical, uint64_t entries, int32_t *pos /* [R] */, Place place)
+#if defined(__x86_64__) && !defined(CELTY_PLAIN_ENCODER)
+// The kept weights of one column of one tile (weight of local row i in values[i], words of its kept bits at a stride of 64), one after
+// the other and zeros up to the end of their last group, and their runs, eight to a word; returns how many.  For a tile without
+// padding entries (a run takes four bits).  A compression of 32 weights or 64 positions is one instruction here, where a scan
+// bit by bit is a dozen per entry.
+__attribute__((target("avx512f,avx512bw,avx512vbmi,avx512vbmi2,popcnt")))
+uint64_t compress_tile(const uint64_t *bits, int64_t words, const uint16_t *values, uint16_t *kept, uint8_t *pos /* and one before */, uint32_t *runs)
 {
-    const int32_t *rows = tr.rows(t);
-    values += (t % 32) * kBlockCols;
+    const __m512i ascending = _mm512_set_epi8(
+        63, 62, 61, 60, 59, 58, 57, 56, 55, 54, 53, 52, 51, 50, 49, 48, 47, 46, 45, 44, 43, 42, 41, 40, 39, 38, 37, 36, 35, 34, 33, 32, 31, 30, 29, 28,
+        27, 26, 25, 24, 23, 22, 21, 20, 19, 18, 17, 16, 15, 14, 13, 12, 11, 10, 9, 8, 7, 6, 5, 4, 3, 2, 1, 0);
     uint64_t n = 0;
+    for (int64_t w = 0; w < words; ++w) {
+        const uint64_t b = bits[w * kBlockCols];
+        const __mmask32 lo = (__mmask32)b, hi = (__mmask32)(b >> 32);
+        const uint64_t half = n + (uint64_t)__builtin_popcountll((uint32_t)b);
+        _mm512_storeu_si512(pos + n, _mm512_maskz_compress_epi8(b, _mm512_add_epi8(ascending, _mm512_set1_epi8((char)(64 * w)))));
+        _mm512_storeu_si512(kept + n, _mm512_maskz_compress_epi16(lo, _mm512_loadu_si512(values + 64 * w)));
+        _mm512_storeu_si512(kept + half, _mm512_maskz_compress_epi16(hi, _mm512_loadu_si512(values + 64 * w + 32)));
+        n += (uint64_t)__builtin_popcountll(b);
+    }
+    _mm_storeu_si128(reinterpret_cast<__m128i *>(kept + n), _mm_setzero_si128());
+    pos[-1] = 0xFF;                                               // the row before the first
+    for (uint64_t k = 0; k < n; k += 64) {
+        const __mmask64 there = n - k >= 64 ? ~0ull : (1ull << (n - k)) - 1;
+        const __m512i gap = _mm512_sub_epi8(_mm512_loadu_si512(pos + k), _mm512_loadu_si512(pos + k - 1));
+        const __m512i run = _mm512_maskz_sub_epi8(there, gap, _mm512_set1_epi8(1));
+        _mm256_storeu_si256(reinterpret_cast<__m256i *>(runs + k / 8), _mm512_cvtepi16_epi8(_mm512_or_si512(run, _mm512_srli_epi16(run, 4))));
+    }
+    return n;
+}
+const bool kCompress = [] {
+    __builtin_cpu_init();
+    return __builtin_cpu_supports("avx512f") && __builtin_cpu_supports("avx512bw") && __builtin_cpu_supports("avx512vbmi") && __builtin_cpu_supports("avx512vbmi2");
+}();
+#else
+constexpr bool kCompress = false;
+uint64_t compress_tile(const uint64_t *, int64_t, const uint16_t *, uint16_t *, uint8_t *, uint32_t *) { return 0; }
+#endif
+
+// Writes the entries of one column of one tile, whose local row i has weight values[kStride i]: group by group into places that
+// `place(q)` gives (16 bytes of values, one run word each, zeroed beforehand), entry e of a group in bits 4e .. 4e+3 of its run word.
+template <int kStride, typename Place>
+void emit_entries(celty_matrix *m, const TileRows &tr, const uint64_t *bits, const uint16_t *values, uint64_t logical, uint64_t entries,
+                  int32_t *pos /* [R] */, Place place)
+{
+    uint64_t n = 0;
+    if (kStride == 1 && kCompress) {
+        alignas(64) uint16_t kept[kMaxTileRows + 96];
+        alignas(64) uint8_t at[64 + kMaxTileRows + 144];
+        alignas(64) uint32_t runs[(kMaxTileRows + 64) / 8 + 8];
+        for (int64_t w = 0; w < tr.words; ++w) n += (uint64_t)__builtin_popcountll(bits[w * kBlockCols]);
+        if (n == entries) {
+            compress_tile(bits, tr.words, values, kept, at + 64, runs);
+            for (uint64_t q = 0; q * kGroup < n; ++q) {
+                uint8_t *vp, *rp;
+                place((uint32_t)q, &vp, &rp);
+                std::memcpy(vp, kept + q * kGroup, 16);
+                std::memcpy(rp, runs + q, 4);
+            }
+            return;
+        }
+        n = 0;
+    }
     for (int64_t w = 0; w < tr.words; ++w)
         for (uint64_t b = bits[w * kBlockCols]; b; b &= b - 1) pos[n++] = (int32_t)(w * 64) + __builtin_ctzll(b);
     if (n == entries) {                                           // no padding entries: whole groups without branches
@@ -175,7 +272,7 @@ void emit_entries(celty_matrix *m, const TileRows &tr, const uint64_t *bits, int
             uint32_t runs = 0;
             auto one = [&](int e) {
                 const int32_t i = pos[k + (uint64_t)e];
-                v[e] = values[(size_t)rows[i] * kBlockCols];
+                v[e] = values[(size_t)i * kStride];
                 runs |= (uint32_t)(i - last - 1) << (4 * e);
                 last = i;
             };
@@ -211,7 +308,7 @@ void emit_entries(celty_matrix *m, const TileRows &tr, const uint64_t *bits, int
             __atomic_fetch_or(&m->pad_bits[(size_t)(logical >> 3)], (uint8_t)(1u << (logical & 7)), __ATOMIC_RELAXED);
             ++logical;
         }
-        put(values[(size_t)rows[i] * kBlockCols], gap);
+        put(values[(size_t)i * kStride], gap);
         ++logical;
         prev = i;
     }
@@ -263,6 +360,44 @@ void choose_shape(int64_t M, int64_t K, double density, int tile_rows, int64_t *
     *C_out = R % 16 == 0 ? 16 : R % 8 == 0 ? 8 : R % 4 == 0 ? 4 : 1;
 }
 
+// Weights of a column of a tile in the encoder's copy: whole vectors of 32 and a row of 64 positions are read.
+inline size_t tile_pitch(int64_t R) { return round_up((size_t)R, 64) + 8; }
+
+// Eight rows of a block of columns (null: zeros), to[c * ld + k] = from[k][c].
+inline void copy_transposed(uint16_t *to, size_t ld, const uint16_t *const from[8], int cols)
+{
+    int c = 0;
+#if defined(__SSE2__) && !defined(CELTY_PLAIN_ENCODER)
+    for (; c + 8 <= cols; c += 8) {
+        __m128i r[8], a[8];
+        for (int k = 0; k < 8; ++k)
+            r[k] = from[k] ? _mm_loadu_si128(reinterpret_cast<const __m128i *>(from[k] + c)) : _mm_setzero_si128();
+        for (int k = 0; k < 4; ++k) {                             // rows 2k and 2k + 1 interleaved, then pairs, then fours
+            a[2 * k] = _mm_unpacklo_epi16(r[2 * k], r[2 * k + 1]);
+            a[2 * k + 1] = _mm_unpackhi_epi16(r[2 * k], r[2 * k + 1]);
+        }
+        for (int h = 0; h < 2; ++h)
+            for (int k = 0; k < 2; ++k) {
+                r[4 * h + 2 * k] = _mm_unpacklo_epi32(a[4 * h + k], a[4 * h + 2 + k]);
+                r[4 * h + 2 * k + 1] = _mm_unpackhi_epi32(a[4 * h + k], a[4 * h + 2 + k]);
+            }
+        for (int k = 0; k < 4; ++k) {
+            _mm_storeu_si128(reinterpret_cast<__m128i *>(to + (c + 2 * k) * ld), _mm_unpacklo_epi64(r[k], r[4 + k]));
+            _mm_storeu_si128(reinterpret_cast<__m128i *>(to + (c + 2 * k + 1) * ld), _mm_unpackhi_epi64(r[k], r[4 + k]));
+        }
+    }
+#endif
+    for (; c < cols; ++c)
+        for (int k = 0; k < 8; ++k) to[(size_t)c * ld + k] = from[k] ? from[k][c] : 0;
+}
+
+// A row of a block of columns.
+inline void copy_row(uint16_t *to, const uint16_t *from, int cols)
+{
+    if (cols == kBlockCols) std::memcpy(to, from, 2 * kBlockCols);
+    else std::memcpy(to, from, (size_t)cols * 2);
+}
+
 // COLUMN image: meta uint2[K] {off16, entries}, then per column its chunks of up to 32 groups;
 // chunk = [groups x 16 B values][groups x 4 B runs]; column block padded to 16 bytes.
 void write_column(celty_matrix *m, const TileRows &tr, const uint64_t *bits, const uint16_t *values, int32_t *pos, int64_t j,
@@ -273,7 +408,7 @@ void write_column(celty_matrix *m, const TileRows &tr, const uint64_t *bits, con
     uint8_t *col = m->image.data() + m->meta_bytes + (size_t)meta[2 * j] * 16;
     meta[2 * j + 1] = (uint32_t)n;
     std::memset(col, 0, round_up((size_t)groups * 20, 16));
-    emit_entries(m, tr, bits + c, 0, values + c, e0, n, pos, [&](uint32_t g, uint8_t **vp, uint8_t **rp) {
+    emit_entries<kBlockCols>(m, tr, bits + c, values + c, e0, n, pos, [&](uint32_t g, uint8_t **vp, uint8_t **rp) {
         const uint64_t chunk = g / kChunkGroups, in = g % kChunkGroups, gc = std::min<uint64_t>(kChunkGroups, groups - chunk * kChunkGroups);
         uint8_t *at = col + chunk * (kChunkGroups * 20);
         *vp = at + 16 * in;
@@ -286,20 +421,27 @@ void write_column(celty_matrix *m, const TileRows &tr, const uint64_t *bits, con
 // padded to 16 bytes,
 // G = sum of the lanes' group counts.  Vectors are stored step-major: for step q = 0, 1, ... the
 // lanes that still have a q-th group, in lane order, so that a warp reads one contiguous span per step.
-void write_lane_tile(celty_matrix *m, const TileRows &tr, const uint64_t *bits, const uint16_t *values, int32_t *pos, int64_t j0,
+// W points at the block's first column.  A tile's rows of the block are copied together, column by column: 8 to 32 KB, which stay in
+// L1 or L2 while the tile is packed.  (Two or four blocks at a time, 256 or 512 bytes of a row: 20 % slower.)
+void write_lane_tile(celty_matrix *m, const TileRows &tr, const uint64_t *bits, const uint16_t *W, int64_t ldw, Scratch &scratch, int64_t j0,
                      int cols)
 {
     const int64_t S = m->S, T = m->T;
+    const size_t ld = tile_pitch(m->R);
     const uint32_t *meta = reinterpret_cast<const uint32_t *>(m->image.data());
-    constexpr int kMaxSteps = (kMaxTileRows + kGroup - 1) / kGroup + 1;
-    struct Sub { uint8_t *at; uint32_t vectors; uint16_t slot[kMaxSteps + 1]; } sub[kBlockCols];   // slot[q]: next free of step q
+    scratch.values.resize((size_t)cols * ld);
+    scratch.pos.resize((size_t)m->R);
+    scratch.subs.resize((size_t)cols);
+    uint16_t *values = scratch.values.data();
+    int32_t *pos = scratch.pos.data();
+    SubBlock *sub = scratch.subs.data();
     for (int64_t s = 0; s < S; ++s) {
         for (int c = 0; c < cols; ++c) {
             const size_t b = (size_t)((j0 + c) * S + s);
-            Sub &sb = sub[c];
+            SubBlock &sb = sub[c];
             sb.at = m->image.data() + m->meta_bytes + (size_t)meta[b] * 16;
             std::memset(sb.at, 0, ((size_t)meta[b + 1] - meta[b]) * 16);
-            uint16_t lanes[kMaxSteps + 1] = {};                     // lanes that have a q-th group
+            uint16_t lanes[(kMaxTileRows + kGroup - 1) / kGroup + 2] = {};                     // lanes that have a q-th group
             uint32_t steps = 0;
             sb.vectors = 0;
             for (int L = 0; L < 32; ++L) {
@@ -317,11 +459,22 @@ void write_lane_tile(celty_matrix *m, const TileRows &tr, const uint64_t *bits, 
         }
         for (int L = 0; L < 32; ++L) {
             const int64_t t = 32 * s + L;
+            const int32_t *rows = tr.rows(t);
+            for (int64_t i = 0; i < m->R; i += 8) {
+                const uint16_t *from[8];
+                for (int k = 0; k < 8; ++k) {
+                    const int64_t r = i + k < m->R ? rows[i + k] + L : m->M;
+                    from[k] = r < m->M ? W + r * ldw : nullptr;
+                    if (r + 1 < m->M)                                // of the next tile
+                        for (int c = 0; c < cols; c += 32) __builtin_prefetch(from[k] + ldw + c);
+                }
+                copy_transposed(values + i, ld, from, cols);
+            }
             for (int c = 0; c < cols; ++c) {
-                Sub &sb = sub[c];
+                SubBlock &sb = sub[c];
                 uint8_t *vbase = sb.at + kSubHeader, *rbase = vbase + 16 * (size_t)sb.vectors;
                 const uint64_t e0 = m->block_ptr[(size_t)((j0 + c) * T + t)], e1 = m->block_ptr[(size_t)((j0 + c) * T + t + 1)];
-                emit_entries(m, tr, bits + t * tr.words * kBlockCols + c, t, values + c, e0, e1 - e0, pos,
+                emit_entries<1>(m, tr, bits + t * tr.words * kBlockCols + c, values + (size_t)c * ld, e0, e1 - e0, pos,
                              [&](uint32_t q, uint8_t **vp, uint8_t **rp) {
                                  const uint32_t slot = sb.slot[q]++;
                                  *vp = vbase + 16 * (size_t)slot;
@@ -376,75 +529,135 @@ extern "C" int celty_encode(const uint16_t *W, int64_t ldw, const uint8_t *mask,
         const TileRows tr(m);
         const int64_t blocks = (K + kBlockCols - 1) / kBlockCols;
         auto columns = [&](int64_t b) { return (int)std::min<int64_t>(kBlockCols, K - b * kBlockCols); };
-        // Pass 1: kept bits of every block of columns, entries of every (column, tile), groups of every unit the
-        // image is made of (COLUMN: a column, LANE_TILE: a sub-block).
-        m->block_ptr.resize((size_t)(K * T + 1));
-        std::vector<uint32_t> unit_groups((size_t)(K * S));
-        std::vector<std::vector<uint64_t>> bits((size_t)blocks);
-        std::atomic<uint64_t> nnz(0), n_pad(0);
-        if (!for_blocks(blocks, threads, [&](int64_t b, Scratch &scratch) {
-                const int n = columns(b);
-                scratch.row_word.resize((size_t)M);
-                for (int64_t r = 0; r < M; ++r) scratch.row_word[(size_t)r] = kept_word(W, ldw, mask, K, r, b * kBlockCols, n);
-                std::vector<uint64_t> &bb = bits[(size_t)b];
-                bb.resize((size_t)(T * tr.words * kBlockCols));
-                tr.bits_of_block(scratch.row_word, bb.data());
-                uint64_t kept_sum = 0, pad_sum = 0;
-                for (int c = 0; c < n; ++c) {
-                    const int64_t j = b * kBlockCols + c;
-                    for (int64_t t = 0; t < T; ++t) {
+        // Phase 0: kept bits of every block of columns, entries of every (column, tile), groups of every unit the image is
+        // made of (COLUMN: a column, LANE_TILE: a sub-block).  Entries and units are summed within the block.
+        m->block_ptr.allocate((size_t)(K * T + 1));
+        const size_t block_bits = (size_t)(T * tr.words * kBlockCols);
+        Raw<uint64_t> bits;
+        bits.allocate(block_bits * (size_t)blocks);
+        Raw<uint32_t> unit_at;                                    // units before unit u in its block, in 16-byte steps
+        unit_at.allocate((size_t)(K * S));
+        struct Sum { uint64_t kept = 0, pads = 0, units16 = 0; uint32_t largest = 0; };
+        std::vector<Sum> sums((size_t)blocks);
+        uint32_t *meta = nullptr;
+        size_t units16 = 0;
+        std::atomic<int64_t> next[3] = {{0}, {0}, {0}}, touched(0);
+        const int64_t want = host_threads(blocks, threads);
+        // blocks that a thread takes together in phase 0, row by row: the mask is read 256 bytes at a time
+        const int64_t together = std::max<int64_t>(1, std::min<int64_t>(4, blocks / want));
+        auto count_block = [&](int64_t b, const uint64_t *row_word) {
+            uint64_t *bb = bits.data() + block_bits * (size_t)b;
+            tr.bits_of_block(row_word, bb);
+            Sum &sum = sums[(size_t)b];
+            uint32_t entries = 0;
+            for (int c = 0; c < columns(b); ++c) {
+                const int64_t j = b * kBlockCols + c;
+                for (int64_t s = 0; s < S; ++s) {
+                    uint32_t groups = 0;
+                    for (int64_t t = s * (T / S); t < (s + 1) * (T / S); ++t) {
                         uint32_t kept, pads;
-                        count_entries(bb.data() + t * tr.words * kBlockCols + c, tr.words, &kept, &pads);
-                        m->block_ptr[(size_t)(j * T + t + 1)] = kept + pads;
-                        unit_groups[(size_t)(j * S + t / 32)] += (kept + pads + kGroup - 1) / kGroup;
-                        kept_sum += kept;
-                        pad_sum += pads;
+                        count_entries(bb + t * tr.words * kBlockCols + c, tr.words, &kept, &pads);
+                        entries += kept + pads;
+                        m->block_ptr[(size_t)(j * T + t + 1)] = entries;
+                        groups += (kept + pads + kGroup - 1) / kGroup;
+                        sum.kept += kept;
+                        sum.pads += pads;
                     }
+                    const uint32_t units16 = (uint32_t)(((lane_tile ? kSubHeader : 0) + (size_t)groups * 20 + 15) / 16);
+                    unit_at[(size_t)(j * S + s)] = (uint32_t)sum.units16;
+                    sum.units16 += units16;
+                    sum.largest = std::max(sum.largest, units16);
                 }
-                nnz += kept_sum;
-                n_pad += pad_sum;
-            }))
-            return CELTY_ENOMEM;
-        m->nnz = (int64_t)nnz.load();
-        m->n_pad = (int64_t)n_pad.load();
-        const uint64_t total = nnz.load() + n_pad.load();
-        if (total > 0xFFFFFFFFull) return CELTY_EINVAL;
-        m->block_ptr[0] = 0;
-        for (int64_t k = 0; k < K * T; ++k) m->block_ptr[(size_t)(k + 1)] += m->block_ptr[(size_t)k];
-        m->pad_bits.assign((size_t)(total + 7) / 8, 0);
-        // Places: offsets of the units, in 16-byte steps.
-        m->meta_bytes = round_up(lane_tile ? (size_t)(K * S + 1) * 4 : (size_t)K * 8, kAlign);
-        uint64_t bytes = 0;
-        auto unit_bytes = [&](int64_t u) { return (uint64_t)round_up((lane_tile ? kSubHeader : 0) + (size_t)unit_groups[(size_t)u] * 20, 16); };
-        for (int64_t u = 0; u < K * S; ++u) bytes += unit_bytes(u);
-        m->stream_bytes = round_up((size_t)bytes, kAlign);
-        m->image.allocate(m->meta_bytes + m->stream_bytes);
-        std::memset(m->image.data(), 0, m->meta_bytes);
-        std::memset(m->image.data() + m->meta_bytes + bytes, 0, m->stream_bytes - (size_t)bytes);
-        uint32_t *meta = reinterpret_cast<uint32_t *>(m->image.data());
-        uint64_t at = 0;
-        for (int64_t u = 0; u < K * S; ++u) {
-            meta[lane_tile ? u : 2 * u] = (uint32_t)(at / 16);
-            m->max_unit16 = std::max<uint32_t>(m->max_unit16, (uint32_t)(unit_bytes(u) / 16));
-            at += unit_bytes(u);
-        }
-        if (lane_tile) meta[K * S] = (uint32_t)(at / 16);
-        // Pass 2: values and runs.  A block's weights are copied together first: read column by column where they
-        // are, a power-of-two row pitch maps them all to a few sets of the cache.
-        if (!for_blocks(blocks, threads, [&](int64_t b, Scratch &scratch) {
+            }
+        };
+        auto work = [&](int phase, Scratch &scratch) {
+            if (phase == 0) {
+                scratch.row_word.resize((size_t)(M * together));
+                for (int64_t b0; (b0 = next[0].fetch_add(together)) < blocks;) {
+                    const int64_t b1 = std::min(blocks, b0 + together);
+                    for (int64_t r = 0; r < M; ++r) {
+                        const int64_t ahead = std::min<int64_t>(M - 1, r + 16);
+                        for (int64_t b = b0; b < b1; ++b) {
+                            if (mask) __builtin_prefetch(mask + ahead * K + b * kBlockCols);
+                            else __builtin_prefetch(W + ahead * ldw + b * kBlockCols);
+                            scratch.row_word[(size_t)((b - b0) * M + r)] = kept_word(W, ldw, mask, K, r, b * kBlockCols, columns(b));
+                        }
+                    }
+                    for (int64_t b = b0; b < b1; ++b) count_block(b, scratch.row_word.data() + (b - b0) * M);
+                }
+                return;
+            }
+            // Phase 1: places of the block's entries and units.  Phase 2: values and runs.  The large arrays are first touched here,
+            // a 2 MB page per thread: in phase 2 all threads would wait for the few pages that they are in at a time.
+            if (phase == 1) {
+                constexpr size_t page = (size_t)2 << 20;
+                const size_t pages = (m->image.size() + page - 1) / page;
+                for (size_t k; (k = (size_t)touched.fetch_add(1)) * page < pages * page + m->pad_bits.size();) {
+                    const size_t at = k < pages ? std::max(k * page, m->meta_bytes) : (k - pages) * page;      // (meta is written below)
+                    if (k >= pages) std::memset(m->pad_bits.data() + at, 0, std::min(page, m->pad_bits.size() - at));
+                    else if (at < std::min((k + 1) * page, m->image.size())) *(volatile uint8_t *)(m->image.data() + at) = 0;
+                }
+            }
+            if (phase == 1) {
+                for (int64_t b; (b = next[1].fetch_add(1)) < blocks;) {
+                    const Sum &before = sums[(size_t)b];          // of all blocks before this one by now
+                    const int64_t j0 = b * kBlockCols, j1 = j0 + columns(b);
+                    const uint32_t entries = (uint32_t)(before.kept + before.pads);
+                    for (int64_t k = j0 * T; k < j1 * T; ++k) m->block_ptr[(size_t)(k + 1)] += entries;
+                    for (int64_t u = j0 * S; u < j1 * S; ++u) meta[lane_tile ? u : 2 * u] = unit_at[(size_t)u] + (uint32_t)before.units16;
+                    if (b + 1 < blocks) continue;
+                    const size_t used = lane_tile ? (size_t)(K * S + 1) * 4 : (size_t)K * 8;
+                    if (lane_tile) meta[K * S] = (uint32_t)units16;
+                    std::memset(m->image.data() + used, 0, m->meta_bytes - used);
+                    std::memset(m->image.data() + m->meta_bytes + units16 * 16, 0, m->stream_bytes - units16 * 16);
+                }
+                return;
+            }
+            for (int64_t b; (b = next[2].fetch_add(1)) < blocks;) {
+                const uint64_t *bb = bits.data() + block_bits * (size_t)b;
                 const int n = columns(b);
-                std::vector<uint16_t> &values = scratch.values;
-                values.resize((size_t)M * kBlockCols);
-                scratch.pos.resize((size_t)m->R);
-                int32_t *pos = scratch.pos.data();
-                for (int64_t r = 0; r < M; ++r)
-                    std::memcpy(&values[(size_t)r * kBlockCols], W + r * ldw + b * kBlockCols, (size_t)n * 2);
-                if (lane_tile) write_lane_tile(m, tr, bits[(size_t)b].data(), values.data(), pos, b * kBlockCols, n);
-                else
-                    for (int c = 0; c < n; ++c) write_column(m, tr, bits[(size_t)b].data(), values.data(), pos, b * kBlockCols + c, c);
-                std::vector<uint64_t>().swap(bits[(size_t)b]);
-            }))
-            return CELTY_ENOMEM;
+                if (lane_tile) {
+                    write_lane_tile(m, tr, bb, W + b * kBlockCols, ldw, scratch, b * kBlockCols, n);
+                    continue;
+                }
+                // (read column by column where they are, a power-of-two row pitch maps them all to a few sets of the cache)
+                scratch.values.resize((size_t)M * kBlockCols);
+                scratch.pos.resize((size_t)M);
+                for (int64_t r = 0; r < M; ++r) copy_row(&scratch.values[(size_t)r * kBlockCols], W + r * ldw + b * kBlockCols, n);
+                for (int c = 0; c < n; ++c) write_column(m, tr, bb, scratch.values.data(), scratch.pos.data(), b * kBlockCols + c, c);
+            }
+        };
+        bool too_large = false;
+        auto between = [&](int phase) {
+            if (phase != 0) return;
+            Sum all;
+            for (Sum &sum : sums) {                               // the sum of a block becomes that of those before it
+                const Sum own = sum;
+                sum = all;
+                all.kept += own.kept;
+                all.pads += own.pads;
+                all.units16 += own.units16;
+                all.largest = std::max(all.largest, own.largest);
+            }
+            const uint64_t total = all.kept + all.pads;
+            m->nnz = (int64_t)all.kept;
+            m->n_pad = (int64_t)all.pads;
+            m->max_unit16 = all.largest;
+            if (total > 0xFFFFFFFFull) {
+                too_large = true;
+                for (auto &n : next) n = blocks;                  // nothing of the later phases
+                return;
+            }
+            m->block_ptr[0] = 0;
+            m->pad_bits.allocate((size_t)(total + 7) / 8);
+            m->meta_bytes = round_up(lane_tile ? (size_t)(K * S + 1) * 4 : (size_t)K * 8, kAlign);
+            units16 = (size_t)all.units16;
+            m->stream_bytes = round_up(units16 * 16, kAlign);
+            m->image.allocate(m->meta_bytes + m->stream_bytes);
+            meta = reinterpret_cast<uint32_t *>(m->image.data());
+        };
+        if (!in_phases(want, 3, work, between)) return CELTY_ENOMEM;
+        if (too_large) return CELTY_EINVAL;
         const int64_t spb = o.slabs_per_block > 0 ? o.slabs_per_block : kSlabsPerBlock;
         m->P = (int32_t)((m->S + spb - 1) / spb);
         m->Sc = (int32_t)((m->S + m->P - 1) / m->P);

@@ -4,9 +4,13 @@
 #include <cmath>
 #include <cstddef>
 #include <cstdint>
+#include <cstdlib>
 #include <cstring>
 #include <memory>
+#include <new>
 #include <vector>
+
+#include <sys/mman.h>
 
 #include "celty.h"
 
@@ -50,19 +54,35 @@ CELTY_HD inline int64_t tile_row(int64_t S, int64_t C, int64_t s, int64_t lane, 
     return (((i / C) * S + s) * C + i % C) * 32 + lane;
 }
 
-// Host bytes that are not cleared when they are allocated: the encoder's threads write (and so first touch) all of them.
-class Bytes {
+// Host memory that is not cleared when it is allocated: the encoder's threads write (and so first touch) all of it.  From 2 MB on
+// in 2 MB pages where the system grants them on request: 16 threads that first touch 12 MB in 4 KB pages take 0.6 ms, most of it in
+// one another's way.
+template <typename T>
+class Raw {
 public:
-    Bytes() = default;
-    Bytes(const Bytes &o) { allocate(o.n_); if (n_) std::memcpy(p_.get(), o.p_.get(), n_); }
-    Bytes &operator=(const Bytes &) = delete;
-    void allocate(size_t n) { p_.reset(new uint8_t[n]); n_ = n; }
-    uint8_t *data() { return p_.get(); }
-    const uint8_t *data() const { return p_.get(); }
+    Raw() = default;
+    Raw(const Raw &o) { allocate(o.n_); if (n_) std::memcpy(p_.get(), o.p_.get(), n_ * sizeof(T)); }
+    Raw &operator=(const Raw &) = delete;
+    void allocate(size_t n)
+    {
+        constexpr size_t huge = (size_t)2 << 20;
+        const size_t bytes = n * sizeof(T), align = bytes >= huge ? huge : 64;
+        p_.reset(static_cast<T *>(std::aligned_alloc(align, round_up(bytes + (bytes == 0), align))));
+        if (!p_) throw std::bad_alloc();
+        n_ = n;
+#ifdef MADV_HUGEPAGE
+        if (align == huge) (void)madvise(p_.get(), round_up(bytes, huge), MADV_HUGEPAGE);
+#endif
+    }
+    T *data() { return p_.get(); }
+    const T *data() const { return p_.get(); }
+    T &operator[](size_t i) { return p_.get()[i]; }
+    const T &operator[](size_t i) const { return p_.get()[i]; }
     size_t size() const { return n_; }
 
 private:
-    std::unique_ptr<uint8_t[]> p_;
+    struct Free { void operator()(void *p) const { std::free(p); } };
+    std::unique_ptr<T, Free> p_;
     size_t n_ = 0;
 };
 
@@ -417,12 +437,12 @@ struct celty_matrix : celty::LaunchKnobs {
     int64_t S = 1;          // slabs of 32 tiles per column (LANE_TILE), 1 for COLUMN
     int32_t P = 1, Sc = 1;  // LANE_TILE: row parts per column and slabs per part (P * Sc >= S)
     int64_t nnz = 0, n_pad = 0;
-    std::vector<uint32_t> block_ptr;   // K*T + 1, stored entries before block (j, t)
-    std::vector<uint8_t> pad_bits;     // one bit per stored entry (logical order): 1 = padding entry
+    celty::Raw<uint32_t> block_ptr;    // K*T + 1, stored entries before block (j, t)
+    celty::Raw<uint8_t> pad_bits;      // one bit per stored entry (logical order): 1 = padding entry
     // image = [meta | stream]
     //   COLUMN:    meta = uint2[K]  {offset/16 of the column block in the stream, entries}
     //   LANE_TILE: meta = uint32[K*S + 1]  offset/16 of sub-block (j, s); sub-blocks are contiguous
-    celty::Bytes image;
+    celty::Raw<uint8_t> image;
     size_t meta_bytes = 0;             // stream starts at image[meta_bytes]
     size_t stream_bytes = 0;
     uint32_t max_unit16 = 0;           // largest column block / sub-block in 16-byte units

@@ -1,0 +1,62 @@
+"""The host encoder with and without vector instructions packs the same image, byte for byte (the plain build's entries are
+held to the oracle's rule where the library runs without them; the vector build's in test_host_encoder).  No GPU needed."""
+import os
+import subprocess
+
+import pytest
+
+from conftest import ROOT
+
+CSRC = os.path.join(ROOT, "paper_2608_01536_b200", "csrc")
+MAIN = r'''
+#include <cstdio>
+#include <cstdlib>
+#include <random>
+#include <vector>
+#include "celty.h"
+int main(int, char **v) {
+    const int M = atoi(v[1]), K = atoi(v[2]), tile_rows = atoi(v[3]), kept = atoi(v[4]), column = atoi(v[5]);
+    std::mt19937 r(M * 31 + K);
+    std::vector<uint16_t> W((size_t)M * K);
+    std::vector<uint8_t> mask((size_t)M * K);
+    for (size_t i = 0; i < W.size(); ++i) { W[i] = (uint16_t)r(); mask[i] = (int)(r() % 1000) < kept; }
+    celty_encode_opts o = {4, column ? CELTY_LAYOUT_COLUMN : CELTY_LAYOUT_LANE_TILE, tile_rows, 0};
+    for (int with_mask = 0; with_mask < 2; ++with_mask) {
+        celty_matrix *m;
+        if (celty_encode(W.data(), K, with_mask ? mask.data() : nullptr, M, K, &o, &m)) return 1;
+        const void *image; size_t bytes, at;
+        celty_host_image(m, &image, &bytes, &at);
+        fwrite(image, 1, bytes, stdout);
+        for (int j = 0; j < K; j += 1 + K / 7) {
+            std::vector<uint8_t> runs(4 * M + 64), pads(4 * M + 64);
+            int64_t n;
+            if (celty_decode_host(m, j, nullptr, nullptr, runs.data(), pads.data(), 4 * M + 64, &n)) return 2;
+            fwrite(runs.data(), 1, n, stdout);
+            fwrite(pads.data(), 1, n, stdout);
+        }
+        celty_destroy(m);
+    }
+}
+'''
+
+
+@pytest.fixture(scope="module")
+def encoders(tmp_path_factory):
+    d = tmp_path_factory.mktemp("encoders")
+    (d / "main.cpp").write_text(MAIN)
+    exes = []
+    for k, flags in enumerate(([], ["-DCELTY_PLAIN_ENCODER"])):
+        exes.append(str(d / ("encoder%d" % k)))
+        subprocess.check_call(["g++", "-O2", "-std=c++17", "-pthread", *flags, "-I", os.path.join(ROOT, "include"), "-I", CSRC,
+                               os.path.join(CSRC, "celty_host.cpp"), str(d / "main.cpp"), "-o", exes[-1]])
+    return exes
+
+
+# rows per tile on both sides of a 64-bit word of kept bits and the largest; ragged rows and columns; all, half, few and no padding
+@pytest.mark.parametrize("M,K,tile_rows,kept,column", [
+    (1, 1, 0, 500, 0), (33, 63, 0, 500, 0), (40, 65, 1, 1000, 0), (2016, 130, 63, 500, 0), (2048, 64, 64, 1000, 0), (2080, 129, 65, 300, 0),
+    (7680, 70, 240, 500, 0), (7681, 70, 240, 900, 0), (4100, 200, 128, 60, 0), (2048, 300, 0, 500, 0), (1000, 200, 0, 1, 0), (777, 130, 0, 500, 1),
+    (3000, 64, 96, 980, 0)])
+def test_plain_and_vector_builds_agree(encoders, M, K, tile_rows, kept, column):
+    outs = [subprocess.check_output([e, *map(str, (M, K, tile_rows, kept, column))]) for e in encoders]
+    assert len(outs[0]) > 0 and outs[0] == outs[1]
