@@ -13,8 +13,13 @@
 // What bounds it: shared memory.  The rows of the 32 lanes fall on the banks as good as at random (8 entries, or
 // some 16 rows at 50 % density, lie between two lanes), so a load or store takes 3 to 4 wavefronts where the lane
 // tiles' takes one; entries per SM / 32 x 7 wavefronts is 3.2 us at 4096 x 4096, 50 % / 50 %.  Measured there:
-// 11.8 us against 41.6 us for warps that each took whole columns and added with shared-memory atomics, behind a
-// one-block compaction kernel.
+// 11.6 us against 41.6 us for warps that each took whole columns and added with shared-memory atomics, behind a
+// one-block compaction kernel; 10.2 with dealt columns.
+//
+// kDealt (column_dealt says where): a block's columns as in k_spmspv_direct, dealt to groups of blocks that share the survivors, instead of
+// every block ranking all of x and looking its share up behind five block barriers.  Device time in us, ranked -> dealt: 4096 x 4096 at 10 % /
+// 50 % 6.88 -> 5.55, 11.59 -> 10.24;  1000 x 1000 5.81 -> 4.15;  2048 x 8192 at 30 % 8.80 -> 7.68;  7000 x 2300 11.41 -> 10.84.  (The next
+// chunk's scan moved under this one's loads: 0.1 to 0.3 us slower, with the loads of x ahead by one chunk more or not.)
 //
 // a0: k_clear clears y ahead of this kernel (11.4 us where every block cleared its share and all waited for one
 // another's ticket, but a call must not need all SMs at once).  a1 as in the fused kernel: every block thresholds all of
@@ -34,6 +39,12 @@ struct ColumnParams {
     int W, groups;              // warps per column, columns in flight per block (W * groups <= 32, groups <= 15 if W > 1)
     int cap;                    // columns a block looks up at a time
     int own_list;               // 1: threshold x here
+    // kDealt: columns are dealt to groups of blocks as in k_spmspv_direct
+    celty::DirectSizes sizes;
+    int rankers;
+    float rankers_inv;
+    uint32_t dealt;             // where the block's columns go in shared memory, {column, x bits} of most, then {offset/16, entries}
+    int most;
 };
 
 constexpr int kColumnThreads = 1024;
@@ -79,13 +90,14 @@ __device__ __forceinline__ uint32_t keep_word(const uint16_t *x, int K, int w, _
     return word;
 }
 
+template <bool kDealt>
 __global__ void __launch_bounds__(kColumnThreads, 1) k_spmspv_column(const ColumnParams p)
 {
     extern __shared__ __align__(128) uint8_t smem[];
     const ColumnSmem lay = column_smem_layout(p.M, p.K, p.groups, p.cap, p.own_list);
     float *acc = reinterpret_cast<float *>(smem + lay.acc);
-    int2 *items = reinterpret_cast<int2 *>(smem + lay.items);
-    uint2 *imeta = reinterpret_cast<uint2 *>(smem + lay.imeta);
+    int2 *items = reinterpret_cast<int2 *>(smem + (kDealt ? p.dealt : lay.items));
+    uint2 *imeta = kDealt ? reinterpret_cast<uint2 *>(items + p.most) : reinterpret_cast<uint2 *>(smem + lay.imeta);
     int *warp_tot = reinterpret_cast<int *>(smem + lay.warps);
     uint32_t *keep = reinterpret_cast<uint32_t *>(smem + lay.keep);
     int *rank = reinterpret_cast<int *>(smem + lay.rank);
@@ -94,18 +106,61 @@ __global__ void __launch_bounds__(kColumnThreads, 1) k_spmspv_column(const Colum
     const int Mp = (p.M + 3) & ~3;
 
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    const float nK_inv = __fdividef(1.f, (float)gridDim.x);
+    const DirectGroup group = kDealt ? direct_group((int)blockIdx.x, p.sizes) : DirectGroup{};
+    const int column = kDealt && warp < p.rankers ? direct_held(tid, group, (int)gridDim.x, nK_inv) : p.K;      // (K or more: none)
+    uint2 place = make_uint2(0u, 0u);
+    if (kDealt && column < p.K) place = __ldg(p.meta + column);
+    if (kDealt && tid == 0) *warp_tot = 0;                         // columns that the block has taken
     for (int i = tid; i < p.groups * Mp / 4; i += kColumnThreads)
         reinterpret_cast<float4 *>(acc)[i] = make_float4(0.f, 0.f, 0.f, 0.f);
     // The block's columns lie around the same fraction of K as the block in the grid: their offsets are fetched now.
     // (The table is part of the image, which no kernel writes.)
     uint2 *const window = reinterpret_cast<uint2 *>(smem + lay.window);
     const int win0 = max(0, min(p.K - kColumnWindow, (int)((float)(2 * blockIdx.x + 1) * (float)p.K / (float)(2 * gridDim.x)) - kColumnWindow / 2));
-    if (p.own_list && tid < kColumnWindow && win0 + tid < p.K) window[tid] = __ldg(p.meta + win0 + tid);
+    if (!kDealt && p.own_list && tid < kColumnWindow && win0 + tid < p.K) window[tid] = __ldg(p.meta + win0 + tid);
+    if (kDealt) __syncthreads();
     asm volatile("griddepcontrol.wait;" ::: "memory");
 
-    // ---- a1: keep words and the survivors before each of them
     int n = 0;
-    if (p.own_list) {
+    if (kDealt) {
+        // ---- a1 as in k_spmspv_direct: the lanes of the ranking warps threshold the columns of the block's group, and every
+        // size-th survivor is this block's.  The list for the API comes from the warps that do not stream, in a few blocks.
+        if (warp < p.rankers) {
+            const uint32_t xb = column < p.K ? p.x[column] : 0u;
+            const bool kept = column < p.K && !(fabsf(__half2float(__ushort_as_half((uint16_t)xb))) <= p.tau);
+            const uint32_t word = __ballot_sync(kFull, kept);
+            if (kept && direct_taker(__popc(word & ((1u << lane) - 1u)), warp, p.rankers_inv, group) == (int)blockIdx.x - group.first) {
+                const int i = atomicAdd(warp_tot, 1);
+                items[i] = make_int2(column, (int)xb);
+                imeta[i] = place;
+            }
+        }
+        __syncthreads();
+        n = *warp_tot;
+        const int streaming = p.W * p.groups, helpers = 32 - streaming, nwords = (p.K + 31) >> 5;
+        const int list_blocks = min((int)gridDim.x, idiv_small(nwords + 2 * helpers - 1, 2 * helpers));
+        if (warp >= streaming && (int)blockIdx.x < list_blocks) {
+            const __half2 tau2 = __half2half2(__float2half_rd(p.tau));
+#pragma unroll 1
+            for (int w = tid - 32 * streaming; w < nwords; w += 32 * helpers) keep[w] = keep_word(p.x, p.K, w, tau2);
+            asm volatile("bar.sync 15, %0;" ::"r"(32 * helpers) : "memory");
+#pragma unroll 1
+            for (int w = (int)blockIdx.x + list_blocks * (warp - streaming); w < nwords; w += list_blocks * helpers) {
+                uint32_t before = 0;
+                for (int e = lane; e < w; e += 32) before += (uint32_t)__popc(keep[e]);
+                before = __reduce_add_sync(kFull, before);
+                const uint32_t word = keep[w];
+                if (word >> lane & 1u) {
+                    const int pos = (int)before + __popc(word & ((1u << lane) - 1u)), j = 32 * w + lane;
+                    p.idx[pos] = j;
+                    p.val[pos] = p.x[j];
+                }
+                if (w == nwords - 1 && lane == 0) *p.count = (int)before + __popc(word);
+            }
+        }
+    } else if (p.own_list) {
+        // ---- a1: keep words and the survivors before each of them
         const __half2 tau2 = __half2half2(__float2half_rd(p.tau));   // |x| > tau decided in FP16, as in the fused kernel
         const int nwords = (p.K + 31) >> 5;
         for (int w0 = 0; w0 < nwords; w0 += kColumnThreads) {          // the same trip count for every thread
@@ -136,7 +191,7 @@ __global__ void __launch_bounds__(kColumnThreads, 1) k_spmspv_column(const Colum
 
     // n / blocks columns each, the first n mod blocks one more
     const int share = n / (int)gridDim.x, extra = n - share * (int)gridDim.x, b = (int)blockIdx.x;
-    const int p0 = b * share + min(b, extra), p1 = p0 + share + (b < extra ? 1 : 0);
+    const int p0 = kDealt ? 0 : b * share + min(b, extra), p1 = kDealt ? n : p0 + share + (b < extra ? 1 : 0);
     const int g = idiv_small(warp, p.W), w = warp - g * p.W;
     const bool works = g < p.groups;
     float *const a = acc + (size_t)(works ? g : 0) * Mp;
@@ -144,10 +199,11 @@ __global__ void __launch_bounds__(kColumnThreads, 1) k_spmspv_column(const Colum
     const uint32_t acc0 = smem_u32(a), dump = smem_u32(smem + lay.dump) + 4u * lane;
     uint32_t parity = 0;
     bool out_of_range = false;
-    for (int b0 = p0; b0 < p1; b0 += p.cap) {
+    for (int b0 = p0; b0 < p1; b0 += kDealt ? n : p.cap) {
         // ---- the columns of ranks b0 .. b0 + cnt - 1
-        const int cnt = min(p.cap, p1 - b0);
-        if (p.own_list) {
+        const int cnt = kDealt ? n : min(p.cap, p1 - b0);
+        if (kDealt) {
+        } else if (p.own_list) {
             const int nwords = (p.K + 31) >> 5;
             for (int i = tid; i < cnt; i += kColumnThreads) {
                 // the last word with rank[] <= r, then the bit: halve the word, keep the half with the wanted set bit
@@ -176,7 +232,7 @@ __global__ void __launch_bounds__(kColumnThreads, 1) k_spmspv_column(const Colum
                 imeta[i] = __ldg(p.meta + j);
             }
         }
-        __syncthreads();
+        if (!kDealt) __syncthreads();
         // ---- a2 - a4: this group's columns of the batch
         if (works) {
             const int i1 = idiv_small((g + 1) * cnt, p.groups);          // cnt <= 1024
@@ -201,6 +257,23 @@ __global__ void __launch_bounds__(kColumnThreads, 1) k_spmspv_column(const Colum
                 }
                 next(li, lc);
             };
+            // The rows a chunk spans (Algorithm 1: inclusive scan over the lanes), posted for the group's other warps.
+            struct Spans { uint32_t even, odd, span, sum; };
+            auto scan = [&](const Chunk &ch, int i, int c) {
+                Spans sp;
+                const uint32_t e0 = ((uint32_t)(c + w) * kChunkGroups + lane) * kGroup;
+                uint32_t total;
+                decode_group(ch.runs, sp.even, sp.odd, total);
+                sp.span = i < i1 && e0 < imeta[i].y ? total + kGroup : 0u;
+                sp.sum = sp.span;
+#pragma unroll
+                for (int d = 1; d < 32; d <<= 1) {
+                    const uint32_t prev = __shfl_up_sync(kFull, sp.sum, d);
+                    if (lane >= d) sp.sum += prev;
+                }
+                if (p.W > 1 && lane == 31) spans[32 * parity + w] = sp.sum;
+                return sp;
+            };
             Chunk c0, c1, c2;
             load(c0);
             load(c1);
@@ -208,42 +281,32 @@ __global__ void __launch_bounds__(kColumnThreads, 1) k_spmspv_column(const Colum
             while (pi < i1) {
                 load(c2);
                 const uint32_t nent = imeta[pi].y, e0 = ((uint32_t)(pc + w) * kChunkGroups + lane) * kGroup;
-                uint32_t even, odd, total;
-                decode_group(c0.runs, even, odd, total);
-                const uint32_t span = e0 < nent ? total + kGroup : 0u;
-                uint32_t sum = span;                                   // Algorithm 1: inclusive scan over the lanes
-#pragma unroll
-                for (int d = 1; d < 32; d <<= 1) {
-                    const uint32_t prev = __shfl_up_sync(kFull, sum, d);
-                    if (lane >= d) sum += prev;
-                }
-                uint32_t row0 = carry + sum - span;
-                const uint32_t mine = __shfl_sync(kFull, sum, 31);
+                const Spans now = scan(c0, pi, pc);
+                uint32_t row0 = carry + now.sum - now.span;
                 if (p.W > 1) {
-                    if (lane == 0) spans[32 * parity + w] = mine;
                     asm volatile("bar.sync %0, %1;" ::"r"(1 + g), "r"(32 * p.W) : "memory");
                     const uint32_t t = lane < p.W ? spans[32 * parity + lane] : 0u;
                     row0 += __reduce_add_sync(kFull, lane < w ? t : 0u);
                     carry += __reduce_add_sync(kFull, t);
                     parity ^= 1u;
                 } else {
-                    carry += mine;
+                    carry += __shfl_sync(kFull, now.sum, 31);
                     __syncwarp();                                      // the lanes' stores of the column before this one
                 }
                 const uint16_t xj = (uint16_t)items[pi].y;
                 const uint32_t have = nent > e0 ? min(nent - e0, (uint32_t)kGroup) : 0u;
                 // A lane's rows grow, so its last one tells whether all are in range.
-                const uint32_t last = row0 + entry_offset(even, odd, kGroup - 1);
+                const uint32_t last = row0 + entry_offset(now.even, now.odd, kGroup - 1);
                 uint32_t cell[kGroup];
                 const uint32_t cell0 = acc0 + 4u * row0;
-                cell[0] = __dp4a(even, 0x00000004u, cell0);
-                cell[1] = __dp4a(odd, 0x00000004u, cell0);
-                cell[2] = __dp4a(even, 0x00000400u, cell0);
-                cell[3] = __dp4a(odd, 0x00000400u, cell0);
-                cell[4] = __dp4a(even, 0x00040000u, cell0);
-                cell[5] = __dp4a(odd, 0x00040000u, cell0);
-                cell[6] = __dp4a(even, 0x04000000u, cell0);
-                cell[7] = __dp4a(odd, 0x04000000u, cell0);
+                cell[0] = __dp4a(now.even, 0x00000004u, cell0);
+                cell[1] = __dp4a(now.odd, 0x00000004u, cell0);
+                cell[2] = __dp4a(now.even, 0x00000400u, cell0);
+                cell[3] = __dp4a(now.odd, 0x00000400u, cell0);
+                cell[4] = __dp4a(now.even, 0x00040000u, cell0);
+                cell[5] = __dp4a(now.odd, 0x00040000u, cell0);
+                cell[6] = __dp4a(now.even, 0x04000000u, cell0);
+                cell[7] = __dp4a(now.odd, 0x04000000u, cell0);
                 if (!__all_sync(kFull, have == kGroup && last < (uint32_t)p.M)) {   // the end of a column, or of the image
 #pragma unroll
                     for (int e = 0; e < kGroup; ++e) {
@@ -255,15 +318,15 @@ __global__ void __launch_bounds__(kColumnThreads, 1) k_spmspv_column(const Colum
                 float c[kGroup], d[kGroup];
 #pragma unroll
                 for (int e = 0; e < kGroup; ++e) c[e] = lds_f32(cell[e]);
+                const int before = pi;                                 // (while these loads are on their way: 0.3 us)
+                next(pi, pc);
+                if (pi != before) carry = 0;
                 fma_pair(c0.v.x, xj, c[0], c[1], d[0], d[1]);
                 fma_pair(c0.v.y, xj, c[2], c[3], d[2], d[3]);
                 fma_pair(c0.v.z, xj, c[4], c[5], d[4], d[5]);
                 fma_pair(c0.v.w, xj, c[6], c[7], d[6], d[7]);
 #pragma unroll
                 for (int e = 0; e < kGroup; ++e) sts_f32(cell[e], d[e]);
-                const int before = pi;
-                next(pi, pc);
-                if (pi != before) carry = 0;
                 c0 = c1;
                 c1 = c2;
             }

@@ -448,7 +448,7 @@ __global__ void k_decode_lane(const uint32_t *__restrict__ meta, const uint8_t *
 // asked for), so that steady-state calls make no attribute calls.  The attribute belongs to the kernel,
 // so every entry point that launches a kernel shares that kernel's cache (g_granted_*): two caches for
 // one kernel could disagree about what the runtime currently allows.
-int g_granted_fused[64], g_granted_lean[2][64], g_granted_fused_extras[64], g_granted_lean_extras[2][64], g_granted_batch[2][64], g_granted_column[64], g_granted_lane[64], g_granted_reg[4][64];
+int g_granted_fused[64], g_granted_lean[2][64], g_granted_fused_extras[64], g_granted_lean_extras[2][64], g_granted_batch[2][64], g_granted_column[2][64], g_granted_lane[64], g_granted_reg[4][64];
 
 template <typename Kernel>
 int ensure_smem(Kernel kernel, size_t bytes, int *granted /* [64], per device */)
@@ -1128,8 +1128,10 @@ int run_product(celty_matrix *m, const void *x_dev, float tau, const ListInput *
     // untouched.
     if (m->layout == CELTY_LAYOUT_COLUMN) {
         const int grid = m->grid > 0 ? m->grid : di.sms;
-        const ColumnShape shape = column_shape(m->M, m->K, m->stream_bytes, (size_t)di.max_smem_optin, grid);
+        ColumnShape shape = column_shape(m->M, m->K, m->stream_bytes, (size_t)di.max_smem_optin, grid);
         if (shape.groups == 0) return CELTY_EINVAL;
+        DirectGroups groups;
+        const bool dealt = column_dealt(m->M, m->K, m->stream_bytes, grid, (size_t)di.max_smem_optin, &shape, &groups);
         ColumnParams cp{};
         cp.meta = reinterpret_cast<const uint2 *>(m->d_image);
         cp.stream = stream_base;
@@ -1139,21 +1141,31 @@ int run_product(celty_matrix *m, const void *x_dev, float tau, const ListInput *
         cp.y = y;
         cp.M = (int)m->M; cp.K = (int)m->K;
         cp.W = shape.W; cp.groups = shape.groups; cp.cap = shape.cap; cp.own_list = shape.own_list;
-        rc = ensure_smem(k_spmspv_column, shape.smem, g_granted_column);
+        size_t smem = shape.smem;
+        if (dealt) {
+            cp.sizes = groups.sizes[0];
+            cp.rankers = groups.rankers;
+            cp.rankers_inv = 1.f / (float)groups.rankers;
+            cp.dealt = (uint32_t)smem;
+            cp.most = groups.most;
+            smem += (size_t)groups.most * 16;
+        }
+        const auto kernel = dealt ? k_spmspv_column<true> : k_spmspv_column<false>;
+        rc = ensure_smem(kernel, smem, g_granted_column[dealt]);
         if (rc) return rc;
         rc = shape.own_list ? launch_clear(y, m->M, st) : launch_compact(x_dev, m->K, tau, idx, val, count, y, m->M, st);
         if (rc) return rc;
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3((unsigned)grid);
         cfg.blockDim = dim3(kColumnThreads);
-        cfg.dynamicSmemBytes = shape.smem;
+        cfg.dynamicSmemBytes = smem;
         cfg.stream = st;
         cudaLaunchAttribute attr[1];
         attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
         attr[0].val.programmaticStreamSerializationAllowed = 1;
         cfg.attrs = attr;
         cfg.numAttrs = 1;
-        CELTY_CUDA(cudaLaunchKernelEx(&cfg, k_spmspv_column, cp));
+        CELTY_CUDA(cudaLaunchKernelEx(&cfg, kernel, cp));
     } else {
         const size_t group_bytes = (size_t)m->S * (m->R + kTileSlack) * 32 * 4;
         if (group_bytes > (size_t)di.max_smem_optin) return CELTY_EINVAL;
