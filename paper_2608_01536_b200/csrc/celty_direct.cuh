@@ -34,10 +34,20 @@
 //   276 (20000 x 8000, 0.5)                 26.15 -> 26.06
 //   332 (16384 x 12288, 0.1 / 0.5 / 0.7)    10.89 -> 9.99, 30.57 -> 30.50, 40.26 -> 39.78
 //   387 (8192 x 28672, 0.3 / 0.5)           24.55 -> 23.59, 35.47 -> 34.38
-// and batches: 4096 x 4096, N = 4 / 8  15.14 -> 13.57, 24.77 -> 23.35;  11008 x 4096, N = 4  27.92 -> 25.74.  The gain shrinks with the
+// The gain shrinks with the
 // columns, whose streaming outgrows what is saved ahead of it; the line, 512 (four members' columns at four per lane), lies beyond
-// what was measured.  One vector of a layer whose left-over blocks serve several row parts is k_spmspv_fused's (28672 x 8192 at
-// 50 %: 33.3, here 33.6, though at 10 % 11.7 and 10.9).
+// what was measured.  Where k_spmspv_fused lets the left-over blocks serve several row parts (one vector, eight or twelve parts), which
+// saves it 2 % of the streaming, the line is 384:
+//   144 (28672 x 2600, 0.1 / 0.3 / 0.5 / 0.7)   7.18 -> 6.19, 11.38 -> 9.79, 15.10 -> 14.44, 18.79 -> 17.80
+//   228 (28672 x 4096, 0.1 / 0.3 / 0.5 / 0.7)   8.30 -> 7.39, 15.06 -> 13.89, 19.94 -> 19.63, 25.63 -> 24.71
+//   361 (28672 x 6500, 0.1 / 0.3 / 0.5 / 0.7)   10.58 -> 9.80, 19.88 -> 19.02, 27.76 -> 27.58, 36.26 -> 36.32
+//   455 (28672 x 8192, 0.1 / 0.5)               11.7 -> 10.9, 33.3 -> 33.6
+// and for several vectors, with so many groups that one of them is far from the mean, columns times rows per lane may be 20 000 (N
+// vectors at 50 %; the last three beyond the line):
+//   4096 x 4096, N = 4 / 5 (14 100, 18 000)     14.3 -> 13.4, 17.3 -> 15.9
+//   2048 x 6200, N = 4 (10 700)                 12.1 -> 11.0;     2000 x 9000, N = 4 (15 600)   15.6 -> 14.1
+//   2558 x 6286, N = 6 (21 000)                 17.7 -> 17.8 (with 39 % of the weights 16.7 -> 18.3)
+//   6000 x 3000, N = 6 (24 000)                 18.2 -> 18.9;     4928 x 3456, N = 7 (27 600)   20.1 -> 19.9 (35 %: 20.7 -> 23.3)
 // Runs of two, so that survivors that lie together in x (zeroed heads of an attention output) are shared about as evenly as independent ones.
 // A list is shared evenly whatever its length; the second
 // product of the 5504 x 2048 MLP chain gains 1.9 of 15.4 us from this kernel.

@@ -503,7 +503,7 @@ int launch_compact(const void *x, int64_t K, float tau, int32_t *idx, uint16_t *
 
 constexpr int kMostToMix = 48;           // left-over blocks are shared between row parts up to this (fit_clusters)
 
-constexpr int kDirectMost = 128, kGroupsMost = 512;      // columns of a block of k_spmspv_direct, of k_spmspv_fused_groups (see there)
+constexpr int kDirectMost = 128, kGroupsMost = 512, kMixesMost = 384, kBatchMost = 20000;      // columns of a block of k_spmspv_direct, of k_spmspv_fused_groups (see there)
 
 int direct_threads(int G, int pairs) { return 32 * (pairs ? 16 + kDirectHelpers + 1 : std::max(16, G + kDirectHelpers + 1)); }
 
@@ -545,8 +545,9 @@ int plan_fused(const celty_matrix *m, const LaunchKnobs &knobs, const DeviceInfo
     const int64_t columns = (m->K + per_part - 1) / per_part;
     const int left = pl.grid % pl.P;
     const bool mixes = left > 0 && pl.P % left == 0 && (int64_t)(pl.P / left) * per_part <= kMostToMix;    // see fit_clusters
+    const int64_t most_columns = vectors > 1 ? std::max<int64_t>(kDirectMost, std::min<int64_t>(kGroupsMost, kBatchMost / m->R)) : mixes ? kMixesMost : kGroupsMost;
     pl.direct = reg_rows == 0 && knobs.merge != 0 && knobs.cluster <= 1 && knobs.lean != 0 && knobs.mix <= 0 && pl.Sc == 1 &&
-                (list ? !mixes && m->K / per_part < 4096 : columns <= (mixes && vectors == 1 ? kDirectMost : kGroupsMost));
+                (list ? !mixes && m->K / per_part < 4096 : columns <= most_columns);
     pl.wide = pl.direct && !list && columns > kDirectMost;
     auto smem_bytes = [&](int G, int D) {
         if (!pl.direct) return fused_smem_bytes(m->R, (int)m->K, G, pl.Sc, D, pl.slot_bytes, pl.cap);
@@ -593,11 +594,12 @@ int plan_fused(const celty_matrix *m, const LaunchKnobs &knobs, const DeviceInfo
     //   6 to 9, at most 7 teams:  1 to 3 % faster from 30 % on (11008 x 2048, 16384 x 2048), level at 10 %;
     //   6 to 9, 8 teams:  1 to 3 % slower at 10 %, level at 50 % (4096 x 4096, 1024 x 4096): not taken;
     //   9 teams, of which pairs leave 8:  5 to 8 % faster (13824 x 5120 with 30 % of the weights, 3000 x 28672);
-    //   11 teams or more:  6 % slower at 70 % (5120 x 13824): not taken.
+    //   10 teams:  2 to 3 % faster at 15 and 50 % (5000 x 17000 with 70 % of the weights 20.1 -> 19.5 us, five vectors of 3000 x 7000 18.8 -> 18.4);
+    //   11 teams or more:  1 to 3 % faster at 15 %, 1 to 6 % slower from 50 % on (5120 x 13824, 2300 x 20000): not taken.
     if (reg_rows == 0 && knobs.pairs != 0 && pl.G > 0 && pl.Sc <= 8) {             // a pair is warps t and t + 8
         const int teams_per_part = std::max(1, pl.grid / pl.P) * pl.G;
         const int64_t columns = m->K / teams_per_part;
-        if (knobs.pairs > 0 || (pl.G * pl.Sc <= 9 && columns >= (pl.G * pl.Sc <= 7 ? 6 : 9))) {
+        if (knobs.pairs > 0 || (pl.G * pl.Sc <= 10 && columns >= (pl.G * pl.Sc <= 7 ? 6 : 9))) {
             const FusedPlan keep = pl;
             fit(1);
             if (pl.G == 0) pl = keep;
