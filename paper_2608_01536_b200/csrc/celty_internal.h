@@ -413,7 +413,8 @@ inline ColumnShape column_shape(int64_t M, int64_t K, size_t stream_bytes, size_
 
 // Whether the COLUMN kernel's blocks get their columns dealt (k_spmspv_direct): up to 128 columns per block, at least two warps that
 // do not stream, for the list, with a named barrier of their own, and room for the columns.  Where all warps stream, four of those that
-// take a column each are given up, or one of several on a column if the others need no pass more for it.  A block may have one or two
+// take a column each are given up, or columns in flight that the block's share does not fill, or one of several warps on a column if the
+// others need no pass more for it.  A block may have one or two
 // columns more than the mean, so where a block's columns take long (more passes over one than there are others in flight) survivors
 // are ranked: dealt, 28672 x 8192 at 20 % took 49.8 us instead of 43.4, 20000 x 4000 at 30 % 29.6 instead of 26.6.
 inline bool column_dealt(int64_t M, int64_t K, size_t stream_bytes, int grid, size_t budget, ColumnShape *shape, DirectGroups *g)
@@ -423,6 +424,8 @@ inline bool column_dealt(int64_t M, int64_t K, size_t stream_bytes, int grid, si
     const double chunks = (double)stream_bytes / 20.0 / (double)K / kChunkGroups + 0.1;
     const int most = s.W == 1 ? 28 : 30;                          // warps that stream
     if (s.W == 1) s.groups = std::min(s.groups, most);
+    const int64_t share = std::max<int64_t>(1, (K / 2 + grid - 1) / grid);           // as in column_shape
+    while (s.W > 1 && s.groups > 1 && (s.W * s.groups > 28 || s.groups > 14) && (share + s.groups - 2) / (s.groups - 1) == (share + s.groups - 1) / s.groups) --s.groups;
     while (s.W > 2 && s.W * s.groups > most && std::ceil(chunks / (s.W - 1)) == std::ceil(chunks / s.W)) --s.W;
     if (std::ceil(chunks / s.W) > s.groups || s.W * s.groups > most || (s.W > 1 && s.groups > 14)) return false;
     const int warps = std::min(16, s.W * s.groups);
