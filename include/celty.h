@@ -412,7 +412,7 @@ int celty_last_status(celty_matrix *m, celty_stream_t stream);
  *            16 = always / 32 = never run warp pairs: two warps per team that take turns at the team's
  *            accumulator, one waiting for its next sub-block and reading its header while the other runs its
  *            steps (by default the library pairs warps where a team has nine or more columns to stream, or six with at most
- *            seven teams to a block, and in place of nine teams),
+ *            seven teams to a block, and in place of nine or ten teams),
  *            64 = never / 128 = wherever possible share a thread block between row parts.  (With the bulk
  *            reduce-add merge and no clusters: when the blocks do not divide by the row parts and the blocks left
  *            over can be shared evenly, each of them can serve several parts with correspondingly fewer teams per
@@ -421,10 +421,9 @@ int celty_last_status(celty_matrix *m, celty_stream_t stream);
  *            256 = run the build of the fused kernel that has every option compiled in even where the launch is
  *            the default one (bulk reduce-add merge, no clusters), for which the library otherwise uses smaller
  *            builds without the other options' code (same results; the smaller builds are faster).  With 128 or 256 the
- *            blocks always share a ranked list of the survivors; by default a layer of at most 128 columns per block has
- *            its columns dealt to the blocks whatever x is, in runs of two.  That takes 5 to 23 % less time on layers of up
- *            to 75 columns per block, whether or not the survivors lie together in x (zeroed heads, one stretch), and
- *            between 18 % less and 3 % more on layers of 84 to 128.
+ *            blocks always share a ranked list of the survivors; by default a layer of at most 512 columns per block (384
+ *            where blocks left over can be shared, 20 000 / tile rows in a batch) has its columns dealt to groups of blocks
+ *            whatever x is, in runs of two, and the blocks of a group share its survivors.  That takes 1 to 25 % less time.
  *   groups   fused kernel: warp teams per slab working on different columns (each has an accumulator)
  *   depth    fused kernel: bulk copies each team keeps in flight (ring slots)
  *   cluster  fused kernel, bulk reduce-add merge: thread blocks per cluster (1, 2 or 4); the blocks of a
