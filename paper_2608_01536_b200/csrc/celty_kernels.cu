@@ -884,6 +884,13 @@ namespace {
 constexpr int kUploadThreads = 8, kUploadSlots = 2;               // slots per thread: one is filled while the other's copy is on its way
 constexpr size_t kUploadPiece = (size_t)512 << 10;
 
+// Another thread's stream capture (of the mode that watches all threads) does not mind this thread's allocations and waits.
+struct RelaxedCapture {
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+    ~RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+};
+
 struct Staging {
     std::mutex mu;
     uint8_t *memory = nullptr;
@@ -919,6 +926,7 @@ cudaError_t upload(void *to, const uint8_t *from, size_t bytes, cudaStream_t st)
     cudaError_t err = cudaStreamIsCapturing(st, &capturing);
     if (err == cudaSuccess) err = cudaGetDevice(&dev);
     if (err != cudaSuccess) return err;
+    RelaxedCapture relaxed;
     Staging &stage = staging();
     std::unique_lock<std::mutex> lock(stage.mu, std::defer_lock);
     const bool staged = capturing == cudaStreamCaptureStatusNone && bytes >= kUploadPiece && lock.try_lock();
@@ -937,6 +945,7 @@ cudaError_t upload(void *to, const uint8_t *from, size_t bytes, cudaStream_t st)
     std::atomic<int64_t> next(0);
     std::atomic<int> failed((int)cudaSuccess);
     auto work = [&](int thread) {
+        RelaxedCapture relaxed_too;
         cudaError_t e = cudaSetDevice(dev);
         for (int64_t i, k = 0; e == cudaSuccess && failed == (int)cudaSuccess && (i = next.fetch_add(1)) < pieces; ++k) {
             const int slot = thread * kUploadSlots + (int)(k % kUploadSlots);
@@ -971,6 +980,7 @@ cudaError_t upload(void *to, const uint8_t *from, size_t bytes, cudaStream_t st)
 
 extern "C" int celty_release_staging(void)
 {
+    RelaxedCapture relaxed;
     Staging &stage = staging();
     std::lock_guard<std::mutex> lock(stage.mu);
     if (!stage.memory) return CELTY_OK;

@@ -57,3 +57,35 @@ def test_uploads_of_several_threads_and_streams():
         t.join()
     celty.release_staging()
     assert not bad
+
+
+def test_an_upload_beside_another_threads_capture():
+    """A capture that watches all threads goes on while another thread takes the page-locked memory and uploads."""
+    celty.release_staging()
+    m, small = _matrix(6 * PIECE, 3), celty.Matrix(synth.integer_weights(1, 64, 64), device="cuda")
+    x = torch.ones(64, dtype=torch.float16, device="cuda")
+    small.spmspv(x, 0.5)
+    buffers = [torch.empty(b, dtype=torch.uint8, device="cuda") for b in m.device_bytes()]
+    stream, bad = torch.cuda.Stream(), []
+    torch.cuda.synchronize()
+
+    def work():
+        try:
+            torch.cuda.set_device(0)
+            celty._check(celty.load().celty_bind_device(m._h, buffers[0].data_ptr(), buffers[0].numel(), buffers[1].data_ptr(),
+                                                        buffers[1].numel(), stream.cuda_stream), "celty_bind_device")
+        except BaseException as e:                                # noqa: BLE001
+            bad.append(e)
+
+    y = torch.empty(64, device="cuda")
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        small.spmspv(x, 0.5, y=y)
+        t = threading.Thread(target=work)
+        t.start()
+        t.join()
+    graph.replay()
+    torch.cuda.synchronize()
+    assert not bad
+    assert np.array_equal(buffers[0].cpu().numpy(), m.host_image()[0])
+    assert np.array_equal(y.cpu().numpy(), small.spmspv(x, 0.5).cpu().numpy())
