@@ -1288,7 +1288,7 @@ extern "C" int celty_spmspv_static(const celty_matrix *m, const void *image_dev,
     // The kernel of celty_spmspv behind one that clears y.  With a ticket in the shared array instead, as the workspace's
     // calls have it, blocks would wait for one another: next to a kernel of another stream that keeps some of the SMs
     // they could give up, and a caller without a workspace has no status word to find out by.  4096 x 4096, 50 % / 50 %:
-    // 28.7 us with the two kernels below, 7.0 us this way (with a ticket 6.1).  The handle's launch choices are for its
+    // 28.7 us with the two kernels below, 6.5 us this way (with a ticket 5.7).  The handle's launch choices are for its
     // workspace's calls and are not looked at, but for the limit of the waits.
     FusedPlan plan;
     LaunchKnobs knobs;
@@ -1334,8 +1334,8 @@ namespace {
 // A batch through the single-launch kernel.  One launch serves several vectors at once, each with its share of the
 // blocks: a vector's product streams no faster than before on as much of the chip as it has, but the part of a call
 // that does not stream -- thresholding, look-ups, the latency of the first copies, the merge, the change of kernels,
-// some 5 us -- is paid once for all of them (50 % / 50 %, 4096 x 4096, four vectors: 26.3 us in four launches,
-// 15.5 us in one; 11008 x 4096, eight vectors: 84.1 and 51.7).  How many vectors share a launch is chosen by that trade:
+// some 5 us -- is paid once for all of them (50 % / 50 %, 4096 x 4096, four vectors: 23.9 us in four launches,
+// 13.9 us in one; 11008 x 4096, eight vectors: 75.5 and 51.7).  How many vectors share a launch is chosen by that trade:
 // fixed time against what the division of the blocks loses when they do not divide by vectors and row parts (5 vectors of a layer of 8 row parts: 29
 // blocks for 8 parts leaves five parts with one block more than the other three).
 int run_batch(celty_matrix *m, const uint16_t *x, int64_t ldx, int N, float tau, float *y, int64_t ldy,
@@ -1418,7 +1418,7 @@ extern "C" int celty_spmspv_batch(celty_matrix *m, const void *x_dev, int64_t ld
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     // Measured, the widened kernels below lose to the single-vector kernel at every N (N accumulators per warp leave room
     // for fewer warps, and the union of N activation patterns is nearly every column from N = 4 on; 4096 x 4096, N = 2 / 4 /
-    // 8: 42 / 94 / 253 us against 9.6 / 15.5 / 25.3): unless the two-launch variant is asked for, the batch goes to
+    // 8: 41 / 94 / 251 us against 9.2 / 13.9 / 25.4): unless the two-launch variant is asked for, the batch goes to
     // run_batch where the handle has its workspace and every row of x and y starts on a 16-byte boundary.
     if (m->variant == 0 && m->d_ws && !(((uintptr_t)x_dev | (uintptr_t)(ldx * 2) | (uintptr_t)y_dev | (uintptr_t)(ldy * 4)) & 15)) {
         return run_batch(m, static_cast<const uint16_t *>(x_dev), ldx, N, tau, static_cast<float *>(y_dev), ldy, stream);
