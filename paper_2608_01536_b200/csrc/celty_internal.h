@@ -333,6 +333,8 @@ struct FusedPlan {
     int lean;                  // 0: every option compiled in; 1 / 2: the builds for the default launch (without / with warp pairs)
     int direct;                // 1: columns are dealt (k_spmspv_direct, k_spmspv_fused_groups)
     int wide;                  // 1: k_spmspv_fused_groups
+    DirectGroups groups;       // of its blocks (not from a list)
+    DirectSmem tables;         // its shared memory
     size_t smem;
 };
 
@@ -436,6 +438,14 @@ inline bool column_dealt(int64_t M, int64_t K, size_t stream_bytes, int grid, si
     return true;
 }
 
+// A COLUMN launch worked out once for a handle and a device.
+struct PreparedColumn {
+    int device = -1;           // -1: not worked out
+    ColumnShape shape{};
+    DirectGroups groups{};
+    bool dealt = false;
+};
+
 // Launch choices of a handle (celty_set_launch and its neighbours); a default-constructed one is the library's.
 struct LaunchKnobs {
     int32_t grid = 0, variant = 0, groups = 0, depth = 0, cluster = 0;
@@ -479,5 +489,10 @@ struct celty_matrix : celty::LaunchKnobs {
     int32_t last_grid = 0, last_merge = -1;   // what the tickets in the workspace were last used with
     int32_t last_batch_grid[9] = {};          // the same for the tickets of launches that serve 2 .. 8 vectors
     celty::PreparedLaunch prepared[9];        // [0] one vector, [1] one from a list, [v] launches that serve v = 2 .. 8
-    void forget_launches() { for (celty::PreparedLaunch &p : prepared) p.device = -1; }   // the handle has changed
+    celty::PreparedColumn prepared_column;
+    void forget_launches()                    // the handle has changed
+    {
+        for (celty::PreparedLaunch &p : prepared) p.device = -1;
+        prepared_column.device = -1;
+    }
 };

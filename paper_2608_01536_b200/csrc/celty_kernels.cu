@@ -621,7 +621,11 @@ int plan_fused(const celty_matrix *m, const LaunchKnobs &knobs, const DeviceInfo
         pl.window = (int)(std::min(wanted, budget - pl.smem) / 128 * 128);
         pl.smem += (size_t)pl.window;
     }
-    if (pl.direct) pl.cap = direct_cap(m, pl.grid, pl.P, pl.G, pl.pp, list, pl.wide);
+    if (pl.direct) {
+        pl.cap = direct_cap(m, pl.grid, pl.P, pl.G, pl.pp, list, pl.wide);
+        if (!list) pl.groups = direct_groups(m, pl.grid, pl.P, pl.threads, pl.wide);
+        pl.tables = direct_smem_layout(m->R, (int)m->K, pl.G, pl.D, pl.slot_bytes, pl.cap);
+    }
     pl.merge = (knobs.merge >= 0 ? knobs.merge : 1);
     // Clusters (bulk reduce-add merge only, on request): as long as the grid is made of whole clusters, every row
     // part gets at least one, and the device can hold them all at once.
@@ -760,6 +764,20 @@ int prepared_launch(celty_matrix *m, const DeviceInfo &di, int vectors, bool lis
     return p.status;
 }
 
+// The same for the COLUMN kernel, whose calls on small layers are bound by the host as well (0.4 us).
+PreparedColumn prepared_column(celty_matrix *m, const DeviceInfo &di, int grid)
+{
+    static std::mutex mu;
+    std::lock_guard<std::mutex> lock(mu);
+    PreparedColumn &p = m->prepared_column;
+    if (p.device != di.device) {
+        p.shape = column_shape(m->M, m->K, m->stream_bytes, (size_t)di.max_smem_optin, grid);
+        p.dealt = p.shape.groups > 0 && column_dealt(m->M, m->K, m->stream_bytes, grid, (size_t)di.max_smem_optin, &p.shape, &p.groups);
+        p.device = di.device;
+    }
+    return p;
+}
+
 // Programmatic dependent launch: the kernel may be scheduled while the previous kernel of the stream drains; it
 // waits for that kernel (griddepcontrol.wait) before it reads or writes anything of the call.
 template <typename Params>
@@ -807,20 +825,20 @@ DirectBuild direct_build(const FusedPlan &plan, bool list, int held)
                      : DirectBuild{k_spmspv_fused_groups<kPairs, kBatch, 4>, granted[4]};
 }
 
-DirectBuild direct_build(const celty_matrix *m, const FusedPlan &plan, bool batch, bool list)
+DirectBuild direct_build(const FusedPlan &plan, bool batch, bool list)
 {
-    const int held = list ? 0 : direct_groups(m, plan.grid, plan.P, plan.threads, plan.wide).held;
+    const int held = list ? 0 : plan.groups.held;
     if (batch) return plan.pp ? direct_build<true, true>(plan, false, held) : direct_build<false, true>(plan, false, held);
     return plan.pp ? direct_build<true, false>(plan, list, held) : direct_build<false, false>(plan, list, held);
 }
 
-int launch_direct(const celty_matrix *m, const LaunchKnobs &knobs, const FusedPlan &plan, int vectors, bool list, const FusedParams &fp, cudaStream_t st)
+int launch_direct(const LaunchKnobs &knobs, const FusedPlan &plan, int vectors, bool list, const FusedParams &fp, cudaStream_t st)
 {
-    const DirectBuild b = direct_build(m, plan, vectors > 1, list);
+    const DirectBuild b = direct_build(plan, vectors > 1, list);
     DirectParams p{};
     p.meta = fp.meta; p.stream = fp.stream;
     p.K = fp.K; p.S = fp.S; p.P = fp.P; p.G = fp.G; p.R = fp.R; p.D = fp.D; p.M = fp.M; p.C = fp.C;
-    p.lay = direct_smem_layout(fp.R, fp.K, plan.G, plan.D, plan.slot_bytes, plan.cap);
+    p.lay = plan.tables;
     p.image_early = fp.image_early;
     p.x = fp.x; p.ldx = fp.ldx; p.tau = fp.tau;
     p.G_inv = (65535u + plan.G) / plan.G;
@@ -833,7 +851,7 @@ int launch_direct(const celty_matrix *m, const LaunchKnobs &knobs, const FusedPl
         p.list.idx = fp.list_idx; p.x = fp.list_val; p.list_count = fp.list_count;
         p.list.units_inv = fp.units_inv; p.list.units_inv_long = fp.units_inv_long;
     } else {
-        const DirectGroups g = direct_groups(m, plan.grid, plan.P, plan.threads, plan.wide);
+        const DirectGroups &g = plan.groups;
         p.sizes[0] = g.sizes[0]; p.sizes[1] = g.sizes[1];
         p.rankers = g.rankers;
         p.rankers_inv = 1.f / (float)g.rankers;
@@ -1113,7 +1131,7 @@ int run_product(celty_matrix *m, const void *x_dev, float tau, const ListInput *
             m->last_merge = plan.merge;
         }
         if (plan.direct)
-            rc = launch_direct(m, *m, plan, 1, list != nullptr, fp, st);
+            rc = launch_direct(*m, plan, 1, list != nullptr, fp, st);
         else if (list)                                           // the list input has builds of its own
             rc = plan.lean == 2 ? launch_fused(k_spmspv_fused<true, 0, 2>, g_granted_lean_extras[1], *m, plan, 1, fp, st)
                : plan.lean == 1 ? launch_fused(k_spmspv_fused<true, 0, 1>, g_granted_lean_extras[0], *m, plan, 1, fp, st)
@@ -1140,10 +1158,11 @@ int run_product(celty_matrix *m, const void *x_dev, float tau, const ListInput *
     // untouched.
     if (m->layout == CELTY_LAYOUT_COLUMN) {
         const int grid = m->grid > 0 ? m->grid : di.sms;
-        ColumnShape shape = column_shape(m->M, m->K, m->stream_bytes, (size_t)di.max_smem_optin, grid);
+        const PreparedColumn pc = prepared_column(m, di, grid);
+        const ColumnShape &shape = pc.shape;
+        const DirectGroups &groups = pc.groups;
+        const bool dealt = pc.dealt;
         if (shape.groups == 0) return CELTY_EINVAL;
-        DirectGroups groups;
-        const bool dealt = column_dealt(m->M, m->K, m->stream_bytes, grid, (size_t)di.max_smem_optin, &shape, &groups);
         ColumnParams cp{};
         cp.meta = reinterpret_cast<const uint2 *>(m->d_image);
         cp.stream = stream_base;
@@ -1307,13 +1326,13 @@ extern "C" int celty_spmspv_static(const celty_matrix *m, const void *image_dev,
         fp.win_cols = 0;
         // (the limit is raised before the first launch: an error return leaves y untouched)
         fp.image_early = 0;
-        const DirectBuild direct = plan.direct ? direct_build(m, plan, false, false) : DirectBuild{};
+        const DirectBuild direct = plan.direct ? direct_build(plan, false, false) : DirectBuild{};
         rc = plan.direct ? ensure_smem(direct.kernel, plan.smem, direct.granted)
            : plan.lean == 2 ? ensure_smem(k_spmspv_fused<false, 0, 2>, plan.smem, g_granted_lean[1])
                             : ensure_smem(k_spmspv_fused<false, 0, 1>, plan.smem, g_granted_lean[0]);
         if (rc == CELTY_OK) rc = launch_clear(y, m->M, st);
         if (rc) return rc;
-        if (plan.direct) return launch_direct(m, knobs, plan, 1, false, fp, st);
+        if (plan.direct) return launch_direct(knobs, plan, 1, false, fp, st);
         return plan.lean == 2 ? launch_fused(k_spmspv_fused<false, 0, 2>, g_granted_lean[1], knobs, plan, 1, fp, st)
                               : launch_fused(k_spmspv_fused<false, 0, 1>, g_granted_lean[0], knobs, plan, 1, fp, st);
     }
@@ -1393,7 +1412,7 @@ int run_batch(celty_matrix *m, const uint16_t *x, int64_t ldx, int N, float tau,
             m->last_batch_grid[v] = plan.grid;
         }
         if (plan.direct)
-            rc = launch_direct(m, *m, plan, v, false, fp, st);
+            rc = launch_direct(*m, plan, v, false, fp, st);
         else
             rc = plan.lean == 2 ? launch_fused(k_spmspv_fused<false, 0, 2, true>, g_granted_batch[1], *m, plan, v, fp, st)
                             : launch_fused(k_spmspv_fused<false, 0, 1, true>, g_granted_batch[0], *m, plan, v, fp, st);
