@@ -1,4 +1,4 @@
-"""Builds the C-ABI CUDA library in-tree, csrc/celty_host.cpp and csrc/*.cu -> libcelty.so (sm_100a only), and the module
+"""Builds the C-ABI CUDA library in-tree, csrc/celty_host.cpp, csrc/celty_upload.cpp and csrc/*.cu -> libcelty.so (sm_100a only), and the module
 behind the Python binding, csrc/celty_torch.cpp -> _celty_torch.so."""
 from __future__ import annotations
 
@@ -10,8 +10,8 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libcelty.so")
-SOURCES = [os.path.join(CSRC, "celty_host.cpp"), os.path.join(CSRC, "celty_kernels.cu")]
-HEADERS = [os.path.join(CSRC, "celty_internal.h"), os.path.join(CSRC, "celty_fused.cuh"), os.path.join(CSRC, "celty_direct.cuh"), os.path.join(CSRC, "celty_column.cuh"),
+SOURCES = [os.path.join(CSRC, "celty_host.cpp"), os.path.join(CSRC, "celty_upload.cpp"), os.path.join(CSRC, "celty_kernels.cu")]
+HEADERS = [os.path.join(CSRC, "celty_internal.h"), os.path.join(CSRC, "celty_upload.h"), os.path.join(CSRC, "celty_fused.cuh"), os.path.join(CSRC, "celty_direct.cuh"), os.path.join(CSRC, "celty_column.cuh"),
            os.path.join(ROOT, "include", "celty.h")]
 
 

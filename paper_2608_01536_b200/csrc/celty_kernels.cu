@@ -5,14 +5,12 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
-#include <atomic>
 #include <cmath>
 #include <cstdio>
-#include <exception>
 #include <mutex>
-#include <thread>
 
 #include "celty_internal.h"
+#include "celty_upload.h"
 
 using namespace celty;
 
@@ -892,120 +890,9 @@ extern "C" int celty_launch_plan(const celty_matrix *m, int32_t *out, int32_t n)
 }
 
 
-namespace {
-
-// Host-to-device copies of images through page-locked memory.  A copy from pageable memory is one host thread's in the driver, 4
-// GB/s; here up to kUploadThreads threads copy pieces into slots of their own and enqueue the copies from there, on the
-// caller's stream.  celty_bind_device of an image of 11 MB: 2.6 -> 0.85 ms, of 56 MB: 6.1 -> 2.6 (4 threads 1.0 and 3.4; pieces of 256 KB 0.97
-// and 3.7; of 1 MB 0.9 and 2.2, for twice the memory).  The 8 MB are taken by the first upload, used by one upload at a time (another one
-// meanwhile goes the pageable way) and given back by celty_release_staging.
-constexpr int kUploadThreads = 8, kUploadSlots = 2;               // slots per thread: one is filled while the other's copy is on its way
-constexpr size_t kUploadPiece = (size_t)512 << 10;
-
-// Another thread's stream capture (of the mode that watches all threads) does not mind this thread's allocations and waits.
-struct RelaxedCapture {
-    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
-    RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
-    ~RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
-};
-
-struct Staging {
-    std::mutex mu;
-    uint8_t *memory = nullptr;
-    cudaEvent_t done[kUploadThreads * kUploadSlots] = {};         // of a slot's last copy; null: the slot is free
-    int device[kUploadThreads * kUploadSlots] = {};               // that the event belongs to
-
-    // All copies have left their slots (mu is held).
-    cudaError_t wait()
-    {
-        cudaError_t first = cudaSuccess;
-        for (cudaEvent_t &e : done) {
-            if (!e) continue;
-            const cudaError_t err = cudaEventSynchronize(e);
-            if (first == cudaSuccess) first = err;
-            cudaEventDestroy(e);
-            e = nullptr;
-        }
-        return first;
-    }
-};
-
-Staging &staging()
-{
-    static Staging *s = new Staging;                              // (never destroyed: the runtime may be gone by then)
-    return *s;
-}
-
-// What a stream capture would have to replay, small images and those that come while the staging memory is in use go the pageable way.
-cudaError_t upload(void *to, const uint8_t *from, size_t bytes, cudaStream_t st)
-{
-    cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusActive;
-    int dev = 0;
-    cudaError_t err = cudaStreamIsCapturing(st, &capturing);
-    if (err == cudaSuccess) err = cudaGetDevice(&dev);
-    if (err != cudaSuccess) return err;
-    RelaxedCapture relaxed;
-    Staging &stage = staging();
-    std::unique_lock<std::mutex> lock(stage.mu, std::defer_lock);
-    const bool staged = capturing == cudaStreamCaptureStatusNone && bytes >= kUploadPiece && lock.try_lock();
-    if (staged && !stage.memory &&
-        cudaHostAlloc(&stage.memory, kUploadThreads * kUploadSlots * kUploadPiece, cudaHostAllocPortable) != cudaSuccess) {
-        stage.memory = nullptr;
-        (void)cudaGetLastError();
-    }
-    if (!staged || !stage.memory) return cudaMemcpyAsync(to, from, bytes, cudaMemcpyHostToDevice, st);
-    for (int i = 0; i < kUploadThreads * kUploadSlots; ++i)       // events of another device cannot be recorded here
-        if (stage.done[i] && stage.device[i] != dev) {
-            if ((err = stage.wait()) != cudaSuccess) return err;
-            break;
-        }
-    const int64_t pieces = (int64_t)((bytes + kUploadPiece - 1) / kUploadPiece);
-    std::atomic<int64_t> next(0);
-    std::atomic<int> failed((int)cudaSuccess);
-    auto work = [&](int thread) {
-        RelaxedCapture relaxed_too;
-        cudaError_t e = cudaSetDevice(dev);
-        for (int64_t i, k = 0; e == cudaSuccess && failed == (int)cudaSuccess && (i = next.fetch_add(1)) < pieces; ++k) {
-            const int slot = thread * kUploadSlots + (int)(k % kUploadSlots);
-            uint8_t *const at = stage.memory + (size_t)slot * kUploadPiece;
-            const size_t n = std::min(kUploadPiece, bytes - (size_t)i * kUploadPiece);
-            if (!stage.done[slot]) {
-                e = cudaEventCreateWithFlags(&stage.done[slot], cudaEventDisableTiming);
-                stage.device[slot] = dev;
-            } else {
-                e = cudaEventSynchronize(stage.done[slot]);
-            }
-            if (e != cudaSuccess) break;
-            std::memcpy(at, from + (size_t)i * kUploadPiece, n);
-            e = cudaMemcpyAsync(static_cast<uint8_t *>(to) + (size_t)i * kUploadPiece, at, n, cudaMemcpyHostToDevice, st);
-            if (e == cudaSuccess) e = cudaEventRecord(stage.done[slot], st);
-        }
-        if (e != cudaSuccess) failed = (int)e;
-    };
-    std::vector<std::thread> threads;
-    try {
-        const int64_t want = std::min<int64_t>({kUploadThreads, (pieces + 2) / 3, std::max(1u, std::thread::hardware_concurrency())});
-        threads.reserve((size_t)want);
-        for (int t = 1; t < want; ++t) threads.emplace_back(work, t);
-    } catch (const std::exception &) {                            // no (more) threads to be had: those there are do it
-    }
-    work(0);
-    for (std::thread &t : threads) t.join();
-    return (cudaError_t)failed.load();
-}
-
-}  // namespace
-
 extern "C" int celty_release_staging(void)
 {
-    RelaxedCapture relaxed;
-    Staging &stage = staging();
-    std::lock_guard<std::mutex> lock(stage.mu);
-    if (!stage.memory) return CELTY_OK;
-    const cudaError_t waited = stage.wait();
-    CELTY_CUDA(cudaFreeHost(stage.memory));
-    stage.memory = nullptr;
-    CELTY_CUDA(waited);
+    CELTY_CUDA(release_staging());
     return CELTY_OK;
 }
 

@@ -1,0 +1,180 @@
+// Host-to-device copies of images through page-locked memory.  A copy from pageable memory is one host thread's in the driver, 4
+// GB/s; here up to kUploadThreads threads copy pieces into slots of page-locked memory, and the caller's thread enqueues the copies from
+// there.  It alone makes CUDA calls: a stream handle may mean another stream in another thread (cudaStreamPerThread), and the
+// caller's context need not be the one that cudaSetDevice would make current.  The 8 MB are taken by the first upload, used by one upload at a
+// time (another one meanwhile goes the pageable way) and given back by celty_release_staging.
+#include "celty_upload.h"
+
+#include <algorithm>
+#include <condition_variable>
+#include <cstring>
+#include <exception>
+#include <mutex>
+#include <thread>
+#include <vector>
+
+namespace celty {
+
+namespace {
+
+constexpr int kUploadThreads = 8, kUploadSlots = 16;
+constexpr size_t kUploadPiece = (size_t)512 << 10;
+
+// Another thread's stream capture (of the mode that watches all threads) does not mind this thread's allocations and waits.
+struct RelaxedCapture {
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+    ~RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+};
+
+struct Staging {
+    std::mutex mu;
+    uint8_t *memory = nullptr;
+    cudaEvent_t done[kUploadSlots] = {};                          // of a slot's last copy; null: the slot is free
+
+    // All copies have left their slots (mu is held).
+    cudaError_t wait()
+    {
+        cudaError_t first = cudaSuccess;
+        for (cudaEvent_t &e : done) {
+            if (!e) continue;
+            const cudaError_t err = cudaEventSynchronize(e);
+            if (first == cudaSuccess) first = err;
+            cudaEventDestroy(e);
+            e = nullptr;
+        }
+        return first;
+    }
+};
+
+Staging &staging()
+{
+    static Staging *s = new Staging;                              // (never destroyed: the runtime may be gone by then)
+    return *s;
+}
+
+// The pieces of an image on their way through the slots, piece i through slot i mod kUploadSlots.
+class Pieces {
+public:
+    Pieces(uint8_t *slots, const uint8_t *from, size_t bytes) : slots_(slots), from_(from), bytes_(bytes) {}
+    int64_t count() const { return (int64_t)((bytes_ + kUploadPiece - 1) / kUploadPiece); }
+    size_t size(int64_t i) const { return std::min(kUploadPiece, bytes_ - (size_t)i * kUploadPiece); }
+    uint8_t *slot(int64_t i) const { return slots_ + (size_t)(i % kUploadSlots) * kUploadPiece; }
+
+    void fill(int64_t i) const { std::memcpy(slot(i), from_ + (size_t)i * kUploadPiece, size(i)); }
+
+    // A thread that fills slots: the next pieces, each as soon as its slot is free.
+    void fill_all()
+    {
+        std::unique_lock<std::mutex> lock(mu_);
+        while (!stopped_ && claimed_ < count()) {
+            const int64_t i = claimed_++;
+            changed_.wait(lock, [&] { return stopped_ || i < copied_ + kUploadSlots; });
+            if (stopped_) return;
+            lock.unlock();
+            fill(i);
+            lock.lock();
+            filled_[i % kUploadSlots] = i + 1;
+            changed_.notify_all();
+        }
+    }
+
+    void wait_filled(int64_t i)
+    {
+        std::unique_lock<std::mutex> lock(mu_);
+        changed_.wait(lock, [&] { return filled_[i % kUploadSlots] == i + 1; });
+    }
+
+    // The copies of the first n pieces have been made: their slots are free.
+    void copied(int64_t n)
+    {
+        std::lock_guard<std::mutex> lock(mu_);
+        copied_ = n;
+        changed_.notify_all();
+    }
+
+    void stop()
+    {
+        std::lock_guard<std::mutex> lock(mu_);
+        stopped_ = true;
+        changed_.notify_all();
+    }
+
+private:
+    uint8_t *const slots_;
+    const uint8_t *const from_;
+    const size_t bytes_;
+    std::mutex mu_;
+    std::condition_variable changed_;
+    int64_t claimed_ = 0, copied_ = 0;
+    int64_t filled_[kUploadSlots] = {};                           // i + 1 when piece i is there
+    bool stopped_ = false;
+};
+
+}  // namespace
+
+// What a stream capture would have to replay, small images and those that come while the staging memory is in use go the pageable way.
+cudaError_t upload(void *to, const uint8_t *from, size_t bytes, cudaStream_t st)
+{
+    cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusActive;
+    cudaError_t err = cudaStreamIsCapturing(st, &capturing);
+    if (err != cudaSuccess) return err;
+    RelaxedCapture relaxed;
+    Staging &stage = staging();
+    std::unique_lock<std::mutex> lock(stage.mu, std::defer_lock);
+    const bool staged = capturing == cudaStreamCaptureStatusNone && bytes >= kUploadPiece && lock.try_lock();
+    if (staged && !stage.memory) {
+        void *memory = nullptr;
+        if (cudaHostAlloc(&memory, kUploadSlots * kUploadPiece, cudaHostAllocPortable) != cudaSuccess) (void)cudaGetLastError();
+        else stage.memory = static_cast<uint8_t *>(memory);
+    }
+    if (!staged || !stage.memory) return cudaMemcpyAsync(to, from, bytes, cudaMemcpyHostToDevice, st);
+    if ((err = stage.wait()) != cudaSuccess) return err;
+    Pieces pieces(stage.memory, from, bytes);
+    std::vector<std::thread> threads;
+    try {
+        // up to three pieces the caller's thread takes no longer than starting another would
+        const int64_t want = std::min<int64_t>({kUploadThreads, (pieces.count() + 2) / 3, std::max(1u, std::thread::hardware_concurrency())});
+        threads.reserve((size_t)want);
+        for (int64_t t = want > 1 ? 0 : 1; t < want; ++t) threads.emplace_back([&] { pieces.fill_all(); });
+    } catch (const std::exception &) {                            // no (more) threads to be had: those there are do it
+    }
+    for (int64_t i = 0, made = 0; i < pieces.count(); ++i) {
+        for (; made < i; ++made) {
+            const cudaEvent_t e = stage.done[made % kUploadSlots];
+            err = i - made == kUploadSlots ? cudaEventSynchronize(e) : cudaEventQuery(e);
+            if (err != cudaSuccess) break;
+        }
+        if (err == cudaErrorNotReady) (void)cudaGetLastError();
+        else if (err != cudaSuccess) break;
+        if (threads.empty()) {
+            pieces.fill(i);
+        } else {
+            pieces.copied(made);
+            pieces.wait_filled(i);
+        }
+        cudaEvent_t &e = stage.done[i % kUploadSlots];
+        if (!e && (err = cudaEventCreateWithFlags(&e, cudaEventDisableTiming)) != cudaSuccess) break;
+        err = cudaMemcpyAsync(static_cast<uint8_t *>(to) + (size_t)i * kUploadPiece, pieces.slot(i), pieces.size(i), cudaMemcpyHostToDevice, st);
+        if (err == cudaSuccess) err = cudaEventRecord(e, st);
+        if (err != cudaSuccess) break;
+    }
+    pieces.stop();
+    for (std::thread &t : threads) t.join();
+    return err;
+}
+
+cudaError_t release_staging()
+{
+    RelaxedCapture relaxed;
+    Staging &stage = staging();
+    std::lock_guard<std::mutex> lock(stage.mu);
+    if (!stage.memory) return cudaSuccess;
+    const cudaError_t waited = stage.wait();
+    const cudaError_t err = cudaFreeHost(stage.memory);
+    if (err != cudaSuccess) return err;
+    stage.memory = nullptr;
+    return waited;
+}
+
+}  // namespace celty

@@ -89,3 +89,22 @@ def test_an_upload_beside_another_threads_capture():
     assert not bad
     assert np.array_equal(buffers[0].cpu().numpy(), m.host_image()[0])
     assert np.array_equal(y.cpu().numpy(), small.spmspv(x, 0.5).cpu().numpy())
+
+
+def test_an_upload_on_the_threads_own_stream():
+    """cudaStreamPerThread (handle 2) means the calling thread's stream: reads enqueued there behind each of several uploads into one
+    buffer find the image that was uploaded last."""
+    ms = [_matrix(40 * PIECE, k) for k in range(2)]
+    assert ms[0].device_bytes() == ms[1].device_bytes()
+    image, ws = [torch.empty(b, dtype=torch.uint8, device="cuda") for b in ms[0].device_bytes()]
+    torch.cuda.synchronize()
+    stream, read = torch.cuda.ExternalStream(2), []
+    for k in range(6):
+        m = ms[k % 2]
+        celty._check(celty.load().celty_bind_device(m._h, image.data_ptr(), image.numel(), ws.data_ptr(), ws.numel(), 2), "celty_bind_device")
+        with torch.cuda.stream(stream):
+            read.append(torch.empty(image.numel(), dtype=torch.uint8, pin_memory=True))
+            read[-1].copy_(image, non_blocking=True)
+    stream.synchronize()
+    for k in range(6):
+        assert np.array_equal(read[k].numpy(), ms[k % 2].host_image()[0]), k

@@ -1,0 +1,163 @@
+"""Uploads of images against a CUDA runtime made of host code: a copy is made when something waits for it (or a query says it is
+ready), and cudaStreamPerThread means a queue of the calling thread's own.  No GPU needed."""
+import os
+import subprocess
+
+import pytest
+
+from conftest import ROOT
+
+CSRC = os.path.join(ROOT, "paper_2608_01536_b200", "csrc")
+CUDA = os.path.join(os.path.dirname(os.path.dirname(os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc"))), "include")
+
+MAIN = r'''
+#include <cstdio>
+#include <cstdlib>
+#include <cstring>
+#include <deque>
+#include <map>
+#include <mutex>
+#include <random>
+#include <set>
+#include <string>
+#include <thread>
+#include <vector>
+#include "celty_upload.h"
+
+// ---- the runtime: queues of copies and event marks
+struct Op { void *to; const void *from; size_t n; std::vector<uint8_t> own; struct Event *mark; };
+struct Event { bool ready = true; int polls = 0; std::string queue; };
+std::recursive_mutex mu;
+std::map<std::string, std::deque<Op>> queues;
+std::map<std::string, int> calls;
+std::set<std::thread::id> callers;
+std::set<Event *> events;
+std::vector<uint8_t *> locked;
+bool capturing = false;
+int waited = 0;                                  // marks that somebody waited for
+
+std::string queue_of(cudaStream_t st)
+{
+    char name[64];
+    snprintf(name, sizeof name, "%p", (void *)st);
+    return st == cudaStreamPerThread ? std::to_string(std::hash<std::thread::id>()(std::this_thread::get_id())) : name;
+}
+void drain(const std::string &q, Event *up_to)
+{
+    auto &ops = queues[q];
+    while (!ops.empty()) {
+        Op op = std::move(ops.front());
+        ops.pop_front();
+        if (op.n) memcpy(op.to, op.own.empty() ? op.from : op.own.data(), op.n);
+        if (op.mark) op.mark->ready = true;
+        if (op.mark && op.mark == up_to) return;
+    }
+}
+void called(const char *name) { ++calls[name]; callers.insert(std::this_thread::get_id()); }
+#define CALL std::lock_guard<std::recursive_mutex> lock(mu); called(__func__)
+extern "C" {
+cudaError_t cudaStreamIsCapturing(cudaStream_t, cudaStreamCaptureStatus *s) { CALL; *s = capturing ? cudaStreamCaptureStatusActive : cudaStreamCaptureStatusNone; return cudaSuccess; }
+cudaError_t cudaThreadExchangeStreamCaptureMode(cudaStreamCaptureMode *) { return cudaSuccess; }
+cudaError_t cudaGetDevice(int *d) { CALL; *d = 0; return cudaSuccess; }
+cudaError_t cudaSetDevice(int) { CALL; return cudaSuccess; }
+cudaError_t cudaGetLastError() { return cudaSuccess; }
+cudaError_t cudaHostAlloc(void **p, size_t n, unsigned) { CALL; locked.push_back((uint8_t *)malloc(n)); *p = locked.back(); return cudaSuccess; }
+cudaError_t cudaFreeHost(void *p) { CALL; free(p); return cudaSuccess; }
+cudaError_t cudaEventCreateWithFlags(cudaEvent_t *e, unsigned) { CALL; Event *ev = new Event; events.insert(ev); *e = (cudaEvent_t)ev; return cudaSuccess; }
+cudaError_t cudaEventDestroy(cudaEvent_t e) { CALL; events.erase((Event *)e); return cudaSuccess; }
+cudaError_t cudaEventRecord(cudaEvent_t e, cudaStream_t st)
+{
+    CALL;
+    Event *ev = (Event *)e;
+    ev->ready = false; ev->polls = 0; ev->queue = queue_of(st);
+    queues[ev->queue].push_back(Op{nullptr, nullptr, 0, {}, ev});
+    return cudaSuccess;
+}
+cudaError_t cudaEventQuery(cudaEvent_t e)
+{
+    CALL;
+    Event *ev = (Event *)e;
+    if (!ev->ready && ++ev->polls >= 3) drain(ev->queue, ev);
+    return ev->ready ? cudaSuccess : cudaErrorNotReady;
+}
+cudaError_t cudaEventSynchronize(cudaEvent_t e)
+{
+    CALL;
+    Event *ev = (Event *)e;
+    if (!ev->ready) { ++waited; drain(ev->queue, ev); }
+    return cudaSuccess;
+}
+cudaError_t cudaMemcpyAsync(void *to, const void *from, size_t n, cudaMemcpyKind, cudaStream_t st)
+{
+    CALL;
+    Op op{to, from, n, {}, nullptr};
+    bool is_locked = false;
+    for (uint8_t *l : locked) is_locked |= (const uint8_t *)from >= l && (const uint8_t *)from < l + ((size_t)8 << 20);
+    if (!is_locked) op.own.assign((const uint8_t *)from, (const uint8_t *)from + n);      // pageable: read before the call returns
+    queues[queue_of(st)].push_back(std::move(op));
+    return cudaSuccess;
+}
+}
+
+std::vector<uint8_t> image(size_t n, unsigned seed)
+{
+    std::vector<uint8_t> v(n);
+    std::mt19937 r(seed);
+    for (size_t i = 0; i + 4 <= n; i += 4) { const uint32_t w = r(); memcpy(&v[i], &w, 4); }
+    return v;
+}
+#define CHECK(c) do { if (!(c)) { printf("line %d: %s\n", __LINE__, #c); return 1; } } while (0)
+
+// A caller's stream: the image, another one into the same place, and reads of it behind each copy, by the stream's order.
+int ordered(cudaStream_t st, size_t n)
+{
+    std::vector<uint8_t> at(n), read[3];
+    const std::string q = queue_of(st);
+    for (int k = 0; k < 3; ++k) {
+        const std::vector<uint8_t> from = image(n, (unsigned)(n + k));
+        CHECK(celty::upload(at.data(), from.data(), n, st) == cudaSuccess);
+        read[k].resize(n);
+        { std::lock_guard<std::recursive_mutex> lock(mu); queues[q].push_back(Op{read[k].data(), at.data(), n, {}, nullptr}); }
+    }
+    { std::lock_guard<std::recursive_mutex> lock(mu); drain(q, nullptr); }
+    for (int k = 0; k < 3; ++k) CHECK(read[k] == image(n, (unsigned)(n + k)));
+    return 0;
+}
+
+int main(int, char **v)
+{
+    const std::string what = v[1];
+    const cudaStream_t st = (cudaStream_t)atol(v[2]);
+    const size_t n = (size_t)atol(v[3]);
+    if (what == "ordered") {
+        if (ordered(st, n)) return 1;
+        CHECK(callers.size() == 1);              // of which a stream handle or a context may be the property
+        CHECK(calls["cudaSetDevice"] == 0);
+    }
+    CHECK(celty::release_staging() == cudaSuccess);
+    CHECK(celty::release_staging() == cudaSuccess);
+    CHECK(events.empty());
+    return 0;
+}
+'''
+
+
+@pytest.fixture(scope="module")
+def program(tmp_path_factory):
+    d = tmp_path_factory.mktemp("upload")
+    (d / "main.cpp").write_text(MAIN)
+    exe = str(d / "upload")
+    subprocess.check_call(["g++", "-O1", "-g", "-std=c++17", "-pthread", "-I", CSRC, "-I", CUDA, os.path.join(CSRC, "celty_upload.cpp"),
+                           str(d / "main.cpp"), "-o", exe])
+
+    def run(*args):
+        r = subprocess.run([exe, *map(str, args)], capture_output=True, text=True, timeout=120)
+        assert r.returncode == 0, r.stdout + r.stderr
+    return run
+
+
+# handles 1 and 2 are cudaStreamLegacy and cudaStreamPerThread; sizes around the pieces of 512 KB, and beyond all slots
+@pytest.mark.parametrize("stream", [0, 1, 2, 4096])
+@pytest.mark.parametrize("size", [1000, (512 << 10) - 1, 512 << 10, (1536 << 10) + 1, (8 << 20) + 5, 20 << 20])
+def test_an_upload_is_work_of_the_callers_stream(program, stream, size):
+    program("ordered", stream, size)
