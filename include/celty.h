@@ -155,15 +155,16 @@ int celty_device_bytes(const celty_matrix *m, size_t *image_bytes, size_t *works
  * the image (and the clearing of the workspace) on `stream`.  The host image is ordinary pageable
  * memory, so the copy may block the calling thread; the handle is usable on `stream` on return
  * and on other streams after the caller has synchronised.
- * Large images go through 8 MB of page-locked memory that the library keeps for later calls (celty_release_staging).
+ * Large images go through 8 MB of page-locked memory that the library keeps for later calls (celty_release_staging), where
+ * `stream` has no earlier work to do; the call then returns when they are on the GPU.
  * Errors: CELTY_EINVAL, CELTY_ENOMEM (buffer too small or misaligned), CELTY_ECUDA.
  */
 int celty_bind_device(celty_matrix *m, void *image_dev, size_t image_bytes, void *workspace_dev,
                       size_t workspace_bytes, celty_stream_t stream);
 
 /*
- * celty_release_staging -- give back the page-locked memory that celty_bind_device keeps (waits for copies that are still on
- * their way from it; the next large image takes it again).  Errors: CELTY_ECUDA.
+ * celty_release_staging -- give back the page-locked memory that celty_bind_device keeps (the next large image takes it again).
+ * Errors: CELTY_ECUDA.
  */
 int celty_release_staging(void);
 

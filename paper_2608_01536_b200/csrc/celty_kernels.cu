@@ -903,8 +903,7 @@ extern "C" int celty_bind_device(celty_matrix *m, void *image_dev, size_t image_
     if (image_bytes < m->image.size() || workspace_bytes < m->ws.total) return CELTY_ENOMEM;
     if (((uintptr_t)image_dev | (uintptr_t)workspace_dev) & (kAlign - 1)) return CELTY_ENOMEM;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    CELTY_CUDA(upload(image_dev, m->image.data(), m->image.size(), st));
-    CELTY_CUDA(cudaMemsetAsync(workspace_dev, 0, m->ws.total, st));
+    CELTY_CUDA(upload(image_dev, m->image.data(), m->image.size(), workspace_dev, m->ws.total, st));
     m->d_image = static_cast<uint8_t *>(image_dev);
     m->d_ws = static_cast<uint8_t *>(workspace_dev);
     m->forget_launches();

@@ -1,8 +1,9 @@
 // Host-to-device copies of images through page-locked memory.  A copy from pageable memory is one host thread's in the driver, 4
-// GB/s; here up to kUploadThreads threads copy pieces into slots of page-locked memory, and the caller's thread enqueues the copies from
-// there.  It alone makes CUDA calls: a stream handle may mean another stream in another thread (cudaStreamPerThread), and the
+// GB/s; here up to kUploadThreads threads copy pieces into slots of page-locked memory, and one of them, the caller's, enqueues the copies
+// from there.  It alone makes CUDA calls: a stream handle may mean another stream in another thread (cudaStreamPerThread), and the
 // caller's context need not be the one that cudaSetDevice would make current.  The 8 MB are taken by the first upload, used by one upload at a
-// time (another one meanwhile goes the pageable way) and given back by celty_release_staging.
+// time and given back by celty_release_staging.  An upload ends when its copies have left the slots, so that it waits for no other stream's
+// work, nor leaves events for another context.
 #include "celty_upload.h"
 
 #include <algorithm>
@@ -30,21 +31,6 @@ struct RelaxedCapture {
 struct Staging {
     std::mutex mu;
     uint8_t *memory = nullptr;
-    cudaEvent_t done[kUploadSlots] = {};                          // of a slot's last copy; null: the slot is free
-
-    // All copies have left their slots (mu is held).
-    cudaError_t wait()
-    {
-        cudaError_t first = cudaSuccess;
-        for (cudaEvent_t &e : done) {
-            if (!e) continue;
-            const cudaError_t err = cudaEventSynchronize(e);
-            if (first == cudaSuccess) first = err;
-            cudaEventDestroy(e);
-            e = nullptr;
-        }
-        return first;
-    }
 };
 
 Staging &staging()
@@ -61,8 +47,6 @@ public:
     size_t size(int64_t i) const { return std::min(kUploadPiece, bytes_ - (size_t)i * kUploadPiece); }
     uint8_t *slot(int64_t i) const { return slots_ + (size_t)(i % kUploadSlots) * kUploadPiece; }
 
-    void fill(int64_t i) const { std::memcpy(slot(i), from_ + (size_t)i * kUploadPiece, size(i)); }
-
     // A thread that fills slots: the next pieces, each as soon as its slot is free.
     void fill_all()
     {
@@ -71,18 +55,18 @@ public:
             const int64_t i = claimed_++;
             changed_.wait(lock, [&] { return stopped_ || i < copied_ + kUploadSlots; });
             if (stopped_) return;
-            lock.unlock();
-            fill(i);
-            lock.lock();
-            filled_[i % kUploadSlots] = i + 1;
-            changed_.notify_all();
+            fill(i, lock);
         }
     }
 
+    // Returns when piece i is there; fills others, or i itself, meanwhile.
     void wait_filled(int64_t i)
     {
         std::unique_lock<std::mutex> lock(mu_);
-        changed_.wait(lock, [&] { return filled_[i % kUploadSlots] == i + 1; });
+        while (filled_[i % kUploadSlots] != i + 1) {
+            if (claimed_ < std::min(count(), copied_ + kUploadSlots)) fill(claimed_++, lock);
+            else changed_.wait(lock);
+        }
     }
 
     // The copies of the first n pieces have been made: their slots are free.
@@ -101,6 +85,15 @@ public:
     }
 
 private:
+    void fill(int64_t i, std::unique_lock<std::mutex> &lock)
+    {
+        lock.unlock();
+        std::memcpy(slot(i), from_ + (size_t)i * kUploadPiece, size(i));
+        lock.lock();
+        filled_[i % kUploadSlots] = i + 1;
+        changed_.notify_all();
+    }
+
     uint8_t *const slots_;
     const uint8_t *const from_;
     const size_t bytes_;
@@ -113,8 +106,9 @@ private:
 
 }  // namespace
 
-// What a stream capture would have to replay, small images and those that come while the staging memory is in use go the pageable way.
-cudaError_t upload(void *to, const uint8_t *from, size_t bytes, cudaStream_t st)
+// The pageable way go what a stream capture would have to replay, small images, those that come while the staging memory is in use, and
+// those behind work that their stream has not done yet: the wait for the copies would be one for that work.
+cudaError_t upload(void *to, const uint8_t *from, size_t bytes, void *clear, size_t clear_bytes, cudaStream_t st)
 {
     cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusActive;
     cudaError_t err = cudaStreamIsCapturing(st, &capturing);
@@ -122,45 +116,55 @@ cudaError_t upload(void *to, const uint8_t *from, size_t bytes, cudaStream_t st)
     RelaxedCapture relaxed;
     Staging &stage = staging();
     std::unique_lock<std::mutex> lock(stage.mu, std::defer_lock);
-    const bool staged = capturing == cudaStreamCaptureStatusNone && bytes >= kUploadPiece && lock.try_lock();
+    bool staged = capturing == cudaStreamCaptureStatusNone && bytes >= kUploadPiece && lock.try_lock();
+    if (staged && cudaStreamQuery(st) != cudaSuccess) {
+        (void)cudaGetLastError();
+        lock.unlock();
+        staged = false;
+    }
     if (staged && !stage.memory) {
         void *memory = nullptr;
         if (cudaHostAlloc(&memory, kUploadSlots * kUploadPiece, cudaHostAllocPortable) != cudaSuccess) (void)cudaGetLastError();
         else stage.memory = static_cast<uint8_t *>(memory);
     }
+    // (first, and waited for with the copies: the next layer's upload finds the stream idle)
+    if ((err = cudaMemsetAsync(clear, 0, clear_bytes, st)) != cudaSuccess) return err;
     if (!staged || !stage.memory) return cudaMemcpyAsync(to, from, bytes, cudaMemcpyHostToDevice, st);
-    if ((err = stage.wait()) != cudaSuccess) return err;
     Pieces pieces(stage.memory, from, bytes);
     std::vector<std::thread> threads;
     try {
-        // up to three pieces the caller's thread takes no longer than starting another would
         const int64_t want = std::min<int64_t>({kUploadThreads, (pieces.count() + 2) / 3, std::max(1u, std::thread::hardware_concurrency())});
         threads.reserve((size_t)want);
-        for (int64_t t = want > 1 ? 0 : 1; t < want; ++t) threads.emplace_back([&] { pieces.fill_all(); });
+        for (int64_t t = 1; t < want; ++t) threads.emplace_back([&] { pieces.fill_all(); });
     } catch (const std::exception &) {                            // no (more) threads to be had: those there are do it
     }
+    cudaEvent_t done[kUploadSlots] = {};                          // of a slot's last copy
+    cudaEvent_t last = nullptr;
     for (int64_t i = 0, made = 0; i < pieces.count(); ++i) {
         for (; made < i; ++made) {
-            const cudaEvent_t e = stage.done[made % kUploadSlots];
+            const cudaEvent_t e = done[made % kUploadSlots];
             err = i - made == kUploadSlots ? cudaEventSynchronize(e) : cudaEventQuery(e);
             if (err != cudaSuccess) break;
         }
         if (err == cudaErrorNotReady) (void)cudaGetLastError();
         else if (err != cudaSuccess) break;
-        if (threads.empty()) {
-            pieces.fill(i);
-        } else {
-            pieces.copied(made);
-            pieces.wait_filled(i);
-        }
-        cudaEvent_t &e = stage.done[i % kUploadSlots];
+        pieces.copied(made);
+        pieces.wait_filled(i);
+        cudaEvent_t &e = done[i % kUploadSlots];
         if (!e && (err = cudaEventCreateWithFlags(&e, cudaEventDisableTiming)) != cudaSuccess) break;
         err = cudaMemcpyAsync(static_cast<uint8_t *>(to) + (size_t)i * kUploadPiece, pieces.slot(i), pieces.size(i), cudaMemcpyHostToDevice, st);
         if (err == cudaSuccess) err = cudaEventRecord(e, st);
         if (err != cudaSuccess) break;
+        last = e;
     }
     pieces.stop();
     for (std::thread &t : threads) t.join();
+    if (last) {
+        const cudaError_t waited = cudaEventSynchronize(last);
+        if (err == cudaSuccess) err = waited;
+    }
+    for (cudaEvent_t e : done)
+        if (e) cudaEventDestroy(e);
     return err;
 }
 
@@ -170,11 +174,9 @@ cudaError_t release_staging()
     Staging &stage = staging();
     std::lock_guard<std::mutex> lock(stage.mu);
     if (!stage.memory) return cudaSuccess;
-    const cudaError_t waited = stage.wait();
     const cudaError_t err = cudaFreeHost(stage.memory);
-    if (err != cudaSuccess) return err;
-    stage.memory = nullptr;
-    return waited;
+    if (err == cudaSuccess) stage.memory = nullptr;
+    return err;
 }
 
 }  // namespace celty

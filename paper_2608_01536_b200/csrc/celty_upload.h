@@ -8,8 +8,8 @@
 
 namespace celty {
 
-// Enqueues the copy on st, with the current device; from has been read when it returns.
-cudaError_t upload(void *to, const uint8_t *from, size_t bytes, cudaStream_t st);
+// Enqueues the copy, and the clearing of another buffer, on st; from has been read when it returns.
+cudaError_t upload(void *to, const uint8_t *from, size_t bytes, void *clear, size_t clear_bytes, cudaStream_t st);
 
 // Gives back the memory that upload keeps.
 cudaError_t release_staging();

@@ -33,8 +33,7 @@ std::map<std::string, int> calls;
 std::set<std::thread::id> callers;
 std::set<Event *> events;
 std::vector<uint8_t *> locked;
-bool capturing = false;
-int waited = 0;                                  // marks that somebody waited for
+std::set<std::string> held;                      // queues that do not get on
 
 std::string queue_of(cudaStream_t st)
 {
@@ -45,6 +44,7 @@ std::string queue_of(cudaStream_t st)
 void drain(const std::string &q, Event *up_to)
 {
     auto &ops = queues[q];
+    if (held.count(q)) { printf("a wait for the work of a queue that is held\n"); exit(3); }
     while (!ops.empty()) {
         Op op = std::move(ops.front());
         ops.pop_front();
@@ -56,8 +56,9 @@ void drain(const std::string &q, Event *up_to)
 void called(const char *name) { ++calls[name]; callers.insert(std::this_thread::get_id()); }
 #define CALL std::lock_guard<std::recursive_mutex> lock(mu); called(__func__)
 extern "C" {
-cudaError_t cudaStreamIsCapturing(cudaStream_t, cudaStreamCaptureStatus *s) { CALL; *s = capturing ? cudaStreamCaptureStatusActive : cudaStreamCaptureStatusNone; return cudaSuccess; }
+cudaError_t cudaStreamIsCapturing(cudaStream_t, cudaStreamCaptureStatus *s) { CALL; *s = cudaStreamCaptureStatusNone; return cudaSuccess; }
 cudaError_t cudaThreadExchangeStreamCaptureMode(cudaStreamCaptureMode *) { return cudaSuccess; }
+cudaError_t cudaStreamQuery(cudaStream_t st) { CALL; return queues[queue_of(st)].empty() ? cudaSuccess : cudaErrorNotReady; }
 cudaError_t cudaGetDevice(int *d) { CALL; *d = 0; return cudaSuccess; }
 cudaError_t cudaSetDevice(int) { CALL; return cudaSuccess; }
 cudaError_t cudaGetLastError() { return cudaSuccess; }
@@ -77,16 +78,17 @@ cudaError_t cudaEventQuery(cudaEvent_t e)
 {
     CALL;
     Event *ev = (Event *)e;
-    if (!ev->ready && ++ev->polls >= 3) drain(ev->queue, ev);
+    if (!ev->ready && ++ev->polls >= 3 && !held.count(ev->queue)) drain(ev->queue, ev);
     return ev->ready ? cudaSuccess : cudaErrorNotReady;
 }
 cudaError_t cudaEventSynchronize(cudaEvent_t e)
 {
     CALL;
     Event *ev = (Event *)e;
-    if (!ev->ready) { ++waited; drain(ev->queue, ev); }
+    if (!ev->ready) drain(ev->queue, ev);
     return cudaSuccess;
 }
+cudaError_t cudaMemsetAsync(void *p, int c, size_t n, cudaStream_t st) { CALL; queues[queue_of(st)].push_back(Op{p, nullptr, n, std::vector<uint8_t>(n, (uint8_t)c), nullptr}); return cudaSuccess; }
 cudaError_t cudaMemcpyAsync(void *to, const void *from, size_t n, cudaMemcpyKind, cudaStream_t st)
 {
     CALL;
@@ -99,6 +101,7 @@ cudaError_t cudaMemcpyAsync(void *to, const void *from, size_t n, cudaMemcpyKind
 }
 }
 
+uint8_t cleared[1000];
 std::vector<uint8_t> image(size_t n, unsigned seed)
 {
     std::vector<uint8_t> v(n);
@@ -108,16 +111,20 @@ std::vector<uint8_t> image(size_t n, unsigned seed)
 }
 #define CHECK(c) do { if (!(c)) { printf("line %d: %s\n", __LINE__, #c); return 1; } } while (0)
 
-// A caller's stream: the image, another one into the same place, and reads of it behind each copy, by the stream's order.
+// A caller's stream: the image, others into the same place, and reads of it behind each copy, by the stream's order; the stream is busy
+// with the read when the second one comes.
 int ordered(cudaStream_t st, size_t n)
 {
     std::vector<uint8_t> at(n), read[3];
     const std::string q = queue_of(st);
     for (int k = 0; k < 3; ++k) {
         const std::vector<uint8_t> from = image(n, (unsigned)(n + k));
-        CHECK(celty::upload(at.data(), from.data(), n, st) == cudaSuccess);
+        memset(cleared, 7, sizeof cleared);
+        CHECK(celty::upload(at.data(), from.data(), n, cleared, sizeof cleared, st) == cudaSuccess);
         read[k].resize(n);
         { std::lock_guard<std::recursive_mutex> lock(mu); queues[q].push_back(Op{read[k].data(), at.data(), n, {}, nullptr}); }
+        if (k != 0) { std::lock_guard<std::recursive_mutex> lock(mu); drain(q, nullptr); }
+        if (k != 0) CHECK(cleared[0] == 0 && cleared[999] == 0);
     }
     { std::lock_guard<std::recursive_mutex> lock(mu); drain(q, nullptr); }
     for (int k = 0; k < 3; ++k) CHECK(read[k] == image(n, (unsigned)(n + k)));
@@ -134,9 +141,25 @@ int main(int, char **v)
         CHECK(callers.size() == 1);              // of which a stream handle or a context may be the property
         CHECK(calls["cudaSetDevice"] == 0);
     }
+    if (what == "held") {                        // a stream that does not get on holds up neither its own small uploads nor another's
+        const cudaStream_t other = (cudaStream_t)77;
+        std::vector<uint8_t> at(n), there(n), from = image(n, 1);
+        CHECK(celty::upload(there.data(), from.data(), n, cleared, sizeof cleared, other) == cudaSuccess);
+        const std::string q = queue_of(st);
+        queues[q].push_back(Op{&at[0], from.data(), 1, {}, nullptr});
+        held.insert(q);
+        CHECK(celty::upload(at.data(), from.data(), n, cleared, sizeof cleared, st) == cudaSuccess);
+        const std::vector<uint8_t> next = image(n, 2);
+        CHECK(celty::upload(there.data(), next.data(), n, cleared, sizeof cleared, other) == cudaSuccess);
+        drain(queue_of(other), nullptr);
+        CHECK(there == next);
+        held.clear();
+        drain(q, nullptr);
+        CHECK(at == from);
+    }
+    CHECK(events.empty());                       // (of the context that was current)
     CHECK(celty::release_staging() == cudaSuccess);
     CHECK(celty::release_staging() == cudaSuccess);
-    CHECK(events.empty());
     return 0;
 }
 '''
@@ -161,3 +184,8 @@ def program(tmp_path_factory):
 @pytest.mark.parametrize("size", [1000, (512 << 10) - 1, 512 << 10, (1536 << 10) + 1, (8 << 20) + 5, 20 << 20])
 def test_an_upload_is_work_of_the_callers_stream(program, stream, size):
     program("ordered", stream, size)
+
+
+@pytest.mark.parametrize("size", [1000, 512 << 10, 3 << 20, 8 << 20])
+def test_an_upload_waits_for_no_other_work(program, size):
+    program("held", 4096, size)
