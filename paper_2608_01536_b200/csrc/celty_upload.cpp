@@ -14,6 +14,8 @@
 #include <thread>
 #include <vector>
 
+#include "celty_internal.h"
+
 namespace celty {
 
 namespace {
@@ -28,9 +30,26 @@ struct RelaxedCapture {
     ~RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
 };
 
+// Ordinary memory that is registered: cudaDeviceReset, or the end of the context that was current, ends the registration and not the memory.
 struct Staging {
     std::mutex mu;
-    uint8_t *memory = nullptr;
+    Raw<uint8_t> memory;
+
+    // The slots, page-locked; null: not to be had (mu is held).
+    uint8_t *slots()
+    {
+        try {
+            if (memory.size() == 0) memory.allocate(kUploadSlots * kUploadPiece);
+        } catch (const std::exception &) {
+            return nullptr;
+        }
+        cudaPointerAttributes is{};
+        if (cudaPointerGetAttributes(&is, memory.data()) == cudaSuccess && is.type == cudaMemoryTypeHost) return memory.data();
+        (void)cudaGetLastError();
+        if (cudaHostRegister(memory.data(), memory.size(), cudaHostRegisterPortable) == cudaSuccess) return memory.data();
+        (void)cudaGetLastError();
+        return nullptr;
+    }
 };
 
 Staging &staging()
@@ -122,15 +141,11 @@ cudaError_t upload(void *to, const uint8_t *from, size_t bytes, void *clear, siz
         lock.unlock();
         staged = false;
     }
-    if (staged && !stage.memory) {
-        void *memory = nullptr;
-        if (cudaHostAlloc(&memory, kUploadSlots * kUploadPiece, cudaHostAllocPortable) != cudaSuccess) (void)cudaGetLastError();
-        else stage.memory = static_cast<uint8_t *>(memory);
-    }
+    uint8_t *const slots = staged ? stage.slots() : nullptr;
     // (first, and waited for with the copies: the next layer's upload finds the stream idle)
     if ((err = cudaMemsetAsync(clear, 0, clear_bytes, st)) != cudaSuccess) return err;
-    if (!staged || !stage.memory) return cudaMemcpyAsync(to, from, bytes, cudaMemcpyHostToDevice, st);
-    Pieces pieces(stage.memory, from, bytes);
+    if (!slots) return cudaMemcpyAsync(to, from, bytes, cudaMemcpyHostToDevice, st);
+    Pieces pieces(slots, from, bytes);
     std::vector<std::thread> threads;
     try {
         const int64_t want = std::min<int64_t>({kUploadThreads, (pieces.count() + 2) / 3, std::max(1u, std::thread::hardware_concurrency())});
@@ -173,9 +188,13 @@ cudaError_t release_staging()
     RelaxedCapture relaxed;
     Staging &stage = staging();
     std::lock_guard<std::mutex> lock(stage.mu);
-    if (!stage.memory) return cudaSuccess;
-    const cudaError_t err = cudaFreeHost(stage.memory);
-    if (err == cudaSuccess) stage.memory = nullptr;
+    if (stage.memory.size() == 0) return cudaSuccess;
+    cudaError_t err = cudaHostUnregister(stage.memory.data());
+    if (err == cudaErrorHostMemoryNotRegistered) {
+        (void)cudaGetLastError();
+        err = cudaSuccess;
+    }
+    if (err == cudaSuccess) stage.memory.reset();
     return err;
 }
 

@@ -22,6 +22,7 @@ MAIN = r'''
 #include <string>
 #include <thread>
 #include <vector>
+#include <sys/mman.h>
 #include "celty_upload.h"
 
 // ---- the runtime: queues of copies and event marks
@@ -32,7 +33,8 @@ std::map<std::string, std::deque<Op>> queues;
 std::map<std::string, int> calls;
 std::set<std::thread::id> callers;
 std::set<Event *> events;
-std::vector<uint8_t *> locked;
+struct Locked { size_t bytes; bool ours; };
+std::map<uint8_t *, Locked> locked;
 std::set<std::string> held;                      // queues that do not get on
 
 std::string queue_of(cudaStream_t st)
@@ -62,8 +64,29 @@ cudaError_t cudaStreamQuery(cudaStream_t st) { CALL; return queues[queue_of(st)]
 cudaError_t cudaGetDevice(int *d) { CALL; *d = 0; return cudaSuccess; }
 cudaError_t cudaSetDevice(int) { CALL; return cudaSuccess; }
 cudaError_t cudaGetLastError() { return cudaSuccess; }
-cudaError_t cudaHostAlloc(void **p, size_t n, unsigned) { CALL; locked.push_back((uint8_t *)malloc(n)); *p = locked.back(); return cudaSuccess; }
-cudaError_t cudaFreeHost(void *p) { CALL; free(p); return cudaSuccess; }
+cudaError_t cudaHostAlloc(void **p, size_t n, unsigned)
+{
+    CALL;
+    *p = mmap(nullptr, n, PROT_READ | PROT_WRITE, MAP_PRIVATE | MAP_ANONYMOUS, -1, 0);
+    locked[(uint8_t *)*p] = Locked{n, true};
+    return cudaSuccess;
+}
+cudaError_t cudaFreeHost(void *p) { CALL; munmap(p, locked.at((uint8_t *)p).bytes); locked.erase((uint8_t *)p); return cudaSuccess; }
+cudaError_t cudaHostRegister(void *p, size_t n, unsigned)
+{
+    CALL;
+    if (locked.count((uint8_t *)p)) return cudaErrorHostMemoryAlreadyRegistered;
+    locked[(uint8_t *)p] = Locked{n, false};
+    return cudaSuccess;
+}
+cudaError_t cudaHostUnregister(void *p) { CALL; return locked.erase((uint8_t *)p) ? cudaSuccess : cudaErrorHostMemoryNotRegistered; }
+cudaError_t cudaPointerGetAttributes(cudaPointerAttributes *a, const void *p) { CALL; a->type = locked.count((uint8_t *)p) ? cudaMemoryTypeHost : cudaMemoryTypeUnregistered; return cudaSuccess; }
+void device_reset()                              // what was allocated page-locked is gone, what was registered is ordinary memory
+{
+    for (auto &l : locked) if (l.second.ours) munmap(l.first, l.second.bytes);
+    locked.clear();
+    events.clear();
+}
 cudaError_t cudaEventCreateWithFlags(cudaEvent_t *e, unsigned) { CALL; Event *ev = new Event; events.insert(ev); *e = (cudaEvent_t)ev; return cudaSuccess; }
 cudaError_t cudaEventDestroy(cudaEvent_t e) { CALL; events.erase((Event *)e); return cudaSuccess; }
 cudaError_t cudaEventRecord(cudaEvent_t e, cudaStream_t st)
@@ -94,7 +117,7 @@ cudaError_t cudaMemcpyAsync(void *to, const void *from, size_t n, cudaMemcpyKind
     CALL;
     Op op{to, from, n, {}, nullptr};
     bool is_locked = false;
-    for (uint8_t *l : locked) is_locked |= (const uint8_t *)from >= l && (const uint8_t *)from < l + ((size_t)8 << 20);
+    for (auto &l : locked) is_locked |= (const uint8_t *)from >= l.first && (const uint8_t *)from < l.first + l.second.bytes;
     if (!is_locked) op.own.assign((const uint8_t *)from, (const uint8_t *)from + n);      // pageable: read before the call returns
     queues[queue_of(st)].push_back(std::move(op));
     return cudaSuccess;
@@ -157,6 +180,13 @@ int main(int, char **v)
         drain(q, nullptr);
         CHECK(at == from);
     }
+    if (what == "reset") {                       // and one that is not followed by another upload
+        if (ordered(st, n)) return 1;
+        device_reset();
+        if (ordered(st, n)) return 1;
+        CHECK(n < (512 << 10) || locked.size() == 1);
+        device_reset();
+    }
     CHECK(events.empty());                       // (of the context that was current)
     CHECK(celty::release_staging() == cudaSuccess);
     CHECK(celty::release_staging() == cudaSuccess);
@@ -170,7 +200,7 @@ def program(tmp_path_factory):
     d = tmp_path_factory.mktemp("upload")
     (d / "main.cpp").write_text(MAIN)
     exe = str(d / "upload")
-    subprocess.check_call(["g++", "-O1", "-g", "-std=c++17", "-pthread", "-I", CSRC, "-I", CUDA, os.path.join(CSRC, "celty_upload.cpp"),
+    subprocess.check_call(["g++", "-O1", "-g", "-std=c++17", "-pthread", "-I", CSRC, "-I", os.path.join(ROOT, "include"), "-I", CUDA, os.path.join(CSRC, "celty_upload.cpp"),
                            str(d / "main.cpp"), "-o", exe])
 
     def run(*args):
@@ -189,3 +219,8 @@ def test_an_upload_is_work_of_the_callers_stream(program, stream, size):
 @pytest.mark.parametrize("size", [1000, 512 << 10, 3 << 20, 8 << 20])
 def test_an_upload_waits_for_no_other_work(program, size):
     program("held", 4096, size)
+
+
+@pytest.mark.parametrize("size", [1000, 2 << 20, 20 << 20])
+def test_uploads_go_on_after_a_device_reset(program, size):
+    program("reset", 4096, size)
