@@ -44,7 +44,7 @@ struct Scratch {
 
 int64_t host_threads(int64_t n, bool worth_threads)
 {
-    return worth_threads ? std::min<int64_t>({n, 16, (int64_t)std::thread::hardware_concurrency()}) : 1;
+    return worth_threads ? std::max<int64_t>(1, std::min<int64_t>({n, 16, (int64_t)std::thread::hardware_concurrency()})) : 1;      // (0: not known)
 }
 
 // Phases of work that several host threads go through together: work(phase, scratch) on each of them, then between(phase) on one

@@ -12,8 +12,12 @@ MAIN = r'''
 #include <cstdio>
 #include <cstdlib>
 #include <random>
+#include <thread>
 #include <vector>
 #include "celty.h"
+#ifdef NO_COUNT                                  // a system that does not say how many processors it has
+unsigned std::thread::hardware_concurrency() noexcept { return 0; }
+#endif
 int main(int, char **v) {
     const int M = atoi(v[1]), K = atoi(v[2]), tile_rows = atoi(v[3]), kept = atoi(v[4]), column = atoi(v[5]);
     std::mt19937 r(M * 31 + K);
@@ -45,7 +49,7 @@ def encoders(tmp_path_factory):
     d = tmp_path_factory.mktemp("encoders")
     (d / "main.cpp").write_text(MAIN)
     exes = []
-    for k, flags in enumerate(([], ["-DCELTY_PLAIN_ENCODER"])):
+    for k, flags in enumerate(([], ["-DCELTY_PLAIN_ENCODER"], ["-DNO_COUNT"])):
         exes.append(str(d / ("encoder%d" % k)))
         subprocess.check_call(["g++", "-O2", "-std=c++17", "-pthread", *flags, "-I", os.path.join(ROOT, "include"), "-I", CSRC,
                                os.path.join(CSRC, "celty_host.cpp"), str(d / "main.cpp"), "-o", exes[-1]])
@@ -58,5 +62,11 @@ def encoders(tmp_path_factory):
     (7680, 70, 240, 500, 0), (7681, 70, 240, 900, 0), (4100, 200, 128, 60, 0), (2048, 300, 0, 500, 0), (1000, 200, 0, 1, 0), (777, 130, 0, 500, 1),
     (3000, 64, 96, 980, 0)])
 def test_plain_and_vector_builds_agree(encoders, M, K, tile_rows, kept, column):
-    outs = [subprocess.check_output([e, *map(str, (M, K, tile_rows, kept, column))]) for e in encoders]
+    outs = [subprocess.check_output([e, *map(str, (M, K, tile_rows, kept, column))]) for e in encoders[:2]]
+    assert len(outs[0]) > 0 and outs[0] == outs[1]
+
+
+@pytest.mark.parametrize("M,K,column", [(1024, 1024, 0), (1024, 1024, 1), (21000, 70, 0), (100, 100, 0)])
+def test_a_system_without_a_processor_count(encoders, M, K, column):
+    outs = [subprocess.check_output([e, *map(str, (M, K, 0, 500, column))]) for e in (encoders[0], encoders[2])]
     assert len(outs[0]) > 0 and outs[0] == outs[1]
