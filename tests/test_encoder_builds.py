@@ -70,3 +70,25 @@ def test_plain_and_vector_builds_agree(encoders, M, K, tile_rows, kept, column):
 def test_a_system_without_a_processor_count(encoders, M, K, column):
     outs = [subprocess.check_output([e, *map(str, (M, K, 0, 500, column))]) for e in (encoders[0], encoders[2])]
     assert len(outs[0]) > 0 and outs[0] == outs[1]
+
+
+def test_encoder_threads_that_wait_leave_the_processor(tmp_path):
+    """One of eight threads takes 0.3 s of wall-clock time over each of two phases: the others look for a moment and sleep."""
+    (tmp_path / "main.cpp").write_text(r'''
+#include "celty_host.cpp"
+#include <cstdio>
+#include <ctime>
+int main() {
+    std::atomic<int> turn[2] = {{0}, {0}}, seen(0), between(0);
+    if (!in_phases(8, 2, [&](int p, Scratch &) {
+            if (between != p) exit(2);                            // nobody is ahead
+            if (turn[p]++ == 3) std::this_thread::sleep_for(std::chrono::milliseconds(300));
+            ++seen;
+        }, [&](int) { if (seen != 8 * ++between) exit(3); }))
+        return 1;
+    printf("%.4f", (double)clock() / CLOCKS_PER_SEC);
+}
+''')
+    exe = str(tmp_path / "phases")
+    subprocess.check_call(["g++", "-O2", "-std=c++17", "-pthread", "-I", os.path.join(ROOT, "include"), "-I", CSRC, str(tmp_path / "main.cpp"), "-o", exe])
+    assert float(subprocess.check_output([exe])) < 0.1            # seconds of processor time; seven threads that poll: up to 4
