@@ -272,8 +272,7 @@ class Matrix:
     def launch_plan(self) -> dict:
         """Shape of the single-launch kernel's launch for this handle on the current device, and which kernel it is; which
         one runs from a list, and (index 2 .. 8) in launches that serve so many vectors of a batch (None: there is none).
-        k_spmspv_direct: at most 128 columns per block, or a list; k_spmspv_fused: more (up to 512 its form that deals columns to groups of
-        blocks, k_spmspv_fused_groups, where no option asks for something else)."""
+        k_spmspv_direct deals columns to groups of blocks, or shares a list evenly; k_spmspv_fused ranks the survivors."""
         out = (_i32 * 19)()
         _check(load().celty_launch_plan(self._h, out, 19), "celty_launch_plan")
         keys = ("grid", "threads", "smem_bytes", "teams_per_slab", "ring_depth", "cluster", "row_parts",

@@ -24,8 +24,7 @@
 //    84 (11008 x 4096, 0.1 / 0.5)           6.92 / 5.63 / 5.22, 11.63 / 11.43 / 10.68
 //   111 (14336 x 4096, 0.5)                 12.86 / 12.97 / 12.19
 //   111 (8192 x 8192, 0.5)                  14.26 / 14.80 / 13.57
-// Beyond 128 columns per block the same code runs as k_spmspv_fused_groups (the form of k_spmspv_fused that a plan's readers
-// expect there), with one, two or four of the group's columns per ranking lane, k_spmspv_fused -> this one, one vector:
+// Beyond 128 columns per block a ranking lane may hold one, two or four of the group's columns, k_spmspv_fused -> this one, one vector:
 //   128 (40 x 18945, 0.5)                   6.83 -> 5.73
 //   139 (13824 x 5120, 0.1 / 0.5)           7.16 -> 5.73, 14.92 -> 14.03
 //   187 (5120 x 13824, 0.1 / 0.5)           7.30 -> 6.01, 15.69 -> 13.75
@@ -62,7 +61,7 @@ constexpr int kDirectThreads = 32 * (16 + kDirectHelpers + 1);
 // (DirectParams::ldx); kHeld: columns of the group per ranking lane; 0: the survivors come as a list (DirectParams::list), in
 // equal shares for all teams.
 template <bool kPairs, bool kBatch, int kHeld>
-__device__ __forceinline__ void dealt_product(const DirectParams p)
+__global__ void __launch_bounds__(kDirectThreads, 1) k_spmspv_direct(const DirectParams p)
 {
     constexpr bool kList = kHeld == 0;
     constexpr int kArray = kList ? 1 : kHeld;
@@ -379,17 +378,4 @@ __device__ __forceinline__ void dealt_product(const DirectParams p)
     }
     asm volatile("cp.async.bulk.commit_group;" ::: "memory");
     asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");   // shared memory may go once it has been read
-}
-
-template <bool kPairs, bool kBatch, int kHeld>
-__global__ void __launch_bounds__(kDirectThreads, 1) k_spmspv_direct(const DirectParams p)
-{
-    dealt_product<kPairs, kBatch, kHeld>(p);
-}
-
-// k_spmspv_fused with dealt columns, for blocks that own more than 128.
-template <bool kPairs, bool kBatch, int kHeld>
-__global__ void __launch_bounds__(kDirectThreads, 1) k_spmspv_fused_groups(const DirectParams p)
-{
-    dealt_product<kPairs, kBatch, kHeld>(p);
 }

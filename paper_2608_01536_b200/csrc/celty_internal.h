@@ -332,8 +332,8 @@ struct FusedPlan {
     int G, Sc, P, D, cl, pp, mix, slot_bytes, cap, threads, grid, merge;
     int window;                // bytes of the offset window where it has a place of its own (several vectors), else -1
     int lean;                  // 0: every option compiled in; 1 / 2: the builds for the default launch (without / with warp pairs)
-    int direct;                // 1: columns are dealt (k_spmspv_direct, k_spmspv_fused_groups)
-    int wide;                  // 1: k_spmspv_fused_groups
+    int direct;                // 1: columns are dealt (k_spmspv_direct)
+    int wide;                  // 1: and a ranking lane may hold several
     DirectGroups groups;       // of its blocks (not from a list)
     DirectSmem tables;         // its shared memory
     size_t smem;

@@ -501,7 +501,9 @@ int launch_compact(const void *x, int64_t K, float tau, int32_t *idx, uint16_t *
 
 constexpr int kMostToMix = 48;           // left-over blocks are shared between row parts up to this (fit_clusters)
 
-constexpr int kDirectMost = 128, kGroupsMost = 512, kMixesMost = 384, kBatchMost = 20000;      // columns of a block of k_spmspv_direct, of k_spmspv_fused_groups (see there)
+// Columns of a block of k_spmspv_direct (see there): with one per ranking lane; at most; where blocks left over can be shared; times rows
+// per lane in launches for several vectors.
+constexpr int kDirectMost = 128, kGroupsMost = 512, kMixesMost = 384, kBatchMost = 20000;
 
 int direct_threads(int G, int pairs) { return 32 * (pairs ? 16 + kDirectHelpers + 1 : std::max(16, G + kDirectHelpers + 1)); }
 
@@ -809,18 +811,17 @@ int launch_fused(void (*kernel)(Params), int *granted, const LaunchKnobs &knobs,
     return CELTY_OK;
 }
 
-// The build of k_spmspv_direct or k_spmspv_fused_groups for a plan, and its shared-memory limit.
+// The build of k_spmspv_direct for a plan, and its shared-memory limit.
 struct DirectBuild { void (*kernel)(DirectParams); int *granted; };
 
 template <bool kPairs, bool kBatch>
 DirectBuild direct_build(const FusedPlan &plan, bool list, int held)
 {
-    static int granted[5][64];
+    static int granted[4][64];
     if (list) return DirectBuild{k_spmspv_direct<kPairs, false, 0>, granted[0]};
-    if (!plan.wide) return DirectBuild{k_spmspv_direct<kPairs, kBatch, 1>, granted[1]};
-    return held == 1 ? DirectBuild{k_spmspv_fused_groups<kPairs, kBatch, 1>, granted[2]}
-         : held == 2 ? DirectBuild{k_spmspv_fused_groups<kPairs, kBatch, 2>, granted[3]}
-                     : DirectBuild{k_spmspv_fused_groups<kPairs, kBatch, 4>, granted[4]};
+    return held == 1 ? DirectBuild{k_spmspv_direct<kPairs, kBatch, 1>, granted[1]}
+         : held == 2 ? DirectBuild{k_spmspv_direct<kPairs, kBatch, 2>, granted[2]}
+                     : DirectBuild{k_spmspv_direct<kPairs, kBatch, 4>, granted[3]};
 }
 
 DirectBuild direct_build(const FusedPlan &plan, bool batch, bool list)
@@ -880,11 +881,11 @@ extern "C" int celty_launch_plan(const celty_matrix *m, int32_t *out, int32_t n)
                            plan.slot_bytes, plan.merge + 16 * plan.pp + 256 * plan.mix};
     for (int i = 0; i < 10; ++i) out[i] = v[i];
     // which kernel: of this launch, of one from a list, of launches that serve 2 .. 8 vectors
-    if (n > 10) out[10] = plan.direct && !plan.wide;
+    if (n > 10) out[10] = plan.direct;
     for (int i = 11; i < std::min(n, 19); ++i) {
         rc = plan_launch(m, *m, di, i == 11 ? 1 : i - 10, &plan, i == 11);
         if (rc == CELTY_ECUDA) return rc;
-        out[i] = rc ? -1 : plan.direct && !plan.wide;
+        out[i] = rc ? -1 : plan.direct;
     }
     return CELTY_OK;
 }

@@ -223,7 +223,8 @@ def test_first_calls_of_several_threads_on_one_handle():
 
 
 def test_the_plan_names_the_kernel():
-    """At most 128 columns per block: dealt; more, several slabs per block, or on request: ranked.  A list is shared by the
+    """At most 512 columns per block (384 where blocks left over can be shared, 20 000 / rows per lane for several vectors): dealt;
+    more, several slabs per block, or on request: ranked.  A list is shared by the
     kernel that deals unless left-over blocks serve several row parts.  A caller of the C entry with room for ten words
     gets ten."""
     def plan(M, K, variant=0, **kw):
@@ -234,13 +235,17 @@ def test_the_plan_names_the_kernel():
         return p
 
     ranked, direct = "k_spmspv_fused", "k_spmspv_direct"
-    for K, kernel in ((148 * 128, direct), (148 * 128 + 1, ranked)):
+    for K, kernel in ((148 * 128, direct), (148 * 128 + 1, direct), (148 * 512, direct), (148 * 512 + 1, ranked)):
         p = plan(40, K)
         assert (p["kernel"], p["list_kernel"]) == (kernel, direct)
+    for K, kernel in ((18 * 384, direct), (18 * 384 + 1, ranked)):                 # eight row parts, four blocks left over
+        p = plan(256, K, tile_rows=1)
+        assert (p["kernel"], p["row_parts"], p["parts_per_spare_block"]) == (kernel, 8, 1 if kernel == direct else 2)
     for N in range(2, 9):
-        columns = 128 * (148 // N)
-        for K, kernel in ((columns, direct), (columns + 1, ranked)):
-            assert plan(40, K)["batch_kernels"][N] == kernel, (N, K)
+        for M, rows, most in ((40, 0, 512), (4096, 128, 156)):
+            columns = most * (148 // N)
+            for K, kernel in ((columns, direct), (columns + 1, ranked)):
+                assert plan(M, K, tile_rows=rows)["batch_kernels"][N] == kernel, (N, K)
     for variant in (2, 128, 256):
         p = plan(300, 400, variant)
         assert p["kernel"] == ranked and p["list_kernel"] in (ranked, None)

@@ -1,5 +1,5 @@
 """Products whose blocks share their columns' survivors in groups, at the edges of what a ranking lane holds (one, two or four
-columns) and where the kernel that ranks all of x takes over (more than 512 columns per block)."""
+columns) and where the kernel that ranks all of x takes over (more than 512 columns per block, 384 where blocks left over can be shared)."""
 import numpy as np
 import pytest
 import torch
@@ -19,8 +19,9 @@ def _lib():
 
 # blocks of the launch; rows, rows per tile (row parts); columns per block of a row part: three members of a group need 512 / 3
 # columns each (384 / 3 without warp pairs) for one column per lane, 341 (256) for two
-@pytest.mark.parametrize("grid,M,tile_rows", [(5, 40, 0), (37, 300, 3), (148, 40, 0), (19, 1100, 4)])
-@pytest.mark.parametrize("columns", [127, 128, 129, 170, 171, 256, 257, 341, 342, 512, 513])
+@pytest.mark.parametrize("grid,M,tile_rows,columns", [(g, M, r, c) for g, M, r in ((5, 40, 0), (37, 300, 3), (148, 40, 0), (19, 1100, 4))
+                                                       for c in (127, 128, 129, 170, 171, 256, 257, 341, 342, 512, 513)] +
+                         [(148, 256, 1, c) for c in (127, 171, 257, 384, 385)])
 def test_groups_at_their_edges(grid, M, tile_rows, columns):
     """Integer data, exact: three densities, survivors that lie together, none and all; the reported list; the call twice."""
     probe = celty.Matrix(synth.integer_weights(1, M, 8), None, tile_rows=tile_rows)
@@ -30,7 +31,9 @@ def test_groups_at_their_edges(grid, M, tile_rows, columns):
     mask = synth.mask_bernoulli(columns + grid, M, K, 0.4)
     m = celty.Matrix(W, mask, tile_rows=tile_rows, device="cuda")
     m.set_launch(grid=grid)
-    assert m.launch_plan()["row_parts"] == parts
+    plan, left = m.launch_plan(), grid % parts
+    mixes = left > 0 and parts % left == 0 and parts // left * (grid // parts) <= 48       # left-over blocks can be shared
+    assert plan["row_parts"] == parts and plan["kernel"] == ("k_spmspv_direct" if columns <= (384 if mixes else 512) else "k_spmspv_fused")
     rng = np.random.default_rng(columns)
     full = synth.integer_activations(9, K)
     full = np.where(full == 0, np.float16(1), full)               # 1 .. in magnitude

@@ -1,6 +1,6 @@
-"""The kernel that ranks the survivors, on layers where it is the default (more than 128 columns per thread block) and in the
-builds that the launch choices ask for, and both kernels where what they decide is their own code: thresholds, batches, waits
-that run out."""
+"""The kernel that ranks the survivors, on layers where it is the default (more than 512 columns per thread block, 384 where left-over
+blocks can be shared) and in the builds that the launch choices ask for, and both kernels where what they decide is their own
+code: thresholds, batches, waits that run out."""
 import numpy as np
 import pytest
 import torch
@@ -35,7 +35,8 @@ SPECIAL_X = np.array([0x0000, 0x8000, 0x7E00, 0xFE00, 0x7C00, 0xFC00, 0x0001, 0x
                       0x7BFF, 0xFBFF, 0x3C00, 0xBC00, 0x3C01, 0x3BFF, 0x3800, 0xB800], np.uint16)
 
 
-@pytest.mark.parametrize("tiles,empty,kernel", [(32, 3, DIRECT), (256, 3, DIRECT), (992, 3, RANKED), (32, 20001, RANKED)])
+@pytest.mark.parametrize("tiles,empty,kernel", [(32, 3, DIRECT), (256, 3, DIRECT), (992, 3, DIRECT), (32, 20001, DIRECT),
+                                                (992, 1300, RANKED), (32, 76001, RANKED)])
 def test_special_values_reach_y_through_every_kernel(tiles, empty, kernel):
     """Every column of W fills one tile of 8 rows with ones, so y shows which columns the product took: +-0, NaNs, infinities,
     subnormals and the neighbours of 1 against thresholds that are 0, below the smallest subnormal, on FP16 values, between
@@ -71,15 +72,16 @@ def test_special_values_reach_y_through_every_kernel(tiles, empty, kernel):
                 n = torch.tensor([oi.size], dtype=torch.int32, device="cuda")
                 ys.append(m.spmspv_list(_dev(np.append(oi, 0).astype(np.int32)), _dev(np.append(ov, 0).astype(np.uint16).view(np.int16)), n))
             if variant == 0:
-                ys += [m.spmspv_static(xd, tau)] + list(m.spmspv_batch(wide[:, :K], tau, y=yb))
+                ys += ([m.spmspv_static(xd, tau)] if K <= 32768 else []) + list(m.spmspv_batch(wide[:, :K], tau, y=yb))
             for k, y in enumerate(ys):
                 assert np.array_equal(y.cpu().numpy(), want, equal_nan=True), (variant, tau, k)
         assert m.last_status() == 0
 
 
-# blocks of a vector at the edges of 32, 64, 96 and 128 columns per block, and beyond, where survivors are ranked
+# blocks of a vector at the edges of 32, 64, 96, 128 and 512 columns per block, or of 20 000 / rows per lane, beyond which survivors are ranked
 @pytest.mark.parametrize("N,M,tile_rows,K", [(2, 40, 0, 74 * 32 * c + e) for c in (1, 2, 3, 4) for e in (0, 1)] +
                          [(5, 40, 0, 29 * 128 + e) for e in (-1, 1)] + [(3, 200, 2, 12 * 128 + e) for e in (0, 1)] +
+                         [(2, 40, 0, 74 * 512 + e) for e in (0, 1)] + [(8, 4096, 128, 18 * 156 + e) for e in (0, 1)] +
                          [(4, 4096, 0, 4096), (3, 4096, 0, 4096), (8, 2048, 0, 4096), (8, 300, 0, 40000), (4, 9000, 0, 3000)])
 def test_batches_on_both_sides_of_the_line(N, M, tile_rows, K):
     """Integer data, exact; also with two teams per block, so that a team has more columns than it looks up at once."""
@@ -94,7 +96,8 @@ def test_batches_on_both_sides_of_the_line(N, M, tile_rows, K):
         m.set_launch(variant=variant, groups=groups)
         plan = m.launch_plan()
         columns = -(-K // (148 // N // plan["row_parts"]))
-        assert plan["batch_kernels"][N] == (DIRECT if columns <= 128 and variant != 128 else RANKED)
+        most = max(128, min(512, 20000 // m.row_map()[1]))
+        assert plan["batch_kernels"][N] == (DIRECT if columns <= most and variant != 128 else RANKED)
         y = torch.full((N, (M + 3) // 4 * 4), 9.0, device="cuda")[:, :M]
         for _ in range(2):
             m.spmspv_batch(wide[:, :K], 1.0, y=y)
@@ -104,14 +107,18 @@ def test_batches_on_both_sides_of_the_line(N, M, tile_rows, K):
         assert m.last_status() == 0
 
 
-@pytest.mark.parametrize("M,K,variant", [(300, 20000, 0), (4096, 12000, 16), (4096, 12000, 32)])
-def test_a_ranked_wait_that_runs_out_is_reported_and_the_handle_recovers(M, K, variant):
+# (tile_rows 64: two row parts; 2: five; 1: eight, between which four blocks left over are shared)
+@pytest.mark.parametrize("M,K,tile_rows,grid,variant,kernel", [
+    (300, 20000, 0, 0, 0, DIRECT), (4096, 12000, 64, 0, 16, DIRECT), (4096, 12000, 64, 0, 32, DIRECT), (300, 15000, 2, 0, 0, RANKED),
+    (300, 15000, 2, 0, 16, RANKED), (300, 15000, 2, 0, 32, RANKED), (4096, 5200, 64, 20, 16, RANKED), (4096, 5200, 64, 20, 32, RANKED),
+    (256, 7000, 1, 0, 0, RANKED)])
+def test_a_wait_that_runs_out_is_reported_and_the_handle_recovers(M, K, tile_rows, grid, variant, kernel):
     """The ticket that tells a block when the others have cleared their shares of y is moved ahead by hand, so that five
     blocks wait for a count that never comes: the launch comes back, the status says so once, the next call is right."""
-    W, mask, m = _layer(61, M, K, tile_rows=64 if M == 4096 else 0)     # (64: two row parts)
-    m.set_launch(variant=variant)
+    W, mask, m = _layer(61, M, K, tile_rows=tile_rows)
+    m.set_launch(variant=variant, grid=grid)
     plan = m.launch_plan()
-    assert plan["kernel"] == RANKED
+    assert plan["kernel"] == kernel and plan["parts_per_spare_block"] == (2 if tile_rows == 1 else 1)
     x = synth.integer_activations(62, K)
     y_ref, _ = orc.masked_gemv(W, mask, x, 1.0, threads=8)
     xd = _dev(x)
@@ -130,16 +137,19 @@ def test_a_ranked_wait_that_runs_out_is_reported_and_the_handle_recovers(M, K, v
         assert m.last_status() == 0
 
 
-@pytest.mark.parametrize("M,K,variant,depth", [(300, 20000, 0, 0), (4096, 12000, 16, 0), (4096, 12000, 16, 4), (4096, 12000, 32, 0)])
-def test_the_shortest_wait_limit_on_ranked_layers(M, K, variant, depth):
-    """One poll per wait in single, list, batch and static calls of layers whose survivors are ranked: the kernels come back,
+@pytest.mark.parametrize("M,K,tile_rows,grid,variant,depth,kernel", [
+    (300, 20000, 0, 0, 0, 0, DIRECT), (4096, 12000, 64, 0, 16, 0, DIRECT), (4096, 12000, 64, 0, 16, 4, DIRECT), (4096, 12000, 64, 0, 32, 0, DIRECT),
+    (300, 15000, 2, 0, 0, 0, RANKED), (300, 15000, 2, 0, 16, 0, RANKED), (300, 15000, 2, 0, 32, 0, RANKED), (4096, 5200, 64, 20, 16, 0, RANKED),
+    (4096, 5200, 64, 20, 16, 4, RANKED), (4096, 5200, 64, 20, 32, 0, RANKED), (256, 7000, 1, 0, 0, 0, RANKED)])
+def test_the_shortest_wait_limit(M, K, tile_rows, grid, variant, depth, kernel):
+    """One poll per wait in single, list, batch and static calls of layers with many columns per block: the kernels come back,
     what they asked for has landed before their blocks end, and the handle is right again after last_status.  In the call
     without a status word every row is right or NaN."""
-    W, mask, m = _layer(63, M, K, tile_rows=64 if M == 4096 else 0)     # (64: two row parts)
+    W, mask, m = _layer(63, M, K, tile_rows=tile_rows)
     beside = m.clone("cuda")
-    m.set_launch(variant=variant, depth=depth)
+    m.set_launch(variant=variant, depth=depth, grid=grid)
     plan = m.launch_plan()
-    assert plan["kernel"] == RANKED and plan["batch_kernels"][4] == RANKED
+    assert plan["kernel"] == kernel and plan["batch_kernels"][4] == RANKED
     x = synth.integer_activations(64, K)
     y_ref, _ = orc.masked_gemv(W, mask, x, 1.0, threads=8)
     oi, ov, _ = orc.compact(x, 1.0)
