@@ -357,18 +357,11 @@ void choose_shape(int64_t M, int64_t K, double density, int tile_rows, int64_t *
         // sub-blocks of half the size.  Measured at 4096 x 4096: 8.3 us against 8.8; at 4096 x 11008, where a team
         // has five sub-blocks to stream, no gain, so the rule stops short of it.
         if (S == 1 && Q >= 32 && K <= 6144) S = 2;
-        // For the same reason slabs of up to 2048 rows on taller layers of few columns: to 56 columns per block on 148 SMs.  Device
-        // time at 10 / 30 / 50 / 70 % of the activations, in us, with slabs of 4096 rows -> of 2048:
-        //   8192 x 2048 (55 columns)    4.63 / 5.31 / 6.06 / 7.08 -> 3.91 / 4.70 / 5.73 / 6.85
-        //   6000 x 2000 (41)            4.36 / 4.69 / 5.11 / 5.89 -> 3.93 / 4.20 / 4.95 / 5.64
-        //   11008 x 1024 (41)           4.59 / 4.84 / 5.34 / 5.84 -> 3.87 / 4.16 / 4.87 / 5.68
-        //   5504 x 2048 (42)            4.19 / 4.55 / 4.87 / 5.65 -> 3.85 / 4.15 / 4.97 / 5.74
-        //   5000 x 1500 (30)            4.05 / 4.23 / 4.42 / 4.79 -> 3.80 / 3.97 / 4.34 / 4.91
-        // and beyond the line:
-        //   6000 x 3072 (62)            4.35 / 4.94 / 5.94 / 6.87 -> 3.95 / 4.94 / 6.11 / 7.17
-        //   11008 x 2048 (83)           4.67 / 5.54 / 6.79 / 8.10 -> 4.00 / 5.50 / 7.05 / 8.85
-        const int64_t lower = (M + 2047) / 2048;
-        if (S > 1 && S < 6 && M > 4096 && K * lower <= 8192) S = lower;
+        // (Taller layers of few columns would gain from slabs of 2048 rows in calls for one vector, 7 to 17 % at 10 % of the
+        // activations and up to 7 at 50, and lose more in batches, whose blocks have N times the columns; the image is the same for both.
+        // Slabs of 4096 -> of 2048 rows, us, one vector at 10 / 50 %, N = 4, 8 at 50 %:  8192 x 2048 4.66 / 5.94, 12.7, 22.0 -> 3.92 /
+        // 6.07, 13.5, 27.2;  5504 x 2048 4.24 / 5.03, 9.3, 16.5 -> 3.87 / 4.99, 10.6, 19.2;  20000 x 800 4.71 / 6.06, 12.6, 24.9 -> 3.93 /
+        // 5.62, 14.7, 29.9;  8192 x 512 4.56 / 4.64, 6.1, 8.3 -> 3.89 / 3.92, 5.9, 9.0.)
         auto rows_for = [&](int64_t slabs) { return std::max<int64_t>(16, ((Q + slabs - 1) / slabs + 15) / 16 * 16); };
         auto teams_that_fit = [&](int64_t rows) {
             const double entries = 32.0 * rows * density;             // of one sub-block, mean; + 3.5 sigma for the largest
