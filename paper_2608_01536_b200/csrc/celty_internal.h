@@ -226,6 +226,22 @@ struct DirectGroups {
     DirectSizes sizes[2];      // in row parts with floor(grid / P) blocks, and in those with one more
 };
 
+// Warps that rank, of `most` that can, where blocks have up to `columns`.  Those that neither rank nor stream make the reported list, and a
+// block of few columns has done the rest before three of them have.  Device time with 12 / 10 / 8 / 6 / 4, us:
+//    512 x 512 (4 columns), 50 % of the activations    -   /  -   / 3.41 / 3.35 / 3.37;  with two 3.32
+//   1024 x 1024 (14), 50 %                            3.25 /  -   / 3.24 / 3.24 / 3.24;  with two 3.28
+//    600 x 3000 (22), 30 %                            3.66 /  -   / 3.55 / 3.55 / 3.55
+//   2048 x 2048 (28), 50 %                            3.57 / 3.54 / 3.52 / 3.54 / 3.56
+//   2048 x 3000 (42), 30 %                            3.65 / 3.51 / 3.49 / 3.52 / 3.53
+//   1000 x 7000 (48), 10 %, 50 %                      3.79, 4.19 / 3.62, 4.21 / 3.61, 4.22 / 3.62, 4.22 / 3.62, 4.38
+//   4096 x 4096 (56), 10 %, 50 %                      3.83, 5.67 / 3.82, 5.66 / 3.83, 5.71 / 3.83, 5.93 / 3.84, 6.01
+//   3001 x 5003 (68), 10 %, 50 %                      4.19, 5.76 / 4.21, 5.87 / 4.20, 5.87 / 4.18, 5.97 / 4.26, 6.29
+// (Pairs stream with 16 warps whatever ranks: fewer rankers are no more list makers.)
+inline int direct_rankers(int columns, int pairs, int most)
+{
+    return pairs ? most : std::min({most, columns <= 64 ? 10 : most, 1 + columns / 4});
+}
+
 inline DirectGroups direct_groups(int64_t K, int grid, int P, int warps, bool wide)
 {
     DirectGroups g;

@@ -507,15 +507,16 @@ constexpr int kDirectMost = 128, kGroupsMost = 512, kMixesMost = 384, kBatchMost
 
 int direct_threads(int G, int pairs) { return 32 * (pairs ? 16 + kDirectHelpers + 1 : std::max(16, G + kDirectHelpers + 1)); }
 
-DirectGroups direct_groups(const celty_matrix *m, int grid, int P, int threads, bool wide)
+DirectGroups direct_groups(const celty_matrix *m, int grid, int P, int G, int pairs, bool wide)
 {
-    return celty::direct_groups(m->K, grid, P, threads / 32 - 1 - kDirectHelpers, wide);
+    const int most = direct_threads(G, pairs) / 32 - 1 - kDirectHelpers;
+    return celty::direct_groups(m->K, grid, P, direct_rankers(direct_columns(m->K, grid / P), pairs, most), wide);
 }
 
 // Columns that a team of k_spmspv_direct may get: of the block's, or of an even split of a list over the teams of a row part.
 int direct_cap(const celty_matrix *m, int grid, int P, int G, int pairs, bool list, bool wide)
 {
-    return list ? (int)(m->K / ((int64_t)(grid / P) * G) + 1) : (direct_groups(m, grid, P, direct_threads(G, pairs), wide).most + G - 1) / G;
+    return list ? (int)(m->K / ((int64_t)(grid / P) * G) + 1) : (direct_groups(m, grid, P, G, pairs, wide).most + G - 1) / G;
 }
 
 // Shape of the fused launch: P row parts of Sc slabs, G teams per slab (teams = G * Sc warps, one accumulator
@@ -623,7 +624,7 @@ int plan_fused(const celty_matrix *m, const LaunchKnobs &knobs, const DeviceInfo
     }
     if (pl.direct) {
         pl.cap = direct_cap(m, pl.grid, pl.P, pl.G, pl.pp, list, pl.wide);
-        if (!list) pl.groups = direct_groups(m, pl.grid, pl.P, pl.threads, pl.wide);
+        if (!list) pl.groups = direct_groups(m, pl.grid, pl.P, pl.G, pl.pp, pl.wide);
         pl.tables = direct_smem_layout(m->R, (int)m->K, pl.G, pl.D, pl.slot_bytes, pl.cap);
     }
     pl.merge = (knobs.merge >= 0 ? knobs.merge : 1);
