@@ -11,7 +11,7 @@ ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libcelty.so")
 SOURCES = [os.path.join(CSRC, "celty_host.cpp"), os.path.join(CSRC, "celty_upload.cpp"), os.path.join(CSRC, "celty_kernels.cu")]
-HEADERS = [os.path.join(CSRC, "celty_internal.h"), os.path.join(CSRC, "celty_upload.h"), os.path.join(CSRC, "celty_fused.cuh"), os.path.join(CSRC, "celty_direct.cuh"), os.path.join(CSRC, "celty_column.cuh"),
+HEADERS = [os.path.join(CSRC, "celty_internal.h"), os.path.join(CSRC, "celty_upload.h"), os.path.join(CSRC, "celty_signal.h"), os.path.join(CSRC, "celty_fused.cuh"), os.path.join(CSRC, "celty_direct.cuh"), os.path.join(CSRC, "celty_column.cuh"),
            os.path.join(ROOT, "include", "celty.h")]
 
 

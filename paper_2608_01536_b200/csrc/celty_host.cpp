@@ -2,13 +2,10 @@
 // host-side decoding for round-trip tests and byte accounting.  No CUDA calls in this file.
 #include <algorithm>
 #include <atomic>
-#include <chrono>
 #include <cmath>
-#include <condition_variable>
 #include <cstring>
 #include <exception>
 #include <memory>
-#include <mutex>
 #include <new>
 #include <thread>
 #ifdef __SSE2__
@@ -16,6 +13,7 @@
 #endif
 
 #include "celty_internal.h"
+#include "celty_signal.h"
 
 using namespace celty;
 
@@ -51,25 +49,14 @@ int64_t host_threads(int64_t n, bool worth_threads)
 }
 
 // Phases of work that several host threads go through together: work(phase, scratch) on each of them, then between(phase) on one
-// while the others wait.  The threads are started once (starting 15 takes 0.2 ms).  Who waits looks for kLook, about what it takes to
-// be woken, and sleeps from then on: the processors may be wanted by other work, another layer's encoding perhaps.  false = memory ran out
-// in one.
-constexpr std::chrono::microseconds kLook(50);
-
+// while the others wait.  The threads are started once (starting 15 takes 0.2 ms).  false = memory ran out in one.
 template <typename Work, typename Between>
 bool in_phases(int64_t want, int phases, Work work, Between between)
 {
     std::atomic<bool> failed(false);
     std::atomic<int64_t> arrived(0);
     std::atomic<int> open(0);                                     // the phase that may run
-    std::mutex mu;
-    std::condition_variable all_arrived, opened;
-    auto wait = [&](std::condition_variable &change, auto there) {
-        for (const auto until = std::chrono::steady_clock::now() + kLook; !there() && std::chrono::steady_clock::now() < until;) std::this_thread::yield();
-        if (there()) return;
-        std::unique_lock<std::mutex> lock(mu);
-        change.wait(lock, there);
-    };
+    Signal all_arrived, opened;
     auto phase = [&](int p, Scratch &scratch) {
         try {
             if (!failed) work(p, scratch);
@@ -84,11 +71,10 @@ bool in_phases(int64_t want, int phases, Work work, Between between)
             threads.emplace_back([&]() {
                 Scratch scratch;
                 for (int p = 0; p < phases; ++p) {
-                    wait(opened, [&] { return open >= p; });
+                    opened.wait([&] { return open >= p; });
                     phase(p, scratch);
-                    std::lock_guard<std::mutex> lock(mu);
                     ++arrived;
-                    all_arrived.notify_one();
+                    all_arrived.raise();
                 }
             });
     } catch (const std::exception &) {                            // no (more) threads to be had: those there are do it
@@ -96,15 +82,14 @@ bool in_phases(int64_t want, int phases, Work work, Between between)
     Scratch scratch;
     for (int p = 0; p < phases; ++p) {
         phase(p, scratch);
-        wait(all_arrived, [&] { return arrived >= (int64_t)threads.size() * (p + 1); });
+        all_arrived.wait([&] { return arrived >= (int64_t)threads.size() * (p + 1); });
         try {
             if (!failed) between(p);
         } catch (const std::exception &) {
             failed = true;
         }
-        std::lock_guard<std::mutex> lock(mu);
         open = p + 1;
-        opened.notify_all();
+        opened.raise();
     }
     for (std::thread &t : threads) t.join();
     return !failed;
