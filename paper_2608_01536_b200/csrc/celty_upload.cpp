@@ -7,7 +7,7 @@
 #include "celty_upload.h"
 
 #include <algorithm>
-#include <condition_variable>
+#include <atomic>
 #include <cstring>
 #include <exception>
 #include <mutex>
@@ -15,6 +15,7 @@
 #include <vector>
 
 #include "celty_internal.h"
+#include "celty_signal.h"
 
 namespace celty {
 
@@ -61,66 +62,61 @@ Staging &staging()
 // The pieces of an image on their way through the slots, piece i through slot i mod kUploadSlots.
 class Pieces {
 public:
-    Pieces(uint8_t *slots, const uint8_t *from, size_t bytes) : slots_(slots), from_(from), bytes_(bytes) {}
-    int64_t count() const { return (int64_t)((bytes_ + kUploadPiece - 1) / kUploadPiece); }
-    size_t size(int64_t i) const { return std::min(kUploadPiece, bytes_ - (size_t)i * kUploadPiece); }
+    Pieces(uint8_t *slots, const uint8_t *from, size_t bytes)
+        : slots_(slots), from_(from), bytes_(bytes), count_((int64_t)((bytes + kUploadPiece - 1) / kUploadPiece)) {}
+    int64_t count() const { return count_; }
     uint8_t *slot(int64_t i) const { return slots_ + (size_t)(i % kUploadSlots) * kUploadPiece; }
+    size_t size(int64_t i, int64_t n) const { return std::min((size_t)n * kUploadPiece, bytes_ - (size_t)i * kUploadPiece); }      // of n pieces from i on
+    bool filled(int64_t i) const { return filled_[i % kUploadSlots] == i + 1; }
 
     // A thread that fills slots: the next pieces, each as soon as its slot is free.
     void fill_all()
     {
-        std::unique_lock<std::mutex> lock(mu_);
-        while (!stopped_ && claimed_ < count()) {
-            const int64_t i = claimed_++;
-            changed_.wait(lock, [&] { return stopped_ || i < copied_ + kUploadSlots; });
-            if (stopped_) return;
-            fill(i, lock);
-        }
+        while (!stopped_ && claimed_ < count_)
+            if (!fill_next()) free_.wait([&] { return stopped_ || claimed_ >= count_ || claimed_ < copied_ + kUploadSlots; });
     }
 
     // Returns when piece i is there; fills others, or i itself, meanwhile.
     void wait_filled(int64_t i)
     {
-        std::unique_lock<std::mutex> lock(mu_);
-        while (filled_[i % kUploadSlots] != i + 1) {
-            if (claimed_ < std::min(count(), copied_ + kUploadSlots)) fill(claimed_++, lock);
-            else changed_.wait(lock);
-        }
+        while (!filled(i))
+            if (!fill_next()) there_.wait([&] { return filled(i); });
     }
 
     // The copies of the first n pieces have been made: their slots are free.
     void copied(int64_t n)
     {
-        std::lock_guard<std::mutex> lock(mu_);
         copied_ = n;
-        changed_.notify_all();
+        free_.raise();
     }
 
     void stop()
     {
-        std::lock_guard<std::mutex> lock(mu_);
         stopped_ = true;
-        changed_.notify_all();
+        free_.raise();
     }
 
 private:
-    void fill(int64_t i, std::unique_lock<std::mutex> &lock)
+    bool fill_next()                                              // false: no piece whose slot is free is left
     {
-        lock.unlock();
-        std::memcpy(slot(i), from_ + (size_t)i * kUploadPiece, size(i));
-        lock.lock();
+        int64_t i = claimed_;
+        do {
+            if (i >= std::min<int64_t>(count_, copied_ + kUploadSlots)) return false;
+        } while (!claimed_.compare_exchange_weak(i, i + 1));
+        std::memcpy(slot(i), from_ + (size_t)i * kUploadPiece, size(i, 1));
         filled_[i % kUploadSlots] = i + 1;
-        changed_.notify_all();
+        there_.raise();
+        return true;
     }
 
     uint8_t *const slots_;
     const uint8_t *const from_;
     const size_t bytes_;
-    std::mutex mu_;
-    std::condition_variable changed_;
-    int64_t claimed_ = 0, copied_ = 0;
-    int64_t filled_[kUploadSlots] = {};                           // i + 1 when piece i is there
-    bool stopped_ = false;
+    const int64_t count_;
+    std::atomic<int64_t> claimed_{0}, copied_{0};
+    std::atomic<int64_t> filled_[kUploadSlots] = {};              // i + 1 when piece i is there
+    std::atomic<bool> stopped_{false};
+    Signal there_, free_;
 };
 
 }  // namespace
@@ -153,31 +149,34 @@ cudaError_t upload(void *to, const uint8_t *from, size_t bytes, void *clear, siz
         for (int64_t t = 1; t < want; ++t) threads.emplace_back([&] { pieces.fill_all(); });
     } catch (const std::exception &) {                            // no (more) threads to be had: those there are do it
     }
-    cudaEvent_t done[kUploadSlots] = {};                          // of a slot's last copy
-    cudaEvent_t last = nullptr;
-    for (int64_t i = 0, made = 0; i < pieces.count(); ++i) {
-        for (; made < i; ++made) {
-            const cudaEvent_t e = done[made % kUploadSlots];
-            err = i - made == kUploadSlots ? cudaEventSynchronize(e) : cudaEventQuery(e);
+    // The pieces that are there are copied together, up to the end of their quarter of the slots, and a quarter is free again behind its event.
+    constexpr int quarter = kUploadSlots / 4;
+    cudaEvent_t done[4] = {};
+    int64_t made = 0, recorded = 0;                               // quarters copied, quarters with an event behind them
+    for (int64_t i = 0, n; i < pieces.count(); i += n) {
+        for (; made < recorded; ++made) {
+            const cudaEvent_t e = done[made % 4];
+            err = i == (made + 4) * quarter ? cudaEventSynchronize(e) : cudaEventQuery(e);
             if (err != cudaSuccess) break;
         }
         if (err == cudaErrorNotReady) (void)cudaGetLastError();
         else if (err != cudaSuccess) break;
-        pieces.copied(made);
+        pieces.copied(made * quarter);
         pieces.wait_filled(i);
-        cudaEvent_t &e = done[i % kUploadSlots];
-        if (!e && (err = cudaEventCreateWithFlags(&e, cudaEventDisableTiming)) != cudaSuccess) break;
-        err = cudaMemcpyAsync(static_cast<uint8_t *>(to) + (size_t)i * kUploadPiece, pieces.slot(i), pieces.size(i), cudaMemcpyHostToDevice, st);
-        if (err == cudaSuccess) err = cudaEventRecord(e, st);
+        const int64_t end = std::min(pieces.count(), (i / quarter + 1) * quarter);
+        for (n = 1; i + n < end && pieces.filled(i + n); ++n) {}
+        err = cudaMemcpyAsync(static_cast<uint8_t *>(to) + (size_t)i * kUploadPiece, pieces.slot(i), pieces.size(i, n), cudaMemcpyHostToDevice, st);
         if (err != cudaSuccess) break;
-        last = e;
+        if (i + n < end) continue;
+        cudaEvent_t &e = done[recorded % 4];
+        if (!e && (err = cudaEventCreateWithFlags(&e, cudaEventDisableTiming)) != cudaSuccess) break;
+        if ((err = cudaEventRecord(e, st)) != cudaSuccess) break;
+        ++recorded;
     }
     pieces.stop();
     for (std::thread &t : threads) t.join();
-    if (last) {
-        const cudaError_t waited = cudaEventSynchronize(last);
-        if (err == cudaSuccess) err = waited;
-    }
+    if (err == cudaSuccess) err = cudaEventSynchronize(done[(recorded - 1) % 4]);
+    else (void)cudaStreamSynchronize(st);                         // (there may be copies without an event)
     for (cudaEvent_t e : done)
         if (e) cudaEventDestroy(e);
     return err;

@@ -111,6 +111,7 @@ cudaError_t cudaEventSynchronize(cudaEvent_t e)
     if (!ev->ready) drain(ev->queue, ev);
     return cudaSuccess;
 }
+cudaError_t cudaStreamSynchronize(cudaStream_t st) { CALL; drain(queue_of(st), nullptr); return cudaSuccess; }
 cudaError_t cudaMemsetAsync(void *p, int c, size_t n, cudaStream_t st) { CALL; queues[queue_of(st)].push_back(Op{p, nullptr, n, std::vector<uint8_t>(n, (uint8_t)c), nullptr}); return cudaSuccess; }
 cudaError_t cudaMemcpyAsync(void *to, const void *from, size_t n, cudaMemcpyKind, cudaStream_t st)
 {
@@ -211,7 +212,7 @@ def program(tmp_path_factory):
 
 # handles 1 and 2 are cudaStreamLegacy and cudaStreamPerThread; sizes around the pieces of 512 KB, and beyond all slots
 @pytest.mark.parametrize("stream", [0, 1, 2, 4096])
-@pytest.mark.parametrize("size", [1000, (512 << 10) - 1, 512 << 10, (1536 << 10) + 1, (8 << 20) + 5, 20 << 20])
+@pytest.mark.parametrize("size", [1000, (512 << 10) - 1, 512 << 10, (1536 << 10) + 1, 2 << 20, (8 << 20) - 1, (8 << 20) + 5, 20 << 20])
 def test_an_upload_is_work_of_the_callers_stream(program, stream, size):
     program("ordered", stream, size)
 
