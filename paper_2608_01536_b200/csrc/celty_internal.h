@@ -74,7 +74,6 @@ public:
         if (align == huge) (void)madvise(p_.get(), round_up(bytes, huge), MADV_HUGEPAGE);
 #endif
     }
-    void reset() { p_.reset(); n_ = 0; }
     T *data() { return p_.get(); }
     const T *data() const { return p_.get(); }
     T &operator[](size_t i) { return p_.get()[i]; }

@@ -14,7 +14,8 @@
 #include <thread>
 #include <vector>
 
-#include "celty_internal.h"
+#include <sys/mman.h>
+
 #include "celty_signal.h"
 
 namespace celty {
@@ -32,22 +33,24 @@ struct RelaxedCapture {
 };
 
 // Ordinary memory that is registered: cudaDeviceReset, or the end of the context that was current, ends the registration and not the memory.
+// (Not of the heap, whose largest blocks it would lie between.)
 struct Staging {
+    static constexpr size_t bytes = kUploadSlots * kUploadPiece;
     std::mutex mu;
-    Raw<uint8_t> memory;
+    uint8_t *memory = nullptr;
 
     // The slots, page-locked; null: not to be had (mu is held).
     uint8_t *slots()
     {
-        try {
-            if (memory.size() == 0) memory.allocate(kUploadSlots * kUploadPiece);
-        } catch (const std::exception &) {
-            return nullptr;
+        if (!memory) {
+            void *const m = mmap(nullptr, bytes, PROT_READ | PROT_WRITE, MAP_PRIVATE | MAP_ANONYMOUS, -1, 0);
+            if (m == MAP_FAILED) return nullptr;
+            memory = static_cast<uint8_t *>(m);
         }
         cudaPointerAttributes is{};
-        if (cudaPointerGetAttributes(&is, memory.data()) == cudaSuccess && is.type == cudaMemoryTypeHost) return memory.data();
+        if (cudaPointerGetAttributes(&is, memory) == cudaSuccess && is.type == cudaMemoryTypeHost) return memory;
         (void)cudaGetLastError();
-        if (cudaHostRegister(memory.data(), memory.size(), cudaHostRegisterPortable) == cudaSuccess) return memory.data();
+        if (cudaHostRegister(memory, bytes, cudaHostRegisterPortable) == cudaSuccess) return memory;
         (void)cudaGetLastError();
         return nullptr;
     }
@@ -138,9 +141,10 @@ cudaError_t upload(void *to, const uint8_t *from, size_t bytes, void *clear, siz
         staged = false;
     }
     uint8_t *const slots = staged ? stage.slots() : nullptr;
-    // (first, and waited for with the copies: the next layer's upload finds the stream idle)
-    if ((err = cudaMemsetAsync(clear, 0, clear_bytes, st)) != cudaSuccess) return err;
-    if (!slots) return cudaMemcpyAsync(to, from, bytes, cudaMemcpyHostToDevice, st);
+    if (!slots) {
+        err = cudaMemcpyAsync(to, from, bytes, cudaMemcpyHostToDevice, st);
+        return err == cudaSuccess ? cudaMemsetAsync(clear, 0, clear_bytes, st) : err;
+    }
     Pieces pieces(slots, from, bytes);
     std::vector<std::thread> threads;
     try {
@@ -175,7 +179,9 @@ cudaError_t upload(void *to, const uint8_t *from, size_t bytes, void *clear, siz
     }
     pieces.stop();
     for (std::thread &t : threads) t.join();
-    if (err == cudaSuccess) err = cudaEventSynchronize(done[(recorded - 1) % 4]);
+    // (the clearing is waited for as well: the next layer's upload finds the stream idle)
+    if (err == cudaSuccess && (err = cudaMemsetAsync(clear, 0, clear_bytes, st)) == cudaSuccess) err = cudaEventRecord(done[0], st);
+    if (err == cudaSuccess) err = cudaEventSynchronize(done[0]);
     else (void)cudaStreamSynchronize(st);                         // (there may be copies without an event)
     for (cudaEvent_t e : done)
         if (e) cudaEventDestroy(e);
@@ -187,14 +193,16 @@ cudaError_t release_staging()
     RelaxedCapture relaxed;
     Staging &stage = staging();
     std::lock_guard<std::mutex> lock(stage.mu);
-    if (stage.memory.size() == 0) return cudaSuccess;
-    cudaError_t err = cudaHostUnregister(stage.memory.data());
+    if (!stage.memory) return cudaSuccess;
+    cudaError_t err = cudaHostUnregister(stage.memory);
     if (err == cudaErrorHostMemoryNotRegistered) {
         (void)cudaGetLastError();
         err = cudaSuccess;
     }
-    if (err == cudaSuccess) stage.memory.reset();
-    return err;
+    if (err != cudaSuccess) return err;
+    munmap(stage.memory, Staging::bytes);
+    stage.memory = nullptr;
+    return cudaSuccess;
 }
 
 }  // namespace celty
