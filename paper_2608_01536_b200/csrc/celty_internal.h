@@ -235,10 +235,11 @@ struct DirectGroups {
 //   1000 x 7000 (48), 10 %, 50 %                      3.79, 4.19 / 3.62, 4.21 / 3.61, 4.22 / 3.62, 4.22 / 3.62, 4.38
 //   4096 x 4096 (56), 10 %, 50 %                      3.83, 5.67 / 3.82, 5.66 / 3.83, 5.71 / 3.83, 5.93 / 3.84, 6.01
 //   3001 x 5003 (68), 10 %, 50 %                      4.19, 5.76 / 4.21, 5.87 / 4.20, 5.87 / 4.18, 5.97 / 4.26, 6.29
-// (Pairs stream with 16 warps whatever ranks: fewer rankers are no more list makers.)
+// (In two runs 4096 x 4096 with a magnitude mask took 5.71 and 5.81 with ten and 5.71 with twelve, so that the line lies at 48.  Pairs stream
+// with 16 warps whatever ranks: fewer rankers are no more list makers.)
 inline int direct_rankers(int columns, int pairs, int most)
 {
-    return pairs ? most : std::min({most, columns <= 64 ? 10 : most, 1 + columns / 4});
+    return pairs ? most : std::min({most, columns <= 48 ? 10 : most, 1 + columns / 4});
 }
 
 inline DirectGroups direct_groups(int64_t K, int grid, int P, int warps, bool wide)

@@ -48,7 +48,7 @@ int main(int, char **v) {
         out = subprocess.check_output([exe, str(K), str(grid), str(P), str(part), str(warps)], input=keep.astype(np.uint8).tobytes())
         rows = np.array(out.split(), dtype=np.int64).reshape(-1, 2)
         most, rankers = rows[0]
-        assert 1 <= rankers <= warps - (2 if warps == 12 and K <= 62 * (grid // P) else 0)      # the others make the list
+        assert 1 <= rankers <= warps - (2 if warps == 12 and K <= 46 * (grid // P) else 0)      # the others make the list
         taken = rows[1:]
         assert np.array_equal(np.sort(taken[:, 0]), np.flatnonzero(keep))      # every survivor once, and nothing else
         return taken[:, 1], most
