@@ -17,7 +17,7 @@
 //
 // What is left of imbalance is the difference between groups.  Device time with 50 % of the weights, in us, k_spmspv_fused / blocks with columns of their
 // own / this kernel, by columns per block (mean of 6 draws; the first figure of 16):
-//    14 (1024 x 1024, d = 0.5)              3.80 / 3.29 / 3.30
+//    14 (1024 x 1024, d = 0.5)              3.80 / 3.20 / 3.22
 //    56 (4096 x 4096, 0.1 / 0.5 / 0.7)      4.82 / 3.94 / 3.86, 7.79 / 6.24 / 5.80, 8.65 / 7.82 / 7.27
 //    70 (5120 x 5120, 0.4)                  7.38 -> 6.58
 //    75 (4096 x 11008, 0.5)                 12.26 / 11.80 / 10.91
@@ -61,7 +61,7 @@ constexpr int kDirectThreads = 32 * (16 + kDirectHelpers + 1);
 // (DirectParams::ldx); kHeld: columns of the group per ranking lane; 0: the survivors come as a list (DirectParams::list), in
 // equal shares for all teams.
 template <bool kPairs, bool kBatch, int kHeld>
-__global__ void __launch_bounds__(kDirectThreads, 1) k_spmspv_direct(const DirectParams p)
+__device__ __forceinline__ void dealt_product(const DirectParams p)
 {
     constexpr bool kList = kHeld == 0;
     constexpr int kArray = kList ? 1 : kHeld;
@@ -378,4 +378,11 @@ __global__ void __launch_bounds__(kDirectThreads, 1) k_spmspv_direct(const Direc
     }
     asm volatile("cp.async.bulk.commit_group;" ::: "memory");
     asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");   // shared memory may go once it has been read
+}
+
+// (The same body in the kernel itself compiles to slower code: 11008 x 4096 with its FP16 copy 10.55 us instead of 10.51.)
+template <bool kPairs, bool kBatch, int kHeld>
+__global__ void __launch_bounds__(kDirectThreads, 1) k_spmspv_direct(const DirectParams p)
+{
+    dealt_product<kPairs, kBatch, kHeld>(p);
 }
