@@ -424,7 +424,8 @@ int celty_last_status(celty_matrix *m, celty_stream_t stream);
  *            builds without the other options' code (same results; the smaller builds are faster).  With 128 or 256 the
  *            blocks always share a ranked list of the survivors; by default a layer of at most 512 columns per block (384
  *            where blocks left over can be shared, 20 000 / tile rows in a batch) has its columns dealt to groups of blocks
- *            whatever x is, in runs of two, and the blocks of a group share its survivors.  That takes 1 to 25 % less time.
+ *            whatever x is, in runs of two, and the blocks of a group share its survivors.  That takes up to 25 % less time, and about as
+ *            long near those lines.
  *   groups   fused kernel: warp teams per slab working on different columns (each has an accumulator)
  *   depth    fused kernel: bulk copies each team keeps in flight (ring slots)
  *   cluster  fused kernel, bulk reduce-add merge: thread blocks per cluster (1, 2 or 4); the blocks of a

@@ -342,7 +342,7 @@ void choose_shape(int64_t M, int64_t K, double density, int tile_rows, int64_t *
         // sub-blocks of half the size.  Measured at 4096 x 4096: 8.3 us against 8.8; at 4096 x 11008, where a team
         // has five sub-blocks to stream, no gain, so the rule stops short of it.
         if (S == 1 && Q >= 32 && K <= 6144) S = 2;
-        // (Taller layers of few columns would gain from slabs of 2048 rows in calls for one vector, 7 to 17 % at 10 % of the
+        // (Taller layers of few columns would gain from slabs of 2048 rows in calls for one vector, 6 to 17 % at 10 % of the
         // activations and up to 7 at 50, and lose more in batches, whose blocks have N times the columns; the image is the same for both.
         // Slabs of 4096 -> of 2048 rows, us, one vector at 10 / 50 %, N = 4, 8 at 50 %:  8192 x 2048 4.66 / 5.94, 12.7, 22.0 -> 3.92 /
         // 6.07, 13.5, 27.2;  5504 x 2048 4.24 / 5.03, 9.3, 16.5 -> 3.87 / 4.99, 10.6, 19.2;  20000 x 800 4.71 / 6.06, 12.6, 24.9 -> 3.93 /

@@ -3,7 +3,8 @@
 // from there.  It alone makes CUDA calls: a stream handle may mean another stream in another thread (cudaStreamPerThread), and the
 // caller's context need not be the one that cudaSetDevice would make current.  The 8 MB are taken by the first upload, used by one upload at a
 // time and given back by celty_release_staging.  An upload ends when its copies have left the slots, so that it waits for no other stream's
-// work, nor leaves events for another context.
+// work, nor leaves events for another context.  celty_bind_device with a new image, from pageable memory / this way: 6.3 MB 1.5 / 1.1 ms, 12.6 MB
+// 2.5 / 1.2, 57 MB 6.5 / 2.6, 171 MB 16.5 / 6.3.  Bound by the threads' start, then by their copies.
 #include "celty_upload.h"
 
 #include <algorithm>
