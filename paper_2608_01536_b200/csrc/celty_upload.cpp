@@ -13,6 +13,7 @@
 #include <exception>
 #include <mutex>
 #include <thread>
+#include <type_traits>
 #include <vector>
 
 #include <sys/mman.h>
@@ -57,11 +58,8 @@ struct Staging {
     }
 };
 
-Staging &staging()
-{
-    static Staging *s = new Staging;                              // (never destroyed: the runtime may be gone by then)
-    return *s;
-}
+Staging stage;
+static_assert(std::is_trivially_destructible<Staging>::value, "at the process's end the runtime may be gone");
 
 // The pieces of an image on their way through the slots, piece i through slot i mod kUploadSlots.
 class Pieces {
@@ -133,7 +131,6 @@ cudaError_t upload(void *to, const uint8_t *from, size_t bytes, void *clear, siz
     cudaError_t err = cudaStreamIsCapturing(st, &capturing);
     if (err != cudaSuccess) return err;
     RelaxedCapture relaxed;
-    Staging &stage = staging();
     std::unique_lock<std::mutex> lock(stage.mu, std::defer_lock);
     bool staged = capturing == cudaStreamCaptureStatusNone && bytes >= kUploadPiece && lock.try_lock();
     if (staged && cudaStreamQuery(st) != cudaSuccess) {
@@ -192,7 +189,6 @@ cudaError_t upload(void *to, const uint8_t *from, size_t bytes, void *clear, siz
 cudaError_t release_staging()
 {
     RelaxedCapture relaxed;
-    Staging &stage = staging();
     std::lock_guard<std::mutex> lock(stage.mu);
     if (!stage.memory) return cudaSuccess;
     cudaError_t err = cudaHostUnregister(stage.memory);

@@ -108,3 +108,21 @@ def test_an_upload_on_the_threads_own_stream():
     stream.synchronize()
     for k in range(6):
         assert np.array_equal(read[k].numpy(), ms[k % 2].host_image()[0]), k
+
+
+@pytest.mark.parametrize("size", [2 * PIECE, 20 * PIECE])
+def test_an_upload_behind_work_of_its_stream(size):
+    """The image of before is read by work that the stream has yet to do when the next one is bound to the same memory."""
+    a, b = _matrix(size, 1), _matrix(size, 2)
+    assert a.device_bytes() == b.device_bytes()
+    image, ws = [torch.empty(n, dtype=torch.uint8, device="cuda") for n in a.device_bytes()]
+    torch.cuda.synchronize()
+    stream, read = torch.cuda.Stream(), []
+    with torch.cuda.stream(stream):
+        for m in (a, b, a):
+            celty._check(celty.load().celty_bind_device(m._h, image.data_ptr(), image.numel(), ws.data_ptr(), ws.numel(), stream.cuda_stream), "celty_bind_device")
+            torch.cuda._sleep(20_000_000)                         # some 10 ms
+            read.append(image.clone())
+    stream.synchronize()
+    for m, r in zip((a, b, a), read):
+        assert np.array_equal(r.cpu().numpy(), m.host_image()[0])
